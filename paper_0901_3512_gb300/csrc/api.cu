@@ -113,6 +113,8 @@ seedcg_status seedcg_create(seedcg_handle** out, const int dims[4], const double
             src = tmp.as<double>();
         }
         seedcg::gauge_to_internal(src, h->u64.as<double2>(), h->u32.as<float2>(), (int)vol, 0);
+        h->fix.ensure(nl * sizeof(int4));
+        seedcg::fix_links(h->g, h->u64.as<double2>(), kappa, h->fix.as<int4>(), &h->fix_k, &h->fix_ok, 0);
         SEEDCG_CUDA_TRY(cudaDeviceSynchronize());
         tmp.release();
     } catch (const Error& e) {
@@ -267,11 +269,7 @@ seedcg_status seedcg_apply(seedcg_handle* h, int op, int prec, int multi, int n,
         if (prec == 0) {
             seedcg::to_internal_f64(in, (double2*)A, vol, n, st);
             auto apply = [&](int dag, const double2* x, double2* y) {
-                if (multi) seedcg::dslash_mrhs_f64(h->g, h->u64.as<double2>(), h->kappa, dag, n, x, y, st);
-                else
-                    for (int r = 0; r < n; r++)
-                        seedcg::dslash_f64(h->g, h->u64.as<double2>(), h->kappa, dag,
-                                           x + (size_t)r * 12 * vol, y + (size_t)r * 12 * vol, st);
+                seedcg::dslash_f64(seedcg::fix_of(h), dag, n, x, y, st);   // one kernel for any n
             };
             const double2* res = nullptr;
             if (op == 0) { apply(0, (double2*)A, (double2*)Bv); res = (double2*)Bv; }
@@ -526,8 +524,7 @@ seedcg_status seedcg_time_dslash(seedcg_handle* h, int prec, int n, int reps, in
             if (flush_l2) SEEDCG_CUDA_TRY(cudaMemsetAsync(flush.p, r & 0xff, fbytes, st));
             SEEDCG_CUDA_TRY(cudaEventRecord(e0, st));
             if (prec == 0)
-                seedcg::dslash_mrhs_f64(h->g, h->u64.as<double2>(), h->kappa, 0, n,
-                                        (const double2*)b0, (double2*)(b0 + nf * esz), st);
+                seedcg::dslash_f64(seedcg::fix_of(h), 0, n, (const double2*)b0, (double2*)(b0 + nf * esz), st);
             else
                 seedcg::dslash_mrhs_f32(h->g, h->u32.as<float2>(), (float)h->kappa, 0, n,
                                         (const float2*)b0, (float2*)(b0 + nf * esz), st);
@@ -562,6 +559,7 @@ void seedcg_destroy(seedcg_handle* h) {
     cudaSetDevice(h->device);
     h->u64.release();
     h->u32.release();
+    h->fix.release();
     h->vbasis.release();
     h->lz_scalars.release();
     h->red.release();

@@ -28,6 +28,7 @@
 
 #include "cg_batch.cuh"
 #include "eo.cuh"
+#include "fixhop.cuh"
 #include "kernels.cuh"
 #include "reduce.cuh"
 #include "wilson.cuh"
@@ -65,6 +66,7 @@ struct GroupDev {
     int ntiles;         // tiles of 32 (half-)sites; every share is one warp's sum
     int tile0;          // first tile of this group in the dslash grid
     Brk b64, b128;      // brick tilings of 64 and 128 sites (single-field full-lattice batches)
+    FixDev fix;         // the FP64 operator's links
 };
 
 struct Rows {
@@ -361,6 +363,76 @@ k_mf_brick(const GroupDev<R>* __restrict__ G, Rows rows, CgS C) {
         }
         put_share(DAG ? gd.part2 : gd.part, gd.ntiles, r, tile32, dr);
     }
+}
+
+// 1/3 in FP64, in fixed point (fixhop.cuh), over the tiles of every field: full lattice STAGE 0 and 3
+// (t = D p; D^dag t), even-odd STAGE 0..3 as in k_mf_eo.  The epilogues are those of the FP32 kernels.
+struct MfFixEpi {
+    static constexpr bool kShare = true;
+    double2* out;         // stored field (null in the last stage)
+    double2* r;           // last stage: r -= alpha val
+    const double* alpha;  // of this group's slot 0
+    double* shares;       // null: none
+    long stride;
+    int ntiles, tile, vo;
+    __device__ __forceinline__ double operator()(int q, int plane, int idx, int, bool live, double2 a, double2 b) {
+        if (!live) return 0.0;
+        const size_t ix = (size_t)q * stride + ((size_t)plane * vo + idx) * 2;
+        if (r) {
+            const double al = alpha[q];
+            const double2 ra = r[ix], rb = r[ix + 1];
+            a = make_double2(ra.x - al * a.x, ra.y - al * a.y);
+            b = make_double2(rb.x - al * b.x, rb.y - al * b.y);
+            r[ix] = a;
+            r[ix + 1] = b;
+        } else {
+            out[ix] = a;
+            out[ix + 1] = b;
+        }
+        return shares ? a.x * a.x + a.y * a.y + (b.x * b.x + b.y * b.y) : 0.0;
+    }
+    __device__ __forceinline__ void put(int q, double v) {
+        if (shares) shares[(size_t)q * ntiles + tile] = v;
+    }
+};
+
+template <int EO, int STAGE>
+__global__ void __launch_bounds__(kFixThreads, 2)
+k_mf_fix(const GroupDev<double>* __restrict__ G, int ng, Rows rows, CgS C) {
+    extern __shared__ __align__(16) unsigned char fix_smem[];
+    int f = 0;
+    while (f + 1 < ng && (int)blockIdx.x >= G[f + 1].tile0) f++;
+    const GroupDev<double>& gd = G[f];
+    const int nsys = rows.nact[f];
+    if ((int)blockIdx.y >= nsys) return;
+    const int tile = blockIdx.x - gd.tile0;
+    const double2* in = STAGE == 0 ? gd.p : (EO && STAGE != 2) ? gd.e : gd.t;
+    FixOp op{STAGE >= 2 ? 1 : 0, EO ? (STAGE & 1) : -1, in, gd.n, EO, 1, 1, nullptr, gd.n, EO};
+    if (EO) {
+        op.diag = STAGE & 1;
+        op.hsgn = (STAGE & 1) ? -1 : 1;
+        op.same = STAGE == 1 ? gd.p : gd.t;
+    } else {
+        op.same = in;
+    }
+    MfFixEpi epi{EO && !(STAGE & 1) ? gd.e : gd.t,
+                 STAGE == 3 ? gd.r : nullptr,
+                 C.alpha + rows.first[f],
+                 STAGE == 3 ? gd.part2 : (STAGE == 1 || !EO) ? gd.part : nullptr,
+                 gd.n,
+                 gd.ntiles,
+                 tile,
+                 EO ? gd.g.vol / 2 : gd.g.vol};
+    fix_tile(gd.fix, op, tile, blockIdx.y, nsys, gridDim.y, fix_smem, epi);
+}
+
+template <int EO, int STAGE>
+void mf_fix(int tiles, int gy, cudaStream_t s, const GroupDev<double>* gdev, int ng, Rows rows, const CgS& C) {
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_mf_fix<EO, STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
+    SEEDCG_CUDA_TRY(attr);
+    k_mf_fix<EO, STAGE><<<dim3(tiles, gy), kFixThreads, kFixSmem, s>>>(gdev, ng, rows, C);
+    SEEDCG_CHECK_LAUNCH();
 }
 
 // a row's shares, summed in a fixed order (one block per row); four independent
@@ -665,7 +737,20 @@ void launch_op(bool eo, int code, int tiles, const Brk& b64, const Brk& b128, cu
         k_mf_alpha<R><<<C.rows_cap, 256, 0, s>>>(gdev, rows, C);
         SEEDCG_CHECK_LAUNCH();
     };
-    if (eo) {
+    if constexpr (sizeof(R) == 8) {
+        // code = the grid rows (systems side by side)
+        if (eo) {
+            mf_fix<1, 0>(tiles, code, s, gdev, ng, rows, C);
+            mf_fix<1, 1>(tiles, code, s, gdev, ng, rows, C);
+            alpha();
+            mf_fix<1, 2>(tiles, code, s, gdev, ng, rows, C);
+            mf_fix<1, 3>(tiles, code, s, gdev, ng, rows, C);
+        } else {
+            mf_fix<0, 0>(tiles, code, s, gdev, ng, rows, C);
+            alpha();
+            mf_fix<0, 3>(tiles, code, s, gdev, ng, rows, C);
+        }
+    } else if (eo) {
         for (int stage = 0; stage < 2; stage++) launch_mf_eo<R>(code, stage, tiles, s, gdev, ng, rows, C);
         alpha();
         for (int stage = 2; stage < 4; stage++) launch_mf_eo<R>(code, stage, tiles, s, gdev, ng, rows, C);
@@ -871,6 +956,7 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
         gd[f].g = h->g;
         gd[f].u = fp64 ? reinterpret_cast<const cx_t<R>*>(h->u64.p) : reinterpret_cast<const cx_t<R>*>(h->u32.p);
         gd[f].kappa = (R)h->kappa;
+        gd[f].fix = fix_of(h);
         gd[f].n = n;
         gd[f].eo = eo ? 1 : 0;
         gd[f].xr = cv.take<cx_t<R>>((size_t)ns * n);
@@ -1003,11 +1089,10 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
             k_mf_ru_flush<R><<<gr, kRedThreads, 0, st>>>(ru_slot, ru_sys, gd[f].xr, groups[f].x64, Gx[f], n);
             SEEDCG_CHECK_LAUNCH();
             if (eo) {
-                eo_apply_mdag_m_f64(h->g, h->u64.as<double2>(), h->kappa, nf, Gx[f], T64[f], T64[f] + n,
-                                    MX[f], st);
+                eo_apply_mdag_m_f64(fix_of(h), nf, Gx[f], T64[f], MX[f], st);
             } else {
-                dslash_mrhs_f64(h->g, h->u64.as<double2>(), h->kappa, 0, nf, Gx[f], T64[f], st);
-                dslash_mrhs_f64(h->g, h->u64.as<double2>(), h->kappa, 1, nf, T64[f], MX[f], st);
+                dslash_f64(fix_of(h), 0, nf, Gx[f], T64[f], st);
+                dslash_f64(fix_of(h), 1, nf, T64[f], MX[f], st);
             }
             k_mf_ru_resid<R><<<gr, kRedThreads, 0, st>>>(ru_row, ru_slot, ru_sys, groups[f].b64, MX[f],
                                                          gd[f].r, n, C, trd, C.partials, C.counters);
@@ -1089,7 +1174,10 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
     // ---- the iteration chunk (graph-captured) ----
     const int gx = rblocks;
     const Brk b64 = gd[0].b64, b128 = gd[0].b128;
-    const int rpb = nrows > 0 ? autotune_rpb<R>(groups, tiles, b64, b128, gdev, ng, rows, C, st) : 8;
+    // FP64: one kernel, its grid rows by a rule; FP32: the autotuner's choice
+    int rpb = 8;
+    if constexpr (sizeof(R) == 8) rpb = fix_grid_y(tiles, nsys_max);
+    else if (nrows > 0) rpb = autotune_rpb<R>(groups, tiles, b64, b128, gdev, ng, rows, C, st);
     out.rpb = rpb;
     auto chunk = [&](cudaStream_t s) {
         for (int it = 0; it < poll; it++) {

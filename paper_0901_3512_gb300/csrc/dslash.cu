@@ -1,4 +1,4 @@
-// Wilson dslash kernels (single- and multi-right-hand-side, FP64 and FP32)
+// FP32 Wilson dslash kernels (single- and multi-right-hand-side; FP64: fixed.cu)
 // and the layout transforms between the boundary's complex128 AoS and the
 // internal site-fastest layouts.
 #include <algorithm>
@@ -443,26 +443,13 @@ void gauge_to_internal(const double* in, double2* u64, float2* u32, int vol, cud
     SEEDCG_CHECK_LAUNCH();
 }
 
-void dslash_f64(const Geom& g, const double2* u, double kappa, int dag, const double2* in,
-                double2* out, cudaStream_t s) {
-    launch_dslash<double>(g, u, kappa, dag, in, out, s);
-}
 void dslash_f32(const Geom& g, const float2* u, float kappa, int dag, const float2* in,
                 float2* out, cudaStream_t s) {
     launch_dslash<float>(g, u, kappa, dag, in, out, s);
 }
-void dslash_mrhs_f64(const Geom& g, const double2* u, double kappa, int dag, int n,
-                     const double2* in, double2* out, cudaStream_t s) {
-    launch_dslash_mrhs<double>(g, u, kappa, dag, n, in, out, s);
-}
 void dslash_mrhs_f32(const Geom& g, const float2* u, float kappa, int dag, int n,
                      const float2* in, float2* out, cudaStream_t s) {
     launch_dslash_mrhs<float>(g, u, kappa, dag, n, in, out, s);
-}
-void dslash_mrhs_fixed_f64(const Geom& g, const double2* u, double kappa, int dag, int n,
-                           const double2* in, double2* out, cudaStream_t s) {
-    const BrickChoice c{128, 0};
-    launch_dslash_mrhs<double>(g, u, kappa, dag, n, in, out, s, &c);
 }
 void dslash_mrhs_fixed_f32(const Geom& g, const float2* u, float kappa, int dag, int n,
                            const float2* in, float2* out, cudaStream_t s) {

@@ -39,22 +39,6 @@ k_eo_hop(Geom g, const cx_t<R>* __restrict__ u, int p_out, const cx_t<R>* __rest
     store_spinor(out, vh, h, acc);
 }
 
-// half[h] = full at the parity-p site of h (scatter = 0) or the reverse (scatter = 1)
-template <typename T>
-__global__ void k_eo_move(Geom g, int p, int scatter, T* __restrict__ full, T* __restrict__ half) {
-    const int vh = g.vol / 2;
-    const int h = blockIdx.x * blockDim.x + threadIdx.x;
-    if (h >= vh) return;
-    const int s = eo_site(g, h, p);
-#pragma unroll
-    for (int k = 0; k < 12; k++) {
-        if (scatter)
-            full[sidx(k, s, g.vol)] = half[sidx(k, h, vh)];
-        else
-            half[sidx(k, h, vh)] = full[sidx(k, s, g.vol)];
-    }
-}
-
 inline int eo_blocks(const Geom& g) { return (g.vol / 2 + 127) / 128; }
 
 template <typename R>
@@ -77,54 +61,6 @@ void apply_a(const Geom& g, const cx_t<R>* u, double kappa, int dag, const cx_t<
 
 }  // namespace
 
-// out_r = A^dag A x_r for n FP64 half vectors (te: one even half vector, y: one odd)
-void eo_apply_mdag_m_f64(const Geom& g, const double2* u, double kappa, int n, const double2* x,
-                         double2* te, double2* y, double2* out, cudaStream_t st) {
-    const size_t hf = (size_t)g.vol / 2 * 12;
-    for (int r = 0; r < n; r++) {
-        apply_a<double>(g, u, kappa, 0, x + r * hf, te, y, st);
-        apply_a<double>(g, u, kappa, 1, y, te, out + r * hf, st);
-    }
-}
-
-// phi = eta_o + kappa H_oe eta_e and b = A^dag phi for n full FP64 fields
-// (internal layout); phi, b: half vectors; ee, eo, te: half scratch
-void eo_rhs_f64(const Geom& g, const double2* u, double kappa, int n, const double2* eta, double2* phi,
-                double2* b, double2* ee, double2* eo, double2* te, cudaStream_t st) {
-    const size_t hf = (size_t)g.vol / 2 * 12, ff = (size_t)g.vol * 12;
-    for (int r = 0; r < n; r++) {
-        k_eo_move<double2><<<eo_blocks(g), 128, 0, st>>>(g, 0, 0, const_cast<double2*>(eta) + r * ff, ee);
-        SEEDCG_CHECK_LAUNCH();
-        k_eo_move<double2><<<eo_blocks(g), 128, 0, st>>>(g, 1, 0, const_cast<double2*>(eta) + r * ff, eo);
-        SEEDCG_CHECK_LAUNCH();
-        eo_hop<double>(g, u, 0, 1, ee, eo, 1.0, kappa, phi + r * hf, st);
-        apply_a<double>(g, u, kappa, 1, phi + r * hf, te, b + r * hf, st);
-    }
-}
-
-void eo_gather_f64(const Geom& g, int p, int n, const double2* full, double2* half, cudaStream_t st) {
-    const size_t hf = (size_t)g.vol / 2 * 12, ff = (size_t)g.vol * 12;
-    for (int r = 0; r < n; r++) {
-        k_eo_move<double2><<<eo_blocks(g), 128, 0, st>>>(g, p, 0, const_cast<double2*>(full) + r * ff, half + r * hf);
-        SEEDCG_CHECK_LAUNCH();
-    }
-}
-
-// x = [x_e, x_o] with x_e = eta_e + kappa H_eo x_o for n fields (x: full; ee, xe: half scratch)
-void eo_reconstruct_f64(const Geom& g, const double2* u, double kappa, int n, const double2* x_odd,
-                        const double2* eta, double2* x, double2* ee, double2* xe, cudaStream_t st) {
-    const size_t hf = (size_t)g.vol / 2 * 12, ff = (size_t)g.vol * 12;
-    for (int r = 0; r < n; r++) {
-        k_eo_move<double2><<<eo_blocks(g), 128, 0, st>>>(g, 0, 0, const_cast<double2*>(eta) + r * ff, ee);
-        SEEDCG_CHECK_LAUNCH();
-        eo_hop<double>(g, u, 0, 0, x_odd + r * hf, ee, 1.0, kappa, xe, st);
-        k_eo_move<double2><<<eo_blocks(g), 128, 0, st>>>(g, 0, 1, x + r * ff, xe);
-        SEEDCG_CHECK_LAUNCH();
-        k_eo_move<double2><<<eo_blocks(g), 128, 0, st>>>(g, 1, 1, x + r * ff, const_cast<double2*>(x_odd) + r * hf);
-        SEEDCG_CHECK_LAUNCH();
-    }
-}
-
 namespace {
 
 bool eo_dims_ok(const Geom& g) {
@@ -133,37 +69,49 @@ bool eo_dims_ok(const Geom& g) {
     return true;
 }
 
-template <typename R>
-void apply_eo_impl(seedcg_handle* h, int op, int n, const double* in, double* out, cudaStream_t st) {
+void apply_eo_f64(seedcg_handle* h, int op, int n, const double* in, double* out, cudaStream_t st) {
+    const int vh = h->g.vol / 2;
+    const size_t hf = (size_t)vh * 12 * n;
+    DevBuf buf;
+    buf.ensure(3 * hf * sizeof(double2));
+    double2* X = buf.as<double2>();
+    double2* Y = X + hf;
+    double2* T = Y + hf;
+    to_internal_f64(in, X, vh, n, st);
+    const FixDev F = fix_of(h);
+    if (op == 2) eo_apply_mdag_m_f64(F, n, X, T, Y, st);
+    else eo_apply_a_f64(F, op, n, X, T, Y, st);
+    from_internal_f64(Y, out, vh, n, st);
+    SEEDCG_CUDA_TRY(cudaStreamSynchronize(st));
+}
+
+void apply_eo_f32(seedcg_handle* h, int op, int n, const double* in, double* out, cudaStream_t st) {
     const Geom& g = h->g;
     const int vh = g.vol / 2;
     const size_t hf = (size_t)vh * 12;
-    const cx_t<R>* u = sizeof(R) == 8 ? reinterpret_cast<const cx_t<R>*>(h->u64.p)
-                                      : reinterpret_cast<const cx_t<R>*>(h->u32.p);
+    const float2* u = h->u32.as<float2>();
     DevBuf buf;
-    buf.ensure((3 * (size_t)n + 1) * hf * sizeof(cx_t<R>));
-    cx_t<R>* X = buf.as<cx_t<R>>();
-    cx_t<R>* Y = X + (size_t)n * hf;
-    cx_t<R>* Z = Y + (size_t)n * hf;
-    cx_t<R>* T = Z + (size_t)n * hf;
-    if (sizeof(R) == 8) to_internal_f64(in, reinterpret_cast<double2*>(X), vh, n, st);
-    else to_internal_f32(in, reinterpret_cast<float2*>(X), vh, n, st);
-    cx_t<R>* res = Y;
+    buf.ensure((3 * (size_t)n + 1) * hf * sizeof(float2));
+    float2* X = buf.as<float2>();
+    float2* Y = X + (size_t)n * hf;
+    float2* Z = Y + (size_t)n * hf;
+    float2* T = Z + (size_t)n * hf;
+    to_internal_f32(in, X, vh, n, st);
+    float2* res = Y;
     for (int r = 0; r < n; r++) {
-        const cx_t<R>* x = X + (size_t)r * hf;
-        cx_t<R>* y = Y + (size_t)r * hf;
+        const float2* x = X + (size_t)r * hf;
+        float2* y = Y + (size_t)r * hf;
         if (op == 0) {
-            apply_a<R>(g, u, h->kappa, 0, x, T, y, st);
+            apply_a<float>(g, u, h->kappa, 0, x, T, y, st);
         } else if (op == 1) {
-            apply_a<R>(g, u, h->kappa, 1, x, T, y, st);
+            apply_a<float>(g, u, h->kappa, 1, x, T, y, st);
         } else {
-            apply_a<R>(g, u, h->kappa, 0, x, T, y, st);
-            apply_a<R>(g, u, h->kappa, 1, y, T, Z + (size_t)r * hf, st);
+            apply_a<float>(g, u, h->kappa, 0, x, T, y, st);
+            apply_a<float>(g, u, h->kappa, 1, y, T, Z + (size_t)r * hf, st);
             res = Z;
         }
     }
-    if (sizeof(R) == 8) from_internal_f64(reinterpret_cast<double2*>(res), out, vh, n, st);
-    else from_internal_f32(reinterpret_cast<float2*>(res), out, vh, n, st);
+    from_internal_f32(res, out, vh, n, st);
     SEEDCG_CUDA_TRY(cudaStreamSynchronize(st));
 }
 
@@ -211,8 +159,8 @@ extern "C" seedcg_status seedcg_apply_eo(seedcg_handle* h, int op, int prec, int
     try {
         SEEDCG_CUDA_TRY(cudaSetDevice(h->device));
         cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-        if (prec == 0) seedcg::apply_eo_impl<double>(h, op, n, in, out, st);
-        else seedcg::apply_eo_impl<float>(h, op, n, in, out, st);
+        if (prec == 0) seedcg::apply_eo_f64(h, op, n, in, out, st);
+        else seedcg::apply_eo_f32(h, op, n, in, out, st);
         return SEEDCG_OK;
     } catch (const Error& e) {
         h->err = e.msg;
@@ -231,20 +179,11 @@ extern "C" seedcg_status seedcg_eo_source(seedcg_handle* h, int n, const double*
         const int vh = g.vol / 2;
         const size_t hf = (size_t)vh * 12, ff = (size_t)g.vol * 12;
         DevBuf buf;
-        buf.ensure(((size_t)n * ff + (size_t)n * hf + 2 * hf) * sizeof(double2));
+        buf.ensure(((size_t)n * ff + (size_t)n * hf) * sizeof(double2));
         double2* E = buf.as<double2>();
         double2* P = E + (size_t)n * ff;
-        double2* Ee = P + (size_t)n * hf;
-        double2* Eo = Ee + hf;
         seedcg::to_internal_f64(eta, E, g.vol, n, st);
-        for (int r = 0; r < n; r++) {
-            seedcg::k_eo_move<double2><<<seedcg::eo_blocks(g), 128, 0, st>>>(g, 0, 0, E + (size_t)r * ff, Ee);
-            SEEDCG_CHECK_LAUNCH();
-            seedcg::k_eo_move<double2><<<seedcg::eo_blocks(g), 128, 0, st>>>(g, 1, 0, E + (size_t)r * ff, Eo);
-            SEEDCG_CHECK_LAUNCH();
-            // phi = eta_o + kappa H_oe eta_e
-            seedcg::eo_hop<double>(g, h->u64.as<double2>(), 0, 1, Ee, Eo, 1.0, h->kappa, P + (size_t)r * hf, st);
-        }
+        seedcg::eo_source_f64(seedcg::fix_of(h), n, E, P, st);   // phi = eta_o + kappa H_oe eta_e
         seedcg::from_internal_f64(P, phi, vh, n, st);
         SEEDCG_CUDA_TRY(cudaStreamSynchronize(st));
         return SEEDCG_OK;
@@ -265,26 +204,13 @@ extern "C" seedcg_status seedcg_eo_reconstruct(seedcg_handle* h, int n, const do
         const int vh = g.vol / 2;
         const size_t hf = (size_t)vh * 12, ff = (size_t)g.vol * 12;
         DevBuf buf;
-        buf.ensure((2 * (size_t)n * ff + (size_t)n * hf + 2 * hf) * sizeof(double2));
+        buf.ensure((2 * (size_t)n * ff + (size_t)n * hf) * sizeof(double2));
         double2* E = buf.as<double2>();
         double2* F = E + (size_t)n * ff;
         double2* Xo = F + (size_t)n * ff;
-        double2* Ee = Xo + (size_t)n * hf;
-        double2* Xe = Ee + hf;
         seedcg::to_internal_f64(eta, E, g.vol, n, st);
         seedcg::to_internal_f64(x_odd, Xo, vh, n, st);
-        for (int r = 0; r < n; r++) {
-            double2* fr = F + (size_t)r * ff;
-            double2* xo = Xo + (size_t)r * hf;
-            seedcg::k_eo_move<double2><<<seedcg::eo_blocks(g), 128, 0, st>>>(g, 0, 0, E + (size_t)r * ff, Ee);
-            SEEDCG_CHECK_LAUNCH();
-            // x_e = eta_e + kappa H_eo x_o
-            seedcg::eo_hop<double>(g, h->u64.as<double2>(), 0, 0, xo, Ee, 1.0, h->kappa, Xe, st);
-            seedcg::k_eo_move<double2><<<seedcg::eo_blocks(g), 128, 0, st>>>(g, 0, 1, fr, Xe);
-            SEEDCG_CHECK_LAUNCH();
-            seedcg::k_eo_move<double2><<<seedcg::eo_blocks(g), 128, 0, st>>>(g, 1, 1, fr, xo);
-            SEEDCG_CHECK_LAUNCH();
-        }
+        seedcg::eo_reconstruct_f64(seedcg::fix_of(h), n, Xo, E, F, st);   // x_e = eta_e + kappa H_eo x_o
         seedcg::from_internal_f64(F, x, g.vol, n, st);
         SEEDCG_CUDA_TRY(cudaStreamSynchronize(st));
         return SEEDCG_OK;

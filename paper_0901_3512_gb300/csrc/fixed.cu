@@ -1,0 +1,168 @@
+// The FP64 operator: links in fixed point, D and D^dag on full fields, and the
+// even-odd operator of Section 3 on half vectors, all through fix_tile (fixhop.cuh).
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
+#include "fixhop.cuh"
+#include "handle.cuh"
+
+namespace seedcg {
+namespace {
+
+// largest and smallest nonzero link component magnitude by link (upper word of the FP64 value:
+// 21 bits are enough for a power of two), range[0] a maximum and range[1] a minimum
+__global__ void k_fix_range(const double2* __restrict__ u, int vol, unsigned* __restrict__ range) {
+    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    unsigned mx = 0;
+    if (t < 4L * vol) {
+        const int mu = (int)(t / vol), s = (int)(t % vol);
+#pragma unroll
+        for (int e = 0; e < 9; e++) {
+            const double2 z = u[(size_t)(mu * 9 + e) * vol + s];
+            mx = max(mx, max((unsigned)__double2hiint(z.x) & 0x7fffffffu, (unsigned)__double2hiint(z.y) & 0x7fffffffu));
+        }
+    }
+    const unsigned hi = __reduce_max_sync(0xffffffffu, mx), lo = __reduce_min_sync(0xffffffffu, mx ? mx : 0x7fffffffu);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(range, hi);
+        atomicMin(range + 1, lo);
+    }
+}
+
+__global__ void k_fix_links(Geom g, const double2* __restrict__ u, double kappa, int k, int4* __restrict__ L) {
+    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (t >= 36L * g.vol) return;
+    const int s = (int)(t % g.vol), mu = (int)(t / g.vol) / 9;
+    const double2 z = u[t];
+    // hops across the t boundary, forward from the last slice and backward from the first, use this link
+    const double c = ldexp(mu == 3 && s / g.stride[3] == g.L[3] - 1 ? kappa : -kappa, k);
+    const long long re = __double2ll_rn(c * z.x), im = __double2ll_rn(c * z.y);
+    constexpr long long kLow = (1ll << 27) - 1;
+    L[t] = make_int4((int)(re >> 27), (int)(re & kLow), (int)(im >> 27), (int)(im & kLow));
+}
+
+struct FixStore {
+    static constexpr bool kShare = false;
+    double2* out;
+    long stride;
+    int vo;       // sites of an output field
+    int half;     // 1: stored at the half index
+    __device__ __forceinline__ double operator()(int r, int plane, int idx, int s, bool live, double2 a, double2 b) {
+        if (live) {
+            double2* q = out + (size_t)r * stride + ((size_t)plane * vo + (half ? idx : s)) * 2;
+            q[0] = a;
+            q[1] = b;
+        }
+        return 0.0;
+    }
+    __device__ __forceinline__ void put(int, double) {}
+};
+
+// At most 128 registers: two blocks per SM.  Instruction issue bounds it: 1270 warp instructions per
+// 32 sites, direction and field, 216 of them multiply-adds of 32 x 32 + 64 bits and 380 the conversion of the
+// neighbour.  16^3 x 32, 12 fields: 900 us, issue 44 % busy at 16 warps per SM, DRAM 12 %.
+__global__ void __launch_bounds__(kFixThreads, 2) k_fix_apply(FixDev F, FixOp op, FixStore st, int n) {
+    extern __shared__ __align__(16) unsigned char fix_smem[];
+    fix_tile(F, op, blockIdx.x, blockIdx.y, n, gridDim.y, fix_smem, st);
+}
+
+void fix_go(const FixDev& F, const FixOp& op, const FixStore& st, int n, cudaStream_t s) {
+    if (n <= 0) return;
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_fix_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
+    SEEDCG_CUDA_TRY(attr);
+    const int sites = op.parity < 0 ? F.g.vol : F.g.vol / 2, tiles = (sites + 31) / 32;
+    k_fix_apply<<<dim3(tiles, fix_grid_y(tiles, n)), kFixThreads, kFixSmem, s>>>(F, op, st, n);
+    SEEDCG_CHECK_LAUNCH();
+}
+
+// half[h] = full at the parity-p site of h (scatter = 0) or the reverse (scatter = 1), field blockIdx.y
+__global__ void k_eo_move(Geom g, int p, int scatter, double2* __restrict__ full, double2* __restrict__ half) {
+    const int vh = g.vol / 2;
+    const int h = blockIdx.x * blockDim.x + threadIdx.x;
+    if (h >= vh) return;
+    full += (size_t)blockIdx.y * 12 * g.vol;
+    half += (size_t)blockIdx.y * 12 * vh;
+    const int s = eo_site(g, h, p);
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+        if (scatter)
+            full[sidx(k, s, g.vol)] = half[sidx(k, h, vh)];
+        else
+            half[sidx(k, h, vh)] = full[sidx(k, s, g.vol)];
+    }
+}
+
+void eo_move(const Geom& g, int p, int scatter, int n, double2* full, double2* half, cudaStream_t st) {
+    k_eo_move<<<dim3((g.vol / 2 + 127) / 128, n), 128, 0, st>>>(g, p, scatter, full, half);
+    SEEDCG_CHECK_LAUNCH();
+}
+
+}  // namespace
+
+void fix_links(const Geom& g, const double2* u, double kappa, int4* L, int* k, int* ok, cudaStream_t s) {
+    DevBuf rb;
+    rb.ensure(2 * sizeof(unsigned));
+    unsigned range[2] = {0u, 0x7fffffffu};
+    SEEDCG_CUDA_TRY(cudaMemcpyAsync(rb.p, range, sizeof(range), cudaMemcpyHostToDevice, s));
+    k_fix_range<<<(4 * g.vol + 255) / 256, 256, 0, s>>>(u, g.vol, rb.as<unsigned>());
+    SEEDCG_CHECK_LAUNCH();
+    SEEDCG_CUDA_TRY(cudaMemcpyAsync(range, rb.p, sizeof(range), cudaMemcpyDeviceToHost, s));
+    SEEDCG_CUDA_TRY(cudaStreamSynchronize(s));
+    // |kappa U| < 2^ex for every component; L = kappa U 2^k stays within 2^55, and the diagonal term's
+    // significand within 2^58 (k <= 57).  Links of very different size would lose relative
+    // accuracy (more than 2^8 apart), as would a scale far from the diagonal's: plain FP64 then.
+    int ex = 0;
+    const bool finite = range[0] < 0x7ff00000u - 1u && std::isfinite(kappa);
+    double mx = 0.0;
+    if (finite) {
+        const unsigned long long bits = (unsigned long long)(range[0] + 1u) << 32;
+        std::memcpy(&mx, &bits, sizeof(mx));
+        if (range[0] == 0) mx = 0.0;
+        frexp(mx * std::fabs(kappa), &ex);
+    }
+    *k = std::min(57, 55 - ex);
+    *ok = finite && ex < 16 && (range[0] == 0 || range[1] + (8u << 20) >= range[0]) ? 1 : 0;
+    if (!*ok) *k = 0;
+    k_fix_links<<<(int)((36L * g.vol + 255) / 256), 256, 0, s>>>(g, u, *ok ? kappa : 0.0, *k, L);
+    SEEDCG_CHECK_LAUNCH();
+}
+
+void dslash_f64(const FixDev& F, int dag, int n, const double2* in, double2* out, cudaStream_t s) {
+    const long nf = 12L * F.g.vol;
+    const FixOp op{dag, -1, in, nf, 0, 1, 1, in, nf, 0};
+    fix_go(F, op, FixStore{out, nf, F.g.vol, 0}, n, s);
+}
+
+// With t = -kappa H_eo x (FP64 half vectors), A x = x - (-kappa H_oe) t: the factors of
+// kappa^2 are in the links.
+void eo_apply_a_f64(const FixDev& F, int dag, int n, const double2* x, double2* te, double2* out, cudaStream_t st) {
+    const int vh = F.g.vol / 2;
+    const long nh = 12L * vh;
+    fix_go(F, FixOp{dag, 0, x, nh, 1, 0, 1, nullptr, 0, 1}, FixStore{te, nh, vh, 1}, n, st);
+    fix_go(F, FixOp{dag, 1, te, nh, 1, 1, -1, x, nh, 1}, FixStore{out, nh, vh, 1}, n, st);
+}
+
+void eo_apply_mdag_m_f64(const FixDev& F, int n, const double2* x, double2* te, double2* out, cudaStream_t st) {
+    eo_apply_a_f64(F, 0, n, x, te, out, st);
+    eo_apply_a_f64(F, 1, n, out, te, out, st);
+}
+
+void eo_source_f64(const FixDev& F, int n, const double2* eta, double2* phi, cudaStream_t st) {
+    const int vh = F.g.vol / 2;
+    fix_go(F, FixOp{0, 1, eta, 12L * F.g.vol, 0, 1, -1, eta, 12L * F.g.vol, 0}, FixStore{phi, 12L * vh, vh, 1}, n, st);
+}
+
+void eo_gather_f64(const Geom& g, int p, int n, const double2* full, double2* half, cudaStream_t st) {
+    eo_move(g, p, 0, n, const_cast<double2*>(full), half, st);
+}
+
+void eo_reconstruct_f64(const FixDev& F, int n, const double2* x_odd, const double2* eta, double2* x,
+                        cudaStream_t st) {
+    const long nf = 12L * F.g.vol, nh = nf / 2;
+    fix_go(F, FixOp{0, 0, x_odd, nh, 1, 1, -1, eta, nf, 0}, FixStore{x, nf, F.g.vol, 0}, n, st);
+    eo_move(F.g, 1, 1, n, x, const_cast<double2*>(x_odd), st);
+}
+
+}  // namespace seedcg

@@ -14,6 +14,8 @@ struct seedcg_handle {
     seedcg_options opt;
     int device = 0;
     seedcg::DevBuf u64, u32;      // links [4][9][V] double2 / float2
+    seedcg::DevBuf fix;           // links in fixed point [4][9][V] int4 (the FP64 operator)
+    int fix_k = 0, fix_ok = 0;    // their scale, and whether every link fits it
     // workspaces
     seedcg::DevBuf vbasis;        // stored Krylov basis V, m_cap rows
     int vbasis_prec = -1;         // precision mode V was written in
@@ -39,6 +41,10 @@ struct seedcg_handle {
 };
 
 namespace seedcg {
+inline FixDev fix_of(const seedcg_handle* h) {
+    return FixDev{h->g, h->fix.as<int4>(), h->u64.as<double2>(), h->kappa, h->fix_k, h->fix_ok};
+}
+
 // learned initial guess (guess.cu); B, X internal FP64 [n][12 V]
 void guess_set_weights(seedcg_handle* h, const double* w, cudaStream_t st);
 void guess_get_weights(seedcg_handle* h, double* w, cudaStream_t st);

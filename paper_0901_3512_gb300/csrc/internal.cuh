@@ -103,6 +103,18 @@ inline Geom make_geom(const int dims[4]) {
     return g;
 }
 
+// One gauge field for the FP64 operator (fixhop.cuh): the links in fixed point,
+// L = -kappa U 2^k with the antiperiodic sign, [4][9][V] (re hi, re lo, im hi, im lo),
+// and the FP64 links for what the fixed point cannot take (ok = 0: for every site).
+struct FixDev {
+    Geom g;
+    const int4* L;
+    const double2* u;
+    double kappa;
+    int k;
+    int ok;
+};
+
 // ----------------------------------------------------------------------------
 // device buffers
 // ----------------------------------------------------------------------------
@@ -153,33 +165,32 @@ void from_internal_f32(const float2* in, double* out, int vol, int n, cudaStream
 void gauge_to_internal(const double* in, double2* u64, float2* u32, int vol, cudaStream_t s);
 
 // out = D in (dag = 0) or D^dag in (dag = 1); single right-hand side
-void dslash_f64(const Geom& g, const double2* u, double kappa, int dag, const double2* in,
-                double2* out, cudaStream_t s);
 void dslash_f32(const Geom& g, const float2* u, float kappa, int dag, const float2* in,
                 float2* out, cudaStream_t s);
 // n right-hand sides at in + r*12*V; links staged once per tile of sites
-void dslash_mrhs_f64(const Geom& g, const double2* u, double kappa, int dag, int n,
-                     const double2* in, double2* out, cudaStream_t s);
 void dslash_mrhs_f32(const Geom& g, const float2* u, float kappa, int dag, int n,
                      const float2* in, float2* out, cudaStream_t s);
-
-// even-odd preconditioned system (evenodd.cu), FP64 half vectors in the internal layout:
-// out_r = A^dag A x_r, A = 1 - kappa^2 H_oe H_eo (te, y: one even / odd half scratch each)
-void eo_apply_mdag_m_f64(const Geom& g, const double2* u, double kappa, int n, const double2* x,
-                         double2* te, double2* y, double2* out, cudaStream_t st);
-// phi = eta_o + kappa H_oe eta_e and b = A^dag phi for n full fields eta
-void eo_rhs_f64(const Geom& g, const double2* u, double kappa, int n, const double2* eta, double2* phi,
-                double2* b, double2* ee, double2* eo, double2* te, cudaStream_t st);
-// half[r] = the parity-p sites of full[r] for n fields
-void eo_gather_f64(const Geom& g, int p, int n, const double2* full, double2* half, cudaStream_t st);
-// full x from x_o: x_e = eta_e + kappa H_eo x_o
-void eo_reconstruct_f64(const Geom& g, const double2* u, double kappa, int n, const double2* x_odd,
-                        const double2* eta, double2* x, double2* ee, double2* xe, cudaStream_t st);
-
-// the multi-RHS kernel with its default tile shape, never timing alternatives
-void dslash_mrhs_fixed_f64(const Geom& g, const double2* u, double kappa, int dag, int n,
-                           const double2* in, double2* out, cudaStream_t s);
+// the same kernel with its default tile shape, never timing alternatives
 void dslash_mrhs_fixed_f32(const Geom& g, const float2* u, float kappa, int dag, int n,
                            const float2* in, float2* out, cudaStream_t s);
+
+// FP64 operator in fixed point (fixed.cu): out = D in or D^dag in for n fields
+void dslash_f64(const FixDev& F, int dag, int n, const double2* in, double2* out, cudaStream_t s);
+// the links of a handle in fixed point: L from u, and the scale k and range flag ok (synchronises)
+void fix_links(const Geom& g, const double2* u, double kappa, int4* L, int* k, int* ok, cudaStream_t s);
+
+// even-odd preconditioned system (fixed.cu), FP64 half vectors in the internal layout:
+// out_r = A x_r (dag = 0) or A^dag x_r, A = 1 - kappa^2 H_oe H_eo, n fields (te: n even half
+// vectors of scratch; out may be x)
+void eo_apply_a_f64(const FixDev& F, int dag, int n, const double2* x, double2* te, double2* out, cudaStream_t st);
+// out_r = A^dag A x_r (te: n even half vectors of scratch)
+void eo_apply_mdag_m_f64(const FixDev& F, int n, const double2* x, double2* te, double2* out, cudaStream_t st);
+// phi = eta_o + kappa H_oe eta_e for n full fields eta
+void eo_source_f64(const FixDev& F, int n, const double2* eta, double2* phi, cudaStream_t st);
+// half[r] = the parity-p sites of full[r] for n fields
+void eo_gather_f64(const Geom& g, int p, int n, const double2* full, double2* half, cudaStream_t st);
+// full x from x_o: x_e = eta_e + kappa H_eo x_o, for n fields
+void eo_reconstruct_f64(const FixDev& F, int n, const double2* x_odd, const double2* eta, double2* x,
+                        cudaStream_t st);
 
 }  // namespace seedcg

@@ -88,12 +88,7 @@ extern "C" seedcg_status seedcg_apply_noalloc(seedcg_handle* h, int op, int prec
         if (prec == 0) {
             seedcg::to_internal_f64(in, (double2*)A, vol, n, st);
             auto apply = [&](int dag, const double2* x, double2* y) {
-                if (multi)
-                    seedcg::dslash_mrhs_fixed_f64(h->g, h->u64.as<double2>(), h->kappa, dag, n, x, y, st);
-                else
-                    for (int r = 0; r < n; r++)
-                        seedcg::dslash_f64(h->g, h->u64.as<double2>(), h->kappa, dag,
-                                           x + (size_t)r * 12 * vol, y + (size_t)r * 12 * vol, st);
+                seedcg::dslash_f64(seedcg::fix_of(h), dag, n, x, y, st);   // one kernel for any n
             };
             const double2* res = (const double2*)Bv;
             if (op == 0) apply(0, (double2*)A, (double2*)Bv);

@@ -15,6 +15,7 @@
 
 #include "cg_batch.cuh"
 #include "eo.cuh"
+#include "fixhop.cuh"
 #include "handle.cuh"
 #include "kernels.cuh"
 #include "reduce.cuh"
@@ -120,7 +121,7 @@ __global__ void k_lz_start(const cx_t<R>* __restrict__ r0, cx_t<R>* __restrict__
 
 // t = D v_i
 template <typename R>
-__global__ void __launch_bounds__(kSiteThreads, sizeof(R) == 4 ? 7 : 4)
+__global__ void __launch_bounds__(kSiteThreads, 7)
 k_lz_D(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict__ v,
        cx_t<R>* __restrict__ t, int i, LzDev L) {
     if (i > L.ctl->m) return;
@@ -139,7 +140,7 @@ k_lz_D(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict
 // Step 5 (and 2): f = D^dag t - beta_{i-1} v_{i-1}; alpha_i = Re v_i^dag f.
 // Step 6 scalars (and 3): gamma_{i-1}, delta_i, zeta_i.
 template <typename R>
-__global__ void __launch_bounds__(kSiteThreads, sizeof(R) == 4 ? 7 : 4)
+__global__ void __launch_bounds__(kSiteThreads, 7)
 k_lz_Ddag(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict__ t,
           const cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ vprev,
           cx_t<R>* __restrict__ f, int i, LzDev L) {
@@ -218,6 +219,83 @@ k_lz_eo(Geom g, const cx_t<R>* __restrict__ u, R kk, const cx_t<R>* __restrict__
     }
     if (STAGE == 3)
         grid_sum<1>(red, L.partials, L.counters + CTR_B, [&](double* tot) { lz_alpha_fin(L, i, tot[0]); });
+}
+
+// FP64 runs apply the operator in fixed point (fixhop.cuh).  The last hop's epilogue forms
+// f = val - beta_{i-1} v_{i-1} and this thread's share of alpha_i = Re v_i^dag f; the others store.
+struct LzFixEpi {
+    static constexpr bool kShare = false;
+    double2* out;
+    const double2* v;       // null: store only
+    const double2* vprev;   // null: no beta_{i-1} v_{i-1}
+    double bprev;
+    int vo;
+    double part;
+    __device__ __forceinline__ double operator()(int, int plane, int idx, int, bool live, double2 a, double2 b) {
+        if (live) {
+            const size_t ix = ((size_t)plane * vo + idx) * 2;
+            if (v) {
+                if (vprev) {
+                    const double2 pa = vprev[ix], pb = vprev[ix + 1];
+                    a.x -= bprev * pa.x;
+                    a.y -= bprev * pa.y;
+                    b.x -= bprev * pb.x;
+                    b.y -= bprev * pb.y;
+                }
+                const double2 va = v[ix], vb = v[ix + 1];
+                part += va.x * a.x + va.y * a.y + vb.x * b.x + vb.y * b.y;
+            }
+            out[ix] = a;
+            out[ix + 1] = b;
+        }
+        return 0.0;
+    }
+    __device__ __forceinline__ void put(int, double) {}
+};
+
+template <bool LAST>
+__global__ void __launch_bounds__(kFixThreads, 2)
+k_lz_fix(FixDev F, FixOp op, const double2* __restrict__ v, const double2* __restrict__ vprev,
+         double2* __restrict__ out, int i, LzDev L) {
+    if (i > L.ctl->m) return;
+    extern __shared__ __align__(16) unsigned char fix_smem[];
+    LzFixEpi epi{out,
+                 LAST ? v : nullptr,
+                 LAST && i > 1 ? vprev : nullptr,
+                 LAST && i > 1 ? L.beta[i - 2] : 0.0,
+                 op.parity < 0 ? F.g.vol : F.g.vol / 2,
+                 0.0};
+    fix_tile(F, op, blockIdx.x, 0, 1, 1, fix_smem, epi);
+    if (LAST) {
+        double red[1] = {epi.part};
+        grid_sum<1>(red, L.partials, L.counters + CTR_B, [&](double* tot) { lz_alpha_fin(L, i, tot[0]); });
+    }
+}
+
+template <bool LAST>
+void lz_fix(const FixDev& F, const FixOp& op, const double2* v, const double2* vprev, double2* out, int i,
+            const LzDev& L, cudaStream_t st) {
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_lz_fix<LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
+    SEEDCG_CUDA_TRY(attr);
+    const int sites = op.parity < 0 ? F.g.vol : F.g.vol / 2;
+    k_lz_fix<LAST><<<(sites + 31) / 32, kFixThreads, kFixSmem, st>>>(F, op, v, vprev, out, i, L);
+    SEEDCG_CHECK_LAUNCH();
+}
+
+// f = M v - beta_{i-1} v_{i-1} and alpha_i in FP64: D and D^dag, or the four half-lattice hops
+// (t, e: full or odd half, and even half scratch)
+void lz_apply_f64(const FixDev& F, bool eo, const double2* v, const double2* vprev, double2* t, double2* e,
+                  double2* f, int i, const LzDev& L, cudaStream_t st) {
+    if (!eo) {
+        lz_fix<false>(F, FixOp{0, -1, v, 0, 0, 1, 1, v, 0, 0}, nullptr, nullptr, t, i, L, st);
+        lz_fix<true>(F, FixOp{1, -1, t, 0, 0, 1, 1, t, 0, 0}, v, vprev, f, i, L, st);
+        return;
+    }
+    lz_fix<false>(F, FixOp{0, 0, v, 0, 1, 0, 1, nullptr, 0, 1}, nullptr, nullptr, e, i, L, st);
+    lz_fix<false>(F, FixOp{0, 1, e, 0, 1, 1, -1, v, 0, 1}, nullptr, nullptr, t, i, L, st);
+    lz_fix<false>(F, FixOp{1, 0, t, 0, 1, 0, 1, nullptr, 0, 1}, nullptr, nullptr, e, i, L, st);
+    lz_fix<true>(F, FixOp{1, 1, e, 0, 1, 1, -1, t, 0, 1}, v, vprev, f, i, L, st);
 }
 
 // Steps 4 and 7 (literal seeding): eta^j = v_i^dag r_0^j - gamma_{i-1} eta^j for
@@ -715,8 +793,8 @@ __global__ void __launch_bounds__(256) k_seed_tridiag(double2* C, int ldc, int n
 // M x for n FP64 fields in internal layout (D then D^dag) via the multi-RHS kernel
 inline void apply_M64(seedcg_handle* h, int n, const double2* x, double2* tmp, double2* out,
                       cudaStream_t st) {
-    dslash_mrhs_f64(h->g, h->u64.as<double2>(), h->kappa, 0, n, x, tmp, st);
-    dslash_mrhs_f64(h->g, h->u64.as<double2>(), h->kappa, 1, n, tmp, out, st);
+    dslash_f64(fix_of(h), 0, n, x, tmp, st);
+    dslash_f64(fix_of(h), 1, n, tmp, out, st);
 }
 
 // bump allocator over one device buffer
@@ -949,7 +1027,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     const int nbl = std::min<long>((n * nrhs + 255) / 256, 152 * 32);
     if (o.x0_given || h->force_x0) {
         if (eo)
-            eo_apply_mdag_m_f64(h->g, h->u64.as<double2>(), h->kappa, nrhs, X64, T64, T64 + n, MX, st);
+            eo_apply_mdag_m_f64(fix_of(h), nrhs, X64, T64, MX, st);
         else
             apply_M64(h, nrhs, X64, T64, MX, st);
         k_resid_init<R><<<nbl, 256, 0, st>>>(B64, MX, R0, n * nrhs);
@@ -998,7 +1076,9 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
         const int sbh = site_blocks(vol / 2);
         const R kk = (R)(h->kappa * h->kappa);
         for (; i <= m_max; i++) {
-            if (eo) {
+            if constexpr (sizeof(R) == 8) {
+                lz_apply_f64(fix_of(h), eo, v, vprev, tv, ev, fv, i, L, st);
+            } else if (eo) {
                 // f = A^dag A v - beta v_prev, alpha: four half-lattice hops
                 k_lz_eo<R, 0><<<sbh, kRedThreads, 0, st>>>(h->g, U, kk, v, nullptr, ev, nullptr, nullptr, i, L);
                 SEEDCG_CHECK_LAUNCH();
@@ -1568,7 +1648,7 @@ seedcg_status cg_only(seedcg_handle* h, int nrhs, double2* B64, double2* X64, do
 void d_residuals(seedcg_handle* h, int nrhs, const double2* E64, const double2* X64, double2* T64,
                  std::vector<double>& ratio, cudaStream_t st) {
     const long n = 12L * h->g.vol;
-    dslash_mrhs_f64(h->g, h->u64.as<double2>(), h->kappa, 0, nrhs, X64, T64, st);
+    dslash_f64(fix_of(h), 0, nrhs, X64, T64, st);
     DevBuf nr;
     nr.ensure(sizeof(double) * (4096 + 2 * nrhs) + sizeof(unsigned) * 64);
     double* part = nr.as<double>();
@@ -1676,7 +1756,7 @@ seedcg_status solve_impl(seedcg_handle* h, int nrhs, const double* B, double* X,
     double2* T64 = dmode ? E64 + (size_t)nrhs * n : nullptr;   // scratch
     if (dmode) {
         to_internal_f64(B, E64, vol, nrhs, st);
-        dslash_mrhs_f64(h->g, h->u64.as<double2>(), h->kappa, 1, nrhs, E64, B64, st);  // b = D^dag eta
+        dslash_f64(fix_of(h), 1, nrhs, E64, B64, st);  // b = D^dag eta
     } else {
         to_internal_f64(B, B64, vol, nrhs, st);
     }
@@ -1692,8 +1772,8 @@ seedcg_status solve_impl(seedcg_handle* h, int nrhs, const double* B, double* X,
         t1.ensure(fb);
         t2.ensure(fb);
         nr.ensure(sizeof(double) * (4096 + 2 * nrhs) + sizeof(unsigned) * 64);
-        dslash_mrhs_f64(h->g, h->u64.as<double2>(), h->kappa, 0, nrhs, X64, t1.as<double2>(), st);
-        dslash_mrhs_f64(h->g, h->u64.as<double2>(), h->kappa, 1, nrhs, t1.as<double2>(), t2.as<double2>(), st);
+        dslash_f64(fix_of(h), 0, nrhs, X64, t1.as<double2>(), st);
+        dslash_f64(fix_of(h), 1, nrhs, t1.as<double2>(), t2.as<double2>(), st);
         double* part = nr.as<double>();
         double* norms = part + 4096;
         unsigned* ctr = reinterpret_cast<unsigned*>(norms + 2 * nrhs);
@@ -1763,20 +1843,18 @@ seedcg_status solve_eo_impl(seedcg_handle* h, int nrhs, const double* E, double*
                             int extra_iters, int reorth_period, seedcg_info* info, cudaStream_t st) {
     const Geom& g = h->g;
     const long nh = 12L * (g.vol / 2), nf = 12L * g.vol;
-    // staging: eta and the full solution (full), then phi, b, x_o (half), 3 half scratch
+    // staging: eta and the full solution (full; the latter also holds scratch), then phi, b, x_o (half)
     const size_t full_b = (size_t)nrhs * nf * sizeof(double2), half_b = (size_t)nrhs * nh * sizeof(double2);
-    h->staging.ensure(2 * full_b + 3 * half_b + 3 * (size_t)nh * sizeof(double2) + 1024);
+    h->staging.ensure(2 * full_b + 3 * half_b + 1024);
     double2* E64 = h->staging.as<double2>();
     double2* F64 = E64 + (size_t)nrhs * nf;
     double2* Phi = F64 + (size_t)nrhs * nf;
     double2* B64 = Phi + (size_t)nrhs * nh;
     double2* X64 = B64 + (size_t)nrhs * nh;
-    double2* s0 = X64 + (size_t)nrhs * nh;
-    double2* s1 = s0 + nh;
-    double2* s2 = s1 + nh;
-    const double2* u = h->u64.as<double2>();
+    const FixDev F = fix_of(h);
     to_internal_f64(E, E64, g.vol, nrhs, st);
-    eo_rhs_f64(g, u, h->kappa, nrhs, E64, Phi, B64, s0, s1, s2, st);
+    eo_source_f64(F, nrhs, E64, Phi, st);
+    eo_apply_a_f64(F, 1, nrhs, Phi, F64, B64, st);   // b = A^dag phi
     if (h->opt.x0_given) {
         to_internal_f64(X, F64, g.vol, nrhs, st);
         eo_gather_f64(g, 1, nrhs, F64, X64, st);
@@ -1791,7 +1869,7 @@ seedcg_status solve_eo_impl(seedcg_handle* h, int nrhs, const double* E, double*
     h->force_x0 = false;
     seedcg_status code = dispatch_solve(h, nrhs, B64, X64, tol, extra_iters, reorth_period, info, st);
     h->eo_active = false;
-    eo_reconstruct_f64(g, u, h->kappa, nrhs, X64, E64, F64, s0, s1, st);
+    eo_reconstruct_f64(F, nrhs, X64, E64, F64, st);
     if (info && info->true_resid_D) {
         // the residual of the original system D x = eta, as Section 3 monitors it
         DevBuf tb;
