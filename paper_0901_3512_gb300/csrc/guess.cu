@@ -39,7 +39,6 @@ namespace seedcg {
 namespace {
 
 using bf2 = __nv_bfloat162;
-constexpr int kG = 256;
 
 // ---------------------------------------------------------------------------
 // bf16 site records: the 12 complex entries of one channel at one site, 48 bytes
@@ -103,44 +102,6 @@ __device__ __forceinline__ void apply_link(const float2* __restrict__ u, int vol
     }
 }
 
-// The adjoint transport used by the backward pass through the data: the
-// contribution to site y of direction d comes from site z (y - mu for +mu,
-// y + mu for -mu) and is carried by U_mu(z)^dag (+mu) or U_mu(y) (-mu), with the
-// sign of the hop from z in direction d.
-struct AdjHop {
-    int z;
-    float sg;
-};
-__device__ __forceinline__ AdjHop adj_hop(int y, int d, const Nbr& nb) {
-    if (d == 0) return AdjHop{y, 1.f};
-    const int mu = (d - 1) >> 1;
-    const bool back = (d - 1) & 1;
-    AdjHop h;
-    h.z = back ? nb.f[mu] : nb.b[mu];
-    h.sg = (mu == 3 && (back ? nb.fwrap_t : nb.bwrap_t)) ? -1.f : 1.f;
-    return h;
-}
-__device__ __forceinline__ void apply_link_adj(const float2* __restrict__ u, int vol, int y, int d,
-                                               const AdjHop& hp, const float2 v[3], float2 o[3]) {
-    const int mu = (d - 1) >> 1;
-    const bool back = (d - 1) & 1;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int b = 0; b < 3; b++) {
-            if (!back) {  // U_mu(z)^dag, z = y - mu
-                const float2 uu = __ldg(u + (size_t)(mu * 9 + 3 * b + a) * vol + hp.z);
-                acc = cfma_conj(uu, v[b], acc);
-            } else {      // U_mu(y)
-                const float2 uu = __ldg(u + (size_t)(mu * 9 + 3 * a + b) * vol + y);
-                acc = cfma(uu, v[b], acc);
-            }
-        }
-        o[a] = make_float2(hp.sg * acc.x, hp.sg * acc.y);
-    }
-}
-
 // gathered input g_d(x) of one channel: 4 spins x 3 colours
 __device__ __forceinline__ void gather(const float2* __restrict__ u, const bf2* __restrict__ in_ch, int vol,
                                        int x, int d, const Nbr& nb, float2 g[4][3]) {
@@ -159,36 +120,115 @@ __device__ __forceinline__ void gather(const float2* __restrict__ u, const bf2* 
 }
 
 // ---------------------------------------------------------------------------
-// SIMT layers (one channel on one side): forward, one thread per (site, co)
+// SIMT layers (one channel on one side).  A block owns 32 sites (a lane each); every transported
+// activation is formed once per (site, direction, channel) and shared through shared memory, where
+// one thread per (site, output channel) formed it anew for each output before.  The sums keep the order
+// direction, input channel, input spin, so the results are those of one thread running the whole chain.
 // ---------------------------------------------------------------------------
-template <int CI, int CO>
-__global__ void __launch_bounds__(kG)
-k_g_fwd(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const bf2* __restrict__ in,
-        bf2* __restrict__ z, bf2* __restrict__ h, int relu) {
-    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+constexpr int SL = 32;   // sites per block
+
+// links of the block's sites in the eight directions, times the boundary sign: U(x,d) (ADJ = false) or the
+// link that carries direction d's contribution back to x (apply_link_adj); sl[(d - 1) * 9 + e][lane]
+template <bool ADJ>
+__device__ __forceinline__ void stage_links(const Geom& gm, const float2* __restrict__ u, int x0,
+                                            float2 (*sl)[SL], int (*snb)[SL]) {
     const int vol = gm.vol;
-    if (t >= (long)vol * CO) return;
-    const int co = (int)(t / vol), x = (int)(t % vol);
-    const Nbr nb = neighbours(gm, x);
+    for (int t = threadIdx.x; t < 8 * SL; t += blockDim.x) {
+        const int j = t % SL, d = 1 + t / SL, x = x0 + j;
+        if (x >= vol) continue;
+        const Nbr nb = neighbours(gm, x);
+        const int mu = (d - 1) >> 1;
+        const bool back = (d - 1) & 1;
+        // ADJ: direction +mu comes from x - mu over U_mu(x - mu)^dag, direction -mu from x + mu over U_mu(x)
+        const bool src_back = ADJ ? !back : back;
+        const int y = src_back ? nb.b[mu] : nb.f[mu];
+        const int site = src_back ? y : x;
+        const float sg = (mu == 3 && (src_back ? nb.bwrap_t : nb.fwrap_t)) ? -1.f : 1.f;
+        snb[d - 1][j] = y;
+#pragma unroll
+        for (int e = 0; e < 9; e++) {
+            const float2 z = __ldg(u + (size_t)(mu * 9 + e) * vol + site);
+            sl[(d - 1) * 9 + e][j] = make_float2(sg * z.x, sg * z.y);
+        }
+    }
+}
+
+// o = L v or L^dag v, L[a][b] = sl[3 a + b][lane]
+__device__ __forceinline__ void staged_link(const float2 (*sl)[SL], int lane, bool dag, const float2 v[3], float2 o[3]) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int b = 0; b < 3; b++) {
+            if (!dag) acc = cfma(sl[3 * a + b][lane], v[b], acc);
+            else acc = cfma_conj(sl[3 * b + a][lane], v[b], acc);
+        }
+        o[a] = acc;
+    }
+}
+
+// g_d(x) of one channel into sg[12][lane]
+__device__ __forceinline__ void stage_gather(const bf2* __restrict__ in_ch, int x, int d, const float2 (*sl)[SL],
+                                             const int (*snb)[SL], int lane, float2 (*sg)[SL]) {
+    float2 v[12];
+    ld_site(in_ch + (size_t)(d == 0 ? x : snb[d - 1][lane]) * 12, v);
+    if (d == 0) {
+#pragma unroll
+        for (int k = 0; k < 12; k++) sg[k][lane] = v[k];
+        return;
+    }
+#pragma unroll
+    for (int s = 0; s < 4; s++) {
+        float2 o[3];
+        staged_link(sl + (d - 1) * 9, lane, (d - 1) & 1, &v[3 * s], o);
+#pragma unroll
+        for (int c = 0; c < 3; c++) sg[3 * s + c][lane] = o[c];
+    }
+}
+
+__device__ __forceinline__ void load_w(const bf2* __restrict__ w, float2 (&o)[16]) {
+    const uint4* q = reinterpret_cast<const uint4*>(w);
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const uint4 a = __ldg(q + j);
+        o[4 * j + 0] = unpack_bf2(a.x);
+        o[4 * j + 1] = unpack_bf2(a.y);
+        o[4 * j + 2] = unpack_bf2(a.z);
+        o[4 * j + 3] = unpack_bf2(a.w);
+    }
+}
+
+// layer 1 (1 -> 8): nine warps transport one direction each, then eight warps run one output channel each.
+// z may be null (inference needs h = ReLU(z) only).  16^3 x 32: see the launch.
+__global__ void __launch_bounds__(288)
+k_g_first(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const bf2* __restrict__ in,
+          bf2* __restrict__ z, bf2* __restrict__ h) {
+    __shared__ float2 sl[72][SL];
+    __shared__ int snb[8][SL];
+    __shared__ float2 sg[9 * 12][SL];
+    const int vol = gm.vol, x0 = blockIdx.x * SL;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, x = x0 + lane;
+    const bool live = x < vol;
+    stage_links<false>(gm, u, x0, sl, snb);
+    __syncthreads();
+    if (live) stage_gather(in, x, warp, sl, snb, lane, sg + 12 * warp);
+    __syncthreads();
+    if (warp >= 8 || !live) return;
     float2 acc[4][3];
 #pragma unroll
-    for (int s = 0; s < 4; s++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) acc[s][c] = make_float2(0.f, 0.f);
+    for (int k = 0; k < 12; k++) acc[k / 3][k % 3] = make_float2(0.f, 0.f);
+#pragma unroll 1
     for (int d = 0; d < 9; d++) {
-        for (int ci = 0; ci < CI; ci++) {
-            float2 g[4][3];
-            gather(u, in + (size_t)ci * vol * 12, vol, x, d, nb, g);
-            const bf2* w = W + (((size_t)d * CO + co) * CI + ci) * 16;
+        float2 w[16], g[12];
+        load_w(W + ((size_t)d * 8 + warp) * 16, w);
 #pragma unroll
-            for (int s = 0; s < 4; s++)
+        for (int k = 0; k < 12; k++) g[k] = sg[12 * d + k][lane];
 #pragma unroll
-                for (int sp = 0; sp < 4; sp++) {
-                    const float2 ww = __bfloat1622float2(w[4 * s + sp]);
+        for (int s = 0; s < 4; s++)
 #pragma unroll
-                    for (int c = 0; c < 3; c++) acc[s][c] = cfma(ww, g[sp][c], acc[s][c]);
-                }
-        }
+            for (int sp = 0; sp < 4; sp++)
+#pragma unroll
+                for (int c = 0; c < 3; c++) acc[s][c] = cfma(w[4 * s + sp], g[3 * sp + c], acc[s][c]);
     }
     float2 v[12], r[12];
 #pragma unroll
@@ -196,156 +236,355 @@ k_g_fwd(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const 
         v[k] = acc[k / 3][k % 3];
         r[k] = make_float2(fmaxf(v[k].x, 0.f), fmaxf(v[k].y, 0.f));
     }
-    st_site(site_ptr(z, co, vol, x), v);
-    if (relu) st_site(site_ptr(h, co, vol, x), r);
+    if (z) st_site(site_ptr(z, warp, vol, x), v);
+    st_site(site_ptr(h, warp, vol, x), r);
 }
 
-// backward through the data of a layer with CO = 1: din[ci](y) = sum_d adjoint
-// transport of W_d^dag dout (one thread per (site, ci)), times the ReLU mask of zprev
-template <int CI, int CO>
-__global__ void __launch_bounds__(kG)
-k_g_bwd_data(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const bf2* __restrict__ dout,
-             const bf2* __restrict__ zprev, bf2* __restrict__ din) {
-    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    const int vol = gm.vol;
-    if (t >= (long)vol * CI) return;
-    const int ci = (int)(t / vol), y = (int)(t % vol);
-    const Nbr nb = neighbours(gm, y);
-    float2 acc[4][3];
-#pragma unroll
-    for (int s = 0; s < 4; s++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) acc[s][c] = make_float2(0.f, 0.f);
+// layer 3 (8 -> 1): eight warps transport one input channel each for direction d + 1 while six warps add
+// direction d, a (colour, spin pair) each, over the eight channels; the buffer of a direction is reused two later
+__global__ void __launch_bounds__(448)
+k_g_last(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const bf2* __restrict__ in,
+         bf2* __restrict__ z) {
+    extern __shared__ __align__(16) unsigned char last_smem[];
+    float2 (*sl)[SL] = reinterpret_cast<float2 (*)[SL]>(last_smem);                        // [72]
+    float2 (*sg)[SL] = sl + 72;                                                            // [2][8 * 12]
+    float2 (*sw)[16] = reinterpret_cast<float2 (*)[16]>(sg + 2 * 96);                      // [9 * 8] weights
+    int (*snb)[SL] = reinterpret_cast<int (*)[SL]>(sw + 72);                               // [8]
+    bf2 (*so)[12] = reinterpret_cast<bf2 (*)[12]>(snb + 8);                                // [SL] results
+    const int vol = gm.vol, x0 = blockIdx.x * SL;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, x = x0 + lane;
+    const bool live = x < vol;
+    stage_links<false>(gm, u, x0, sl, snb);
+    for (int t = threadIdx.x; t < 72 * 16; t += blockDim.x) sw[t / 16][t % 16] = __bfloat1622float2(W[t]);
+    __syncthreads();
+    const bool producer = warp < 8;
+    if (producer && live) stage_gather(in + (size_t)warp * vol * 12, x, 0, sl, snb, lane, sg + 12 * warp);
+    const int cw = warp - 8, c = cw % 3, s0 = cw < 3 ? 0 : 2;   // consumer: spins s0, s0 + 1 of colour c
+    float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+#pragma unroll 1
     for (int d = 0; d < 9; d++) {
-        const AdjHop hp = adj_hop(y, d, nb);
-        float2 dg[4][3];
+        __syncthreads();
+        if (producer) {
+            if (d < 8 && live)
+                stage_gather(in + (size_t)warp * vol * 12, x, d + 1, sl, snb, lane, sg + ((d + 1) & 1) * 96 + 12 * warp);
+        } else {
+            const float2 (*g)[SL] = sg + (d & 1) * 96;
 #pragma unroll
-        for (int s = 0; s < 4; s++)
-#pragma unroll
-            for (int c = 0; c < 3; c++) dg[s][c] = make_float2(0.f, 0.f);
-        for (int co = 0; co < CO; co++) {
-            float2 dv[12];
-            ld_site(site_ptr(dout, co, vol, hp.z), dv);
-            const bf2* w = W + (((size_t)d * CO + co) * CI + ci) * 16;
-#pragma unroll
-            for (int s = 0; s < 4; s++)
+            for (int ci = 0; ci < 8; ci++) {
+                const float2* w = sw[d * 8 + ci];
 #pragma unroll
                 for (int sp = 0; sp < 4; sp++) {
-                    const float2 ww = __bfloat1622float2(w[4 * s + sp]);
-#pragma unroll
-                    for (int c = 0; c < 3; c++) dg[sp][c] = cfma_conj(ww, dv[3 * s + c], dg[sp][c]);
+                    const float2 gv = g[12 * ci + 3 * sp + c][lane];
+                    a0 = cfma(w[4 * s0 + sp], gv, a0);
+                    a1 = cfma(w[4 * s0 + 4 + sp], gv, a1);
                 }
-        }
-        if (d == 0) {
-#pragma unroll
-            for (int s = 0; s < 4; s++)
-#pragma unroll
-                for (int c = 0; c < 3; c++) acc[s][c] = cadd(acc[s][c], dg[s][c]);
-        } else {
-#pragma unroll
-            for (int s = 0; s < 4; s++) {
-                float2 o[3];
-                apply_link_adj(u, vol, y, d, hp, dg[s], o);
-#pragma unroll
-                for (int c = 0; c < 3; c++) acc[s][c] = cadd(acc[s][c], o[c]);
             }
         }
     }
+    if (!producer) {
+        so[lane][3 * s0 + c] = __float22bfloat162_rn(a0);
+        so[lane][3 * s0 + 3 + c] = __float22bfloat162_rn(a1);
+    }
+    __syncthreads();
+    // the block's results are contiguous in z: [site][12]
+    const int cnt = min(SL, vol - x0) * 12;
+    for (int t = threadIdx.x; t < cnt; t += blockDim.x) z[(size_t)x0 * 12 + t] = so[t / 12][t % 12];
+}
+
+constexpr size_t kLastSmem = (72 + 2 * 96) * SL * sizeof(float2) + 72 * 16 * sizeof(float2) + 8 * SL * sizeof(int) +
+                             SL * 12 * sizeof(bf2);
+
+// backward through the data of layer 3: din[ci](y) = sum_d adjoint transport of W_d^dag dout (a warp per ci),
+// times the ReLU mask of zprev; links, weights and the neighbours' dout come from shared memory
+__global__ void __launch_bounds__(256)
+k_g_bwd_data(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const bf2* __restrict__ dout,
+             const bf2* __restrict__ zprev, bf2* __restrict__ din) {
+    __shared__ float2 sl[72][SL];
+    __shared__ int snb[8][SL];
+    __shared__ float2 sd[3][12][SL];   // dout of direction d at d % 3
+    const int vol = gm.vol, y0 = blockIdx.x * SL;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, y = y0 + lane;
+    const bool live = y < vol;
+    stage_links<true>(gm, u, y0, sl, snb);
+    __syncthreads();
+    // the warps take turns to widen a direction's dout, two directions ahead
+    auto fetch = [&](int d) {
+        if (warp == d % 8 && live) {
+            float2 v[12];
+            ld_site(dout + (size_t)(d == 0 ? y : snb[d - 1][lane]) * 12, v);
+#pragma unroll
+            for (int k = 0; k < 12; k++) sd[d % 3][k][lane] = v[k];
+        }
+    };
+    fetch(0);
+    fetch(1);
+    float2 acc[4][3];
+#pragma unroll
+    for (int k = 0; k < 12; k++) acc[k / 3][k % 3] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int d = 0; d < 9; d++) {
+        __syncthreads();
+        if (d + 2 < 9) fetch(d + 2);
+        if (!live) continue;
+        float2 w[16], dg[4][3];
+        load_w(W + ((size_t)d * 8 + warp) * 16, w);
+#pragma unroll
+        for (int k = 0; k < 12; k++) dg[k / 3][k % 3] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int s = 0; s < 4; s++)
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const float2 dv = sd[d % 3][3 * s + c][lane];
+#pragma unroll
+                for (int sp = 0; sp < 4; sp++) dg[sp][c] = cfma_conj(w[4 * s + sp], dv, dg[sp][c]);
+            }
+#pragma unroll
+        for (int s = 0; s < 4; s++) {
+            float2 o[3];
+            if (d == 0) {
+#pragma unroll
+                for (int c = 0; c < 3; c++) o[c] = dg[s][c];
+            } else {
+                // direction +mu (odd d) comes back over the adjoint link
+                staged_link(sl + (d - 1) * 9, lane, d & 1, dg[s], o);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; c++) acc[s][c] = cadd(acc[s][c], o[c]);
+        }
+    }
+    if (!live) return;
     float2 v[12], zz[12];
-    ld_site(site_ptr(zprev, ci, vol, y), zz);
+    ld_site(site_ptr(zprev, warp, vol, y), zz);
 #pragma unroll
     for (int k = 0; k < 12; k++) {
         const float2 a = acc[k / 3][k % 3];
         v[k] = make_float2(zz[k].x > 0.f ? a.x : 0.f, zz[k].y > 0.f ? a.y : 0.f);
     }
-    st_site(site_ptr(din, ci, vol, y), v);
+    st_site(site_ptr(din, warp, vol, y), v);
 }
 
-// backward to the weights: dW[d][co][ci][s][s'] = sum_{x,c} dout[co](x)[s][c] conj(g_d(a_ci)(x)[s'][c])
-// block (d, slice of sites); the slice's gathered inputs and output gradients are
-// staged in shared memory 32 sites at a time; each thread owns output entries and
-// accumulates over the slice; partials [slice][9][CO][CI][16]
-template <int CI, int CO>
-__global__ void __launch_bounds__(kG)
-k_g_bwd_w(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ a, const bf2* __restrict__ dout,
-          int sites_per_slice, float2* __restrict__ part) {
-    constexpr int S = 32;
-    constexpr int NO = CO * CI * 16;
-    __shared__ float2 sg[S][3][CI * 4];   // [site][colour][ci*4 + s']
-    __shared__ float2 sd[S][3][CO * 4];   // [site][colour][co*4 + s]
-    const int d = blockIdx.x;
-    const int slice = blockIdx.y;
-    const int vol = gm.vol;
-    const int x0 = slice * sites_per_slice;
-    const int x1 = min(x0 + sites_per_slice, vol);
-    constexpr int PER = (NO + kG - 1) / kG;
-    float2 acc[PER];
-#pragma unroll
-    for (int k = 0; k < PER; k++) acc[k] = make_float2(0.f, 0.f);
-    for (int xs = x0; xs < x1; xs += S) {
-        const int cnt = min(S, x1 - xs);
-        __syncthreads();
-        for (int w = threadIdx.x; w < S * (CI + CO); w += blockDim.x) {
-            const int j = w % S, ch = w / S;
-            const int x = xs + j;
-            if (j >= cnt) continue;
-            const Nbr nb = neighbours(gm, x);
-            if (ch < CI) {
-                float2 g[4][3];
-                gather(u, a + (size_t)ch * vol * 12, vol, x, d, nb, g);
-#pragma unroll
-                for (int s = 0; s < 4; s++)
-#pragma unroll
-                    for (int c = 0; c < 3; c++) sg[j][c][ch * 4 + s] = g[s][c];
-            } else {
-                const int co = ch - CI;
-                float2 dv[12];
-                ld_site(site_ptr(dout, co, vol, x), dv);
-#pragma unroll
-                for (int k = 0; k < 12; k++) sd[j][k % 3][co * 4 + k / 3] = dv[k];
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < PER; k++) {
-            const int o = threadIdx.x + k * kG;
-            if (o < NO) {
-                // o = ((co*CI + ci)*4 + s)*4 + sp
-                const int sp = o % 4, s = (o / 4) % 4, ci = (o / 16) % CI, co = o / (16 * CI);
-                float2 v = acc[k];
-                for (int j = 0; j < cnt; j++)
-#pragma unroll
-                    for (int c = 0; c < 3; c++)
-                        v = cfma_conj(sg[j][c][ci * 4 + sp], sd[j][c][co * 4 + s], v);
-                acc[k] = v;
-            }
-        }
-    }
-    float2* out = part + ((size_t)slice * 9 + d) * NO;
-#pragma unroll
-    for (int k = 0; k < PER; k++) {
-        const int o = threadIdx.x + k * kG;
-        if (o < NO) out[o] = acc[k];
-    }
-}
-
-// grad[e] += sum over slices of part[slice][e]  (e over 9*NO entries), in FP64
-__global__ void k_g_reduce_w(const float2* __restrict__ part, int nslice, int ne,
-                             double2* __restrict__ grad) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= ne) return;
+// grad[e] += sum over slices of part[slice][e]  (e over 9*NO entries), in FP64: eight threads per entry,
+// each over every eighth slice, added in a fixed order (one thread per entry walked 128 slices: 40 us)
+__global__ void __launch_bounds__(256)
+k_g_reduce_w(const float2* __restrict__ part, int nslice, int ne, double2* __restrict__ grad) {
+    __shared__ double2 sh[8][32];
+    const int el = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + el;
     double re = 0.0, im = 0.0;
-    for (int p = 0; p < nslice; p++) {
-        const float2 z = part[(size_t)p * ne + e];
-        re += z.x;
-        im += z.y;
+    if (e < ne)
+        for (int p = q; p < nslice; p += 8) {
+            const float2 z = part[(size_t)p * ne + e];
+            re += z.x;
+            im += z.y;
+        }
+    sh[q][el] = make_double2(re, im);
+    __syncthreads();
+    if (q == 0 && e < ne) {
+        for (int k = 1; k < 8; k++) {
+            re += sh[k][el].x;
+            im += sh[k][el].y;
+        }
+        grad[e].x += re;
+        grad[e].y += im;
     }
-    grad[e].x += re;
-    grad[e].y += im;
+}
+
+// byte offset of (row r, 16-byte chunk j) in a tile of 128-byte rows with 128-byte swizzle
+__device__ __forceinline__ uint32_t sw128(int r, int j) {
+    return (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + ((j ^ (r & 7)) << 4));
 }
 
 // ---------------------------------------------------------------------------
-// layer 2 on tcgen05 (see the file header).  One CTA = 128 sites, 256 threads.
+// backward to the weights on tcgen05:
+//   dW[d][co][ci][s][s'] = sum_{x,c} dout[co](x)[s][c] conj(g_d(a_ci)(x)[s'][c])
+// as real GEMMs with K = (site, colour): P[n][m] = sum g[n] dout[m], n = (ci, s', re/im), m = (co, s, re/im);
+// Re = P[r][r] + P[i][i], Im = P[r][i] - P[i][r].  Both operands are MN-major: a tile row is one site's 64 real
+// entries of one colour, which is how a thread (site, channel) has them, one 16-byte chunk.
+// dout is bf16.  The transported activations g are FP32 and stay so: they enter as three bf16 terms
+// hi + mid + lo (24 bits) in two MMAs, [hi; mid] in the 128 rows of A and [lo; 0] on top.  The FP32 sums of TMEM
+// run over TW_FLUSH tiles (24 accumulations each) and are then added to this CTA's partial in FP32, so that
+// a chain is no longer than the 3072-term FP32 chains of the SIMT kernel this replaced; k_g_reduce_w adds the
+// partials in FP64.
+// One CTA: 64-site tiles of a slice, 512 threads = 64 sites x 8 channels, directions 3y .. 3y+2 (CI = 8) or, for one
+// input channel (CI = 1), directions 1..8 in the place of the channels and direction 0 after them.  Two stage
+// buffers (72 KB each): the transport of the next direction overlaps the MMAs of this one; the transport bounds it.
+// 16^3 x 32: 8 -> 8 layer 2137 us on SIMT (the gather and 32 x 32 complex products per site from shared memory),
+// 8 -> 1 776 us, 1 -> 8 688 us; here see the launch.
+// ---------------------------------------------------------------------------
+constexpr int TW_SITES = 64;
+constexpr int TW_FLUSH = 4;
+constexpr uint32_t TW_TILE = TW_SITES * 128;             // 64 rows x 64 bf16
+constexpr uint32_t TW_STAGE = 9 * TW_TILE;               // 3 colours x (hi, mid, lo)
+constexpr uint32_t TW_SMEM = 2 * TW_STAGE + 2 * 3 * TW_TILE + TW_TILE + 1024 + 64;
+
+template <int CI, int CO>
+__global__ void __launch_bounds__(512, 1)
+k_g_tw(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ a, const bf2* __restrict__ dout,
+       float* __restrict__ part, int* __restrict__ err) {
+    using namespace tc;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* sG = smem;                                    // [2][3 colours][hi, mid, lo]
+    uint8_t* sD = sG + 2 * TW_STAGE;                       // [2][3 colours]
+    uint8_t* sZ = sD + 2 * 3 * TW_TILE;                    // zeros
+    uint64_t* done = reinterpret_cast<uint64_t*>(sZ + TW_TILE);   // [2]
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 2);
+    volatile int* s_fail = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    constexpr int ND = CI == 8 ? 3 : 2;                    // stages per tile
+    constexpr int NO = CO * CI * 16;
+    constexpr int NCOL = CO == 8 ? 64 : 16;                // columns of the MMA (8 used when CO = 1)
+    const int vol = gm.vol;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        mbar_init(&done[0], 1);
+        mbar_init(&done[1], 1);
+        *s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"(256u));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    for (int i = threadIdx.x; i < (int)(TW_TILE / 16); i += blockDim.x)
+        reinterpret_cast<uint4*>(sZ)[i] = make_uint4(0, 0, 0, 0);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_d = *tmem_slot;
+
+    const int row = threadIdx.x & (TW_SITES - 1), ch = threadIdx.x >> 6;
+    const int ntiles = (vol + TW_SITES - 1) / TW_SITES;
+    int q = 0, tcount = 0;
+    bool first = true, ok = true;
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, tcount++) {
+        const int x = t * TW_SITES + row;
+        const bool live = x < vol;
+        Nbr nb;
+        if (live) nb = neighbours(gm, x);
+        const uint32_t dbase = (tcount & 1) * 3 * TW_TILE;
+        for (int dl = 0; dl < ND; dl++, q++) {
+            const int b = q & 1;
+            // the MMAs that read buffer b (stage q - 2) and everything before them are done
+            if (q >= 2 && !mbar_wait(&done[b], (uint32_t)((q - 2) >> 1) & 1u)) *s_fail = 1;
+            __syncthreads();
+            if (*s_fail) {
+                ok = false;
+                break;
+            }
+            if (dl == 0 && ch < CO) {
+                float2 v[12];
+                uint4 w[3] = {};
+                if (live) {
+                    ld_site(site_ptr(dout, ch, vol, x), v);   // bf16 values: packing them again is exact
+#pragma unroll
+                    for (int c = 0; c < 3; c++)
+                        w[c] = make_uint4(pack_bf2(v[c]), pack_bf2(v[3 + c]), pack_bf2(v[6 + c]), pack_bf2(v[9 + c]));
+                }
+#pragma unroll
+                for (int c = 0; c < 3; c++)
+                    *reinterpret_cast<uint4*>(sD + dbase + c * TW_TILE + sw128(row, ch)) = w[c];
+            }
+            const int d = CI == 8 ? blockIdx.y * 3 + dl : dl == 0 ? 1 + ch : 0;
+            if (CI == 8 || dl == 0 || ch == 0) {
+                float2 g[4][3];
+                if (live) {
+                    gather(u, a + (CI == 8 ? (size_t)ch * vol * 12 : 0), vol, x, d, nb, g);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 12; k++) g[k / 3][k % 3] = make_float2(0.f, 0.f);
+                }
+                uint8_t* sb = sG + b * TW_STAGE;
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    unsigned w[3][4];
+#pragma unroll
+                    for (int s = 0; s < 4; s++) {
+                        float2 r = g[s][c];
+#pragma unroll
+                        for (int k = 0; k < 3; k++) {
+                            w[k][s] = pack_bf2(r);
+                            const float2 h = unpack_bf2(w[k][s]);
+                            r = make_float2(r.x - h.x, r.y - h.y);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < 3; k++)
+                        *reinterpret_cast<uint4*>(sb + (3 * c + k) * TW_TILE + sw128(row, ch)) =
+                            make_uint4(w[k][0], w[k][1], w[k][2], w[k][3]);
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                constexpr uint32_t idesc = umma_idesc_bf16(NCOL, 128) | UMMA_MN_MAJOR_AB;
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const uint32_t hi = smem_u32(sG + b * TW_STAGE + 3 * c * TW_TILE), lo = hi + 2 * TW_TILE;
+                    const uint32_t dd = smem_u32(sD + dbase + c * TW_TILE);
+#pragma unroll
+                    for (int kk = 0; kk < TW_SITES / 16; kk++) {
+                        const uint64_t db = umma_desc_mn_sw128(dd + kk * 2048, TW_TILE);
+                        umma_bf16(tmem_d + (uint32_t)(dl * 64), umma_desc_mn_sw128(hi + kk * 2048, TW_TILE), db, idesc,
+                                  (first && c == 0 && kk == 0) ? 0u : 1u);
+                        umma_bf16(tmem_d + (uint32_t)(dl * 64),
+                                  umma_desc_mn_sw128(lo + kk * 2048, smem_u32(sZ) - lo - kk * 2048), db, idesc, 1u);
+                    }
+                }
+                umma_commit(&done[b]);
+            }
+        }
+        if (!ok) break;
+        first = false;
+        const bool last = t + (int)gridDim.x >= ntiles;
+        if (tcount % TW_FLUSH == TW_FLUSH - 1 || last) {
+            if (!mbar_wait(&done[(q - 1) & 1], (uint32_t)((q - 1) >> 1) & 1u)) *s_fail = 1;
+            __syncwarp();
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int lg = warp & 3, cq = warp >> 2;
+            const int r = lg * 32 + lane, n = r & 63, half = r >> 6;
+            const int pt = n & 1, sp = (n >> 1) & 3, cn = n >> 3;
+            if (CO == 8 || cq == 0) {
+                for (int dl = 0; dl < ND; dl++) {
+                    float v[16];
+                    tmem_ld16<16>(tmem_d + ((uint32_t)(lg * 32) << 16) + (uint32_t)(dl * 64 + cq * 16), v);
+                    const int d = CI == 8 ? blockIdx.y * 3 + dl : dl == 0 ? 1 + cn : 0;
+                    const int ci = CI == 8 ? cn : 0;
+                    const bool used = CI == 8 || dl == 0 || cn == 0;
+                    float* out = part + (((size_t)(blockIdx.x * 2 + half) * 9 + d) * NO) * 2 + pt;
+#pragma unroll
+                    for (int j = 0; j < 8; j++) {
+                        // even column: re of dout, odd: im; this lane holds g's re (pt = 0) or im (pt = 1)
+                        const float o = __shfl_xor_sync(0xffffffffu, v[2 * j + 1], 1);
+                        const float z = pt == 0 ? v[2 * j] + o : o - v[2 * j];
+                        const int m = cq * 8 + j, co = m >> 2, s = m & 3;
+                        if (used && co < CO) {
+                            float* p = out + (size_t)(((co * CI + ci) * 4 + s) * 4 + sp) * 2;
+                            *p = tcount < TW_FLUSH ? z : *p + z;
+                        }
+                    }
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncthreads();
+            first = true;
+            if (*s_fail) ok = false;
+        }
+    }
+    if (!ok && threadIdx.x == 0) atomicExch(err, SEEDCG_ERR_TIMEOUT);
+    // on a timeout MMAs may still be in flight: wait for the last committed group (bounded) before TMEM is freed
+    if (!ok && q > 0) mbar_wait(&done[(q - 1) & 1], (uint32_t)((q - 1) >> 1) & 1u);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(256u));
+    }
+}
+
+// ---------------------------------------------------------------------------
+// layer 2 on tcgen05 (see the file header).  One CTA = 128 sites, 512 threads (two channels each).
 // MODE 0 (forward):  A = U(x,d) h1_ci(x+d), B = W in real form; epilogue z2, h2 = ReLU(z2).
 // MODE 1 (backward through the data): A = adjoint transport of d2_co, B = W^dag in
 //        real form; epilogue d1 = D masked by z1 > 0 (real and imaginary parts).
@@ -358,13 +597,8 @@ constexpr uint32_t TC_B_BYTES = 64 * 128;            // 64 rows x 64 bf16
 constexpr uint32_t TC_SMEM = 2 * 3 * TC_A_BYTES + 2 * TC_B_BYTES + 1024 + 256;
 constexpr uint32_t TC_TMEM_COLS = 256;               // 3 colours x 64 columns
 
-// byte offset of (row r, 16-byte chunk j) in a K-major 128-byte-swizzled tile
-__device__ __forceinline__ uint32_t sw128(int r, int j) {
-    return (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + ((j ^ (r & 7)) << 4));
-}
-
 template <int MODE>
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(512, 1)
 k_g_tc(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ in, const uint4* __restrict__ wimg,
        const bf2* __restrict__ zprev, bf2* __restrict__ out0, bf2* __restrict__ out1, int* __restrict__ err) {
     using namespace tc;
@@ -394,9 +628,9 @@ k_g_tc(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ in, const 
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_d = *tmem_slot;
 
-    // this thread's site and half of the input channels
+    // this thread's site and quarter of the input channels
     const int row = threadIdx.x & (TC_SITES - 1);
-    const int half = threadIdx.x >> 7;
+    const int quarter = threadIdx.x >> 7;
     const int x = x0 + row;
     const bool live = x < vol;
     Nbr nb;
@@ -416,7 +650,7 @@ k_g_tc(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ in, const 
             uint4* dst = reinterpret_cast<uint4*>(sB + b * TC_B_BYTES);
             for (int i = threadIdx.x; i < (int)(TC_B_BYTES / 16); i += blockDim.x) dst[i] = __ldg(src + i);
         }
-        // A: the transported activations of channels [4 half, 4 half + 4) at this site
+        // A: the transported activations of channels 2 quarter and 2 quarter + 1 at this site
         float2 lk[9];   // the link of this direction at this site (already with its sign)
         int src_site = x;
         float sgn = 1.f;
@@ -440,8 +674,8 @@ k_g_tc(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ in, const 
             for (int e = 0; e < 9; e++) lk[e] = __ldg(u + (size_t)(mu * 9 + e) * vol + lsite);
         }
 #pragma unroll 1
-        for (int q = 0; q < 4; q++) {
-            const int ch = 4 * half + q;
+        for (int q = 0; q < 2; q++) {
+            const int ch = 2 * quarter + q;
             float2 v[12];
             if (live) {
                 ld_site(site_ptr(in, ch, vol, src_site), v);
@@ -502,15 +736,15 @@ k_g_tc(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ in, const 
     __syncthreads();
     if (*s_fail || issued < 9) {
         if (threadIdx.x == 0) atomicExch(err, SEEDCG_ERR_TIMEOUT);
-    } else if (warp < 4) {
-        // warp w reads TMEM lanes [32 w, 32 w + 32): the rows (sites) of its threads
-        const int r = warp * 32 + lane;
+    } else {
+        // warp w reads TMEM lanes [32 (w % 4), + 32), the rows (sites) of its threads, for two output channels
+        const int lg = warp & 3, r = lg * 32 + lane;
         const int xs = x0 + r;
-        for (int o = 0; o < 8; o++) {
+        for (int o = 2 * (warp >> 2); o < 2 * (warp >> 2) + 2; o++) {
             float cv[3][8];
 #pragma unroll
             for (int c = 0; c < 3; c++)
-                tmem_ld8(tmem_d + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * 64 + o * 8), cv[c]);
+                tmem_ld8(tmem_d + ((uint32_t)(lg * 32) << 16) + (uint32_t)(c * 64 + o * 8), cv[c]);
             if (xs < vol) {
                 float2 z[12];
 #pragma unroll
@@ -521,7 +755,7 @@ k_g_tc(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ in, const 
                     float2 hr[12];
 #pragma unroll
                     for (int k = 0; k < 12; k++) hr[k] = make_float2(fmaxf(z[k].x, 0.f), fmaxf(z[k].y, 0.f));
-                    st_site(site_ptr(out0, o, vol, xs), z);
+                    if (out0) st_site(site_ptr(out0, o, vol, xs), z);   // not kept for inference
                     st_site(site_ptr(out1, o, vol, xs), hr);
                 } else {
                     float2 zz[12];
@@ -644,8 +878,6 @@ __global__ void k_g_round(const float2* __restrict__ W, bf2* __restrict__ Wb, in
     if (e < ne) Wb[e] = __float22bfloat162_rn(W[e]);
 }
 
-inline int gblocks(long n) { return (int)((n + kG - 1) / kG); }
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -731,9 +963,9 @@ void layer2_tc(seedcg_handle* h, GuessState* G, int mode, const bf2* in, const b
         attr[mode] = true;
     }
     if (mode == 0)
-        k_g_tc<0><<<blocks, 256, TC_SMEM, st>>>(gm, h->u32.as<float2>(), in, img, zprev, out0, out1, err);
+        k_g_tc<0><<<blocks, 512, TC_SMEM, st>>>(gm, h->u32.as<float2>(), in, img, zprev, out0, out1, err);
     else
-        k_g_tc<1><<<blocks, 256, TC_SMEM, st>>>(gm, h->u32.as<float2>(), in, img, zprev, out0, out1, err);
+        k_g_tc<1><<<blocks, 512, TC_SMEM, st>>>(gm, h->u32.as<float2>(), in, img, zprev, out0, out1, err);
     SEEDCG_CHECK_LAUNCH();
 }
 
@@ -751,7 +983,8 @@ void check_tc(const Acts& A, cudaStream_t st) {
     if (e) throw Error{SEEDCG_ERR_TIMEOUT, "a tensor-core wait of the learned guess expired"};
 }
 
-void forward(seedcg_handle* h, GuessState* G, const Acts& A, const double2* b64, cudaStream_t st) {
+// keep_z: the backward pass will need the pre-activations z1, z2
+void forward(seedcg_handle* h, GuessState* G, const Acts& A, const double2* b64, bool keep_z, cudaStream_t st) {
     const Geom& gm = h->g;
     const long n = 12L * gm.vol;
     const float2* u = h->u32.as<float2>();
@@ -761,26 +994,34 @@ void forward(seedcg_handle* h, GuessState* G, const Acts& A, const double2* b64,
     k_norm2_public(b64, n, partials, ctr, A.nb, st);
     k_g_scale_in<<<std::min<long>((n + 255) / 256, 4096), 256, 0, st>>>(b64, A.nb, A.a0, gm.vol);
     SEEDCG_CHECK_LAUNCH();
-    k_g_fwd<1, 8><<<gblocks(8L * gm.vol), kG, 0, st>>>(gm, u, W, A.a0, A.z1, A.h1, 1);
+    const int tiles = (gm.vol + SL - 1) / SL;
+    k_g_first<<<tiles, 288, 0, st>>>(gm, u, W, A.a0, keep_z ? A.z1 : nullptr, A.h1);
     SEEDCG_CHECK_LAUNCH();
-    layer2_tc(h, G, 0, A.h1, nullptr, A.z2, A.h2, A.tc_err, st);
-    k_g_fwd<8, 1><<<gblocks((long)gm.vol), kG, 0, st>>>(gm, u, W + GuessState::NW1 + GuessState::NW2, A.h2, A.z3,
-                                                        A.z3, 0);
+    layer2_tc(h, G, 0, A.h1, nullptr, keep_z ? A.z2 : nullptr, A.h2, A.tc_err, st);
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_g_last, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLastSmem);
+    SEEDCG_CUDA_TRY(attr);
+    k_g_last<<<tiles, 448, kLastSmem, st>>>(gm, u, W + GuessState::NW1 + GuessState::NW2, A.h2, A.z3);
     SEEDCG_CHECK_LAUNCH();
 }
 
 template <int CI, int CO>
-void weight_grad(seedcg_handle* h, GuessState* G, const bf2* a, const bf2* dout, double2* grad, cudaStream_t st) {
+void weight_grad(seedcg_handle* h, GuessState* G, const bf2* a, const bf2* dout, double2* grad, int* err,
+                 cudaStream_t st) {
     const Geom& gm = h->g;
-    const int per = 1024;
-    const int nslice = (gm.vol + per - 1) / per;
+    // one CTA per SM: the directions' three groups share the chip (CI = 8)
+    const int ntiles = (gm.vol + TW_SITES - 1) / TW_SITES;
+    const int groups = CI == 8 ? 3 : 1;
+    const int nslice = std::min(ntiles, 152 / groups);
     constexpr int NO = CO * CI * 16;
     const size_t ne = (size_t)9 * NO;
-    G->part.ensure((size_t)nslice * ne * sizeof(float2));
-    dim3 grid(9, nslice);
-    k_g_bwd_w<CI, CO><<<grid, kG, 0, st>>>(gm, h->u32.as<float2>(), a, dout, per, G->part.as<float2>());
+    G->part.ensure((size_t)nslice * 2 * ne * sizeof(float2));
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_g_tw<CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TW_SMEM);
+    SEEDCG_CUDA_TRY(attr);
+    k_g_tw<CI, CO><<<dim3(nslice, groups), 512, TW_SMEM, st>>>(gm, h->u32.as<float2>(), a, dout, G->part.as<float>(), err);
     SEEDCG_CHECK_LAUNCH();
-    k_g_reduce_w<<<(int)((ne + 255) / 256), 256, 0, st>>>(G->part.as<float2>(), nslice, (int)ne, grad);
+    k_g_reduce_w<<<(int)((ne + 31) / 32), 256, 0, st>>>(G->part.as<float2>(), 2 * nslice, (int)ne, grad);
     SEEDCG_CHECK_LAUNCH();
 }
 
@@ -799,15 +1040,15 @@ void backward_pair(seedcg_handle* h, GuessState* G, const Acts& A, const double2
                                                                              A.d3, gm.vol, partials, ctr + 1, A.loss);
     SEEDCG_CHECK_LAUNCH();
     // layer 3 (8 -> 1)
-    weight_grad<8, 1>(h, G, A.h2, A.d3, grad + GuessState::NW1 + GuessState::NW2, st);
-    k_g_bwd_data<8, 1><<<gblocks(8L * gm.vol), kG, 0, st>>>(gm, u, W + GuessState::NW1 + GuessState::NW2, A.d3,
-                                                            A.z2, A.d2);
+    weight_grad<8, 1>(h, G, A.h2, A.d3, grad + GuessState::NW1 + GuessState::NW2, A.tc_err, st);
+    k_g_bwd_data<<<(gm.vol + SL - 1) / SL, 256, 0, st>>>(gm, u, W + GuessState::NW1 + GuessState::NW2, A.d3, A.z2,
+                                                         A.d2);
     SEEDCG_CHECK_LAUNCH();
     // layer 2 (8 -> 8)
-    weight_grad<8, 8>(h, G, A.h1, A.d2, grad + GuessState::NW1, st);
+    weight_grad<8, 8>(h, G, A.h1, A.d2, grad + GuessState::NW1, A.tc_err, st);
     layer2_tc(h, G, 1, A.d2, A.z1, A.d1, nullptr, A.tc_err, st);
     // layer 1 (1 -> 8): only the weight gradient is needed
-    weight_grad<1, 8>(h, G, A.a0, A.d1, grad, st);
+    weight_grad<1, 8>(h, G, A.a0, A.d1, grad, A.tc_err, st);
 }
 
 }  // namespace
@@ -854,7 +1095,7 @@ double guess_loss_grad(seedcg_handle* h, int npairs, const double2* B, const dou
     SEEDCG_CUDA_TRY(cudaMemsetAsync(G->grad.p, 0, GuessState::NW * sizeof(double2), st));
     SEEDCG_CUDA_TRY(cudaMemsetAsync(A.nb, 0, G->scal.bytes, st));
     for (int k = 0; k < npairs; k++) {
-        forward(h, G, A, B + (size_t)k * n, st);
+        forward(h, G, A, B + (size_t)k * n, true, st);
         backward_pair(h, G, A, X + (size_t)k * n, 1.0 / npairs, st);
     }
     double loss = 0.0;
@@ -901,7 +1142,7 @@ void guess_predict(seedcg_handle* h, int n_fields, const double2* B, double2* X0
     Acts A = carve_acts(G, h->g.vol);
     SEEDCG_CUDA_TRY(cudaMemsetAsync(A.nb, 0, G->scal.bytes, st));
     for (int k = 0; k < n_fields; k++) {
-        forward(h, G, A, B + (size_t)k * n, st);
+        forward(h, G, A, B + (size_t)k * n, false, st);
         k_g_scale_out<<<std::min<long>((n + 255) / 256, 4096), 256, 0, st>>>(A.z3, A.nb, X0 + (size_t)k * n,
                                                                             h->g.vol);
         SEEDCG_CHECK_LAUNCH();

@@ -70,6 +70,19 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
     d |= (uint64_t)2 << 61;                           // SWIZZLE_128B
     return d;
 }
+// MN-major, 128-byte swizzle: rows of 64 MN elements (128 B), one per k; 8-k groups 1024 B apart,
+// the next 64 MN elements lbo bytes on
+__device__ __forceinline__ uint64_t umma_desc_mn_sw128(uint32_t saddr, uint32_t lbo) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr >> 4) & 0x3FFF);
+    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
+    d |= (uint64_t)(1024 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+constexpr uint32_t UMMA_MN_MAJOR_AB = (1u << 15) | (1u << 16);   // instruction descriptor: A and B MN-major
+
 // instruction descriptor: kind::f16, A = B = bf16, D = f32, both K-major, M = m, N = n
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int n, int m = 128) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
