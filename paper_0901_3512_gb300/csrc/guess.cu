@@ -78,45 +78,87 @@ __device__ __forceinline__ bf2* site_ptr(bf2* a, int ch, int vol, int x) {
     return a + ((size_t)ch * vol + x) * 12;
 }
 
-// U(x,d) applied to colour vector v (3 complex), with the boundary sign
-__device__ __forceinline__ void apply_link(const float2* __restrict__ u, int vol, int x, int d,
-                                           const Nbr& nb, const float2 v[3], float2 o[3]) {
-    const int mu = (d - 1) >> 1;
-    const bool back = (d - 1) & 1;
-    const float sg = (mu == 3 && (back ? nb.bwrap_t : nb.fwrap_t)) ? -1.f : 1.f;
-    const int site = back ? nb.b[mu] : x;
+// Where direction d's term at site x comes from: the activation of site src, carried by the link at site
+// lsite in direction mu (its adjoint when dag), times sg.  ADJ: the adjoint transport of the backward pass
+// through the data (the hop from src in direction d, seen from x).
+struct HopFrom {
+    int src, lsite, mu;
+    bool dag;
+    float sg;
+};
+template <bool ADJ>
+__device__ __forceinline__ HopFrom hop_from(const Geom& g, int x, int d) {
+    HopFrom h{x, x, 0, false, 1.f};
+    if (d == 0) return h;
+    h.mu = (d - 1) >> 1;
+    const bool back = ((d - 1) & 1) != (ADJ ? 1 : 0);   // src = x - mu
+    const int str = h.mu == 0 ? g.stride[0] : h.mu == 1 ? g.stride[1] : h.mu == 2 ? g.stride[2] : g.stride[3];
+    const int ext = h.mu == 0 ? g.L[0] : h.mu == 1 ? g.L[1] : h.mu == 2 ? g.L[2] : g.L[3];
+    const int c = (x / str) % ext;
+    const bool wrap = back ? c == 0 : c == ext - 1;
+    h.src = back ? (wrap ? x + (ext - 1) * str : x - str) : (wrap ? x - (ext - 1) * str : x + str);
+    h.lsite = back ? h.src : x;
+    h.dag = back;
+    h.sg = h.mu == 3 && wrap ? -1.f : 1.f;
+    return h;
+}
+
+// One thread's loads for a direction, issued ahead of their use: the link and NCH channels of the source site
+template <int NCH>
+struct HopLoad {
+    float2 lk[9];
+    uint4 act[NCH][3];
+    bool dag;
+    float sg;
+};
+template <bool ADJ, int NCH>
+__device__ __forceinline__ void hop_load(HopLoad<NCH>& p, const Geom& g, const float2* __restrict__ u,
+                                         const bf2* __restrict__ in, int ch0, int x, int d) {
+    const HopFrom h = hop_from<ADJ>(g, x, d);
+    p.dag = h.dag;
+    p.sg = h.sg;
+#pragma unroll
+    for (int k = 0; k < NCH; k++) {
+        const uint4* q = reinterpret_cast<const uint4*>(site_ptr(in, ch0 + k, g.vol, h.src));
+#pragma unroll
+        for (int j = 0; j < 3; j++) p.act[k][j] = __ldg(q + j);
+    }
+    if (d > 0) {
+        const float2* l = u + (size_t)(h.mu * 9) * g.vol + h.lsite;
+#pragma unroll
+        for (int e = 0; e < 9; e++) p.lk[e] = __ldg(l + (size_t)e * g.vol);
+    }
+}
+// the link as the matrix that transports colour vectors (sign and adjoint applied)
+template <int NCH>
+__device__ __forceinline__ void hop_matrix(const HopLoad<NCH>& p, float2 (&m)[9]) {
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int b = 0; b < 3; b++) {
+            const float2 z = p.dag ? p.lk[3 * b + a] : p.lk[3 * a + b];
+            m[3 * a + b] = make_float2(p.sg * z.x, p.dag ? -p.sg * z.y : p.sg * z.y);
+        }
+}
+__device__ __forceinline__ void unpack_site(const uint4 (&w)[3], float2 (&o)[12]) {
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        o[4 * j + 0] = unpack_bf2(w[j].x);
+        o[4 * j + 1] = unpack_bf2(w[j].y);
+        o[4 * j + 2] = unpack_bf2(w[j].z);
+        o[4 * j + 3] = unpack_bf2(w[j].w);
+    }
+}
+
+// o = m v
+__device__ __forceinline__ void colour_mul(const float2 (&m)[9], const float2* v, float2* o) {
 #pragma unroll
     for (int a = 0; a < 3; a++) {
         float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int b = 0; b < 3; b++) {
-            if (!back) {
-                const float2 uu = __ldg(u + (size_t)(mu * 9 + 3 * a + b) * vol + site);
-                acc = cfma(uu, v[b], acc);
-            } else {
-                const float2 uu = __ldg(u + (size_t)(mu * 9 + 3 * b + a) * vol + site);
-                acc = cfma_conj(uu, v[b], acc);
-            }
-        }
-        o[a] = make_float2(sg * acc.x, sg * acc.y);
+        for (int b = 0; b < 3; b++) acc = cfma(m[3 * a + b], v[b], acc);
+        o[a] = acc;
     }
-}
-
-// gathered input g_d(x) of one channel: 4 spins x 3 colours
-__device__ __forceinline__ void gather(const float2* __restrict__ u, const bf2* __restrict__ in_ch, int vol,
-                                       int x, int d, const Nbr& nb, float2 g[4][3]) {
-    float2 v[12];
-    if (d == 0) {
-        ld_site(in_ch + (size_t)x * 12, v);
-#pragma unroll
-        for (int k = 0; k < 12; k++) g[k / 3][k % 3] = v[k];
-        return;
-    }
-    const int mu = (d - 1) >> 1;
-    const int y = ((d - 1) & 1) ? nb.b[mu] : nb.f[mu];
-    ld_site(in_ch + (size_t)y * 12, v);
-#pragma unroll
-    for (int s = 0; s < 4; s++) apply_link(u, vol, x, d, nb, &v[3 * s], g[s]);
 }
 
 // ---------------------------------------------------------------------------
@@ -153,18 +195,15 @@ __device__ __forceinline__ void stage_links(const Geom& gm, const float2* __rest
     }
 }
 
-// o = L v or L^dag v, L[a][b] = sl[3 a + b][lane]
-__device__ __forceinline__ void staged_link(const float2 (*sl)[SL], int lane, bool dag, const float2 v[3], float2 o[3]) {
+// the matrix that transports colour vectors, in registers: L or L^dag with L[a][b] = sl[3 a + b][lane]
+__device__ __forceinline__ void staged_link(const float2 (*sl)[SL], int lane, bool dag, float2 (&m)[9]) {
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        float2 acc = make_float2(0.f, 0.f);
+    for (int a = 0; a < 3; a++)
 #pragma unroll
         for (int b = 0; b < 3; b++) {
-            if (!dag) acc = cfma(sl[3 * a + b][lane], v[b], acc);
-            else acc = cfma_conj(sl[3 * b + a][lane], v[b], acc);
+            const float2 z = sl[dag ? 3 * b + a : 3 * a + b][lane];
+            m[3 * a + b] = make_float2(z.x, dag ? -z.y : z.y);
         }
-        o[a] = acc;
-    }
 }
 
 // g_d(x) of one channel into sg[12][lane]
@@ -177,13 +216,12 @@ __device__ __forceinline__ void stage_gather(const bf2* __restrict__ in_ch, int 
         for (int k = 0; k < 12; k++) sg[k][lane] = v[k];
         return;
     }
+    float2 m[9], o[12];
+    staged_link(sl + (d - 1) * 9, lane, (d - 1) & 1, m);
 #pragma unroll
-    for (int s = 0; s < 4; s++) {
-        float2 o[3];
-        staged_link(sl + (d - 1) * 9, lane, (d - 1) & 1, &v[3 * s], o);
+    for (int s = 0; s < 4; s++) colour_mul(m, &v[3 * s], &o[3 * s]);
 #pragma unroll
-        for (int c = 0; c < 3; c++) sg[3 * s + c][lane] = o[c];
-    }
+    for (int k = 0; k < 12; k++) sg[k][lane] = o[k];
 }
 
 __device__ __forceinline__ void load_w(const bf2* __restrict__ w, float2 (&o)[16]) {
@@ -199,7 +237,8 @@ __device__ __forceinline__ void load_w(const bf2* __restrict__ w, float2 (&o)[16
 }
 
 // layer 1 (1 -> 8): nine warps transport one direction each, then eight warps run one output channel each.
-// z may be null (inference needs h = ReLU(z) only).  16^3 x 32: see the launch.
+// z may be null (inference needs h = ReLU(z) only).  16^3 x 32: 294 us with a thread per (site, output
+// channel), 108 us here.
 __global__ void __launch_bounds__(288)
 k_g_first(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const bf2* __restrict__ in,
           bf2* __restrict__ z, bf2* __restrict__ h) {
@@ -241,7 +280,8 @@ k_g_first(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, cons
 }
 
 // layer 3 (8 -> 1): eight warps transport one input channel each for direction d + 1 while six warps add
-// direction d, a (colour, spin pair) each, over the eight channels; the buffer of a direction is reused two later
+// direction d, a (colour, spin pair) each, over the eight channels; the buffer of a direction is reused two later.
+// 16^3 x 32: 346 us with one thread per site, 214 us here (issue 62 % busy, shared memory 74 %).
 __global__ void __launch_bounds__(448)
 k_g_last(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const bf2* __restrict__ in,
          bf2* __restrict__ z) {
@@ -255,7 +295,9 @@ k_g_last(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, x = x0 + lane;
     const bool live = x < vol;
     stage_links<false>(gm, u, x0, sl, snb);
-    for (int t = threadIdx.x; t < 72 * 16; t += blockDim.x) sw[t / 16][t % 16] = __bfloat1622float2(W[t]);
+    // weights [d][ci][input spin][output spin]: one 16-byte load gives the two output spins of a warp
+    for (int t = threadIdx.x; t < 72 * 16; t += blockDim.x)
+        sw[t / 16][(t % 4) * 4 + (t / 4) % 4] = __bfloat1622float2(W[t]);
     __syncthreads();
     const bool producer = warp < 8;
     if (producer && live) stage_gather(in + (size_t)warp * vol * 12, x, 0, sl, snb, lane, sg + 12 * warp);
@@ -275,8 +317,9 @@ k_g_last(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const
 #pragma unroll
                 for (int sp = 0; sp < 4; sp++) {
                     const float2 gv = g[12 * ci + 3 * sp + c][lane];
-                    a0 = cfma(w[4 * s0 + sp], gv, a0);
-                    a1 = cfma(w[4 * s0 + 4 + sp], gv, a1);
+                    const float4 ww = *reinterpret_cast<const float4*>(w + 4 * sp + s0);
+                    a0 = cfma(make_float2(ww.x, ww.y), gv, a0);
+                    a1 = cfma(make_float2(ww.z, ww.w), gv, a1);
                 }
             }
         }
@@ -295,7 +338,7 @@ constexpr size_t kLastSmem = (72 + 2 * 96) * SL * sizeof(float2) + 72 * 16 * siz
                              SL * 12 * sizeof(bf2);
 
 // backward through the data of layer 3: din[ci](y) = sum_d adjoint transport of W_d^dag dout (a warp per ci),
-// times the ReLU mask of zprev; links, weights and the neighbours' dout come from shared memory
+// times the ReLU mask of zprev; links and the neighbours' dout come from shared memory.  16^3 x 32: 410 -> 188 us.
 __global__ void __launch_bounds__(256)
 k_g_bwd_data(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const bf2* __restrict__ dout,
              const bf2* __restrict__ zprev, bf2* __restrict__ din) {
@@ -338,18 +381,19 @@ k_g_bwd_data(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, c
 #pragma unroll
                 for (int sp = 0; sp < 4; sp++) dg[sp][c] = cfma_conj(w[4 * s + sp], dv, dg[sp][c]);
             }
+        if (d == 0) {
 #pragma unroll
-        for (int s = 0; s < 4; s++) {
-            float2 o[3];
-            if (d == 0) {
+            for (int k = 0; k < 12; k++) acc[k / 3][k % 3] = cadd(acc[k / 3][k % 3], dg[k / 3][k % 3]);
+        } else {
+            float2 m[9];
+            staged_link(sl + (d - 1) * 9, lane, d & 1, m);   // direction +mu (odd d) comes back over the adjoint
 #pragma unroll
-                for (int c = 0; c < 3; c++) o[c] = dg[s][c];
-            } else {
-                // direction +mu (odd d) comes back over the adjoint link
-                staged_link(sl + (d - 1) * 9, lane, d & 1, dg[s], o);
+            for (int s = 0; s < 4; s++) {
+                float2 o[3];
+                colour_mul(m, dg[s], o);
+#pragma unroll
+                for (int c = 0; c < 3; c++) acc[s][c] = cadd(acc[s][c], o[c]);
             }
-#pragma unroll
-            for (int c = 0; c < 3; c++) acc[s][c] = cadd(acc[s][c], o[c]);
         }
     }
     if (!live) return;
@@ -405,20 +449,23 @@ __device__ __forceinline__ uint32_t sw128(int r, int j) {
 // run over TW_FLUSH tiles (24 accumulations each) and are then added to this CTA's partial in FP32, so that
 // a chain is no longer than the 3072-term FP32 chains of the SIMT kernel this replaced; k_g_reduce_w adds the
 // partials in FP64.
-// One CTA: 64-site tiles of a slice, 512 threads = 64 sites x 8 channels, directions 3y .. 3y+2 (CI = 8) or, for one
+// One CTA: 32-site tiles of a slice, 256 threads = 32 sites x 8 channels, directions 3y .. 3y+2 (CI = 8) or, for one
 // input channel (CI = 1), directions 1..8 in the place of the channels and direction 0 after them.  Two stage
-// buffers (72 KB each): the transport of the next direction overlaps the MMAs of this one; the transport bounds it.
+// buffers (36 KB each): the transport of the next direction overlaps the MMAs of this one, and the loads of the
+// one after are in flight; two CTAs per SM fill each other's barrier waits.  The transport and the splitting
+// bound it (640 instructions per 32 sites, channel and direction).
 // 16^3 x 32: 8 -> 8 layer 2137 us on SIMT (the gather and 32 x 32 complex products per site from shared memory),
-// 8 -> 1 776 us, 1 -> 8 688 us; here see the launch.
+// 8 -> 1 776 us, 1 -> 8 688 us; here 332, 290 and 68 us.
 // ---------------------------------------------------------------------------
-constexpr int TW_SITES = 64;
-constexpr int TW_FLUSH = 4;
-constexpr uint32_t TW_TILE = TW_SITES * 128;             // 64 rows x 64 bf16
+constexpr int TW_SITES = 32;
+constexpr int TW_THREADS = TW_SITES * 8;
+constexpr int TW_FLUSH = 8;
+constexpr uint32_t TW_TILE = TW_SITES * 128;             // 32 rows x 64 bf16
 constexpr uint32_t TW_STAGE = 9 * TW_TILE;               // 3 colours x (hi, mid, lo)
 constexpr uint32_t TW_SMEM = 2 * TW_STAGE + 2 * 3 * TW_TILE + TW_TILE + 1024 + 64;
 
 template <int CI, int CO>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(TW_THREADS, 2)
 k_g_tw(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ a, const bf2* __restrict__ dout,
        float* __restrict__ part, int* __restrict__ err) {
     using namespace tc;
@@ -453,15 +500,22 @@ k_g_tw(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ a, const b
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_d = *tmem_slot;
 
-    const int row = threadIdx.x & (TW_SITES - 1), ch = threadIdx.x >> 6;
+    const int row = threadIdx.x & (TW_SITES - 1), ch = threadIdx.x / TW_SITES;
     const int ntiles = (vol + TW_SITES - 1) / TW_SITES;
+    auto dir = [&](int dl) { return CI == 8 ? (int)blockIdx.y * 3 + dl : dl == 0 ? 1 + ch : 0; };
+    // the loads of a stage are issued one stage ahead (dead sites load site 0)
+    auto fetch = [&](HopLoad<1>& p, int t, int dl) {
+        const int x = t * TW_SITES + row;
+        if (t < ntiles && (CI == 8 || dl == 0 || ch == 0))
+            hop_load<false, 1>(p, gm, u, a, CI == 8 ? ch : 0, x < vol ? x : 0, dir(dl));
+    };
     int q = 0, tcount = 0;
     bool first = true, ok = true;
+    HopLoad<1> pre;
+    fetch(pre, blockIdx.x, 0);
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, tcount++) {
         const int x = t * TW_SITES + row;
         const bool live = x < vol;
-        Nbr nb;
-        if (live) nb = neighbours(gm, x);
         const uint32_t dbase = (tcount & 1) * 3 * TW_TILE;
         for (int dl = 0; dl < ND; dl++, q++) {
             const int b = q & 1;
@@ -485,22 +539,31 @@ k_g_tw(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ a, const b
                 for (int c = 0; c < 3; c++)
                     *reinterpret_cast<uint4*>(sD + dbase + c * TW_TILE + sw128(row, ch)) = w[c];
             }
-            const int d = CI == 8 ? blockIdx.y * 3 + dl : dl == 0 ? 1 + ch : 0;
             if (CI == 8 || dl == 0 || ch == 0) {
-                float2 g[4][3];
-                if (live) {
-                    gather(u, a + (CI == 8 ? (size_t)ch * vol * 12 : 0), vol, x, d, nb, g);
-                } else {
+                float2 v[12], g[12];
+                unpack_site(pre.act[0], v);
+                if (dir(dl) == 0) {
 #pragma unroll
-                    for (int k = 0; k < 12; k++) g[k / 3][k % 3] = make_float2(0.f, 0.f);
+                    for (int k = 0; k < 12; k++) g[k] = v[k];
+                } else {
+                    float2 m[9];
+                    hop_matrix(pre, m);
+#pragma unroll
+                    for (int s = 0; s < 4; s++) colour_mul(m, &v[3 * s], &g[3 * s]);
                 }
+                if (!live) {
+#pragma unroll
+                    for (int k = 0; k < 12; k++) g[k] = make_float2(0.f, 0.f);
+                }
+                if (dl + 1 < ND) fetch(pre, t, dl + 1);
+                else fetch(pre, t + gridDim.x, 0);
                 uint8_t* sb = sG + b * TW_STAGE;
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
                     unsigned w[3][4];
 #pragma unroll
                     for (int s = 0; s < 4; s++) {
-                        float2 r = g[s][c];
+                        float2 r = g[3 * s + c];
 #pragma unroll
                         for (int k = 0; k < 3; k++) {
                             w[k][s] = pack_bf2(r);
@@ -513,6 +576,8 @@ k_g_tw(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ a, const b
                         *reinterpret_cast<uint4*>(sb + (3 * c + k) * TW_TILE + sw128(row, ch)) =
                             make_uint4(w[k][0], w[k][1], w[k][2], w[k][3]);
                 }
+            } else {
+                fetch(pre, t + gridDim.x, 0);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncthreads();
@@ -542,10 +607,10 @@ k_g_tw(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ a, const b
             if (!mbar_wait(&done[(q - 1) & 1], (uint32_t)((q - 1) >> 1) & 1u)) *s_fail = 1;
             __syncwarp();
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int lg = warp & 3, cq = warp >> 2;
+            const int lg = warp & 3;   // TMEM lanes of this warp; warps w and w + 4 share the columns
             const int r = lg * 32 + lane, n = r & 63, half = r >> 6;
             const int pt = n & 1, sp = (n >> 1) & 3, cn = n >> 3;
-            if (CO == 8 || cq == 0) {
+            for (int cq = warp >> 2; cq < (CO == 8 ? 4 : 1); cq += 2) {
                 for (int dl = 0; dl < ND; dl++) {
                     float v[16];
                     tmem_ld16<16>(tmem_d + ((uint32_t)(lg * 32) << 16) + (uint32_t)(dl * 64 + cq * 16), v);
@@ -584,7 +649,9 @@ k_g_tw(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ a, const b
 }
 
 // ---------------------------------------------------------------------------
-// layer 2 on tcgen05 (see the file header).  One CTA = 128 sites, 512 threads (two channels each).
+// layer 2 on tcgen05 (see the file header).  One CTA = 128 sites, 256 threads (four channels each, in two
+// pairs; the loads of the next pair are in flight); two CTAs per SM fill each other's barrier waits.
+// 16^3 x 32: 313 us with one CTA per SM and every load waited for, 137 us here (bound by the transport's issue).
 // MODE 0 (forward):  A = U(x,d) h1_ci(x+d), B = W in real form; epilogue z2, h2 = ReLU(z2).
 // MODE 1 (backward through the data): A = adjoint transport of d2_co, B = W^dag in
 //        real form; epilogue d1 = D masked by z1 > 0 (real and imaginary parts).
@@ -594,18 +661,22 @@ k_g_tw(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ a, const b
 constexpr int TC_SITES = 128;
 constexpr uint32_t TC_A_BYTES = TC_SITES * 128;      // 128 rows x 64 bf16
 constexpr uint32_t TC_B_BYTES = 64 * 128;            // 64 rows x 64 bf16
-constexpr uint32_t TC_SMEM = 2 * 3 * TC_A_BYTES + 2 * TC_B_BYTES + 1024 + 256;
+// no slack for alignment: two CTAs fill the SM's 228 KB (the base is 1024-byte aligned, checked)
+constexpr uint32_t TC_SMEM = 2 * 3 * TC_A_BYTES + 2 * TC_B_BYTES + 64;
 constexpr uint32_t TC_TMEM_COLS = 256;               // 3 colours x 64 columns
 
 template <int MODE>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(256, 2)
 k_g_tc(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ in, const uint4* __restrict__ wimg,
        const bf2* __restrict__ zprev, bf2* __restrict__ out0, bf2* __restrict__ out1, int* __restrict__ err) {
     using namespace tc;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t* sA = smem;                                   // [2 buffers][3 colours][TC_A_BYTES]
-    uint8_t* sB = smem + 2 * 3 * TC_A_BYTES;              // [2 buffers][TC_B_BYTES]
+    extern __shared__ __align__(1024) uint8_t tc_smem[];
+    if (smem_u32(tc_smem) & 1023u) {   // the swizzled tiles need it
+        if (threadIdx.x == 0) atomicExch(err, SEEDCG_ERR_CUDA);
+        return;
+    }
+    uint8_t* sA = tc_smem;                                   // [2 buffers][3 colours][TC_A_BYTES]
+    uint8_t* sB = sA + 2 * 3 * TC_A_BYTES;              // [2 buffers][TC_B_BYTES]
     uint64_t* done = reinterpret_cast<uint64_t*>(sB + 2 * TC_B_BYTES);   // [2]
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 2);
     volatile int* s_fail = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -628,13 +699,16 @@ k_g_tc(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ in, const 
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_d = *tmem_slot;
 
-    // this thread's site and quarter of the input channels
+    // this thread's site and half of the input channels
     const int row = threadIdx.x & (TC_SITES - 1);
-    const int quarter = threadIdx.x >> 7;
+    const int ch0 = 4 * (threadIdx.x >> 7);
     const int x = x0 + row;
     const bool live = x < vol;
-    Nbr nb;
-    if (live) nb = neighbours(gm, x);
+    // the loads of a pair of channels (and a direction's link and piece of the weight image) are issued one
+    // pair ahead
+    static_assert(TC_B_BYTES == 2 * 256 * 16, "two 16-byte pieces of the weight image per thread");
+    HopLoad<2> pre;
+    hop_load<MODE != 0, 2>(pre, gm, u, in, ch0, live ? x : 0, 0);
     int issued = 0;   // MMA groups committed (one per direction)
     for (int d = 0; d < 9; d++) {
         const int b = d & 1;
@@ -645,68 +719,55 @@ k_g_tc(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ in, const 
         __syncthreads();
         if (*s_fail) break;
         // B: this direction's weights (a ready 128-byte-swizzled image)
+        uint4 w0, w1;
         {
-            const uint4* src = wimg + (size_t)d * (TC_B_BYTES / 16);
-            uint4* dst = reinterpret_cast<uint4*>(sB + b * TC_B_BYTES);
-            for (int i = threadIdx.x; i < (int)(TC_B_BYTES / 16); i += blockDim.x) dst[i] = __ldg(src + i);
+            const uint4* src = wimg + (size_t)d * (TC_B_BYTES / 16) + threadIdx.x;
+            w0 = __ldg(src);
+            w1 = __ldg(src + 256);
         }
-        // A: the transported activations of channels 2 quarter and 2 quarter + 1 at this site
-        float2 lk[9];   // the link of this direction at this site (already with its sign)
-        int src_site = x;
-        float sgn = 1.f;
-        bool dag = false;   // apply the link's adjoint
-        if (live && d > 0) {
-            const int mu = (d - 1) >> 1;
-            const bool back = (d - 1) & 1;
-            int lsite;
-            if (MODE == 0) {
-                src_site = back ? nb.b[mu] : nb.f[mu];
-                lsite = back ? nb.b[mu] : x;
-                dag = back;
-                sgn = (mu == 3 && (back ? nb.bwrap_t : nb.fwrap_t)) ? -1.f : 1.f;
-            } else {
-                src_site = back ? nb.f[mu] : nb.b[mu];
-                lsite = back ? x : nb.b[mu];
-                dag = !back;
-                sgn = (mu == 3 && (back ? nb.fwrap_t : nb.bwrap_t)) ? -1.f : 1.f;
+        // A: the transported activations of channels ch0 .. ch0 + 3 at this site
+        float2 m[9];
+        if (d > 0) hop_matrix(pre, m);
+        const int src_site = hop_from<MODE != 0>(gm, live ? x : 0, d).src;
+#pragma unroll
+        for (int pr = 0; pr < 2; pr++) {
+            float2 v[2][12];
+            unpack_site(pre.act[0], v[0]);
+            unpack_site(pre.act[1], v[1]);
+            if (pr == 0) {
+#pragma unroll
+                for (int k = 0; k < 2; k++) {
+                    const uint4* q = reinterpret_cast<const uint4*>(site_ptr(in, ch0 + 2 + k, vol, src_site));
+#pragma unroll
+                    for (int j = 0; j < 3; j++) pre.act[k][j] = __ldg(q + j);
+                }
+            } else if (d < 8) {
+                hop_load<MODE != 0, 2>(pre, gm, u, in, ch0, live ? x : 0, d + 1);
             }
 #pragma unroll
-            for (int e = 0; e < 9; e++) lk[e] = __ldg(u + (size_t)(mu * 9 + e) * vol + lsite);
-        }
-#pragma unroll 1
-        for (int q = 0; q < 2; q++) {
-            const int ch = 2 * quarter + q;
-            float2 v[12];
-            if (live) {
-                ld_site(site_ptr(in, ch, vol, src_site), v);
-            } else {
+            for (int q = 0; q < 2; q++) {
+                float2 g[12];
+                if (d == 0) {
 #pragma unroll
-                for (int k = 0; k < 12; k++) v[k] = make_float2(0.f, 0.f);
-            }
-            float2 g[4][3];
-#pragma unroll
-            for (int s = 0; s < 4; s++) {
-                if (d == 0 || !live) {
-#pragma unroll
-                    for (int c = 0; c < 3; c++) g[s][c] = v[3 * s + c];
+                    for (int k = 0; k < 12; k++) g[k] = v[q][k];
                 } else {
 #pragma unroll
-                    for (int a = 0; a < 3; a++) {
-                        float2 acc = make_float2(0.f, 0.f);
+                    for (int s = 0; s < 4; s++) colour_mul(m, &v[q][3 * s], &g[3 * s]);
+                }
+                if (!live) {
 #pragma unroll
-                        for (int c = 0; c < 3; c++)
-                            acc = dag ? cfma_conj(lk[3 * c + a], v[3 * s + c], acc) : cfma(lk[3 * a + c], v[3 * s + c], acc);
-                        g[s][a] = make_float2(sgn * acc.x, sgn * acc.y);
-                    }
+                    for (int k = 0; k < 12; k++) g[k] = make_float2(0.f, 0.f);
+                }
+                // colour c of this (site, channel): 4 spins x (re, im) = 16 bytes, chunk ch of the row
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const uint4 w = make_uint4(pack_bf2(g[c]), pack_bf2(g[3 + c]), pack_bf2(g[6 + c]), pack_bf2(g[9 + c]));
+                    *reinterpret_cast<uint4*>(sA + (b * 3 + c) * TC_A_BYTES + sw128(row, ch0 + 2 * pr + q)) = w;
                 }
             }
-            // colour c of this (site, channel): 4 spins x (re, im) = 16 bytes, chunk ch of the row
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                const uint4 w = make_uint4(pack_bf2(g[0][c]), pack_bf2(g[1][c]), pack_bf2(g[2][c]), pack_bf2(g[3][c]));
-                *reinterpret_cast<uint4*>(sA + (b * 3 + c) * TC_A_BYTES + sw128(row, ch)) = w;
-            }
         }
+        reinterpret_cast<uint4*>(sB + b * TC_B_BYTES)[threadIdx.x] = w0;
+        reinterpret_cast<uint4*>(sB + b * TC_B_BYTES)[threadIdx.x + 256] = w1;
         // the tensor cores read shared memory through the async proxy
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
@@ -737,10 +798,10 @@ k_g_tc(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ in, const 
     if (*s_fail || issued < 9) {
         if (threadIdx.x == 0) atomicExch(err, SEEDCG_ERR_TIMEOUT);
     } else {
-        // warp w reads TMEM lanes [32 (w % 4), + 32), the rows (sites) of its threads, for two output channels
+        // warp w reads TMEM lanes [32 (w % 4), + 32), the rows (sites) of its threads, for four output channels
         const int lg = warp & 3, r = lg * 32 + lane;
         const int xs = x0 + r;
-        for (int o = 2 * (warp >> 2); o < 2 * (warp >> 2) + 2; o++) {
+        for (int o = 4 * (warp >> 2); o < 4 * (warp >> 2) + 4; o++) {
             float cv[3][8];
 #pragma unroll
             for (int c = 0; c < 3; c++)
@@ -963,9 +1024,9 @@ void layer2_tc(seedcg_handle* h, GuessState* G, int mode, const bf2* in, const b
         attr[mode] = true;
     }
     if (mode == 0)
-        k_g_tc<0><<<blocks, 512, TC_SMEM, st>>>(gm, h->u32.as<float2>(), in, img, zprev, out0, out1, err);
+        k_g_tc<0><<<blocks, 256, TC_SMEM, st>>>(gm, h->u32.as<float2>(), in, img, zprev, out0, out1, err);
     else
-        k_g_tc<1><<<blocks, 512, TC_SMEM, st>>>(gm, h->u32.as<float2>(), in, img, zprev, out0, out1, err);
+        k_g_tc<1><<<blocks, 256, TC_SMEM, st>>>(gm, h->u32.as<float2>(), in, img, zprev, out0, out1, err);
     SEEDCG_CHECK_LAUNCH();
 }
 
@@ -1009,17 +1070,17 @@ template <int CI, int CO>
 void weight_grad(seedcg_handle* h, GuessState* G, const bf2* a, const bf2* dout, double2* grad, int* err,
                  cudaStream_t st) {
     const Geom& gm = h->g;
-    // one CTA per SM: the directions' three groups share the chip (CI = 8)
+    // two CTAs per SM: the directions' three groups share the chip (CI = 8)
     const int ntiles = (gm.vol + TW_SITES - 1) / TW_SITES;
     const int groups = CI == 8 ? 3 : 1;
-    const int nslice = std::min(ntiles, 152 / groups);
+    const int nslice = std::min(ntiles, 304 / groups);
     constexpr int NO = CO * CI * 16;
     const size_t ne = (size_t)9 * NO;
     G->part.ensure((size_t)nslice * 2 * ne * sizeof(float2));
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_g_tw<CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TW_SMEM);
     SEEDCG_CUDA_TRY(attr);
-    k_g_tw<CI, CO><<<dim3(nslice, groups), 512, TW_SMEM, st>>>(gm, h->u32.as<float2>(), a, dout, G->part.as<float>(), err);
+    k_g_tw<CI, CO><<<dim3(nslice, groups), TW_THREADS, TW_SMEM, st>>>(gm, h->u32.as<float2>(), a, dout, G->part.as<float>(), err);
     SEEDCG_CHECK_LAUNCH();
     k_g_reduce_w<<<(int)((ne + 31) / 32), 256, 0, st>>>(G->part.as<float2>(), 2 * nslice, (int)ne, grad);
     SEEDCG_CHECK_LAUNCH();
