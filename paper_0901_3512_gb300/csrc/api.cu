@@ -257,40 +257,15 @@ seedcg_status seedcg_apply(seedcg_handle* h, int op, int prec, int multi, int n,
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     try {
         SEEDCG_CUDA_TRY(cudaSetDevice(h->device));
-        const int vol = h->g.vol;
-        const size_t nf = (size_t)n * vol * 12;
-        const size_t esz = prec == 0 ? sizeof(double2) : sizeof(float2);
-        seedcg::DevBuf buf;
-        buf.ensure(3 * nf * esz + 512);
-        char* b0 = buf.as<char>();
-        void* A = b0;
-        void* Bv = b0 + nf * esz;
-        void* Cv = b0 + 2 * nf * esz;
+        // the operator reads and writes the caller's fields; what lies between is kept in the handle
+        const size_t nf = (size_t)n * h->g.vol * 12;
         if (prec == 0) {
-            seedcg::to_internal_f64(in, (double2*)A, vol, n, st);
-            auto apply = [&](int dag, const double2* x, double2* y) {
-                seedcg::dslash_f64(seedcg::fix_of(h), dag, n, x, y, st);   // one kernel for any n
-            };
-            const double2* res = nullptr;
-            if (op == 0) { apply(0, (double2*)A, (double2*)Bv); res = (double2*)Bv; }
-            else if (op == 1) { apply(1, (double2*)A, (double2*)Bv); res = (double2*)Bv; }
-            else { apply(0, (double2*)A, (double2*)Bv); apply(1, (double2*)Bv, (double2*)Cv); res = (double2*)Cv; }
-            seedcg::from_internal_f64(res, out, vol, n, st);
+            if (op == 2) h->apply.ensure(nf * sizeof(double2));
+            seedcg::apply_spinors_f64(seedcg::fix_of(h), op, n, in, out, h->apply.as<double2>(), st);
         } else {
-            seedcg::to_internal_f32(in, (float2*)A, vol, n, st);
-            const float k = (float)h->kappa;
-            auto apply = [&](int dag, const float2* x, float2* y) {
-                if (multi) seedcg::dslash_mrhs_f32(h->g, h->u32.as<float2>(), k, dag, n, x, y, st);
-                else
-                    for (int r = 0; r < n; r++)
-                        seedcg::dslash_f32(h->g, h->u32.as<float2>(), k, dag,
-                                           x + (size_t)r * 12 * vol, y + (size_t)r * 12 * vol, st);
-            };
-            const float2* res = nullptr;
-            if (op == 0) { apply(0, (float2*)A, (float2*)Bv); res = (float2*)Bv; }
-            else if (op == 1) { apply(1, (float2*)A, (float2*)Bv); res = (float2*)Bv; }
-            else { apply(0, (float2*)A, (float2*)Bv); apply(1, (float2*)Bv, (float2*)Cv); res = (float2*)Cv; }
-            seedcg::from_internal_f32(res, out, vol, n, st);
+            h->apply.ensure((op == 2 ? 2 : 1) * nf * sizeof(float2));
+            seedcg::apply_spinors_f32(h->g, h->u32.as<float2>(), (float)h->kappa, op, multi, false, n, in, out,
+                                      h->apply.as<float2>(), st);
         }
         SEEDCG_CUDA_TRY(cudaStreamSynchronize(st));
         return SEEDCG_OK;
@@ -526,8 +501,8 @@ seedcg_status seedcg_time_dslash(seedcg_handle* h, int prec, int n, int reps, in
             if (prec == 0)
                 seedcg::dslash_f64(seedcg::fix_of(h), 0, n, (const double2*)b0, (double2*)(b0 + nf * esz), st);
             else
-                seedcg::dslash_mrhs_f32(h->g, h->u32.as<float2>(), (float)h->kappa, 0, n,
-                                        (const float2*)b0, (float2*)(b0 + nf * esz), st);
+                seedcg::dslash_mrhs_f32(h->g, h->u32.as<float2>(), (float)h->kappa, 0, n, (const float2*)b0,
+                                        seedcg::OutF32{(float2*)(b0 + nf * esz)}, false, st);
             SEEDCG_CUDA_TRY(cudaEventRecord(e1, st));
             SEEDCG_CUDA_TRY(cudaEventSynchronize(e1));
             float t = 0.f;
@@ -568,6 +543,7 @@ void seedcg_destroy(seedcg_handle* h) {
     h->tcbuf.release();
     h->cgbuf.release();
     h->hostio.release();
+    h->apply.release();
     seedcg::guess_free(h);
     h->staging.release();
     if (h->pinned) cudaFreeHost(h->pinned);

@@ -407,13 +407,13 @@ k_mf_fix(const GroupDev<double>* __restrict__ G, int ng, Rows rows, CgS C) {
     if ((int)blockIdx.y >= nsys) return;
     const int tile = blockIdx.x - gd.tile0;
     const double2* in = STAGE == 0 ? gd.p : (EO && STAGE != 2) ? gd.e : gd.t;
-    FixOp op{STAGE >= 2 ? 1 : 0, EO ? (STAGE & 1) : -1, in, gd.n, EO, 1, 1, nullptr, gd.n, EO};
+    const int vs = EO ? gd.g.vol / 2 : gd.g.vol;
+    const FixView vi{in, gd.n, 2, 2 * vs, EO};
+    FixOp op{STAGE >= 2 ? 1 : 0, EO ? (STAGE & 1) : -1, vi, 1, 1, vi};
     if (EO) {
         op.diag = STAGE & 1;
         op.hsgn = (STAGE & 1) ? -1 : 1;
-        op.same = STAGE == 1 ? gd.p : gd.t;
-    } else {
-        op.same = in;
+        op.same.p = STAGE == 1 ? gd.p : gd.t;
     }
     MfFixEpi epi{EO && !(STAGE & 1) ? gd.e : gd.t,
                  STAGE == 3 ? gd.r : nullptr,

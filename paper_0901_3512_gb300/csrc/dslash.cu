@@ -7,6 +7,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "internal.cuh"
 #include "wilson.cuh"
@@ -56,20 +57,6 @@ __global__ void k_to_internal_f32(const double2* __restrict__ in, float2* __rest
     for (int k = 0; k < 12; k++) dst[sidx(k, s, vol)] = make_float2((float)src[k].x, (float)src[k].y);
 }
 
-__global__ void k_from_internal_f32(const float2* __restrict__ in, double2* __restrict__ out,
-                                    int vol, int n) {
-    long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (t >= (long)vol * n) return;
-    int r = (int)(t / vol), s = (int)(t % vol);
-    const float2* src = in + (size_t)r * 12 * vol;
-    double2* dst = out + ((size_t)r * vol + s) * 12;
-#pragma unroll
-    for (int k = 0; k < 12; k++) {
-        float2 q = src[sidx(k, s, vol)];
-        dst[k] = make_double2(q.x, q.y);
-    }
-}
-
 __global__ void k_gauge_to_internal(const double2* __restrict__ in, double2* __restrict__ u64,
                                     float2* __restrict__ u32, int vol) {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -83,24 +70,34 @@ __global__ void k_gauge_to_internal(const double2* __restrict__ in, double2* __r
     }
 }
 
+// The result of field r at site s: internal planes, or the boundary's complex128 spinor, written in place of
+// a separate widening pass (6 full 32-byte sectors per thread; 8^3 x 16, 12 fields: that pass took 8.2 us)
+__device__ __forceinline__ void put_site(const OutF32& o, int r, int vol, int s, const Spinor<float>& v) {
+    store_spinor(o.p + (size_t)r * 12 * vol, vol, s, v);
+}
+__device__ __forceinline__ void put_site(const OutF64& o, int r, int vol, int s, const Spinor<float>& v) {
+    put_spinor_f64(o, (size_t)r * vol + s, v);
+}
+
 // ---------------------------------------------------------------------------
-// single right-hand side: one thread per site, links and neighbours from
+// one thread per site, field blockIdx.y, links and neighbours from
 // global memory (coalesced: neighbouring threads read neighbouring sites)
 // ---------------------------------------------------------------------------
-template <typename R, int DAG>
+template <int DAG, typename Out>
 __global__ void __launch_bounds__(kThreads)
-k_dslash(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict__ in,
-         cx_t<R>* __restrict__ out) {
+k_dslash(Geom g, const float2* __restrict__ u, float kappa, const float2* __restrict__ in, Out out) {
+    using R = float;
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.vol) return;
     const int vol = g.vol;
+    in += (size_t)blockIdx.y * 12 * vol;
     Nbr n = neighbours(g, s);
     Spinor<R> res;
     auto load = [&](int y, Spinor<R>& p) { load_spinor(in, vol, y, p); };
     auto fl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + s); };
     auto bl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + n.b[mu]); };
     wilson_site<DAG, R>(n, s, load, fl, bl, kappa, res);
-    store_spinor(out, vol, s, res);
+    put_site(out, blockIdx.y, vol, s, res);
 }
 
 // ---------------------------------------------------------------------------
@@ -109,10 +106,10 @@ k_dslash(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restri
 // staged once in shared memory and reused for every right-hand side.
 // blockDim = TS * RPB; thread (site j, group q) handles rhs q, q+RPB, ...
 // ---------------------------------------------------------------------------
-template <typename R, int DAG, int TS>
-__global__ void __launch_bounds__(384, (sizeof(R) == 4 ? 2 : 1))
-k_dslash_mrhs(Geom g, const cx_t<R>* __restrict__ u, R kappa, int n,
-              const cx_t<R>* __restrict__ in, cx_t<R>* __restrict__ out) {
+template <int DAG, int TS, typename Out>
+__global__ void __launch_bounds__(384, 2)
+k_dslash_mrhs(Geom g, const float2* __restrict__ u, float kappa, int n, const float2* __restrict__ in, Out out) {
+    using R = float;
     // links of the tile, already multiplied by -kappa and the t-boundary sign
     __shared__ cx_t<R> sl[2][4][9][TS];   // [fwd/bwd][mu][3a+b][site]
     __shared__ int sb[4][TS];              // x - mu for each tile site
@@ -155,11 +152,10 @@ k_dslash_mrhs(Geom g, const cx_t<R>* __restrict__ u, R kappa, int n,
     auto bl = [&](int mu, int e) { return sl[1][mu][e][j]; };
     for (int r = q; r < n; r += rpb) {
         const cx_t<R>* inr = in + (size_t)r * 12 * vol;
-        cx_t<R>* outr = out + (size_t)r * 12 * vol;
         Spinor<R> res;
         auto load = [&](int y, Spinor<R>& p) { load_spinor(inr, vol, y, p); };
         wilson_site_prescaled<DAG, R>(nb, s, load, fl, bl, res);
-        store_spinor(outr, vol, s, res);
+        put_site(out, r, vol, s, res);
     }
 }
 
@@ -177,10 +173,11 @@ struct Brick {
 
 // PIPE: at most 256 threads and up to 128 registers per thread, spent on
 // keeping more neighbour spinors in flight (wilson_site_prescaled_pipe)
-template <typename R, int DAG, int TB, bool PIPE = false>
-__global__ void __launch_bounds__(PIPE ? 256 : 384, (sizeof(R) == 4 ? 2 : 1))
-k_dslash_brick(Geom g, Brick br, const cx_t<R>* __restrict__ u, R kappa, int n,
-               const cx_t<R>* __restrict__ in, cx_t<R>* __restrict__ out) {
+template <int DAG, int TB, bool PIPE, typename Out>
+__global__ void __launch_bounds__(PIPE ? 256 : 384, 2)
+k_dslash_brick(Geom g, Brick br, const float2* __restrict__ u, float kappa, int n, const float2* __restrict__ in,
+               Out out) {
+    using R = float;
     extern __shared__ unsigned char smem_raw[];
     cx_t<R>* sl = reinterpret_cast<cx_t<R>*>(smem_raw);            // [2][4][9][TB]
     int* ss = reinterpret_cast<int*>(sl + 72 * TB);                  // [TB] site index
@@ -221,14 +218,13 @@ k_dslash_brick(Geom g, Brick br, const cx_t<R>* __restrict__ u, R kappa, int n,
     auto bl = [&](int mu, int e) { return sl[((1 * 4 + mu) * 9 + e) * TB + j]; };
     for (int r = q; r < n; r += rpb) {
         const cx_t<R>* inr = in + (size_t)r * 12 * vol;
-        cx_t<R>* outr = out + (size_t)r * 12 * vol;
         Spinor<R> res;
         auto load = [&](int y, Spinor<R>& p) { load_spinor(inr, vol, y, p); };
         if constexpr (PIPE)
             wilson_site_prescaled_pipe<DAG, R>(nb, s, load, fl, bl, res);
         else
             wilson_site_prescaled<DAG, R>(nb, s, load, fl, bl, res);
-        store_spinor(outr, vol, s, res);
+        put_site(out, r, vol, s, res);
     }
 }
 
@@ -252,27 +248,16 @@ bool make_brick(const Geom& g, Brick& br, int cap = 128) {
 
 // one launch of a brick kernel; the dynamic shared memory limit is raised once
 // per instantiation (each has its own static flag)
-template <typename R, int DAG, int TB, bool PIPE = false>
+template <int DAG, int TB, bool PIPE, typename Out>
 void brick_go(int nb, int threads, size_t smem, cudaStream_t st, const Geom& g, const Brick& br,
-              const cx_t<R>* u, R kappa, int n, const cx_t<R>* in, cx_t<R>* out) {
+              const float2* u, float kappa, int n, const float2* in, Out out) {
     static bool attr = false;
     if (!attr) {
-        SEEDCG_CUDA_TRY(cudaFuncSetAttribute(k_dslash_brick<R, DAG, TB, PIPE>,
+        SEEDCG_CUDA_TRY(cudaFuncSetAttribute(k_dslash_brick<DAG, TB, PIPE, Out>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
         attr = true;
     }
-    k_dslash_brick<R, DAG, TB, PIPE><<<nb, threads, smem, st>>>(g, br, u, kappa, n, in, out);
-    SEEDCG_CHECK_LAUNCH();
-}
-
-template <typename R>
-void launch_dslash(const Geom& g, const cx_t<R>* u, R kappa, int dag, const cx_t<R>* in,
-                   cx_t<R>* out, cudaStream_t st) {
-    int nb = blocks_for(g.vol, kThreads);
-    if (dag)
-        k_dslash<R, 1><<<nb, kThreads, 0, st>>>(g, u, kappa, in, out);
-    else
-        k_dslash<R, 0><<<nb, kThreads, 0, st>>>(g, u, kappa, in, out);
+    k_dslash_brick<DAG, TB, PIPE, Out><<<nb, threads, smem, st>>>(g, br, u, kappa, n, in, out);
     SEEDCG_CHECK_LAUNCH();
 }
 
@@ -288,19 +273,19 @@ struct BrickChoice {
     int pipe;   // 1 = the register-pipelined site kernel (<= 256 threads)
 };
 
-template <typename R>
-void launch_dslash_mrhs(const Geom& g, const cx_t<R>* u, R kappa, int dag, int n,
-                        const cx_t<R>* in, cx_t<R>* out, cudaStream_t st,
+template <typename Out>
+void launch_dslash_mrhs(const Geom& g, const float2* u, float kappa, int dag, int n,
+                        const float2* in, Out out, cudaStream_t st,
                         const BrickChoice* force = nullptr);
 
-template <typename R>
-BrickChoice tuned_brick(const Geom& g, const cx_t<R>* u, R kappa, int dag, int n, const cx_t<R>* in,
-                        cx_t<R>* out, cudaStream_t st) {
+template <typename Out>
+BrickChoice tuned_brick(const Geom& g, const float2* u, float kappa, int dag, int n, const float2* in,
+                        Out out, cudaStream_t st) {
     static std::mutex mu;
     static std::map<std::string, BrickChoice> cache;
     char key[160];
-    snprintf(key, sizeof(key), "brick_%s_%dx%dx%dx%d_n%d_dag%d", sizeof(R) == 8 ? "f64" : "f32",
-             g.L[0], g.L[1], g.L[2], g.L[3], n, dag);
+    snprintf(key, sizeof(key), "brick_%s_%dx%dx%dx%d_n%d_dag%d",
+             std::is_same<Out, OutF64>::value ? "f32w" : "f32", g.L[0], g.L[1], g.L[2], g.L[3], n, dag);
     {
         std::lock_guard<std::mutex> lk(mu);
         auto it = cache.find(key);
@@ -334,10 +319,10 @@ BrickChoice tuned_brick(const Geom& g, const cx_t<R>* u, R kappa, int dag, int n
     for (const BrickChoice& c : cands) {
         Brick br;
         if (!make_brick(g, br, c.cap) || !(br.tb == 64 || br.tb == 96 || br.tb == 128)) continue;
-        launch_dslash_mrhs<R>(g, u, kappa, dag, n, in, out, st, &c);
+        launch_dslash_mrhs<Out>(g, u, kappa, dag, n, in, out, st, &c);
         SEEDCG_CUDA_TRY(cudaEventRecord(a, st));
         for (int r = 0; r < 3; r++)
-            launch_dslash_mrhs<R>(g, u, kappa, dag, n, in, out, st, &c);
+            launch_dslash_mrhs<Out>(g, u, kappa, dag, n, in, out, st, &c);
         SEEDCG_CUDA_TRY(cudaEventRecord(b, st));
         SEEDCG_CUDA_TRY(cudaEventSynchronize(b));
         float ms = 0.f;
@@ -364,15 +349,16 @@ BrickChoice tuned_brick(const Geom& g, const cx_t<R>* u, R kappa, int dag, int n
     return best;
 }
 
-template <typename R>
-void launch_dslash_mrhs(const Geom& g, const cx_t<R>* u, R kappa, int dag, int n,
-                        const cx_t<R>* in, cx_t<R>* out, cudaStream_t st,
+template <typename Out>
+void launch_dslash_mrhs(const Geom& g, const float2* u, float kappa, int dag, int n,
+                        const float2* in, Out out, cudaStream_t st,
                         const BrickChoice* force) {
+    using R = float;
     if (n <= 0) return;
     Brick br;
     BrickChoice ch{128, 0, 0};
     if (force) ch = *force;
-    else ch = tuned_brick<R>(g, u, kappa, dag, n, in, out, st);
+    else ch = tuned_brick<Out>(g, u, kappa, dag, n, in, out, st);
     if (make_brick(g, br, ch.cap) && (br.tb == 64 || br.tb == 96 || br.tb == 128)) {
         const int maxr = (ch.pipe ? 256 : 384) / br.tb;
         const int passes = (n + maxr - 1) / maxr;
@@ -381,20 +367,20 @@ void launch_dslash_mrhs(const Geom& g, const cx_t<R>* u, R kappa, int dag, int n
         const size_t smem = (size_t)br.tb * (72 * sizeof(cx_t<R>) + 5 * sizeof(int) + 2 * sizeof(R));
         const int nb = br.ny * br.nz * g.L[3];
         if (ch.pipe && br.tb == 128) {
-            if (dag) brick_go<R, 1, 128, true>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
-            else brick_go<R, 0, 128, true>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
+            if (dag) brick_go<1, 128, true, Out>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
+            else brick_go<0, 128, true, Out>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
         } else if (ch.pipe && br.tb == 64) {
-            if (dag) brick_go<R, 1, 64, true>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
-            else brick_go<R, 0, 64, true>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
+            if (dag) brick_go<1, 64, true, Out>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
+            else brick_go<0, 64, true, Out>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
         } else if (br.tb == 128) {
-            if (dag) brick_go<R, 1, 128>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
-            else brick_go<R, 0, 128>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
+            if (dag) brick_go<1, 128, false, Out>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
+            else brick_go<0, 128, false, Out>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
         } else if (br.tb == 96) {
-            if (dag) brick_go<R, 1, 96>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
-            else brick_go<R, 0, 96>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
+            if (dag) brick_go<1, 96, false, Out>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
+            else brick_go<0, 96, false, Out>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
         } else {
-            if (dag) brick_go<R, 1, 64>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
-            else brick_go<R, 0, 64>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
+            if (dag) brick_go<1, 64, false, Out>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
+            else brick_go<0, 64, false, Out>(nb, threads, smem, st, g, br, u, kappa, n, in, out);
         }
         return;
     }
@@ -405,9 +391,9 @@ void launch_dslash_mrhs(const Geom& g, const cx_t<R>* u, R kappa, int dag, int n
     const int threads = TS * rpb;
     const int nb = blocks_for(g.vol, TS);
     if (dag)
-        k_dslash_mrhs<R, 1, TS><<<nb, threads, 0, st>>>(g, u, kappa, n, in, out);
+        k_dslash_mrhs<1, TS, Out><<<nb, threads, 0, st>>>(g, u, kappa, n, in, out);
     else
-        k_dslash_mrhs<R, 0, TS><<<nb, threads, 0, st>>>(g, u, kappa, n, in, out);
+        k_dslash_mrhs<0, TS, Out><<<nb, threads, 0, st>>>(g, u, kappa, n, in, out);
     SEEDCG_CHECK_LAUNCH();
 }
 
@@ -431,29 +417,48 @@ void to_internal_f32(const double* in, float2* out, int vol, int n, cudaStream_t
         reinterpret_cast<const double2*>(in), out, vol, n);
     SEEDCG_CHECK_LAUNCH();
 }
-void from_internal_f32(const float2* in, double* out, int vol, int n, cudaStream_t s) {
-    if ((long)vol * n == 0) return;
-    k_from_internal_f32<<<blocks_for((long)vol * n, 256), 256, 0, s>>>(
-        in, reinterpret_cast<double2*>(out), vol, n);
-    SEEDCG_CHECK_LAUNCH();
-}
 void gauge_to_internal(const double* in, double2* u64, float2* u32, int vol, cudaStream_t s) {
     k_gauge_to_internal<<<blocks_for(vol, 256), 256, 0, s>>>(
         reinterpret_cast<const double2*>(in), u64, u32, vol);
     SEEDCG_CHECK_LAUNCH();
 }
 
-void dslash_f32(const Geom& g, const float2* u, float kappa, int dag, const float2* in,
-                float2* out, cudaStream_t s) {
-    launch_dslash<float>(g, u, kappa, dag, in, out, s);
+template <typename Out>
+void dslash_f32(const Geom& g, const float2* u, float kappa, int dag, int n, const float2* in, Out out,
+                cudaStream_t s) {
+    // fields side by side in the grid (at most 65535 per launch)
+    for (int r0 = 0; r0 < n; r0 += 65535) {
+        const dim3 grid(blocks_for(g.vol, kThreads), std::min(n - r0, 65535));
+        const size_t off = (size_t)r0 * 12 * g.vol;
+        Out o = out;
+        if constexpr (std::is_same<Out, OutF64>::value) o.p += 2 * off;
+        else o.p += off;
+        if (dag) k_dslash<1, Out><<<grid, kThreads, 0, s>>>(g, u, kappa, in + off, o);
+        else k_dslash<0, Out><<<grid, kThreads, 0, s>>>(g, u, kappa, in + off, o);
+        SEEDCG_CHECK_LAUNCH();
+    }
 }
-void dslash_mrhs_f32(const Geom& g, const float2* u, float kappa, int dag, int n,
-                     const float2* in, float2* out, cudaStream_t s) {
-    launch_dslash_mrhs<float>(g, u, kappa, dag, n, in, out, s);
+template <typename Out>
+void dslash_mrhs_f32(const Geom& g, const float2* u, float kappa, int dag, int n, const float2* in, Out out,
+                     bool fixed, cudaStream_t s) {
+    const BrickChoice c{128, 0, 0};
+    launch_dslash_mrhs<Out>(g, u, kappa, dag, n, in, out, s, fixed ? &c : nullptr);
 }
-void dslash_mrhs_fixed_f32(const Geom& g, const float2* u, float kappa, int dag, int n,
-                           const float2* in, float2* out, cudaStream_t s) {
-    const BrickChoice c{128, 0};
-    launch_dslash_mrhs<float>(g, u, kappa, dag, n, in, out, s, &c);
+template void dslash_mrhs_f32<OutF32>(const Geom&, const float2*, float, int, int, const float2*, OutF32, bool, cudaStream_t);
+
+void apply_spinors_f32(const Geom& g, const float2* u, float kappa, int op, int multi, bool fixed, int n,
+                       const double* in, double* out, float2* work, cudaStream_t s) {
+    to_internal_f32(in, work, g.vol, n, s);
+    auto go = [&](int dag, const float2* x, auto y) {
+        if (multi) dslash_mrhs_f32(g, u, kappa, dag, n, x, y, fixed, s);
+        else dslash_f32(g, u, kappa, dag, n, x, y, s);
+    };
+    float2* t = work + (size_t)n * 12 * g.vol;
+    if (op < 2) {
+        go(op, work, make_out_f64(out));
+    } else {
+        go(0, work, OutF32{t});
+        go(1, t, make_out_f64(out));
+    }
 }
 }  // namespace seedcg

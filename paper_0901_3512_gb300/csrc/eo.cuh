@@ -24,16 +24,14 @@ __device__ __forceinline__ int eo_site(const Geom& g, int h, int p) {
 
 // acc += c_hop * (H other)(s): the eight hops of D = 1 - kappa H (DAG: of D^dag)
 // from site s, whose neighbours all have the opposite parity and are read from
-// the half vector `other` at index >> 1; the antiperiodic sign on hops that wrap t
-template <typename R, int DAG>
-__device__ __forceinline__ void eo_hops(const Geom& g, const cx_t<R>* __restrict__ u, int s, const Nbr& nb,
-                                        const cx_t<R>* __restrict__ other, R c_hop, Spinor<R>& acc) {
-    const int vol = g.vol, vh = g.vol / 2;
+// the half vector `other` at index >> 1; the antiperiodic sign on hops that wrap t.
+// Fwd(mu, e) / Bwd(mu, e) give element e = 3a+b of U_mu(s) / U_mu(s - mu).
+template <typename R, int DAG, typename Fwd, typename Bwd>
+__device__ __forceinline__ void eo_hops(const Nbr& nb, Fwd fl, Bwd bl, const cx_t<R>* __restrict__ other, int vh,
+                                        R c_hop, Spinor<R>& acc) {
     constexpr int SF = DAG ? 1 : -1;
     constexpr int SB = -SF;
     Spinor<R> p;
-    auto fl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + s); };
-    auto bl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + nb.b[mu]); };
 #define SEEDCG_EO_HOP(MU)                                                                            \
     {                                                                                                \
         const R cf = (MU == 3 && nb.fwrap_t) ? -c_hop : c_hop;                                       \
@@ -97,7 +95,10 @@ __device__ __forceinline__ void eo_site_apply(const Geom& g, const cx_t<R>* __re
 #pragma unroll
             for (int c = 0; c < 3; c++) acc.c[a][c] = mk<R>(0, 0);
     }
-    eo_hops<R, DAG>(g, u, s, nb, other, c_hop, acc);
+    const int vol = g.vol;
+    auto fl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + s); };
+    auto bl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + nb.b[mu]); };
+    eo_hops<R, DAG>(nb, fl, bl, other, vh, c_hop, acc);
 }
 
 }  // namespace seedcg

@@ -45,14 +45,18 @@ __global__ void k_fix_links(Geom g, const double2* __restrict__ u, double kappa,
 struct FixStore {
     static constexpr bool kShare = false;
     double2* out;
-    long stride;
-    int vo;       // sites of an output field
-    int half;     // 1: stored at the half index
+    FixView v;    // layout of out
+    int wide;     // every pair of entries is 32-byte aligned
     __device__ __forceinline__ double operator()(int r, int plane, int idx, int s, bool live, double2 a, double2 b) {
         if (live) {
-            double2* q = out + (size_t)r * stride + ((size_t)plane * vo + (half ? idx : s)) * 2;
-            q[0] = a;
-            q[1] = b;
+            double2* q = out + (size_t)r * v.field + (size_t)(v.half ? idx : s) * v.site + (size_t)plane * v.pair;
+            if (wide) {
+                asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(q), "d"(a.x), "d"(a.y), "d"(b.x), "d"(b.y)
+                             : "memory");
+            } else {
+                q[0] = a;
+                q[1] = b;
+            }
         }
         return 0.0;
     }
@@ -61,14 +65,16 @@ struct FixStore {
 
 // At most 128 registers: two blocks per SM.  Instruction issue bounds it: 1270 warp instructions per
 // 32 sites, direction and field, 216 of them multiply-adds of 32 x 32 + 64 bits and 380 the conversion of the
-// neighbour.  16^3 x 32, 12 fields: 900 us, issue 44 % busy at 16 warps per SM, DRAM 12 %.
+// neighbour.  16^3 x 32, 12 fields: 900 us between internal fields, issue 44 % busy at 16 warps per SM, DRAM
+// 12 %; 1037 us from and to the boundary's spinors, where two layout passes took another 303 us.
 __global__ void __launch_bounds__(kFixThreads, 2) k_fix_apply(FixDev F, FixOp op, FixStore st, int n) {
     extern __shared__ __align__(16) unsigned char fix_smem[];
     fix_tile(F, op, blockIdx.x, blockIdx.y, n, gridDim.y, fix_smem, st);
 }
 
-void fix_go(const FixDev& F, const FixOp& op, const FixStore& st, int n, cudaStream_t s) {
+void fix_go(const FixDev& F, const FixOp& op, double2* out, const FixView& layout, int n, cudaStream_t s) {
     if (n <= 0) return;
+    const FixStore st{out, layout, (reinterpret_cast<uintptr_t>(out) & 31) == 0};
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_fix_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
     SEEDCG_CUDA_TRY(attr);
@@ -129,19 +135,52 @@ void fix_links(const Geom& g, const double2* u, double kappa, int4* L, int* k, i
     SEEDCG_CHECK_LAUNCH();
 }
 
-void dslash_f64(const FixDev& F, int dag, int n, const double2* in, double2* out, cudaStream_t s) {
-    const long nf = 12L * F.g.vol;
-    const FixOp op{dag, -1, in, nf, 0, 1, 1, in, nf, 0};
-    fix_go(F, op, FixStore{out, nf, F.g.vol, 0}, n, s);
+namespace {
+void fix_d(const FixDev& F, int dag, int n, const FixView& in, double2* out, const FixView& layout, cudaStream_t s) {
+    fix_go(F, FixOp{dag, -1, in, 1, 1, in}, out, layout, n, s);
 }
 
 // With t = -kappa H_eo x (FP64 half vectors), A x = x - (-kappa H_oe) t: the factors of
 // kappa^2 are in the links.
+void fix_a(const FixDev& F, int dag, int n, const FixView& x, double2* te, double2* out, const FixView& layout,
+           cudaStream_t st) {
+    const FixView t = fix_planes(te, F.g, 1);
+    fix_go(F, FixOp{dag, 0, x, 0, 1, x}, te, t, n, st);
+    fix_go(F, FixOp{dag, 1, t, 1, -1, x}, out, layout, n, st);
+}
+}  // namespace
+
+void dslash_f64(const FixDev& F, int dag, int n, const double2* in, double2* out, cudaStream_t s) {
+    fix_d(F, dag, n, fix_planes(in, F.g, 0), out, fix_planes(out, F.g, 0), s);
+}
+
+void apply_spinors_f64(const FixDev& F, int op, int n, const double* in, double* out, double2* tmp, cudaStream_t s) {
+    const double2* x = reinterpret_cast<const double2*>(in);
+    double2* y = reinterpret_cast<double2*>(out);
+    const FixView vx = fix_spinors(x, F.g, 0), vy = fix_spinors(y, F.g, 0), vt = fix_planes(tmp, F.g, 0);
+    if (op < 2) {
+        fix_d(F, op, n, vx, y, vy, s);
+    } else {
+        fix_d(F, 0, n, vx, tmp, vt, s);
+        fix_d(F, 1, n, vt, y, vy, s);
+    }
+}
+
+void apply_eo_spinors_f64(const FixDev& F, int op, int n, const double* in, double* out, double2* te, double2* tmp,
+                          cudaStream_t s) {
+    const double2* x = reinterpret_cast<const double2*>(in);
+    double2* y = reinterpret_cast<double2*>(out);
+    const FixView vx = fix_spinors(x, F.g, 1), vy = fix_spinors(y, F.g, 1), vt = fix_planes(tmp, F.g, 1);
+    if (op < 2) {
+        fix_a(F, op, n, vx, te, y, vy, s);
+    } else {
+        fix_a(F, 0, n, vx, te, tmp, vt, s);
+        fix_a(F, 1, n, vt, te, y, vy, s);
+    }
+}
+
 void eo_apply_a_f64(const FixDev& F, int dag, int n, const double2* x, double2* te, double2* out, cudaStream_t st) {
-    const int vh = F.g.vol / 2;
-    const long nh = 12L * vh;
-    fix_go(F, FixOp{dag, 0, x, nh, 1, 0, 1, nullptr, 0, 1}, FixStore{te, nh, vh, 1}, n, st);
-    fix_go(F, FixOp{dag, 1, te, nh, 1, 1, -1, x, nh, 1}, FixStore{out, nh, vh, 1}, n, st);
+    fix_a(F, dag, n, fix_planes(x, F.g, 1), te, out, fix_planes(out, F.g, 1), st);
 }
 
 void eo_apply_mdag_m_f64(const FixDev& F, int n, const double2* x, double2* te, double2* out, cudaStream_t st) {
@@ -150,8 +189,8 @@ void eo_apply_mdag_m_f64(const FixDev& F, int n, const double2* x, double2* te, 
 }
 
 void eo_source_f64(const FixDev& F, int n, const double2* eta, double2* phi, cudaStream_t st) {
-    const int vh = F.g.vol / 2;
-    fix_go(F, FixOp{0, 1, eta, 12L * F.g.vol, 0, 1, -1, eta, 12L * F.g.vol, 0}, FixStore{phi, 12L * vh, vh, 1}, n, st);
+    const FixView v = fix_planes(eta, F.g, 0);
+    fix_go(F, FixOp{0, 1, v, 1, -1, v}, phi, fix_planes(phi, F.g, 1), n, st);
 }
 
 void eo_gather_f64(const Geom& g, int p, int n, const double2* full, double2* half, cudaStream_t st) {
@@ -160,8 +199,7 @@ void eo_gather_f64(const Geom& g, int p, int n, const double2* full, double2* ha
 
 void eo_reconstruct_f64(const FixDev& F, int n, const double2* x_odd, const double2* eta, double2* x,
                         cudaStream_t st) {
-    const long nf = 12L * F.g.vol, nh = nf / 2;
-    fix_go(F, FixOp{0, 0, x_odd, nh, 1, 1, -1, eta, nf, 0}, FixStore{x, nf, F.g.vol, 0}, n, st);
+    fix_go(F, FixOp{0, 0, fix_planes(x_odd, F.g, 1), 1, -1, fix_planes(eta, F.g, 0)}, x, fix_planes(x, F.g, 0), n, st);
     eo_move(F.g, 1, 1, n, x, const_cast<double2*>(x_odd), st);
 }
 

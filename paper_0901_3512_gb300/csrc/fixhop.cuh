@@ -95,13 +95,28 @@ __device__ __forceinline__ double fix_combine(long long S, int E, int k, int dia
     return T == 0 ? 0.0 : fix_to_double(T, Ec, k);
 }
 
+// FP64 fields as the tiles read them: entry k of site y of field r at p[r * field + y * site + (k / 2) * pair + k % 2].
+// Internal fields are pair planes (site 2, pair 2 * sites), the boundary's fields spinors (site 12, pair 2), which the
+// operator reads and writes in place: no layout pass.  half = 1: half vectors (y is the half index).
+struct FixView {
+    const double2* p;
+    long field;
+    int site, pair, half;
+};
+inline FixView fix_planes(const double2* p, const Geom& g, int half) {
+    return FixView{p, 12L * (g.vol >> half), 2, 2 * (g.vol >> half), half};
+}
+inline FixView fix_spinors(const double2* p, const Geom& g, int half) {
+    return FixView{p, 12L * (g.vol >> half), 12, 2, half};
+}
+
 // The two complex entries of pair-plane `plane` of -kappa H psi (dag: of D^dag's hopping term) at full
-// site s, by the plain FP64 chain; psi in full (sh = 0) or half vectors (sh = 1).
-static __device__ __noinline__ void fix_slow(const FixDev& F, int dag, int s, const double2* in, int sh, int plane,
+// site s, by the plain FP64 chain; psi: field r of `in`.
+static __device__ __noinline__ void fix_slow(const FixDev& F, int dag, int s, const FixView& in, int r, int plane,
                                              double2* a, double2* b) {
     const Geom& g = F.g;
     const Nbr nb = neighbours(g, s);
-    const int vol = g.vol, vs = g.vol >> sh;
+    const int vol = g.vol, sh = in.half;
     Spinor<double> acc;
 #pragma unroll
     for (int k = 0; k < 12; k++) acc.c[k / 3][k % 3] = make_double2(0.0, 0.0);
@@ -118,7 +133,9 @@ static __device__ __noinline__ void fix_slow(const FixDev& F, int dag, int s, co
 #pragma unroll
             for (int k = 0; k < 12; k++) p.c[k / 3][k % 3] = make_double2(0.0, 0.0);
         } else {
-            load_spinor(in, vs, y, p);
+            const double2* q = in.p + (size_t)r * in.field + (size_t)y * in.site;
+#pragma unroll
+            for (int k = 0; k < 12; k++) p.c[k / 3][k % 3] = __ldg(q + (size_t)(k >> 1) * in.pair + (k & 1));
         }
     };
     if (dag) wilson_site<1, double>(idx, -1, load, fl, bl, F.kappa, acc);
@@ -135,14 +152,10 @@ static __device__ __noinline__ void fix_slow(const FixDev& F, int dag, int s, co
 struct FixOp {
     int dag;             // the hopping term of D^dag
     int parity;          // -1: every site; 0 / 1: the sites of that parity (tile index = half index)
-    const double2* in;   // field r at in + r * in_stride; in_sh = 1: half vectors of the other parity
-    long in_stride;
-    int in_sh;
+    FixView in;          // full fields, or half vectors of the other parity
     int diag;            // 1: same is added
     int hsgn;            // +1 or -1
-    const double2* same;
-    long same_stride;
-    int same_sh;
+    FixView same;
 };
 
 // sums of the eight directions for one complex component: SPIN 0 (upper, component c = 3 spin + colour of
@@ -231,16 +244,15 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
     // factor c (times i when swap): re part flips, im part flips
     const unsigned fr0 = swap ? (f0 > 0 ? kNeg : 0u) : (f0 < 0 ? kNeg : 0u), fi0 = f0 < 0 ? kNeg : 0u;
     const unsigned fr1 = swap ? (f1 > 0 ? kNeg : 0u) : (f1 < 0 ? kNeg : 0u), fi1 = f1 < 0 ? kNeg : 0u;
-    const int vs = vol >> op.in_sh;
-    const double2* pin = op.in + (size_t)(nsite_idx >> op.in_sh) * 2;
+    const double2* pin = op.in.p + (size_t)(nsite_idx >> op.in.half) * op.in.site;
     int buf = 0, rprev = -1;
     for (int r = r0; r < nr; r += rstep, buf ^= 1) {
         long long* R = reinterpret_cast<long long*>(smem + buf * kFixBufBytes);
         int* sE = reinterpret_cast<int*>(smem + buf * kFixBufBytes + 8 * 12 * 32 * sizeof(long long));
         {
             double2 p[12];   // 0-5: spins 0 and 1; 6-8: spin q0; 9-11: spin q1
-            const double2* q = pin + (size_t)r * op.in_stride;
-            auto at = [&](int k) { return __ldg(q + (size_t)(k >> 1) * 2 * vs + (k & 1)); };
+            const double2* q = pin + (size_t)r * op.in.field;
+            auto at = [&](int k) { return __ldg(q + (size_t)(k >> 1) * op.in.pair + (k & 1)); };
 #pragma unroll
             for (int c = 0; c < 6; c++) p[c] = at(c);
 #pragma unroll
@@ -319,9 +331,8 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
             for (int d = 0; d < 8; d++) D[d] = Em - D[d];
             double2 pa = make_double2(0.0, 0.0), pb = pa;
             if (op.diag) {
-                const int vd = vol >> op.same_sh;
-                const int si = op.parity < 0 ? idx : (op.same_sh ? idx : s);
-                const double2* q = op.same + (size_t)r * op.same_stride + ((size_t)warp * vd + si) * 2;
+                const int si = op.same.half ? idx : s;
+                const double2* q = op.same.p + (size_t)r * op.same.field + (size_t)si * op.same.site + (size_t)warp * op.same.pair;
                 pa = q[0];
                 pb = q[1];
             }
@@ -332,7 +343,7 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
                 return h != 0 && ((h >> 20) < kFixEMin || (h >> 20) > kFixEMax);
             };
             if (bad || (op.diag && (far(pa.x) || far(pa.y) || far(pb.x) || far(pb.y)))) {
-                fix_slow(F, op.dag, s, op.in + (size_t)r * op.in_stride, op.in_sh, warp, &va, &vb);
+                fix_slow(F, op.dag, s, op.in, r, warp, &va, &vb);
                 const double hs = (double)op.hsgn;
                 va = make_double2(pa.x + hs * va.x, pa.y + hs * va.y);
                 vb = make_double2(pb.x + hs * vb.x, pb.y + hs * vb.y);

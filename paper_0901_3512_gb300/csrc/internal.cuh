@@ -161,21 +161,31 @@ struct DevBuf {
 void to_internal_f64(const double* in, double2* out, int vol, int n, cudaStream_t s);
 void from_internal_f64(const double2* in, double* out, int vol, int n, cudaStream_t s);
 void to_internal_f32(const double* in, float2* out, int vol, int n, cudaStream_t s);
-void from_internal_f32(const float2* in, double* out, int vol, int n, cudaStream_t s);
 void gauge_to_internal(const double* in, double2* u64, float2* u32, int vol, cudaStream_t s);
 
-// out = D in (dag = 0) or D^dag in (dag = 1); single right-hand side
-void dslash_f32(const Geom& g, const float2* u, float kappa, int dag, const float2* in,
-                float2* out, cudaStream_t s);
-// n right-hand sides at in + r*12*V; links staged once per tile of sites
-void dslash_mrhs_f32(const Geom& g, const float2* u, float kappa, int dag, int n,
-                     const float2* in, float2* out, cudaStream_t s);
-// the same kernel with its default tile shape, never timing alternatives
-void dslash_mrhs_fixed_f32(const Geom& g, const float2* u, float kappa, int dag, int n,
-                           const float2* in, float2* out, cudaStream_t s);
+// FP32: out = D in (dag = 0) or D^dag in (dag = 1) for n fields at in + r*12*V; out: internal
+// (OutF32) or the boundary's complex128 [n][V][4][3] (OutF64, widened at the store)
+struct OutF32 { float2* p; };
+struct OutF64 { double* p; int wide; };   // wide: p is 32-byte aligned (make_out_f64)
+inline OutF64 make_out_f64(double* p) { return OutF64{p, (reinterpret_cast<uintptr_t>(p) & 31) == 0}; }
+// links staged once per tile of sites; fixed: the default tile shape, never timing alternatives
+template <typename Out>
+void dslash_mrhs_f32(const Geom& g, const float2* u, float kappa, int dag, int n, const float2* in, Out out,
+                     bool fixed, cudaStream_t s);
+
+// op 0 = D, 1 = D^dag, 2 = M on the boundary's fields in FP32 arithmetic: in is rounded into `work` (n internal
+// fields; 2 n for op 2), the last operator writes out.  multi = 0: links from global memory.
+void apply_spinors_f32(const Geom& g, const float2* u, float kappa, int op, int multi, bool fixed, int n,
+                       const double* in, double* out, float2* work, cudaStream_t s);
 
 // FP64 operator in fixed point (fixed.cu): out = D in or D^dag in for n fields
 void dslash_f64(const FixDev& F, int dag, int n, const double2* in, double2* out, cudaStream_t s);
+// the same on the boundary's complex128 fields [n][V][4][3], without a layout pass: op 0 = D, 1 = D^dag,
+// 2 = M (tmp: n internal fields of scratch, op 2 only)
+void apply_spinors_f64(const FixDev& F, int op, int n, const double* in, double* out, double2* tmp, cudaStream_t s);
+// A, A^dag or A^dag A on complex128 half fields (te: n half vectors of scratch; tmp: n more, op 2 only)
+void apply_eo_spinors_f64(const FixDev& F, int op, int n, const double* in, double* out, double2* te, double2* tmp,
+                          cudaStream_t s);
 // the links of a handle in fixed point: L from u, and the scale k and range flag ok (synchronises)
 void fix_links(const Geom& g, const double2* u, double kappa, int4* L, int* k, int* ok, cudaStream_t s);
 

@@ -81,37 +81,12 @@ extern "C" seedcg_status seedcg_apply_noalloc(seedcg_handle* h, int op, int prec
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     try {
         SEEDCG_CUDA_TRY(cudaSetDevice(h->device));
-        char* b0 = static_cast<char*>(seedcg::scratch_on(h->device));
-        void* A = b0;
-        void* Bv = b0 + nf * esz;
-        void* Cv = b0 + 2 * nf * esz;
-        if (prec == 0) {
-            seedcg::to_internal_f64(in, (double2*)A, vol, n, st);
-            auto apply = [&](int dag, const double2* x, double2* y) {
-                seedcg::dslash_f64(seedcg::fix_of(h), dag, n, x, y, st);   // one kernel for any n
-            };
-            const double2* res = (const double2*)Bv;
-            if (op == 0) apply(0, (double2*)A, (double2*)Bv);
-            else if (op == 1) apply(1, (double2*)A, (double2*)Bv);
-            else { apply(0, (double2*)A, (double2*)Bv); apply(1, (double2*)Bv, (double2*)Cv); res = (double2*)Cv; }
-            seedcg::from_internal_f64(res, out, vol, n, st);
-        } else {
-            seedcg::to_internal_f32(in, (float2*)A, vol, n, st);
-            const float k = (float)h->kappa;
-            auto apply = [&](int dag, const float2* x, float2* y) {
-                if (multi)
-                    seedcg::dslash_mrhs_fixed_f32(h->g, h->u32.as<float2>(), k, dag, n, x, y, st);
-                else
-                    for (int r = 0; r < n; r++)
-                        seedcg::dslash_f32(h->g, h->u32.as<float2>(), k, dag,
-                                           x + (size_t)r * 12 * vol, y + (size_t)r * 12 * vol, st);
-            };
-            const float2* res = (const float2*)Bv;
-            if (op == 0) apply(0, (float2*)A, (float2*)Bv);
-            else if (op == 1) apply(1, (float2*)A, (float2*)Bv);
-            else { apply(0, (float2*)A, (float2*)Bv); apply(1, (float2*)Bv, (float2*)Cv); res = (float2*)Cv; }
-            seedcg::from_internal_f32(res, out, vol, n, st);
-        }
+        void* work = seedcg::scratch_on(h->device);
+        if (prec == 0)
+            seedcg::apply_spinors_f64(seedcg::fix_of(h), op, n, in, out, static_cast<double2*>(work), st);
+        else
+            seedcg::apply_spinors_f32(h->g, h->u32.as<float2>(), (float)h->kappa, op, multi, true, n, in, out,
+                                      static_cast<float2*>(work), st);
         SEEDCG_CUDA_TRY(cudaStreamSynchronize(st));
         return SEEDCG_OK;
     } catch (const Error& e) {

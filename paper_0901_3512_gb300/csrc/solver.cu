@@ -287,15 +287,16 @@ void lz_fix(const FixDev& F, const FixOp& op, const double2* v, const double2* v
 // (t, e: full or odd half, and even half scratch)
 void lz_apply_f64(const FixDev& F, bool eo, const double2* v, const double2* vprev, double2* t, double2* e,
                   double2* f, int i, const LzDev& L, cudaStream_t st) {
+    const FixView vv = fix_planes(v, F.g, eo), vt = fix_planes(t, F.g, eo), ve = fix_planes(e, F.g, eo);
     if (!eo) {
-        lz_fix<false>(F, FixOp{0, -1, v, 0, 0, 1, 1, v, 0, 0}, nullptr, nullptr, t, i, L, st);
-        lz_fix<true>(F, FixOp{1, -1, t, 0, 0, 1, 1, t, 0, 0}, v, vprev, f, i, L, st);
+        lz_fix<false>(F, FixOp{0, -1, vv, 1, 1, vv}, nullptr, nullptr, t, i, L, st);
+        lz_fix<true>(F, FixOp{1, -1, vt, 1, 1, vt}, v, vprev, f, i, L, st);
         return;
     }
-    lz_fix<false>(F, FixOp{0, 0, v, 0, 1, 0, 1, nullptr, 0, 1}, nullptr, nullptr, e, i, L, st);
-    lz_fix<false>(F, FixOp{0, 1, e, 0, 1, 1, -1, v, 0, 1}, nullptr, nullptr, t, i, L, st);
-    lz_fix<false>(F, FixOp{1, 0, t, 0, 1, 0, 1, nullptr, 0, 1}, nullptr, nullptr, e, i, L, st);
-    lz_fix<true>(F, FixOp{1, 1, e, 0, 1, 1, -1, t, 0, 1}, v, vprev, f, i, L, st);
+    lz_fix<false>(F, FixOp{0, 0, vv, 0, 1, vv}, nullptr, nullptr, e, i, L, st);
+    lz_fix<false>(F, FixOp{0, 1, ve, 1, -1, vv}, nullptr, nullptr, t, i, L, st);
+    lz_fix<false>(F, FixOp{1, 0, vt, 0, 1, vt}, nullptr, nullptr, e, i, L, st);
+    lz_fix<true>(F, FixOp{1, 1, ve, 1, -1, vt}, v, vprev, f, i, L, st);
 }
 
 // Steps 4 and 7 (literal seeding): eta^j = v_i^dag r_0^j - gamma_{i-1} eta^j for
@@ -921,6 +922,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     // V basis and coefficient scratch
     const size_t vrow = (size_t)n * sizeof(VT);
     if (h->vbasis.bytes < vrow * (size_t)m_max) {
+        h->apply.release();   // scratch of earlier operator applications must not stand in a basis's way
         // refuse a basis that cannot fit before allocating it (m_max rows of one vector each)
         size_t free_b = 0, total_b = 0;
         SEEDCG_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));

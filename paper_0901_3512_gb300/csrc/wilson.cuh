@@ -133,6 +133,23 @@ __device__ __forceinline__ void store_spinor(double2* __restrict__ p, int vol, i
     for (int k = 0; k < 12; k++) p[sidx(k, s, vol)] = v.c[k / 3][k % 3];
 }
 
+// an FP32 spinor widened into the boundary's complex128 layout at site record `rec`
+__device__ __forceinline__ void put_spinor_f64(const OutF64& o, size_t rec, const Spinor<float>& v) {
+    double* q = o.p + rec * 24;
+    if (o.wide) {
+#pragma unroll
+        for (int c = 0; c < 6; c++) {
+            const float2 a = v.c[(2 * c) / 3][(2 * c) % 3], b = v.c[(2 * c + 1) / 3][(2 * c + 1) % 3];
+            asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(q + 4 * c), "d"((double)a.x),
+                         "d"((double)a.y), "d"((double)b.x), "d"((double)b.y) : "memory");
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 12; k++)
+            reinterpret_cast<double2*>(q)[k] = make_double2((double)v.c[k / 3][k % 3].x, (double)v.c[k / 3][k % 3].y);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // neighbours
 // ---------------------------------------------------------------------------
