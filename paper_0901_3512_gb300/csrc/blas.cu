@@ -251,6 +251,7 @@ template <typename R, typename VT, int NV, int RPW, int CHUNK>
 __global__ void __launch_bounds__(256, (sizeof(R) == 4 && NV == 2) ? 4 : 1)
 k_proj_partial(const VT* __restrict__ V, long ldv, int na, const cx_t<R>* __restrict__ X,
                long ldx, int nv, long n, int chunk, int rg, double2* __restrict__ part) {
+    pdl_enter();
     // block (x, y): one chunk of entries (X chunk staged in shared memory)
     // against the rows of group y (rg rows); warp: RPW rows at a time; lane: W
     // consecutive entries per 16-byte load.  chunk and n are multiples of W
@@ -317,6 +318,7 @@ k_proj_partial(const VT* __restrict__ V, long ldv, int na, const cx_t<R>* __rest
 template <int NV>
 __global__ void k_proj_reduce(const double2* __restrict__ part, int nblk, int na, int nv,
                               double2* __restrict__ C, int ldc, int c0) {
+    pdl_enter();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (w >= na * nv) return;
@@ -443,22 +445,19 @@ void proj(const AT* A, long lda, int na, const cx_t<R>* X, long ldx, int nx, lon
             const int nblk = (int)((n + ch - 1) / ch);
             if ((size_t)nblk * na * 2 > scratch_elems) throw Error{SEEDCG_ERR_OOM, "proj scratch"};
             constexpr int RG = 8 * 4 * 4;
-            k_proj_partial<R, AT, 2, 4, CH><<<dim3(nblk, (na + RG - 1) / RG), 256, 0, s>>>(
+            launch_pdl(pdl_for(n), k_proj_partial<R, AT, 2, 4, CH>, dim3(nblk, (na + RG - 1) / RG), 256, 0, s, 
                 A, lda, na, Xc, ldx, nv, n, ch, RG, scratch);
-            SEEDCG_CHECK_LAUNCH();
-            k_proj_reduce<2><<<(na * nv + 7) / 8, 256, 0, s>>>(scratch, nblk, na, nv, C, ldc, c0);
+            launch_pdl(pdl_for(n), k_proj_reduce<2>, (na * nv + 7) / 8, 256, 0, s, scratch, nblk, na, nv, C, ldc, c0);
         } else {
             constexpr int CH = proj_chunk<R, 4>();
             const int ch = proj_chunk_for(n, CH);
             const int nblk = (int)((n + ch - 1) / ch);
             if ((size_t)nblk * na * 4 > scratch_elems) throw Error{SEEDCG_ERR_OOM, "proj scratch"};
             constexpr int RG = 8 * 2 * 4;
-            k_proj_partial<R, AT, 4, 2, CH><<<dim3(nblk, (na + RG - 1) / RG), 256, 0, s>>>(
+            launch_pdl(pdl_for(n), k_proj_partial<R, AT, 4, 2, CH>, dim3(nblk, (na + RG - 1) / RG), 256, 0, s, 
                 A, lda, na, Xc, ldx, nv, n, ch, RG, scratch);
-            SEEDCG_CHECK_LAUNCH();
-            k_proj_reduce<4><<<(na * nv + 7) / 8, 256, 0, s>>>(scratch, nblk, na, nv, C, ldc, c0);
+            launch_pdl(pdl_for(n), k_proj_reduce<4>, (na * nv + 7) / 8, 256, 0, s, scratch, nblk, na, nv, C, ldc, c0);
         }
-        SEEDCG_CHECK_LAUNCH();
     }
 }
 

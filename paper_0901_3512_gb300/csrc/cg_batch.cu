@@ -90,6 +90,7 @@ struct CgS {
     double tol, delta2;
     int maxiter;
     int rows_cap;   // rows of every per-row array (grid of the per-row kernels)
+    bool pdl;       // programmatic dependent launch of the iteration's kernels
 };
 
 __device__ __forceinline__ int find_group(int b, int ng, const int* tile0) {
@@ -136,6 +137,7 @@ __device__ __forceinline__ void put_share(double* shares, int ntiles, int slot, 
 template <typename R, int DAG, int RPB>
 __global__ void __launch_bounds__(TS * RPB, (sizeof(R) == 4 ? (RPB <= 8 ? 3 : 2) : 1))
 k_mf_dslash(const GroupDev<R>* __restrict__ G, int ng, Rows rows, CgS C) {
+    pdl_enter();
     __shared__ cx_t<R> sl[2][4][9][TS];
     __shared__ int sb[4][TS];
     __shared__ Nbr snb[TS];   // neighbours of the tile's sites (kept out of the registers)
@@ -214,6 +216,7 @@ k_mf_dslash(const GroupDev<R>* __restrict__ G, int ng, Rows rows, CgS C) {
 template <typename R, int STAGE, int RPB>
 __global__ void __launch_bounds__(TS * RPB, (sizeof(R) == 4 ? 2 : 1))
 k_mf_eo(const GroupDev<R>* __restrict__ G, int ng, Rows rows, CgS C) {
+    pdl_enter();
     constexpr int DAG = STAGE >= 2 ? 1 : 0;
     constexpr int POUT = (STAGE & 1) ? 1 : 0;
     __shared__ cx_t<R> sl[2][4][9][TS];
@@ -303,6 +306,7 @@ k_mf_eo(const GroupDev<R>* __restrict__ G, int ng, Rows rows, CgS C) {
 template <typename R, int DAG, int TB, int RPB>
 __global__ void __launch_bounds__(TB * RPB, (sizeof(R) == 4 && TB * RPB <= 256) ? 3 : 1)
 k_mf_brick(const GroupDev<R>* __restrict__ G, Rows rows, CgS C) {
+    pdl_enter();
     extern __shared__ unsigned char smem_raw[];
     cx_t<R>* sl = reinterpret_cast<cx_t<R>*>(smem_raw);   // [2][4][9][TB]
     Nbr* snb = reinterpret_cast<Nbr*>(sl + 72 * TB);        // [TB] neighbours of the brick's sites
@@ -399,6 +403,7 @@ struct MfFixEpi {
 template <int EO, int STAGE>
 __global__ void __launch_bounds__(kFixThreads, 2)
 k_mf_fix(const GroupDev<double>* __restrict__ G, int ng, Rows rows, CgS C) {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char fix_smem[];
     int f = 0;
     while (f + 1 < ng && (int)blockIdx.x >= G[f + 1].tile0) f++;
@@ -431,8 +436,7 @@ void mf_fix(int tiles, int gy, cudaStream_t s, const GroupDev<double>* gdev, int
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_mf_fix<EO, STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
     SEEDCG_CUDA_TRY(attr);
-    k_mf_fix<EO, STAGE><<<dim3(tiles, gy), kFixThreads, kFixSmem, s>>>(gdev, ng, rows, C);
-    SEEDCG_CHECK_LAUNCH();
+    launch_pdl(C.pdl, k_mf_fix<EO, STAGE>, dim3(tiles, gy), kFixThreads, kFixSmem, s, gdev, ng, rows, C);
 }
 
 // a row's shares, summed in a fixed order (one block per row); four independent
@@ -457,6 +461,7 @@ __device__ __forceinline__ double row_shares(const double* __restrict__ sh, int 
 template <typename R>
 __global__ void __launch_bounds__(256)
 k_mf_alpha(const GroupDev<R>* __restrict__ G, Rows rows, CgS C) {
+    pdl_enter();
     const int row = blockIdx.x;
     const int f = rows.group[row];
     if (f < 0) return;
@@ -474,6 +479,7 @@ k_mf_alpha(const GroupDev<R>* __restrict__ G, Rows rows, CgS C) {
 template <typename R>
 __global__ void __launch_bounds__(256)
 k_mf_beta(const GroupDev<R>* __restrict__ G, Rows rows, CgS C) {
+    pdl_enter();
     const int row = blockIdx.x;
     const int f = rows.group[row];
     if (f < 0 || !C.active[row]) return;
@@ -557,6 +563,7 @@ template <> struct Pack16<double> {
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
 k_mf_xp(const GroupDev<R>* __restrict__ G, Rows rows, CgS C) {
+    pdl_enter();
     using P = Pack16<R>;
     using T = typename P::T;
     constexpr int W = P::W;
@@ -681,8 +688,8 @@ template <typename R>
 void launch_mf(int rpb, int dag, int tiles, cudaStream_t s, const GroupDev<R>* gdev, int ng, Rows rows,
                const CgS& C) {
 #define SEEDCG_MF(RP)                                                                          \
-    if (dag) k_mf_dslash<R, 1, RP><<<tiles, TS * RP, 0, s>>>(gdev, ng, rows, C);               \
-    else k_mf_dslash<R, 0, RP><<<tiles, TS * RP, 0, s>>>(gdev, ng, rows, C);
+    if (dag) launch_pdl(C.pdl, k_mf_dslash<R, 1, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C);               \
+    else launch_pdl(C.pdl, k_mf_dslash<R, 0, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C);
     if (rpb == 4) { SEEDCG_MF(4) }
     else if (rpb == 12) { SEEDCG_MF(12) }
     else { SEEDCG_MF(8) }
@@ -695,10 +702,10 @@ void launch_mf_eo(int rpb, int stage, int tiles, cudaStream_t s, const GroupDev<
                   const CgS& C) {
 #define SEEDCG_MFE(RP)                                                                          \
     switch (stage) {                                                                           \
-        case 0: k_mf_eo<R, 0, RP><<<tiles, TS * RP, 0, s>>>(gdev, ng, rows, C); break;         \
-        case 1: k_mf_eo<R, 1, RP><<<tiles, TS * RP, 0, s>>>(gdev, ng, rows, C); break;         \
-        case 2: k_mf_eo<R, 2, RP><<<tiles, TS * RP, 0, s>>>(gdev, ng, rows, C); break;         \
-        default: k_mf_eo<R, 3, RP><<<tiles, TS * RP, 0, s>>>(gdev, ng, rows, C); break;        \
+        case 0: launch_pdl(C.pdl, k_mf_eo<R, 0, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;         \
+        case 1: launch_pdl(C.pdl, k_mf_eo<R, 1, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;         \
+        case 2: launch_pdl(C.pdl, k_mf_eo<R, 2, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;         \
+        default: launch_pdl(C.pdl, k_mf_eo<R, 3, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;        \
     }
     if (rpb == 4) { SEEDCG_MFE(4) }
     else if (rpb == 12) { SEEDCG_MFE(12) }
@@ -718,8 +725,7 @@ void brick_launch(int nb, cudaStream_t s, const GroupDev<R>* gdev, Rows rows, co
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         attr = true;
     }
-    k_mf_brick<R, DAG, TB, RPB><<<nb, TB * RPB, smem, s>>>(gdev, rows, C);
-    SEEDCG_CHECK_LAUNCH();
+    launch_pdl(C.pdl, k_mf_brick<R, DAG, TB, RPB>, nb, TB * RPB, smem, s, gdev, rows, C);
 }
 
 // Launch shape of the operator, chosen by the autotuner: codes 4, 8, 12 are the
@@ -734,8 +740,7 @@ void launch_op(bool eo, int code, int tiles, const Brk& b64, const Brk& b128, cu
                const GroupDev<R>* gdev, int ng, Rows rows, const CgS& C, bool with_alpha) {
     auto alpha = [&]() {
         if (!with_alpha) return;
-        k_mf_alpha<R><<<C.rows_cap, 256, 0, s>>>(gdev, rows, C);
-        SEEDCG_CHECK_LAUNCH();
+        launch_pdl(C.pdl, k_mf_alpha<R>, C.rows_cap, 256, 0, s, gdev, rows, C);
     };
     if constexpr (sizeof(R) == 8) {
         // code = the grid rows (systems side by side)
@@ -918,8 +923,9 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
     // sites of a system's vectors: the lattice, or its odd half for the even-odd system
     auto nsites = [&](const CgGroup& gr) { return eo ? gr.h->g.vol / 2 : gr.h->g.vol; };
     int rows_cap = 0, tiles = 0, nsys_max = 0;
-    long nmax = 0;
+    long nmax = 0, entries = 0;
     for (auto& gr : groups) {
+        entries += 12L * nsites(gr) * gr.nsys;
         rows_cap += gr.nsys;
         tiles += (nsites(gr) + TS - 1) / TS;
         nsys_max = std::max(nsys_max, gr.nsys);
@@ -1006,6 +1012,7 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
     C.delta2 = reliable_delta > 0.0 ? reliable_delta * reliable_delta : 0.0;
     C.maxiter = maxiter;
     C.rows_cap = rows_cap;
+    C.pdl = pdl_for(entries);
     SEEDCG_CUDA_TRY(cudaMemsetAsync(C.counters, 0, sizeof(unsigned) * (rows_cap + 64), st));
     SEEDCG_CUDA_TRY(cudaMemsetAsync(C.iters, 0, sizeof(int) * rows_cap, st));
     SEEDCG_CUDA_TRY(cudaMemsetAsync(C.flag, 0, sizeof(int) * rows_cap, st));
@@ -1182,10 +1189,8 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
     auto chunk = [&](cudaStream_t s) {
         for (int it = 0; it < poll; it++) {
             launch_op<R>(eo, rpb, tiles, b64, b128, s, gdev, ng, rows, C, true);   // steps 1-3
-            k_mf_beta<R><<<rows_cap, 256, 0, s>>>(gdev, rows, C);
-            SEEDCG_CHECK_LAUNCH();
-            k_mf_xp<R><<<dim3(gx, rows_cap), kRedThreads, 0, s>>>(gdev, rows, C);
-            SEEDCG_CHECK_LAUNCH();
+            launch_pdl(C.pdl, k_mf_beta<R>, rows_cap, 256, 0, s, gdev, rows, C);
+            launch_pdl(C.pdl, k_mf_xp<R>, dim3(gx, rows_cap), kRedThreads, 0, s, gdev, rows, C);
         }
     };
     cudaGraphExec_t gexec = nullptr;

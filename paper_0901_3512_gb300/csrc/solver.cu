@@ -111,6 +111,7 @@ __device__ __forceinline__ void lz_alpha_fin(const LzDev& L, int i, double a) {
 template <typename R>
 __global__ void k_lz_start(const cx_t<R>* __restrict__ r0, cx_t<R>* __restrict__ v, long n,
                            LzDev L) {
+    pdl_enter();
     const double inv = 1.0 / L.ctl->beta0;
     for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n;
          e += (long)gridDim.x * blockDim.x) {
@@ -124,6 +125,7 @@ template <typename R>
 __global__ void __launch_bounds__(kSiteThreads, 7)
 k_lz_D(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict__ v,
        cx_t<R>* __restrict__ t, int i, LzDev L) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.vol) return;
@@ -144,6 +146,7 @@ __global__ void __launch_bounds__(kSiteThreads, 7)
 k_lz_Ddag(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict__ t,
           const cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ vprev,
           cx_t<R>* __restrict__ f, int i, LzDev L) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     const int vol = g.vol;
     const R bprev = i > 1 ? (R)L.beta[i - 2] : R(0);
@@ -187,6 +190,7 @@ __global__ void __launch_bounds__(kRedThreads)
 k_lz_eo(Geom g, const cx_t<R>* __restrict__ u, R kk, const cx_t<R>* __restrict__ other,
         const cx_t<R>* __restrict__ same, cx_t<R>* __restrict__ out, const cx_t<R>* __restrict__ v,
         const cx_t<R>* __restrict__ vprev, int i, LzDev L) {
+    pdl_enter();
     constexpr int DAG = STAGE >= 2 ? 1 : 0;
     constexpr int POUT = (STAGE & 1) ? 1 : 0;
     if (i > L.ctl->m) return;
@@ -257,6 +261,7 @@ template <bool LAST>
 __global__ void __launch_bounds__(kFixThreads, 2)
 k_lz_fix(FixDev F, FixOp op, const double2* __restrict__ v, const double2* __restrict__ vprev,
          double2* __restrict__ out, int i, LzDev L) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     extern __shared__ __align__(16) unsigned char fix_smem[];
     LzFixEpi epi{out,
@@ -279,8 +284,7 @@ void lz_fix(const FixDev& F, const FixOp& op, const double2* v, const double2* v
         cudaFuncSetAttribute(k_lz_fix<LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
     SEEDCG_CUDA_TRY(attr);
     const int sites = op.parity < 0 ? F.g.vol : F.g.vol / 2;
-    k_lz_fix<LAST><<<(sites + 31) / 32, kFixThreads, kFixSmem, st>>>(F, op, v, vprev, out, i, L);
-    SEEDCG_CHECK_LAUNCH();
+    launch_pdl(pdl_for(12L * sites), k_lz_fix<LAST>, (sites + 31) / 32, kFixThreads, kFixSmem, st, F, op, v, vprev, out, i, L);
 }
 
 // f = M v - beta_{i-1} v_{i-1} and alpha_i in FP64: D and D^dag, or the four half-lattice hops
@@ -305,6 +309,7 @@ template <typename R, int NE>
 __global__ void __launch_bounds__(kRedThreads)
 k_lz_eta(const cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ r0, long n, int j0, int ne,
          int i, LzDev L, unsigned* ctr) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     double red[2 * NE];
     R acc[2 * NE];
@@ -343,6 +348,7 @@ template <typename R, bool LIT>
 __global__ void __launch_bounds__(kRedThreads)
 k_lz_update(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, cx_t<R>* __restrict__ w,
             cx_t<R>* __restrict__ X, int nrhs, long n, int i, int final_beta, LzDev L) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     const R a = (R)L.alpha[i - 1];
     R dl = 0, bp = 0, zt = 0;
@@ -392,6 +398,7 @@ template <typename R, bool X1>
 __global__ void __launch_bounds__(kRedThreads)
 k_lz_update_v(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, cx_t<R>* __restrict__ w,
               double2* __restrict__ x1, long n, int i, int final_beta, LzDev L) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     constexpr int W = 16 / (int)sizeof(cx_t<R>);
     const R a = (R)L.alpha[i - 1];
@@ -540,6 +547,7 @@ template <typename R, typename VT>
 __global__ void __launch_bounds__(kRedThreads)
 k_po_sub(const VT* __restrict__ V, long ldv, int na, const double2* __restrict__ coef, int cv,
          cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, long n, int i, LzDev L) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     constexpr int W = VLoad<R, VT>::N;
     __shared__ cx_t<R> sc[256][2];
@@ -571,6 +579,7 @@ template <typename R, typename VT>
 __global__ void __launch_bounds__(kRedThreads)
 k_po_sub_seg(const VT* __restrict__ V, long ldv, int na, int seg, const double2* __restrict__ coef,
              int cv, long n, cx_t<R>* __restrict__ part, int i, LzDev L) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     constexpr int W = VLoad<R, VT>::N;
     __shared__ cx_t<R> sc[256][2];
@@ -594,6 +603,7 @@ template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
 k_po_sub_fin(const cx_t<R>* __restrict__ part, int nseg, cx_t<R>* __restrict__ v,
              cx_t<R>* __restrict__ f, long n, int i, LzDev L) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     R acc = 0;
     for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n;
@@ -616,6 +626,7 @@ k_po_sub_fin(const cx_t<R>* __restrict__ part, int nseg, cx_t<R>* __restrict__ v
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
 k_po_normalise(cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f, long n, int i, LzDev L) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     const R inv = (R)(1.0 / L.ctl->nv);
     R pr = 0, pi = 0;
@@ -636,6 +647,7 @@ k_po_normalise(cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f, long n, i
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
 k_po_finish(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, long n, int i, LzDev L) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     const double2 d = L.ctl->dvf;
     const cx_t<R> dc = mk<R>((R)d.x, (R)d.y);
@@ -668,6 +680,7 @@ template <typename R, typename VT>
 __global__ void k_lz_advance(const cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f,
                              cx_t<R>* __restrict__ vnext, VT* __restrict__ Vrow, long n, int i,
                              LzDev L) {
+    pdl_enter();
     if (i > L.ctl->m) return;
     const double b = L.beta[i - 1];
     const bool go = b > 0.0 && i < L.ctl->m;
@@ -861,6 +874,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     // the even-odd system (Section 3) works on odd-site half vectors
     const bool eo = h->eo_active;
     const long n = 12L * (eo ? vol / 2 : vol);
+    const bool pdl = pdl_for(n);
     const bool fp64 = sizeof(R) == 8;
     const bool literal = (o.seed_mode == 0) && fp64;
     const int m_max = std::max(o.m_max, 1);
@@ -1003,19 +1017,16 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
             nseg = std::min<long>({8, (6 * resident + po_gb - 1) / po_gb, na / 128, seg_cap});
         }
         if (nseg <= 1) {
-            k_po_sub<R, VT><<<vec_blocks(n, kW), kRedThreads, 0, st>>>(Vb, n, na, Cc, cvcol, vv, ff, n,
+            launch_pdl(pdl, k_po_sub<R, VT>, vec_blocks(n, kW), kRedThreads, 0, st, Vb, n, na, Cc, cvcol, vv, ff, n,
                                                                        i, L);
-            SEEDCG_CHECK_LAUNCH();
             return;
         }
         const int seg = (int)((na + nseg - 1) / nseg);
         const int ns = (na + seg - 1) / seg;
         cx_t<R>* sp = reinterpret_cast<cx_t<R>*>(split);
-        k_po_sub_seg<R, VT><<<dim3((unsigned)po_gb, ns), kRedThreads, 0, st>>>(Vb, n, na, seg, Cc, cvcol,
+        launch_pdl(pdl, k_po_sub_seg<R, VT>, dim3((unsigned)po_gb, ns), kRedThreads, 0, st, Vb, n, na, seg, Cc, cvcol,
                                                                               n, sp, i, L);
-        SEEDCG_CHECK_LAUNCH();
-        k_po_sub_fin<R><<<rb, kRedThreads, 0, st>>>(sp, ns, vv, ff, n, i, L);
-        SEEDCG_CHECK_LAUNCH();
+        launch_pdl(pdl, k_po_sub_fin<R>, rb, kRedThreads, 0, st, sp, ns, vv, ff, n, i, L);
     };
 
     int* pin = reinterpret_cast<int*>(h->pinned);
@@ -1070,8 +1081,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     int m = 0, m_conv = 0, po_count = 0, lz_status = SEEDCG_OK, breakdown = 0;
     if (beta0 > 0.0) {
         const int sb = site_blocks(vol);
-        k_lz_start<R><<<rb, kRedThreads, 0, st>>>(R0, vA, n, L);
-        SEEDCG_CHECK_LAUNCH();
+        launch_pdl(pdl, k_lz_start<R>, rb, kRedThreads, 0, st, R0, vA, n, L);
         cx_t<R>* v = vA;
         cx_t<R>* vprev = vB;
         int i = 1;
@@ -1082,36 +1092,28 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                 lz_apply_f64(fix_of(h), eo, v, vprev, tv, ev, fv, i, L, st);
             } else if (eo) {
                 // f = A^dag A v - beta v_prev, alpha: four half-lattice hops
-                k_lz_eo<R, 0><<<sbh, kRedThreads, 0, st>>>(h->g, U, kk, v, nullptr, ev, nullptr, nullptr, i, L);
-                SEEDCG_CHECK_LAUNCH();
-                k_lz_eo<R, 1><<<sbh, kRedThreads, 0, st>>>(h->g, U, kk, ev, v, tv, nullptr, nullptr, i, L);
-                SEEDCG_CHECK_LAUNCH();
-                k_lz_eo<R, 2><<<sbh, kRedThreads, 0, st>>>(h->g, U, kk, tv, nullptr, ev, nullptr, nullptr, i, L);
-                SEEDCG_CHECK_LAUNCH();
-                k_lz_eo<R, 3><<<sbh, kRedThreads, 0, st>>>(h->g, U, kk, ev, tv, fv, v, vprev, i, L);
-                SEEDCG_CHECK_LAUNCH();
+                launch_pdl(pdl, k_lz_eo<R, 0>, sbh, kRedThreads, 0, st, h->g, U, kk, v, nullptr, ev, nullptr, nullptr, i, L);
+                launch_pdl(pdl, k_lz_eo<R, 1>, sbh, kRedThreads, 0, st, h->g, U, kk, ev, v, tv, nullptr, nullptr, i, L);
+                launch_pdl(pdl, k_lz_eo<R, 2>, sbh, kRedThreads, 0, st, h->g, U, kk, tv, nullptr, ev, nullptr, nullptr, i, L);
+                launch_pdl(pdl, k_lz_eo<R, 3>, sbh, kRedThreads, 0, st, h->g, U, kk, ev, tv, fv, v, vprev, i, L);
             } else {
-                k_lz_D<R><<<site_blocks_lz(vol), kSiteThreads, 0, st>>>(h->g, U, kap, v, tv, i, L);
-                SEEDCG_CHECK_LAUNCH();
-                k_lz_Ddag<R><<<site_blocks_lz(vol), kSiteThreads, 0, st>>>(h->g, U, kap, tv, v, vprev, fv, i, L);
-                SEEDCG_CHECK_LAUNCH();
+                launch_pdl(pdl, k_lz_D<R>, site_blocks_lz(vol), kSiteThreads, 0, st, h->g, U, kap, v, tv, i, L);
+                launch_pdl(pdl, k_lz_Ddag<R>, site_blocks_lz(vol), kSiteThreads, 0, st, h->g, U, kap, tv, v, vprev, fv, i, L);
             }
             if (literal) {
                 for (int j0 = 2; j0 <= nrhs; j0 += 8) {
                     int ne = std::min(8, nrhs - j0 + 1);
-                    k_lz_eta<R, 8><<<rb, kRedThreads, 0, st>>>(v, R0, n, j0, ne, i, L,
+                    launch_pdl(pdl, k_lz_eta<R, 8>, rb, kRedThreads, 0, st, v, R0, n, j0, ne, i, L,
                                                                  L.counters + CTR_ETA0 + j0);
-                    SEEDCG_CHECK_LAUNCH();
                 }
             }
             const bool po_now = k_po > 0 && i >= 2 && (i % k_po) == 0;
             if (literal)
-                k_lz_update<R, true><<<rb, kRedThreads, 0, st>>>(
+                launch_pdl(pdl, k_lz_update<R, true>, rb, kRedThreads, 0, st, 
                     v, fv, wv, reinterpret_cast<cx_t<R>*>(X64), nrhs, n, i, po_now ? 0 : 1, L);
             else
-                k_lz_update_v<R, true><<<lean_blocks(n, 16 / (int)sizeof(cx_t<R>)), kRedThreads, 0, st>>>(
+                launch_pdl(pdl, k_lz_update_v<R, true>, lean_blocks(n, 16 / (int)sizeof(cx_t<R>)), kRedThreads, 0, st, 
                     v, fv, wv, X64, n, i, po_now ? 0 : 1, L);
-            SEEDCG_CHECK_LAUNCH();
             if (po_now) {
                 cudaEvent_t e0, e1;
                 cudaEventCreate(&e0);
@@ -1124,16 +1126,13 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                     project(na, Bst, 2, 2);
                     po_subtract(na, cvcol, v, fv, i);
                 }
-                k_po_normalise<R><<<rb, kRedThreads, 0, st>>>(v, fv, n, i, L);
-                SEEDCG_CHECK_LAUNCH();
-                k_po_finish<R><<<rb, kRedThreads, 0, st>>>(v, fv, n, i, L);
-                SEEDCG_CHECK_LAUNCH();
+                launch_pdl(pdl, k_po_normalise<R>, rb, kRedThreads, 0, st, v, fv, n, i, L);
+                launch_pdl(pdl, k_po_finish<R>, rb, kRedThreads, 0, st, v, fv, n, i, L);
                 cudaEventRecord(e1, st);
                 po_ev.push_back({e0, e1});
             }
-            k_lz_advance<R, VT><<<rb, kRedThreads, 0, st>>>(v, fv, vprev, Vb + (size_t)(i - 1) * n, n,
+            launch_pdl(pdl, k_lz_advance<R, VT>, rb, kRedThreads, 0, st, v, fv, vprev, Vb + (size_t)(i - 1) * n, n,
                                                            i, L);
-            SEEDCG_CHECK_LAUNCH();
             std::swap(v, vprev);
             if (i % poll == 0 || i == m_max) {
                 SEEDCG_CUDA_TRY(cudaMemcpyAsync(pin, L.ctl, sizeof(int) * 8, cudaMemcpyDeviceToHost, st));
