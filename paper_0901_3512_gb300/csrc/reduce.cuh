@@ -39,10 +39,12 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
     }
     __syncthreads();
     if (warp == 0) {
+        // at most 8 warps: three steps (an FP64 addition takes 68 clocks, and these are all in a row)
 #pragma unroll
         for (int k = 0; k < NV; k++) {
             double t = lane < nw ? sh[k][lane] : 0.0;
-            t = warp_sum(t);
+#pragma unroll
+            for (int o = kRedThreads / 64; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
             if (lane == 0) sh[k][0] = t;
         }
     }
@@ -53,12 +55,15 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
 }
 
 // Grid-wide sum over a 1-D or 2-D grid.  partials holds NV * nblocks doubles,
-// counter one unsigned that is zero on entry (it is reset on exit).  fin(tot)
-// runs once, on thread 0 of the last block, with the grid totals.
-template <int NV, typename Fin>
+// counter one unsigned that is zero on entry (it is reset on exit).  fin(tot, aux)
+// runs once, on thread 0 of the last block, with the grid totals; aux() is scalar work
+// that does not need them (an FP64 division is about 900 clocks here), done
+// by another warp of that block meanwhile.
+template <int NV, typename Aux, typename Fin>
 __device__ __forceinline__ void grid_sum(double (&v)[NV], double* partials, unsigned* counter,
-                                         Fin fin) {
+                                         Aux aux, Fin fin) {
     __shared__ bool s_last;
+    __shared__ double s_aux;
     block_sum<NV>(v);
     const unsigned nblk = gridDim.x * gridDim.y;
     const unsigned bid = blockIdx.y * gridDim.x + blockIdx.x;
@@ -72,6 +77,7 @@ __device__ __forceinline__ void grid_sum(double (&v)[NV], double* partials, unsi
     __syncthreads();
     if (!s_last) return;
     __threadfence();
+    if (threadIdx.x == blockDim.x - 1) s_aux = aux();
     double tot[NV];
 #pragma unroll
     for (int k = 0; k < NV; k++) tot[k] = 0.0;
@@ -81,10 +87,15 @@ __device__ __forceinline__ void grid_sum(double (&v)[NV], double* partials, unsi
     }
     block_sum<NV>(tot);
     if (threadIdx.x == 0) {
-        fin(tot);
+        fin(tot, s_aux);
         *counter = 0u;
         __threadfence();
     }
+}
+template <int NV, typename Fin>
+__device__ __forceinline__ void grid_sum(double (&v)[NV], double* partials, unsigned* counter,
+                                         Fin fin) {
+    grid_sum<NV>(v, partials, counter, [] { return 0.0; }, [&](double* tot, double) { fin(tot); });
 }
 
 // ---------------------------------------------------------------------------

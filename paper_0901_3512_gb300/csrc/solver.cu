@@ -64,17 +64,20 @@ inline int lean_blocks(long n, int w) { return std::min(vec_blocks(n, w), 2 * 15
 // may queue iterations ahead of its next poll.
 // ===========================================================================
 
-// Algorithm 1 step 9 bookkeeping after beta_i is final.
-__device__ void lz_after_beta(const LzDev& L, int i) {
+// |zeta_i / delta_i| of the residual estimate, known before beta_i
+__device__ __forceinline__ double lz_ratio(const LzDev& L, int i) { return fabs(L.zeta[i - 1] / L.delta[i - 1]); }
+
+// Algorithm 1 step 9 bookkeeping after beta_i is final (ratio: lz_ratio).
+__device__ void lz_after_beta(const LzDev& L, int i, double ratio) {
     LzCtl* c = L.ctl;
     const double b = L.beta[i - 1], a = L.alpha[i - 1];
-    const double d = L.delta[i - 1], z = L.zeta[i - 1];
+    const double d = L.delta[i - 1];
     if (!isfinite(b) || !isfinite(d) || !isfinite(a)) {
         c->status = SEEDCG_ERR_NAN;
         c->m = i;
         return;
     }
-    const double est = b * fabs(z / d);
+    const double est = b * ratio;
     if (c->m_conv == 0 && est <= c->tol * c->bnorm1) {
         c->m_conv = i;
         int m1 = i + c->extra_iters;
@@ -88,15 +91,19 @@ __device__ void lz_after_beta(const LzDev& L, int i) {
     }
 }
 
+// gamma_{i-1} = beta_{i-1} / delta_{i-1}, known before alpha_i
+__device__ __forceinline__ double lz_gamma(const LzDev& L, int i) {
+    return i == 1 ? 0.0 : L.beta[i - 2] / L.delta[i - 2];
+}
+
 // alpha_i is final: the LU recurrence of T (Algorithm 1 steps 3 and 6, Eq. 2)
-__device__ __forceinline__ void lz_alpha_fin(const LzDev& L, int i, double a) {
+__device__ __forceinline__ void lz_alpha_fin(const LzDev& L, int i, double a, double gm) {
     L.alpha[i - 1] = a;
     if (i == 1) {
         L.delta[0] = a;
         L.zeta[0] = L.ctl->beta0;
     } else {
         const double bp = L.beta[i - 2];
-        const double gm = bp / L.delta[i - 2];
         L.gamma[i - 2] = gm;
         L.delta[i - 1] = a - gm * bp;
         L.zeta[i - 1] = -gm * L.zeta[i - 2];
@@ -107,35 +114,46 @@ __device__ __forceinline__ void lz_alpha_fin(const LzDev& L, int i, double a) {
     }
 }
 
-// v_1 = r_0^1 / beta_0 (step 2); beta_0 already in ctl
+// Steps 2 and 9, folded into the operator's first kernel: v_i = w / ||w|| with w = f of the last iteration
+// (||w|| = beta_{i-1}) or r_0^1 (beta_0).  The kernel applies D to w and scales the result, and every thread
+// forms its own entries of v_i and stores them as vector and as row of V (a PO step rewrites both).
 template <typename R>
-__global__ void k_lz_start(const cx_t<R>* __restrict__ r0, cx_t<R>* __restrict__ v, long n,
-                           LzDev L) {
-    pdl_enter();
-    const double inv = 1.0 / L.ctl->beta0;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n;
-         e += (long)gridDim.x * blockDim.x) {
-        cx_t<R> z = r0[e];
-        v[e] = mk<R>((R)(z.x * inv), (R)(z.y * inv));
-    }
+__device__ __forceinline__ R lz_inv(const LzDev& L, int i) {
+    return R(1) / (R)(i == 1 ? L.ctl->beta0 : L.beta[i - 2]);
 }
 
-// t = D v_i
-template <typename R>
+// v_i and its row of V at one site
+template <typename R, typename VT>
+__device__ __forceinline__ void lz_put_v(const Spinor<R>& w, R inv, cx_t<R>* v, VT* Vrow, int vol, int s) {
+    Spinor<R> sc;
+#pragma unroll
+    for (int k = 0; k < 12; k++) sc.c[k / 3][k % 3] = cscale(w.c[k / 3][k % 3], inv);
+    store_spinor(v, vol, s, sc);
+#pragma unroll
+    for (int k = 0; k < 12; k++) st_cx(Vrow, sidx(k, s, vol), sc.c[k / 3][k % 3]);
+}
+
+// v_i = w / ||w||, t = D v_i
+template <typename R, typename VT>
 __global__ void __launch_bounds__(kSiteThreads, 7)
-k_lz_D(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict__ v,
-       cx_t<R>* __restrict__ t, int i, LzDev L) {
+k_lz_D(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict__ w, cx_t<R>* __restrict__ v,
+       VT* __restrict__ Vrow, cx_t<R>* __restrict__ t, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.vol) return;
     const int vol = g.vol;
+    const R inv = lz_inv<R>(L, i);
     Nbr n = neighbours(g, s);
     Spinor<R> res;
-    auto load = [&](int y, Spinor<R>& p) { load_spinor(v, vol, y, p); };
+    load_spinor(w, vol, s, res);
+    lz_put_v(res, inv, v, Vrow, vol, s);
+    auto load = [&](int y, Spinor<R>& p) { load_spinor(w, vol, y, p); };
     auto fl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + s); };
     auto bl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + n.b[mu]); };
     wilson_site<0, R>(n, s, load, fl, bl, kappa, res);
+#pragma unroll
+    for (int k = 0; k < 12; k++) res.c[k / 3][k % 3] = cscale(res.c[k / 3][k % 3], inv);
     store_spinor(t, vol, s, res);
 }
 
@@ -175,21 +193,22 @@ k_lz_Ddag(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restr
         }
         red[0] = (double)part;
     }
-    grid_sum<1>(red, L.partials, L.counters + CTR_B, [&](double* tot) { lz_alpha_fin(L, i, tot[0]); });
+    grid_sum<1>(red, L.partials, L.counters + CTR_B, [&] { return lz_gamma(L, i); },
+                    [&](double* tot, double gm) { lz_alpha_fin(L, i, tot[0], gm); });
 }
 
 // Even-odd system (Section 3): M = A^dag A on odd-site half vectors, A = 1 - kappa^2 H_oe H_eo,
 // applied in four parity-restricted hops per Lanczos iteration:
-//   STAGE 0  e = H_eo v                 (even sites)
-//   STAGE 1  y = v - kappa^2 H_oe e     (A v)
+//   STAGE 0  e = H_eo w                 (even sites; w as in k_lz_D)
+//   STAGE 1  y = (w - kappa^2 H_oe e) / ||w|| = A v_i, and v_i = w / ||w|| with its row of V
 //   STAGE 2  e = H^dag_eo y
 //   STAGE 3  f = y - kappa^2 H^dag_oe e - beta_{i-1} v_{i-1};  alpha_i = Re v_i^dag f
 //            (the hops of D^dag give A^dag = g5 A g5), with the LU finaliser of k_lz_Ddag.
-template <typename R, int STAGE>
+template <typename R, typename VT, int STAGE>
 __global__ void __launch_bounds__(kRedThreads)
 k_lz_eo(Geom g, const cx_t<R>* __restrict__ u, R kk, const cx_t<R>* __restrict__ other,
-        const cx_t<R>* __restrict__ same, cx_t<R>* __restrict__ out, const cx_t<R>* __restrict__ v,
-        const cx_t<R>* __restrict__ vprev, int i, LzDev L) {
+        const cx_t<R>* __restrict__ same, cx_t<R>* __restrict__ out, cx_t<R>* __restrict__ v,
+        const cx_t<R>* __restrict__ vprev, VT* __restrict__ Vrow, int i, LzDev L) {
     pdl_enter();
     constexpr int DAG = STAGE >= 2 ? 1 : 0;
     constexpr int POUT = (STAGE & 1) ? 1 : 0;
@@ -201,6 +220,14 @@ k_lz_eo(Geom g, const cx_t<R>* __restrict__ u, R kk, const cx_t<R>* __restrict__
         Spinor<R> acc;
         eo_site_apply<R, DAG>(g, u, POUT, hh, other, POUT ? same : nullptr, R(1), POUT ? -kk : R(1), acc);
         if (STAGE < 3) {
+            if (STAGE == 1) {
+                const R inv = lz_inv<R>(L, i);
+                Spinor<R> w;
+                load_spinor(same, vh, hh, w);
+                lz_put_v(w, inv, v, Vrow, vh, hh);
+#pragma unroll
+                for (int k = 0; k < 12; k++) acc.c[k / 3][k % 3] = cscale(acc.c[k / 3][k % 3], inv);
+            }
             store_spinor(out, vh, hh, acc);
         } else {
             const R bprev = i > 1 ? (R)L.beta[i - 2] : R(0);
@@ -222,15 +249,23 @@ k_lz_eo(Geom g, const cx_t<R>* __restrict__ u, R kk, const cx_t<R>* __restrict__
         }
     }
     if (STAGE == 3)
-        grid_sum<1>(red, L.partials, L.counters + CTR_B, [&](double* tot) { lz_alpha_fin(L, i, tot[0]); });
+        grid_sum<1>(red, L.partials, L.counters + CTR_B, [&] { return lz_gamma(L, i); },
+                    [&](double* tot, double gm) { lz_alpha_fin(L, i, tot[0], gm); });
 }
 
-// FP64 runs apply the operator in fixed point (fixhop.cuh).  The last hop's epilogue forms
-// f = val - beta_{i-1} v_{i-1} and this thread's share of alpha_i = Re v_i^dag f; the others store.
+// FP64 runs apply the operator in fixed point (fixhop.cuh).  The epilogues: PUT (D, or A's second hop)
+// scales by 1 / ||w|| and stores v_i and its row of V as k_lz_D does; LAST forms f = val - beta_{i-1} v_{i-1}
+// and this thread's share of alpha_i = Re v_i^dag f; the other hops store.
+enum { LZ_STORE = 0, LZ_PUT = 1, LZ_LAST = 2 };
+template <int KIND>
 struct LzFixEpi {
     static constexpr bool kShare = false;
     double2* out;
-    const double2* v;       // null: store only
+    const double2* w;       // LZ_PUT
+    double2* vout;
+    double2* Vrow;
+    double inv;
+    const double2* v;       // LZ_LAST
     const double2* vprev;   // null: no beta_{i-1} v_{i-1}
     double bprev;
     int vo;
@@ -238,7 +273,16 @@ struct LzFixEpi {
     __device__ __forceinline__ double operator()(int, int plane, int idx, int, bool live, double2 a, double2 b) {
         if (live) {
             const size_t ix = ((size_t)plane * vo + idx) * 2;
-            if (v) {
+            if (KIND == LZ_PUT) {
+                const double2 wa = w[ix], wb = w[ix + 1];
+                const double2 sa = cscale(wa, inv), sb = cscale(wb, inv);
+                vout[ix] = sa;
+                vout[ix + 1] = sb;
+                Vrow[ix] = sa;
+                Vrow[ix + 1] = sb;
+                a = cscale(a, inv);
+                b = cscale(b, inv);
+            } else if (KIND == LZ_LAST) {
                 if (vprev) {
                     const double2 pa = vprev[ix], pb = vprev[ix + 1];
                     a.x -= bprev * pa.x;
@@ -257,50 +301,56 @@ struct LzFixEpi {
     __device__ __forceinline__ void put(int, double) {}
 };
 
-template <bool LAST>
+template <int KIND>
 __global__ void __launch_bounds__(kFixThreads, 2)
-k_lz_fix(FixDev F, FixOp op, const double2* __restrict__ v, const double2* __restrict__ vprev,
-         double2* __restrict__ out, int i, LzDev L) {
+k_lz_fix(FixDev F, FixOp op, const double2* __restrict__ w, double2* __restrict__ v,
+         const double2* __restrict__ vprev, double2* __restrict__ Vrow, double2* __restrict__ out, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
     extern __shared__ __align__(16) unsigned char fix_smem[];
-    LzFixEpi epi{out,
-                 LAST ? v : nullptr,
-                 LAST && i > 1 ? vprev : nullptr,
-                 LAST && i > 1 ? L.beta[i - 2] : 0.0,
-                 op.parity < 0 ? F.g.vol : F.g.vol / 2,
-                 0.0};
+    LzFixEpi<KIND> epi{out,
+                       w,
+                       v,
+                       Vrow,
+                       KIND == LZ_PUT ? lz_inv<double>(L, i) : 1.0,
+                       v,
+                       KIND == LZ_LAST && i > 1 ? vprev : nullptr,
+                       KIND == LZ_LAST && i > 1 ? L.beta[i - 2] : 0.0,
+                       op.parity < 0 ? F.g.vol : F.g.vol / 2,
+                       0.0};
     fix_tile(F, op, blockIdx.x, 0, 1, 1, fix_smem, epi);
-    if (LAST) {
+    if (KIND == LZ_LAST) {
         double red[1] = {epi.part};
-        grid_sum<1>(red, L.partials, L.counters + CTR_B, [&](double* tot) { lz_alpha_fin(L, i, tot[0]); });
+        grid_sum<1>(red, L.partials, L.counters + CTR_B, [&] { return lz_gamma(L, i); },
+                    [&](double* tot, double gm) { lz_alpha_fin(L, i, tot[0], gm); });
     }
 }
 
-template <bool LAST>
-void lz_fix(const FixDev& F, const FixOp& op, const double2* v, const double2* vprev, double2* out, int i,
-            const LzDev& L, cudaStream_t st) {
+template <int KIND>
+void lz_fix(const FixDev& F, const FixOp& op, const double2* w, double2* v, const double2* vprev, double2* Vrow,
+            double2* out, int i, const LzDev& L, cudaStream_t st) {
     static const cudaError_t attr =
-        cudaFuncSetAttribute(k_lz_fix<LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
+        cudaFuncSetAttribute(k_lz_fix<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
     SEEDCG_CUDA_TRY(attr);
     const int sites = op.parity < 0 ? F.g.vol : F.g.vol / 2;
-    launch_pdl(pdl_for(12L * sites), k_lz_fix<LAST>, (sites + 31) / 32, kFixThreads, kFixSmem, st, F, op, v, vprev, out, i, L);
+    launch_pdl(pdl_for(12L * sites), k_lz_fix<KIND>, (sites + 31) / 32, kFixThreads, kFixSmem, st, F, op, w, v, vprev,
+               Vrow, out, i, L);
 }
 
-// f = M v - beta_{i-1} v_{i-1} and alpha_i in FP64: D and D^dag, or the four half-lattice hops
-// (t, e: full or odd half, and even half scratch)
-void lz_apply_f64(const FixDev& F, bool eo, const double2* v, const double2* vprev, double2* t, double2* e,
-                  double2* f, int i, const LzDev& L, cudaStream_t st) {
-    const FixView vv = fix_planes(v, F.g, eo), vt = fix_planes(t, F.g, eo), ve = fix_planes(e, F.g, eo);
+// v_i = w / ||w||, f = M v_i - beta_{i-1} v_{i-1} and alpha_i in FP64: D and D^dag, or the four half-lattice
+// hops (t, e: full or odd half, and even half scratch)
+void lz_apply_f64(const FixDev& F, bool eo, const double2* w, double2* v, const double2* vprev, double2* Vrow,
+                  double2* t, double2* e, double2* f, int i, const LzDev& L, cudaStream_t st) {
+    const FixView vw = fix_planes(w, F.g, eo), vt = fix_planes(t, F.g, eo), ve = fix_planes(e, F.g, eo);
     if (!eo) {
-        lz_fix<false>(F, FixOp{0, -1, vv, 1, 1, vv}, nullptr, nullptr, t, i, L, st);
-        lz_fix<true>(F, FixOp{1, -1, vt, 1, 1, vt}, v, vprev, f, i, L, st);
+        lz_fix<LZ_PUT>(F, FixOp{0, -1, vw, 1, 1, vw}, w, v, nullptr, Vrow, t, i, L, st);
+        lz_fix<LZ_LAST>(F, FixOp{1, -1, vt, 1, 1, vt}, nullptr, v, vprev, nullptr, f, i, L, st);
         return;
     }
-    lz_fix<false>(F, FixOp{0, 0, vv, 0, 1, vv}, nullptr, nullptr, e, i, L, st);
-    lz_fix<false>(F, FixOp{0, 1, ve, 1, -1, vv}, nullptr, nullptr, t, i, L, st);
-    lz_fix<false>(F, FixOp{1, 0, vt, 0, 1, vt}, nullptr, nullptr, e, i, L, st);
-    lz_fix<true>(F, FixOp{1, 1, ve, 1, -1, vt}, v, vprev, f, i, L, st);
+    lz_fix<LZ_STORE>(F, FixOp{0, 0, vw, 0, 1, vw}, nullptr, nullptr, nullptr, nullptr, e, i, L, st);
+    lz_fix<LZ_PUT>(F, FixOp{0, 1, ve, 1, -1, vw}, w, v, nullptr, Vrow, t, i, L, st);
+    lz_fix<LZ_STORE>(F, FixOp{1, 0, vt, 0, 1, vt}, nullptr, nullptr, nullptr, nullptr, e, i, L, st);
+    lz_fix<LZ_LAST>(F, FixOp{1, 1, ve, 1, -1, vt}, nullptr, v, vprev, nullptr, f, i, L, st);
 }
 
 // Steps 4 and 7 (literal seeding): eta^j = v_i^dag r_0^j - gamma_{i-1} eta^j for
@@ -383,9 +433,9 @@ k_lz_update(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, cx_t<R>* __r
         }
     }
     double red[1] = {(double)part};
-    grid_sum<1>(red, L.partials, L.counters + CTR_D, [&](double* tot) {
+    grid_sum<1>(red, L.partials, L.counters + CTR_D, [&] { return lz_ratio(L, i); }, [&](double* tot, double ratio) {
         L.beta[i - 1] = sqrt(tot[0]);
-        if (final_beta) lz_after_beta(L, i);
+        if (final_beta) lz_after_beta(L, i, ratio);
     });
 }
 
@@ -476,9 +526,9 @@ k_lz_update_v(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, cx_t<R>* _
         }
     }
     double red[1] = {(double)part};
-    grid_sum<1>(red, L.partials, L.counters + CTR_D, [&](double* tot) {
+    grid_sum<1>(red, L.partials, L.counters + CTR_D, [&] { return lz_ratio(L, i); }, [&](double* tot, double ratio) {
         L.beta[i - 1] = sqrt(tot[0]);
-        if (final_beta) lz_after_beta(L, i);
+        if (final_beta) lz_after_beta(L, i, ratio);
     });
 }
 
@@ -622,10 +672,10 @@ k_po_sub_fin(const cx_t<R>* __restrict__ part, int nseg, cx_t<R>* __restrict__ v
     grid_sum<1>(red, L.partials, L.counters + CTR_PO2, [&](double* tot) { po_check_nv(L, i, tot[0]); });
 }
 
-// v_i /= ||v_i||; dvf = v_i^dag f
-template <typename R>
+// v_i /= ||v_i|| (and its row of V); dvf = v_i^dag f
+template <typename R, typename VT>
 __global__ void __launch_bounds__(kRedThreads)
-k_po_normalise(cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f, long n, int i, LzDev L) {
+k_po_normalise(cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f, VT* __restrict__ Vrow, long n, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
     const R inv = (R)(1.0 / L.ctl->nv);
@@ -634,6 +684,7 @@ k_po_normalise(cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f, long n, i
          e += (long)gridDim.x * blockDim.x) {
         cx_t<R> vv = cscale(v[e], inv);
         v[e] = vv;
+        st_cx(Vrow, e, vv);
         cx_t<R> fv = f[e];
         pr += vv.x * fv.x + vv.y * fv.y;
         pi += vv.x * fv.y - vv.y * fv.x;
@@ -659,7 +710,7 @@ k_po_finish(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, long n, int 
         part += fv.x * fv.x + fv.y * fv.y;
     }
     double red[1] = {(double)part};
-    grid_sum<1>(red, L.partials, L.counters + CTR_PO4, [&](double* tot) {
+    grid_sum<1>(red, L.partials, L.counters + CTR_PO4, [&] { return lz_ratio(L, i); }, [&](double* tot, double ratio) {
         const double bnew = sqrt(tot[0]);
         L.ctl->po_count += 1;
         // an orthogonal projection never lengthens f; growth means the stored
@@ -670,40 +721,8 @@ k_po_finish(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, long n, int 
             return;
         }
         L.beta[i - 1] = bnew;
-        lz_after_beta(L, i);
+        lz_after_beta(L, i, ratio);
     });
-}
-
-// Step 9: store v_i into V (storage type VT); v_{i+1} = f / beta_i
-// (FP32: a thread moves two complex entries, 16-byte loads of v and f)
-template <typename R, typename VT>
-__global__ void k_lz_advance(const cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f,
-                             cx_t<R>* __restrict__ vnext, VT* __restrict__ Vrow, long n, int i,
-                             LzDev L) {
-    pdl_enter();
-    if (i > L.ctl->m) return;
-    const double b = L.beta[i - 1];
-    const bool go = b > 0.0 && i < L.ctl->m;
-    const R inv = go ? (R)(1.0 / b) : R(0);
-    if constexpr (sizeof(R) == 4) {
-        const long ng = n / 2;   // n = 12 * sites is even
-        for (long g = blockIdx.x * (long)blockDim.x + threadIdx.x; g < ng;
-             g += (long)gridDim.x * blockDim.x) {
-            const float4 a = reinterpret_cast<const float4*>(v)[g];
-            float4 c;
-            if (go) c = reinterpret_cast<const float4*>(f)[g];
-            st_cx(Vrow, 2 * g, make_float2(a.x, a.y));
-            st_cx(Vrow, 2 * g + 1, make_float2(a.z, a.w));
-            if (go) reinterpret_cast<float4*>(vnext)[g] = make_float4(c.x * inv, c.y * inv, c.z * inv, c.w * inv);
-        }
-    } else {
-        for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n;
-             e += (long)gridDim.x * blockDim.x) {
-            cx_t<R> vv = v[e];
-            st_cx(Vrow, e, vv);
-            if (go) vnext[e] = cscale(f[e], inv);
-        }
-    }
 }
 
 // ||x||^2 of one flat vector into *out (FP64)
@@ -1080,24 +1099,25 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> po_ev;
     int m = 0, m_conv = 0, po_count = 0, lz_status = SEEDCG_OK, breakdown = 0;
     if (beta0 > 0.0) {
-        const int sb = site_blocks(vol);
-        launch_pdl(pdl, k_lz_start<R>, rb, kRedThreads, 0, st, R0, vA, n, L);
         cx_t<R>* v = vA;
         cx_t<R>* vprev = vB;
         int i = 1;
         const int sbh = site_blocks(vol / 2);
         const R kk = (R)(h->kappa * h->kappa);
         for (; i <= m_max; i++) {
+            VT* Vrow = Vb + (size_t)(i - 1) * n;
+            const cx_t<R>* w = i == 1 ? R0 : fv;   // v_i = w / ||w||
             if constexpr (sizeof(R) == 8) {
-                lz_apply_f64(fix_of(h), eo, v, vprev, tv, ev, fv, i, L, st);
+                lz_apply_f64(fix_of(h), eo, w, v, vprev, Vrow, tv, ev, fv, i, L, st);
             } else if (eo) {
                 // f = A^dag A v - beta v_prev, alpha: four half-lattice hops
-                launch_pdl(pdl, k_lz_eo<R, 0>, sbh, kRedThreads, 0, st, h->g, U, kk, v, nullptr, ev, nullptr, nullptr, i, L);
-                launch_pdl(pdl, k_lz_eo<R, 1>, sbh, kRedThreads, 0, st, h->g, U, kk, ev, v, tv, nullptr, nullptr, i, L);
-                launch_pdl(pdl, k_lz_eo<R, 2>, sbh, kRedThreads, 0, st, h->g, U, kk, tv, nullptr, ev, nullptr, nullptr, i, L);
-                launch_pdl(pdl, k_lz_eo<R, 3>, sbh, kRedThreads, 0, st, h->g, U, kk, ev, tv, fv, v, vprev, i, L);
+                const cx_t<R>* none = nullptr;
+                launch_pdl(pdl, k_lz_eo<R, VT, 0>, sbh, kRedThreads, 0, st, h->g, U, kk, w, none, ev, v, none, Vrow, i, L);
+                launch_pdl(pdl, k_lz_eo<R, VT, 1>, sbh, kRedThreads, 0, st, h->g, U, kk, ev, w, tv, v, none, Vrow, i, L);
+                launch_pdl(pdl, k_lz_eo<R, VT, 2>, sbh, kRedThreads, 0, st, h->g, U, kk, tv, none, ev, v, none, Vrow, i, L);
+                launch_pdl(pdl, k_lz_eo<R, VT, 3>, sbh, kRedThreads, 0, st, h->g, U, kk, ev, tv, fv, v, vprev, Vrow, i, L);
             } else {
-                launch_pdl(pdl, k_lz_D<R>, site_blocks_lz(vol), kSiteThreads, 0, st, h->g, U, kap, v, tv, i, L);
+                launch_pdl(pdl, k_lz_D<R, VT>, site_blocks_lz(vol), kSiteThreads, 0, st, h->g, U, kap, w, v, Vrow, tv, i, L);
                 launch_pdl(pdl, k_lz_Ddag<R>, site_blocks_lz(vol), kSiteThreads, 0, st, h->g, U, kap, tv, v, vprev, fv, i, L);
             }
             if (literal) {
@@ -1126,13 +1146,11 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                     project(na, Bst, 2, 2);
                     po_subtract(na, cvcol, v, fv, i);
                 }
-                launch_pdl(pdl, k_po_normalise<R>, rb, kRedThreads, 0, st, v, fv, n, i, L);
+                launch_pdl(pdl, k_po_normalise<R, VT>, rb, kRedThreads, 0, st, v, fv, Vrow, n, i, L);
                 launch_pdl(pdl, k_po_finish<R>, rb, kRedThreads, 0, st, v, fv, n, i, L);
                 cudaEventRecord(e1, st);
                 po_ev.push_back({e0, e1});
             }
-            launch_pdl(pdl, k_lz_advance<R, VT>, rb, kRedThreads, 0, st, v, fv, vprev, Vb + (size_t)(i - 1) * n, n,
-                                                           i, L);
             std::swap(v, vprev);
             if (i % poll == 0 || i == m_max) {
                 SEEDCG_CUDA_TRY(cudaMemcpyAsync(pin, L.ctl, sizeof(int) * 8, cudaMemcpyDeviceToHost, st));
