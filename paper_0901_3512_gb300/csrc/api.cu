@@ -540,6 +540,7 @@ void seedcg_destroy(seedcg_handle* h) {
     h->red.release();
     h->work.release();
     h->coef.release();
+    h->row_exp.release();
     h->tcbuf.release();
     h->cgbuf.release();
     h->hostio.release();

@@ -23,6 +23,7 @@ struct seedcg_handle {
     seedcg::DevBuf lz_scalars;    // LzCtl + alpha/beta/... arrays
     seedcg::DevBuf red;           // reduction partials + counters
     seedcg::DevBuf work;          // working vectors of the solve
+    seedcg::DevBuf row_exp;       // FP64 basis: largest exponent per block of entries over the stored rows
     seedcg::DevBuf coef;          // projection coefficients / gemm split scratch
     seedcg::DevBuf staging;       // complex128 staging of host B / X
     seedcg::DevBuf tcbuf;         // tensor-core projection: bf16 B operand + FP32 partials

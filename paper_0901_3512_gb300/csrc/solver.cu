@@ -15,7 +15,7 @@
 
 #include "cg_batch.cuh"
 #include "eo.cuh"
-#include "fixhop.cuh"
+#include "fixproj.cuh"
 #include "handle.cuh"
 #include "kernels.cuh"
 #include "reduce.cuh"
@@ -264,6 +264,7 @@ struct LzFixEpi {
     const double2* w;       // LZ_PUT
     double2* vout;
     double2* Vrow;
+    int* runE;              // running exponents of the stored rows
     double inv;
     const double2* v;       // LZ_LAST
     const double2* vprev;   // null: no beta_{i-1} v_{i-1}
@@ -271,8 +272,14 @@ struct LzFixEpi {
     int vo;
     double part;
     __device__ __forceinline__ double operator()(int, int plane, int idx, int, bool live, double2 a, double2 b) {
+        const size_t ix = ((size_t)plane * vo + idx) * 2;
+        if (KIND == LZ_PUT) {
+            // groups of 8 lanes hold a block of 16 entries and are live or not as a whole
+            const double2 za = live ? cscale(w[ix], inv) : make_double2(0.0, 0.0);
+            const double2 zb = live ? cscale(w[ix + 1], inv) : make_double2(0.0, 0.0);
+            fix_row_exponent<2>(runE, live ? (long)ix : 1, max(fix_absword(za), fix_absword(zb)), 0xffffffffu);
+        }
         if (live) {
-            const size_t ix = ((size_t)plane * vo + idx) * 2;
             if (KIND == LZ_PUT) {
                 const double2 wa = w[ix], wb = w[ix + 1];
                 const double2 sa = cscale(wa, inv), sb = cscale(wb, inv);
@@ -304,7 +311,8 @@ struct LzFixEpi {
 template <int KIND>
 __global__ void __launch_bounds__(kFixThreads, 2)
 k_lz_fix(FixDev F, FixOp op, const double2* __restrict__ w, double2* __restrict__ v,
-         const double2* __restrict__ vprev, double2* __restrict__ Vrow, double2* __restrict__ out, int i, LzDev L) {
+         const double2* __restrict__ vprev, double2* __restrict__ Vrow, int* __restrict__ runE,
+         double2* __restrict__ out, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
     extern __shared__ __align__(16) unsigned char fix_smem[];
@@ -312,6 +320,7 @@ k_lz_fix(FixDev F, FixOp op, const double2* __restrict__ w, double2* __restrict_
                        w,
                        v,
                        Vrow,
+                       runE,
                        KIND == LZ_PUT ? lz_inv<double>(L, i) : 1.0,
                        v,
                        KIND == LZ_LAST && i > 1 ? vprev : nullptr,
@@ -328,29 +337,29 @@ k_lz_fix(FixDev F, FixOp op, const double2* __restrict__ w, double2* __restrict_
 
 template <int KIND>
 void lz_fix(const FixDev& F, const FixOp& op, const double2* w, double2* v, const double2* vprev, double2* Vrow,
-            double2* out, int i, const LzDev& L, cudaStream_t st) {
+            int* runE, double2* out, int i, const LzDev& L, cudaStream_t st) {
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_lz_fix<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
     SEEDCG_CUDA_TRY(attr);
     const int sites = op.parity < 0 ? F.g.vol : F.g.vol / 2;
     launch_pdl(pdl_for(12L * sites), k_lz_fix<KIND>, (sites + 31) / 32, kFixThreads, kFixSmem, st, F, op, w, v, vprev,
-               Vrow, out, i, L);
+               Vrow, runE, out, i, L);
 }
 
 // v_i = w / ||w||, f = M v_i - beta_{i-1} v_{i-1} and alpha_i in FP64: D and D^dag, or the four half-lattice
 // hops (t, e: full or odd half, and even half scratch)
 void lz_apply_f64(const FixDev& F, bool eo, const double2* w, double2* v, const double2* vprev, double2* Vrow,
-                  double2* t, double2* e, double2* f, int i, const LzDev& L, cudaStream_t st) {
+                  int* runE, double2* t, double2* e, double2* f, int i, const LzDev& L, cudaStream_t st) {
     const FixView vw = fix_planes(w, F.g, eo), vt = fix_planes(t, F.g, eo), ve = fix_planes(e, F.g, eo);
     if (!eo) {
-        lz_fix<LZ_PUT>(F, FixOp{0, -1, vw, 1, 1, vw}, w, v, nullptr, Vrow, t, i, L, st);
-        lz_fix<LZ_LAST>(F, FixOp{1, -1, vt, 1, 1, vt}, nullptr, v, vprev, nullptr, f, i, L, st);
+        lz_fix<LZ_PUT>(F, FixOp{0, -1, vw, 1, 1, vw}, w, v, nullptr, Vrow, runE, t, i, L, st);
+        lz_fix<LZ_LAST>(F, FixOp{1, -1, vt, 1, 1, vt}, nullptr, v, vprev, nullptr, nullptr, f, i, L, st);
         return;
     }
-    lz_fix<LZ_STORE>(F, FixOp{0, 0, vw, 0, 1, vw}, nullptr, nullptr, nullptr, nullptr, e, i, L, st);
-    lz_fix<LZ_PUT>(F, FixOp{0, 1, ve, 1, -1, vw}, w, v, nullptr, Vrow, t, i, L, st);
-    lz_fix<LZ_STORE>(F, FixOp{1, 0, vt, 0, 1, vt}, nullptr, nullptr, nullptr, nullptr, e, i, L, st);
-    lz_fix<LZ_LAST>(F, FixOp{1, 1, ve, 1, -1, vt}, nullptr, v, vprev, nullptr, f, i, L, st);
+    lz_fix<LZ_STORE>(F, FixOp{0, 0, vw, 0, 1, vw}, nullptr, nullptr, nullptr, nullptr, nullptr, e, i, L, st);
+    lz_fix<LZ_PUT>(F, FixOp{0, 1, ve, 1, -1, vw}, w, v, nullptr, Vrow, runE, t, i, L, st);
+    lz_fix<LZ_STORE>(F, FixOp{1, 0, vt, 0, 1, vt}, nullptr, nullptr, nullptr, nullptr, nullptr, e, i, L, st);
+    lz_fix<LZ_LAST>(F, FixOp{1, 1, ve, 1, -1, vt}, nullptr, v, vprev, nullptr, nullptr, f, i, L, st);
 }
 
 // Steps 4 and 7 (literal seeding): eta^j = v_i^dag r_0^j - gamma_{i-1} eta^j for
@@ -649,6 +658,40 @@ k_po_sub_seg(const VT* __restrict__ V, long ldv, int na, int seg, const double2*
     }
 }
 
+// the FP64 subtraction in fixed point (fixproj.cuh): one entry per thread; SEG: sums of row segment blockIdx.y to
+// part, as k_po_sub_seg.  8^3 x 16, 320 rows on average: 460 us on the FP64 pipe, 190 us here.
+template <bool SEG>
+__global__ void __launch_bounds__(kRedThreads, 2)
+k_po_sub_fix(const double2* __restrict__ V, long ldv, int na, int seg, const int* __restrict__ runE,
+             const double2* __restrict__ coef, int cv, double2* __restrict__ v, double2* __restrict__ f, long n,
+             double2* __restrict__ part, int i, LzDev L) {
+    pdl_enter();
+    if (i > L.ctl->m) return;
+    __shared__ FixColumns<2> S;
+    const long e = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    const int r0 = blockIdx.y * seg, r1 = r0 + seg < na ? r0 + seg : na;
+    const int col[2] = {cv, 1 - cv};
+    double2 av[2];
+    fix_accumulate<2>(V, ldv, r0, r1, runE, coef, 2, col, e, e < n, av, S);
+    if (SEG) {
+        if (e < n) {
+            double2* pv = part + (size_t)blockIdx.y * 2 * n + e;
+            pv[0] = av[0];
+            pv[n] = av[1];
+        }
+        return;
+    }
+    double acc = 0.0;
+    if (e < n) {
+        const double2 vv = csub(v[e], av[0]);
+        v[e] = vv;
+        f[e] = csub(f[e], av[1]);
+        acc = vv.x * vv.x + vv.y * vv.y;
+    }
+    double red[1] = {acc};
+    grid_sum<1>(red, L.partials, L.counters + CTR_PO2, [&](double* tot) { po_check_nv(L, i, tot[0]); });
+}
+
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
 k_po_sub_fin(const cx_t<R>* __restrict__ part, int nseg, cx_t<R>* __restrict__ v,
@@ -675,7 +718,8 @@ k_po_sub_fin(const cx_t<R>* __restrict__ part, int nseg, cx_t<R>* __restrict__ v
 // v_i /= ||v_i|| (and its row of V); dvf = v_i^dag f
 template <typename R, typename VT>
 __global__ void __launch_bounds__(kRedThreads)
-k_po_normalise(cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f, VT* __restrict__ Vrow, long n, int i, LzDev L) {
+k_po_normalise(cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f, VT* __restrict__ Vrow, int* __restrict__ runE,
+               long n, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
     const R inv = (R)(1.0 / L.ctl->nv);
@@ -685,6 +729,8 @@ k_po_normalise(cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f, VT* __res
         cx_t<R> vv = cscale(v[e], inv);
         v[e] = vv;
         st_cx(Vrow, e, vv);
+        if constexpr (std::is_same<VT, double2>::value)
+            fix_row_exponent<1>(runE, e, fix_absword(vv), 0xffffu << (threadIdx.x & 16));
         cx_t<R> fv = f[e];
         pr += vv.x * fv.x + vv.y * fv.y;
         pi += vv.x * fv.y - vv.y * fv.x;
@@ -970,6 +1016,12 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     }
     h->vbasis.ensure(vrow * (size_t)m_max);
     VT* Vb = h->vbasis.as<VT>();
+    int* runE = nullptr;   // FP64: the stored rows' exponents for the fixed-point products
+    if (fp64) {
+        h->row_exp.ensure((size_t)(n / kFixBlock) * sizeof(int));
+        SEEDCG_CUDA_TRY(cudaMemsetAsync(h->row_exp.p, 0, (size_t)(n / kFixBlock) * sizeof(int), st));
+        runE = h->row_exp.as<int>();
+    }
     h->vbasis_prec = o.precision;
     h->vbasis_eo = eo;
     h->vbasis_m = 0;
@@ -980,7 +1032,8 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     const size_t seg3 = 3 * 2 * (size_t)n * sizeof(cx_t<R>) / sizeof(double2);
     const size_t split_elems = std::max<size_t>(
         std::max<size_t>(std::max<size_t>(coef_elems * 48, (size_t)1 << 20), seg3),
-        seeds_streamed ? proj_scratch_elems<R, VT>(n, m_max) : proj_scratch_elems<R, VT>(n, m_max) / 2);
+        fp64 ? proj_fix_scratch(n, m_max)
+             : seeds_streamed ? proj_scratch_elems<R, VT>(n, m_max) : proj_scratch_elems<R, VT>(n, m_max) / 2);
     h->coef.ensure((coef_elems + split_elems) * sizeof(double2));
     double2* Cc = h->coef.as<double2>();
     double2* split = Cc + coef_elems;
@@ -1011,7 +1064,9 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                 return;
             }
         }
-        if (nvec <= 2 || seeds_streamed)
+        if constexpr (sizeof(R) == 8)
+            proj_fix(Vb, n, rows, runE, X, n, nvec, n, Cc, ldc, split, split_elems, st);
+        else if (nvec <= 2 || seeds_streamed)
             proj<R, VT>(Vb, n, rows, X, n, nvec, n, Cc, ldc, split, split_elems, st);
         else
             gemm_t<R, VT>(Vb, n, rows, X, n, nvec, n, Cc, ldc, split, split_elems, st);
@@ -1022,15 +1077,31 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     int nsm = 0;
     SEEDCG_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device));
     static int seg_occ = 0;
-    if (!seg_occ)
-        SEEDCG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&seg_occ, k_po_sub_seg<R, VT>,
-                                                                      kRedThreads, 0));
+    if constexpr (sizeof(R) == 4)
+        if (!seg_occ)
+            SEEDCG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&seg_occ, k_po_sub_seg<R, VT>,
+                                                                          kRedThreads, 0));
     constexpr int kW = 16 / (int)sizeof(VT);
     if (n % 4 != 0) throw Error{SEEDCG_ERR_ARG, "spinor length not a multiple of 4"};
     const long po_gb = (n / kW + kRedThreads - 1) / kRedThreads;
     const long seg_cap = (long)(split_elems * sizeof(double2) / (2 * (size_t)n * sizeof(cx_t<R>)));
     auto po_subtract = [&](int na, int cvcol, cx_t<R>* vv, cx_t<R>* ff, int i) {
         long nseg = 1;
+        if constexpr (sizeof(R) == 8) {
+            // the issue rate bounds it: segments of at least 32 rows until four blocks per SM are there
+            nseg = std::max(1L, std::min<long>({8, (4 * (long)nsm + po_gb - 1) / po_gb, na / 32, seg_cap}));
+            const int seg = (int)((na + nseg - 1) / nseg), ns = (na + seg - 1) / seg;
+            double2* sp = split;
+            if (ns > 1) {
+                launch_pdl(pdl, k_po_sub_fix<true>, dim3((unsigned)po_gb, ns), kRedThreads, 0, st, Vb, n, na, seg, runE,
+                           Cc, cvcol, vv, ff, n, sp, i, L);
+                launch_pdl(pdl, k_po_sub_fin<R>, rb, kRedThreads, 0, st, sp, ns, vv, ff, n, i, L);
+            } else {
+                launch_pdl(pdl, k_po_sub_fix<false>, dim3((unsigned)po_gb), kRedThreads, 0, st, Vb, n, na, na, runE, Cc,
+                           cvcol, vv, ff, n, sp, i, L);
+            }
+            return;
+        } else {
         if (na >= 256) {
             const long resident = (long)nsm * std::max(seg_occ, 1);
             nseg = std::min<long>({8, (6 * resident + po_gb - 1) / po_gb, na / 128, seg_cap});
@@ -1046,6 +1117,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
         launch_pdl(pdl, k_po_sub_seg<R, VT>, dim3((unsigned)po_gb, ns), kRedThreads, 0, st, Vb, n, na, seg, Cc, cvcol,
                                                                               n, sp, i, L);
         launch_pdl(pdl, k_po_sub_fin<R>, rb, kRedThreads, 0, st, sp, ns, vv, ff, n, i, L);
+        }
     };
 
     int* pin = reinterpret_cast<int*>(h->pinned);
@@ -1108,7 +1180,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
             VT* Vrow = Vb + (size_t)(i - 1) * n;
             const cx_t<R>* w = i == 1 ? R0 : fv;   // v_i = w / ||w||
             if constexpr (sizeof(R) == 8) {
-                lz_apply_f64(fix_of(h), eo, w, v, vprev, Vrow, tv, ev, fv, i, L, st);
+                lz_apply_f64(fix_of(h), eo, w, v, vprev, Vrow, runE, tv, ev, fv, i, L, st);
             } else if (eo) {
                 // f = A^dag A v - beta v_prev, alpha: four half-lattice hops
                 const cx_t<R>* none = nullptr;
@@ -1146,7 +1218,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                     project(na, Bst, 2, 2);
                     po_subtract(na, cvcol, v, fv, i);
                 }
-                launch_pdl(pdl, k_po_normalise<R, VT>, rb, kRedThreads, 0, st, v, fv, Vrow, n, i, L);
+                launch_pdl(pdl, k_po_normalise<R, VT>, rb, kRedThreads, 0, st, v, fv, Vrow, runE, n, i, L);
                 launch_pdl(pdl, k_po_finish<R>, rb, kRedThreads, 0, st, v, fv, n, i, L);
                 cudaEventRecord(e1, st);
                 po_ev.push_back({e0, e1});
@@ -1195,7 +1267,8 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
         project(m, R0 + n, ns, ns);
         k_seed_tridiag<<<(ns + 31) / 32, 256, 0, st>>>(Cc, ns, ns, m, L);
         SEEDCG_CHECK_LAUNCH();
-        gemm_n<R, VT, double2>(Vb, n, m, Cc, ns, ns, X64 + n, n, n, 1.0, st);
+        if constexpr (sizeof(R) == 8) gemm_n_fix(Vb, n, m, runE, Cc, ns, ns, X64 + n, n, n, st);
+        else gemm_n<R, VT, double2>(Vb, n, m, Cc, ns, ns, X64 + n, n, n, 1.0, st);
     }
     t_seed.stop(st);
 

@@ -102,3 +102,40 @@ def test_non_finite_values_stay_where_the_stencil_puts_them():
         ok = ~touched
         assert np.abs(got[k][ok] - clean[k].reshape(v, 4, 3)[ok]).max() <= 1e-13 * np.abs(clean[k]).max()
     s.close()
+
+
+@pytest.mark.parametrize("dims,nrhs,eo", [((2, 2, 2, 2), 3, 0), ((2, 2, 2, 4), 4, 1), ((2, 4, 6, 10), 6, 0),
+                                          ((8, 8, 8, 8), 8, 0), ((8, 8, 8, 8), 3, 1)])
+def test_fp64_basis_products_in_fixed_point(dims, nrhs, eo):
+    """Re-orthogonalisation (V^dag [v, f] and the subtraction) and the seeds V T^-1 V^dag r against
+    numpy's FP64 products with the stored basis itself: one block of entries, ragged chunks, one to four
+    vectors per pass, rows in one segment and in several.  Bars: V^dag V = 1 to the 1e-10 that step 8
+    promises, and seeds to 1e-9, which covers cond(T) below 1e4 times the rounding of either side."""
+    need_gpu()
+    u = W.gauge_field(dims, 0.5, 81)
+    eta = W.point_sources(dims, nrhs) if not eo else W.z2_sources(dims, nrhs, 82)
+    s = seedcg.Solver(dims, u, 0.19, precision="fp64", past_factor=1.0, stop_after_seed=1, m_max=400)
+    X = dev(np.zeros_like(eta))
+    if eo:
+        code, info = seedcg.seedcg_solve_eo(s.h, dev(eta), X, 1e-8, 0, 5)
+    else:
+        B = dev(np.zeros_like(eta))
+        s.apply(seedcg.OP_DDAG, dev(eta), B, prec=0, multi=1)
+        code, info = s.solve(B, X, 1e-8, 0, 5)
+    m, v = info["m"], W.volume(dims) // (2 if eo else 1)
+    assert info["po_count"] > 0
+    basis = np.zeros((m, v, 4, 3), dtype=np.complex128)
+    seedcg.seedcg_get_basis(s.h, 0, m, basis)
+    V = basis.reshape(m, -1)
+    last = 5 * (m // 5)          # vectors up to the last re-orthogonalisation
+    gram = V[:last].conj() @ V[:last].T
+    assert np.abs(gram[last - 1] - np.eye(last)[last - 1]).max() <= 1e-10
+    if not eo:
+        a, b, _, _ = seedcg.seedcg_get_lanczos(s.h, m)
+        T = np.diag(a) + np.diag(b[:m - 1], 1) + np.diag(b[:m - 1], -1)
+        Bh = host(B).reshape(nrhs, -1)
+        want = (V.T @ np.linalg.solve(T, V.conj() @ Bh[1:].T)).T
+        got = host(X).reshape(nrhs, -1)[1:]
+        for g, w in zip(got, want):
+            assert np.linalg.norm(g - w) <= 1e-9 * np.linalg.norm(w)
+    s.close()
