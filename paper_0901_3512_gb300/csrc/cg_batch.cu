@@ -40,14 +40,7 @@ namespace {
 constexpr int kMaxGroups = 16;
 constexpr int TS = 32;       // sites per dslash tile (one warp per right-hand side)
 // right-hand sides processed side by side per tile (warps per block): picked
-// per batch by the autotuner below from {4, 8, 12}
-
-// brick tiling of one field's lattice: Lx x by x bz sites at one t per tile
-// (x neighbours always in the tile, most y and z neighbours too); n = 0 when
-// the lattice admits no brick of that many sites
-struct Brk {
-    int bx, by, bz, ny, nz, n;
-};
+// per batch by the autotuner below from {3, 4, 6, 8, 12}
 
 template <typename R>
 struct GroupDev {
@@ -65,7 +58,6 @@ struct GroupDev {
     double* part2;      // [cap][ntiles] shares of ||r||^2 after the update of step 3
     int ntiles;         // tiles of 32 (half-)sites; every share is one warp's sum
     int tile0;          // first tile of this group in the dslash grid
-    Brk b64, b128;      // brick tilings of 64 and 128 sites (single-field full-lattice batches)
     FixDev fix;         // the FP64 operator's links
 };
 
@@ -104,20 +96,24 @@ __device__ __forceinline__ int find_group(int b, int ng, const int* tile0) {
 // ||r||^2.  Each warp's sum (32 sites of one system) is one share, written to
 // shares[slot * ntiles + tile32]; k_mf_alpha / k_mf_beta add a system's shares in
 // a fixed order, so no block barrier is needed and the result is reproducible.
-template <typename R>
-__device__ __forceinline__ R r_update_site(cx_t<R>* rr, int vol, int s, const Spinor<R>& q, R a) {
-    Spinor<R> v;
-    load_spinor_rw(rr, vol, s, v);
-    R acc = 0;
+__device__ __forceinline__ float r_update_site(char* rr, size_t plane, unsigned off, const Spinor<float>& q, float a) {
+    Spinor<float> v;
+#pragma unroll
+    for (int c = 0; c < 6; c++) {
+        const float4 z = *reinterpret_cast<const float4*>(rr + c * plane + off);
+        v.c[(2 * c) / 3][(2 * c) % 3] = make_float2(z.x, z.y);
+        v.c[(2 * c + 1) / 3][(2 * c + 1) % 3] = make_float2(z.z, z.w);
+    }
+    float acc = 0;
 #pragma unroll
     for (int k = 0; k < 12; k++) {
-        cx_t<R>& z = v.c[k / 3][k % 3];
-        const cx_t<R> w = q.c[k / 3][k % 3];
+        float2& z = v.c[k / 3][k % 3];
+        const float2 w = q.c[k / 3][k % 3];
         z.x -= a * w.x;
         z.y -= a * w.y;
         acc += z.x * z.x + z.y * z.y;
     }
-    store_spinor(rr, vol, s, v);
+    store_spinor_at(rr, plane, off, v);
     return acc;
 }
 
@@ -125,40 +121,35 @@ __device__ __forceinline__ void put_share(double* shares, int ntiles, int slot, 
     const double d = (double)warp_sum_t(v);
     if ((threadIdx.x & 31) == 0) shares[(size_t)slot * ntiles + tile32] = d;
 }
-__device__ __forceinline__ void put_share(double* shares, int ntiles, int slot, int tile32, double v) {
-    const double d = warp_sum_t(v);
-    if ((threadIdx.x & 31) == 0) shares[(size_t)slot * ntiles + tile32] = d;
-}
-
 // ---------------------------------------------------------------------------
 // 1/3: multi-field multi-RHS dslash (DAG = 0: t = D p and ||t||^2;
 //      DAG = 1: q = D^dag t, r -= alpha q and ||r||^2)
 // ---------------------------------------------------------------------------
-template <typename R, int DAG, int RPB>
-__global__ void __launch_bounds__(TS * RPB, (sizeof(R) == 4 ? (RPB <= 8 ? 3 : 2) : 1))
-k_mf_dslash(const GroupDev<R>* __restrict__ G, int ng, Rows rows, CgS C) {
+template <int DAG, int RPB>
+__global__ void __launch_bounds__(TS * RPB, tile_blocks(RPB))
+k_mf_dslash(const GroupDev<float>* __restrict__ G, int ng, Rows rows, CgS C) {
     pdl_enter();
-    __shared__ cx_t<R> sl[2][4][9][TS];
+    __shared__ float2 sl[72 * TS];   // [fwd/bwd][mu][3a+b][site], times -kappa and the boundary sign
     __shared__ int sb[4][TS];
-    __shared__ Nbr snb[TS];   // neighbours of the tile's sites (kept out of the registers)
-    __shared__ R sgn[2][TS];
+    __shared__ OffNbr snb[TS];       // neighbours of the tile's sites (kept out of the registers)
+    __shared__ float sgn[2][TS];
     __shared__ int s_tile0[kMaxGroups];
     if (threadIdx.x < ng) s_tile0[threadIdx.x] = G[threadIdx.x].tile0;
     __syncthreads();
     const int f = find_group(blockIdx.x, ng, s_tile0);
-    const GroupDev<R>& gd = G[f];
+    const GroupDev<float>& gd = G[f];
     const int nsys = rows.nact[f];
     if (nsys == 0) return;
     const Geom g = gd.g;
     const int vol = g.vol;
     const int tile = blockIdx.x - gd.tile0;
     const int s0 = tile * TS;
-    const R kappa = gd.kappa;
+    const float kappa = gd.kappa;
     if (threadIdx.x < TS) {
         const int s = s0 + threadIdx.x;
         if (s < vol) {
-            Nbr nb = neighbours(g, s);
-            snb[threadIdx.x] = nb;
+            const Nbr nb = neighbours(g, s);
+            snb[threadIdx.x] = offsets_of(nb, 0);
 #pragma unroll
             for (int mu = 0; mu < 4; mu++) sb[mu][threadIdx.x] = nb.b[mu];
             sgn[0][threadIdx.x] = nb.fwrap_t ? kappa : -kappa;
@@ -166,40 +157,35 @@ k_mf_dslash(const GroupDev<R>* __restrict__ G, int ng, Rows rows, CgS C) {
         }
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < 72 * TS; e += blockDim.x) {
-        const int j = e % TS;
-        const int c = (e / TS) % 9;
-        const int mu = (e / (9 * TS)) % 4;
-        const int dir = e / (36 * TS);
-        const int s = s0 + j;
-        cx_t<R> z = mk<R>(0, 0);
-        if (s < vol) {
-            z = __ldg(gd.u + (size_t)(mu * 9 + c) * vol + (dir ? sb[mu][j] : s));
-            z = cscale(z, mu == 3 ? sgn[dir][j] : -kappa);
-        }
-        sl[dir][mu][c][j] = z;
-    }
+    stage_tile_links<TS>(sl, gd.u, vol, [&](int dir, int mu, int j, unsigned& site, float& scale) {
+        if (s0 + j >= vol) return false;
+        site = dir ? sb[mu][j] : s0 + j;
+        scale = mu == 3 ? sgn[dir][j] : -kappa;
+        return true;
+    });
     __syncthreads();
-    const int j = threadIdx.x % TS;   // lane = site of the tile
-    const int qg = threadIdx.x / TS;  // warp = right-hand-side group
-    const int s = s0 + j;
-    const bool live = s < vol;
-    const Nbr& nb = snb[j];
-    auto fl = [&](int mu, int e) { return sl[0][mu][e][j]; };
-    auto bl = [&](int mu, int e) { return sl[1][mu][e][j]; };
-    const cx_t<R>* in = DAG ? gd.t : gd.p;
+    const int j = threadIdx.x % TS;                    // lane = site of the tile
+    const int qg = uniform_warp(threadIdx.x / TS);     // warp = right-hand-side group
+    const bool live = s0 + j < vol;
+    const unsigned off = (unsigned)(s0 + j) * 16u;
+    const OffNbr& nb = snb[j];
+    auto fl = [&](int mu, int e) { return sl[(mu * 9 + e) * TS + j]; };
+    auto bl = [&](int mu, int e) { return sl[(36 + mu * 9 + e) * TS + j]; };
+    const size_t field = (size_t)gd.n * sizeof(float2), plane = (size_t)vol * 16;
+    const char* in = reinterpret_cast<const char*>(DAG ? gd.t : gd.p);
     for (int r = qg; r < nsys; r += RPB) {
-        R dr = 0;
+        float dr = 0;
         if (live) {
-            const cx_t<R>* inr = in + (size_t)r * gd.n;
-            Spinor<R> res;
-            auto load = [&](int y, Spinor<R>& sp) { load_spinor(inr, vol, y, sp); };
-            wilson_site_prescaled<DAG, R>(nb, s, load, fl, bl, res);
+            const char* inr = in + r * field;
+            Spinor<float> res;
+            auto load = [&](unsigned o, Spinor<float>& sp) { load_spinor_at(inr, plane, o, sp); };
+            wilson_site_prescaled<DAG, float>(nb, off, load, fl, bl, res);
             if (DAG) {
-                dr = r_update_site(gd.r + (size_t)r * gd.n, vol, s, res, (R)C.alpha[rows.first[f] + r]);
+                dr = r_update_site(reinterpret_cast<char*>(gd.r) + r * field, plane, off, res,
+                                   (float)C.alpha[rows.first[f] + r]);
             } else {
                 dr = spinor_norm2(res);   // before the store: fewer live registers
-                store_spinor(gd.t + (size_t)r * gd.n, vol, s, res);
+                store_spinor_at(reinterpret_cast<char*>(gd.t) + r * field, plane, off, res);
             }
         }
         put_share(DAG ? gd.part2 : gd.part, gd.ntiles, r, tile, dr);
@@ -213,36 +199,36 @@ k_mf_dslash(const GroupDev<R>* __restrict__ G, int ng, Rows rows, CgS C) {
 // The tile's links (U_mu(x) and U_mu(x - mu) of its 32 sites of the output parity) are
 // staged once in shared memory, times the hop coefficient (1, or -kappa^2 in stages 1
 // and 3) and the t-boundary sign, and reused by every system of the tile.
-template <typename R, int STAGE, int RPB>
-__global__ void __launch_bounds__(TS * RPB, (sizeof(R) == 4 ? 2 : 1))
-k_mf_eo(const GroupDev<R>* __restrict__ G, int ng, Rows rows, CgS C) {
+template <int STAGE, int RPB>
+__global__ void __launch_bounds__(TS * RPB, tile_blocks(RPB))
+k_mf_eo(const GroupDev<float>* __restrict__ G, int ng, Rows rows, CgS C) {
     pdl_enter();
     constexpr int DAG = STAGE >= 2 ? 1 : 0;
     constexpr int POUT = (STAGE & 1) ? 1 : 0;
-    __shared__ cx_t<R> sl[2][4][9][TS];
+    __shared__ float2 sl[72 * TS];
     __shared__ int ssite[TS];
     __shared__ int sb[4][TS];                 // x - mu (full site)
-    __shared__ Nbr snb[TS];                   // neighbours of the tile's sites
-    __shared__ R sgn[2][TS];
+    __shared__ OffNbr snb[TS];                // neighbours of the tile's sites in the other parity
+    __shared__ float sgn[2][TS];
     __shared__ int s_tile0[kMaxGroups];
     if (threadIdx.x < ng) s_tile0[threadIdx.x] = G[threadIdx.x].tile0;
     __syncthreads();
     const int f = find_group(blockIdx.x, ng, s_tile0);
-    const GroupDev<R>& gd = G[f];
+    const GroupDev<float>& gd = G[f];
     const int nsys = rows.nact[f];
     if (nsys == 0) return;
     const Geom g = gd.g;
     const int vol = g.vol, vh = g.vol / 2;
     const int tile = blockIdx.x - gd.tile0;
-    const R kk = gd.kappa * gd.kappa;
-    const R chop = POUT ? -kk : R(1);
+    const float kk = gd.kappa * gd.kappa;
+    const float chop = POUT ? -kk : 1.f;
     if (threadIdx.x < TS) {
         const int h = tile * TS + threadIdx.x;
         if (h < vh) {
             const int s = eo_site(g, h, POUT);
             const Nbr nb = neighbours(g, s);
             ssite[threadIdx.x] = s;
-            snb[threadIdx.x] = nb;
+            snb[threadIdx.x] = offsets_of(nb, 1);
 #pragma unroll
             for (int mu = 0; mu < 4; mu++) sb[mu][threadIdx.x] = nb.b[mu];
             sgn[0][threadIdx.x] = nb.fwrap_t ? -chop : chop;
@@ -250,122 +236,47 @@ k_mf_eo(const GroupDev<R>* __restrict__ G, int ng, Rows rows, CgS C) {
         }
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < 72 * TS; e += blockDim.x) {
-        const int j = e % TS;
-        const int c = (e / TS) % 9;
-        const int mu = (e / (9 * TS)) % 4;
-        const int dir = e / (36 * TS);
-        cx_t<R> z = mk<R>(0, 0);
-        if (tile * TS + j < vh) {
-            z = __ldg(gd.u + (size_t)(mu * 9 + c) * vol + (dir ? sb[mu][j] : ssite[j]));
-            z = cscale(z, mu == 3 ? sgn[dir][j] : chop);
-        }
-        sl[dir][mu][c][j] = z;
-    }
+    stage_tile_links<TS>(sl, gd.u, vol, [&](int dir, int mu, int j, unsigned& site, float& scale) {
+        if (tile * TS + j >= vh) return false;
+        site = dir ? sb[mu][j] : ssite[j];
+        scale = mu == 3 ? sgn[dir][j] : chop;
+        return true;
+    });
     __syncthreads();
     const int j = threadIdx.x % TS;
-    const int qg = threadIdx.x / TS;
+    const int qg = uniform_warp(threadIdx.x / TS);
     const int hh = tile * TS + j;
     const bool live = hh < vh;
-    const Nbr& nb = snb[j];
-    auto fl = [&](int mu, int e) { return sl[0][mu][e][j]; };
-    auto bl = [&](int mu, int e) { return sl[1][mu][e][j]; };
-    const cx_t<R>* in = STAGE == 0 ? gd.p : STAGE == 2 ? gd.t : gd.e;
-    const cx_t<R>* same = STAGE == 1 ? gd.p : STAGE == 3 ? gd.t : nullptr;
-    cx_t<R>* out = (STAGE == 0 || STAGE == 2) ? gd.e : gd.t;   // STAGE 3 stores nothing
+    const unsigned off = (unsigned)hh * 16u;
+    const OffNbr& nb = snb[j];
+    auto fl = [&](int mu, int e) { return sl[(mu * 9 + e) * TS + j]; };
+    auto bl = [&](int mu, int e) { return sl[(36 + mu * 9 + e) * TS + j]; };
+    const size_t field = (size_t)gd.n * sizeof(float2), plane = (size_t)vh * 16;
+    const char* in = reinterpret_cast<const char*>(STAGE == 0 ? gd.p : STAGE == 2 ? gd.t : gd.e);
+    const char* same = reinterpret_cast<const char*>(STAGE == 1 ? gd.p : gd.t);
+    char* out = reinterpret_cast<char*>((STAGE == 0 || STAGE == 2) ? gd.e : gd.t);   // STAGE 3 stores nothing
     for (int r = qg; r < nsys; r += RPB) {
-        R dr = 0;
+        float dr = 0;
         if (live) {
-            const size_t off = (size_t)r * gd.n;
-            Spinor<R> acc;
+            const char* inr = in + r * field;
+            Spinor<float> acc;
             if (POUT) {
-                load_spinor(same + off, vh, hh, acc);
+                load_spinor_at(same + r * field, plane, off, acc);
             } else {
 #pragma unroll
-                for (int k = 0; k < 12; k++) acc.c[k / 3][k % 3] = mk<R>(0, 0);
+                for (int k = 0; k < 12; k++) acc.c[k / 3][k % 3] = make_float2(0.f, 0.f);
             }
-            eo_hops_prescaled<R, DAG>(nb, in + off, vh, fl, bl, acc);
+            auto load = [&](unsigned o, Spinor<float>& sp) { load_spinor_at(inr, plane, o, sp); };
+            wilson_hops_prescaled<DAG, float>(nb, load, fl, bl, acc);
             if (STAGE == 3) {
-                dr = r_update_site(gd.r + off, vh, hh, acc, (R)C.alpha[rows.first[f] + r]);
+                dr = r_update_site(reinterpret_cast<char*>(gd.r) + r * field, plane, off, acc,
+                                   (float)C.alpha[rows.first[f] + r]);
             } else {
                 if (STAGE == 1) dr = spinor_norm2(acc);
-                store_spinor(out + off, vh, hh, acc);
+                store_spinor_at(out + r * field, plane, off, acc);
             }
         }
         if (STAGE == 1 || STAGE == 3) put_share(STAGE == 1 ? gd.part : gd.part2, gd.ntiles, r, tile, dr);
-    }
-}
-
-// 1/3 for a batch of one full-lattice field: the same two kernels over brick
-// tiles of TB sites (TB / 32 warps per right-hand-side group, RPB groups per block).
-// The brick's links (U_mu(x) and U_mu(x - mu), scaled by -kappa and the boundary
-// sign) are staged once in shared memory and reused by every right-hand side;
-// the neighbours in x (always) and mostly in y and z are sites of the same
-// brick, so their spinor loads hit in L1.  The bricks tile the lattice, so the
-// warps of brick b are the 32-site tiles b * TB / 32 ... of the shares.
-template <typename R, int DAG, int TB, int RPB>
-__global__ void __launch_bounds__(TB * RPB, (sizeof(R) == 4 && TB * RPB <= 256) ? 3 : 1)
-k_mf_brick(const GroupDev<R>* __restrict__ G, Rows rows, CgS C) {
-    pdl_enter();
-    extern __shared__ unsigned char smem_raw[];
-    cx_t<R>* sl = reinterpret_cast<cx_t<R>*>(smem_raw);   // [2][4][9][TB]
-    Nbr* snb = reinterpret_cast<Nbr*>(sl + 72 * TB);        // [TB] neighbours of the brick's sites
-    int* ss = reinterpret_cast<int*>(snb + TB);             // [TB] site
-    R* sg = reinterpret_cast<R*>(ss + TB);                  // [2][TB]
-    const GroupDev<R>& gd = G[0];
-    const int nsys = rows.nact[0];
-    if (nsys == 0) return;
-    const Brk br = TB == 64 ? gd.b64 : gd.b128;
-    const Geom g = gd.g;
-    const int vol = g.vol;
-    const R kappa = gd.kappa;
-    int b = blockIdx.x;
-    const int iy = b % br.ny;
-    b /= br.ny;
-    const int iz = b % br.nz;
-    const int t = b / br.nz;
-    if (threadIdx.x < TB) {
-        const int j = threadIdx.x;
-        const int x = j % br.bx, dy = (j / br.bx) % br.by, dz = j / (br.bx * br.by);
-        const int s = x + g.stride[1] * (iy * br.by + dy) + g.stride[2] * (iz * br.bz + dz) + g.stride[3] * t;
-        ss[j] = s;
-        const Nbr nb = neighbours(g, s);
-        snb[j] = nb;
-        sg[j] = nb.fwrap_t ? kappa : -kappa;
-        sg[TB + j] = nb.bwrap_t ? kappa : -kappa;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < 72 * TB; e += blockDim.x) {
-        const int j = e % TB;
-        const int c = (e / TB) % 9;
-        const int mu = (e / (9 * TB)) % 4;
-        const int dir = e / (36 * TB);
-        const cx_t<R> z = __ldg(gd.u + (size_t)(mu * 9 + c) * vol + (dir ? snb[j].b[mu] : ss[j]));
-        sl[e] = cscale(z, mu == 3 ? sg[dir * TB + j] : -kappa);
-    }
-    __syncthreads();
-    const int j = threadIdx.x % TB;
-    const int q = threadIdx.x / TB;
-    const int s = ss[j];
-    const int tile32 = blockIdx.x * (TB / 32) + (j >> 5);
-    const Nbr& nb = snb[j];
-    auto fl = [&](int mu, int e) { return sl[((0 * 4 + mu) * 9 + e) * TB + j]; };
-    auto bl = [&](int mu, int e) { return sl[((1 * 4 + mu) * 9 + e) * TB + j]; };
-    const cx_t<R>* in = DAG ? gd.t : gd.p;
-    // a warp's 32 threads share one system: the loop bound is warp-uniform
-    for (int r = q; r < nsys; r += RPB) {
-        const cx_t<R>* inr = in + (size_t)r * gd.n;
-        Spinor<R> res;
-        auto load = [&](int y, Spinor<R>& sp) { load_spinor(inr, vol, y, sp); };
-        wilson_site_prescaled<DAG, R>(nb, s, load, fl, bl, res);
-        R dr;
-        if (DAG) {
-            dr = r_update_site(gd.r + (size_t)r * gd.n, vol, s, res, (R)C.alpha[rows.first[0] + r]);
-        } else {
-            dr = spinor_norm2(res);
-            store_spinor(gd.t + (size_t)r * gd.n, vol, s, res);
-        }
-        put_share(DAG ? gd.part2 : gd.part, gd.ntiles, r, tile32, dr);
     }
 }
 
@@ -684,60 +595,45 @@ k_norm_rows(const T* __restrict__ base, long n, double* partials, unsigned* coun
 // and the fastest kept; results are cached in memory per batch signature and,
 // when SEEDCG_TUNE_CACHE names a file, in that file ("key rpb" lines).
 // ---------------------------------------------------------------------------
-template <typename R>
-void launch_mf(int rpb, int dag, int tiles, cudaStream_t s, const GroupDev<R>* gdev, int ng, Rows rows,
+void launch_mf(int rpb, int dag, int tiles, cudaStream_t s, const GroupDev<float>* gdev, int ng, Rows rows,
                const CgS& C) {
 #define SEEDCG_MF(RP)                                                                          \
-    if (dag) launch_pdl(C.pdl, k_mf_dslash<R, 1, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C);               \
-    else launch_pdl(C.pdl, k_mf_dslash<R, 0, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C);
-    if (rpb == 4) { SEEDCG_MF(4) }
+    if (dag) launch_pdl(C.pdl, k_mf_dslash<1, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C);               \
+    else launch_pdl(C.pdl, k_mf_dslash<0, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C);
+    if (rpb == 3) { SEEDCG_MF(3) }
+    else if (rpb == 4) { SEEDCG_MF(4) }
+    else if (rpb == 6) { SEEDCG_MF(6) }
     else if (rpb == 12) { SEEDCG_MF(12) }
     else { SEEDCG_MF(8) }
 #undef SEEDCG_MF
     SEEDCG_CHECK_LAUNCH();
 }
 
-template <typename R>
-void launch_mf_eo(int rpb, int stage, int tiles, cudaStream_t s, const GroupDev<R>* gdev, int ng, Rows rows,
+void launch_mf_eo(int rpb, int stage, int tiles, cudaStream_t s, const GroupDev<float>* gdev, int ng, Rows rows,
                   const CgS& C) {
 #define SEEDCG_MFE(RP)                                                                          \
     switch (stage) {                                                                           \
-        case 0: launch_pdl(C.pdl, k_mf_eo<R, 0, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;         \
-        case 1: launch_pdl(C.pdl, k_mf_eo<R, 1, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;         \
-        case 2: launch_pdl(C.pdl, k_mf_eo<R, 2, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;         \
-        default: launch_pdl(C.pdl, k_mf_eo<R, 3, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;        \
+        case 0: launch_pdl(C.pdl, k_mf_eo<0, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;         \
+        case 1: launch_pdl(C.pdl, k_mf_eo<1, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;         \
+        case 2: launch_pdl(C.pdl, k_mf_eo<2, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;         \
+        default: launch_pdl(C.pdl, k_mf_eo<3, RP>, tiles, TS * RP, 0, s, gdev, ng, rows, C); break;        \
     }
-    if (rpb == 4) { SEEDCG_MFE(4) }
+    if (rpb == 3) { SEEDCG_MFE(3) }
+    else if (rpb == 4) { SEEDCG_MFE(4) }
+    else if (rpb == 6) { SEEDCG_MFE(6) }
     else if (rpb == 12) { SEEDCG_MFE(12) }
     else { SEEDCG_MFE(8) }
 #undef SEEDCG_MFE
     SEEDCG_CHECK_LAUNCH();
 }
 
-template <typename R, int DAG, int TB, int RPB>
-void brick_launch(int nb, cudaStream_t s, const GroupDev<R>* gdev, Rows rows, const CgS& C) {
-    const size_t smem = (size_t)TB * (72 * sizeof(cx_t<R>) + sizeof(Nbr) + sizeof(int) + 2 * sizeof(R));
-    static_assert(sizeof(Nbr) % 4 == 0 && (TB * (sizeof(Nbr) + sizeof(int))) % sizeof(R) == 0,
-                  "brick shared-memory layout alignment");
-    static bool attr = false;
-    if (!attr) {
-        SEEDCG_CUDA_TRY(cudaFuncSetAttribute(k_mf_brick<R, DAG, TB, RPB>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr = true;
-    }
-    launch_pdl(C.pdl, k_mf_brick<R, DAG, TB, RPB>, nb, TB * RPB, smem, s, gdev, rows, C);
-}
-
-// Launch shape of the operator, chosen by the autotuner: codes 4, 8, 12 are the
-// multi-field kernel with that many warps per tile of TS sites; code TB * 1000 +
-// RPB is the brick kernel of TB sites with RPB right-hand-side groups (one field).
-constexpr bool is_brick_code(int code) { return code >= 1000; }
+// Launch shape of the operator, chosen by the autotuner: warps per tile of TS sites (FP32), or the grid rows of
+// the fixed-point kernel (FP64).
 
 // steps 1 and 3 of an iteration for every active system: 2 launches (D, D^dag)
 // or 4 (even-odd hops); step 2 (alpha) runs between them in the iteration proper
 template <typename R>
-void launch_op(bool eo, int code, int tiles, const Brk& b64, const Brk& b128, cudaStream_t s,
-               const GroupDev<R>* gdev, int ng, Rows rows, const CgS& C, bool with_alpha) {
+void launch_op(bool eo, int code, int tiles, cudaStream_t s, const GroupDev<R>* gdev, int ng, Rows rows, const CgS& C, bool with_alpha) {
     auto alpha = [&]() {
         if (!with_alpha) return;
         launch_pdl(C.pdl, k_mf_alpha<R>, C.rows_cap, 256, 0, s, gdev, rows, C);
@@ -756,53 +652,20 @@ void launch_op(bool eo, int code, int tiles, const Brk& b64, const Brk& b128, cu
             mf_fix<0, 3>(tiles, code, s, gdev, ng, rows, C);
         }
     } else if (eo) {
-        for (int stage = 0; stage < 2; stage++) launch_mf_eo<R>(code, stage, tiles, s, gdev, ng, rows, C);
+        for (int stage = 0; stage < 2; stage++) launch_mf_eo(code, stage, tiles, s, gdev, ng, rows, C);
         alpha();
-        for (int stage = 2; stage < 4; stage++) launch_mf_eo<R>(code, stage, tiles, s, gdev, ng, rows, C);
-    } else if (is_brick_code(code)) {
-#define SEEDCG_BRICK(TB, RP, BR)                                                               \
-    brick_launch<R, 0, TB, RP>(BR.n, s, gdev, rows, C);                                        \
-    alpha();                                                                                   \
-    brick_launch<R, 1, TB, RP>(BR.n, s, gdev, rows, C);
-        switch (code) {
-            case 64004: SEEDCG_BRICK(64, 4, b64) break;
-            case 64008: SEEDCG_BRICK(64, 8, b64) break;
-            case 128002: SEEDCG_BRICK(128, 2, b128) break;
-            default: SEEDCG_BRICK(128, 4, b128) break;
-        }
-#undef SEEDCG_BRICK
+        for (int stage = 2; stage < 4; stage++) launch_mf_eo(code, stage, tiles, s, gdev, ng, rows, C);
     } else {
-        launch_mf<R>(code, 0, tiles, s, gdev, ng, rows, C);
+        launch_mf(code, 0, tiles, s, gdev, ng, rows, C);
         alpha();
-        launch_mf<R>(code, 1, tiles, s, gdev, ng, rows, C);
+        launch_mf(code, 1, tiles, s, gdev, ng, rows, C);
     }
-}
-
-int largest_divisor_le(int L, int cap) {
-    int best = 1;
-    for (int d = 1; d <= L && d <= cap; d++)
-        if (L % d == 0) best = d;
-    return best;
-}
-
-// the brick of about `cap` sites for g: Lx x by x bz, by preferring a share of
-// the y extent before z (n = 0 when it does not come to exactly TB sites)
-Brk brick_for(const Geom& g, int tb) {
-    Brk b{};
-    b.bx = g.L[0];
-    if (b.bx > 64 || b.bx > tb) return b;
-    b.by = largest_divisor_le(g.L[1], (tb / 2 > b.bx ? tb / 2 : tb) / b.bx);
-    b.bz = largest_divisor_le(g.L[2], tb / (b.bx * b.by));
-    if (b.bx * b.by * b.bz != tb) return Brk{};
-    b.ny = g.L[1] / b.by;
-    b.nz = g.L[2] / b.bz;
-    b.n = b.ny * b.nz * g.L[3];
-    return b;
 }
 
 std::string tune_key(const std::vector<CgGroup>& groups, bool fp64) {
     std::string k = fp64 ? "mf_dslash f64" : "mf_dslash f32";
     if (!groups.empty() && groups[0].h->eo_active) k += " eo";
+    k += " t32";   // the launch shapes: entries of caches written for other shapes are not read
     for (auto& g : groups) {
         char b[96];
         snprintf(b, sizeof(b), " %dx%dx%dx%d:%d", g.h->g.L[0], g.h->g.L[1], g.h->g.L[2], g.h->g.L[3], g.nsys);
@@ -817,7 +680,7 @@ std::string tune_key(const std::vector<CgGroup>& groups, bool fp64) {
 }
 
 // the process-wide table of tuned warps per tile (guarded by tune_mutex); the
-// optional SEEDCG_TUNE_CACHE file is shared with the brick-dslash tuner, so only
+// optional SEEDCG_TUNE_CACHE file is shared with the operator's tuner, so only
 // its "mf_dslash..." lines are read here
 std::mutex& tune_mutex() {
     static std::mutex m;
@@ -846,8 +709,7 @@ std::vector<std::pair<std::string, int>>& tune_table() {
 }
 
 template <typename R>
-int autotune_rpb(const std::vector<CgGroup>& groups, int tiles, const Brk& b64, const Brk& b128,
-                 const GroupDev<R>* gdev, int ng, Rows rows, const CgS& C, cudaStream_t st) {
+int autotune_rpb(const std::vector<CgGroup>& groups, int tiles, const GroupDev<R>* gdev, int ng, Rows rows, const CgS& C, cudaStream_t st) {
     const std::string key = tune_key(groups, sizeof(R) == 8);
     {
         std::lock_guard<std::mutex> lk(tune_mutex());
@@ -855,11 +717,7 @@ int autotune_rpb(const std::vector<CgGroup>& groups, int tiles, const Brk& b64, 
             if (e.first == key) return e.second;
     }
     const bool eo = groups[0].h->eo_active;
-    std::vector<int> cands{4, 8, 12};
-    if (!eo && ng == 1) {
-        if (b64.n) cands.insert(cands.end(), {64004, 64008});
-        if (b128.n) cands.insert(cands.end(), {128002, 128004});
-    }
+    const std::vector<int> cands{3, 4, 6, 8, 12};
     cudaEvent_t a, b;
     SEEDCG_CUDA_TRY(cudaEventCreate(&a));
     SEEDCG_CUDA_TRY(cudaEventCreate(&b));
@@ -869,9 +727,9 @@ int autotune_rpb(const std::vector<CgGroup>& groups, int tiles, const Brk& b64, 
     for (int c : cands) {
         // alpha is zero here: the D^dag kernel rewrites r unchanged, as it would for a
         // stopped system, so the candidates are timed on the whole of steps 1 and 3
-        launch_op<R>(eo, c, tiles, b64, b128, st, gdev, ng, rows, C, false);  // warm-up
+        launch_op<R>(eo, c, tiles, st, gdev, ng, rows, C, false);  // warm-up
         SEEDCG_CUDA_TRY(cudaEventRecord(a, st));
-        for (int r = 0; r < 3; r++) launch_op<R>(eo, c, tiles, b64, b128, st, gdev, ng, rows, C, false);
+        for (int r = 0; r < 3; r++) launch_op<R>(eo, c, tiles, st, gdev, ng, rows, C, false);
         SEEDCG_CUDA_TRY(cudaEventRecord(b, st));
         SEEDCG_CUDA_TRY(cudaEventSynchronize(b));
         float ms = 0.f;
@@ -974,13 +832,6 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
         MX[f] = cv.take<double2>((size_t)ns * n);
         T64[f] = cv.take<double2>((size_t)std::max(ns, 2) * n);
         gd[f].ntiles = (nsites(groups[f]) + TS - 1) / TS;
-        gd[f].b64 = (ng == 1 && !eo) ? brick_for(h->g, 64) : Brk{};
-        gd[f].b128 = (ng == 1 && !eo) ? brick_for(h->g, 128) : Brk{};
-        // the brick kernels write one share per warp of 32 sites: the bricks must tile
-        // the lattice exactly, so that their warps are the ntiles site tiles
-        if ((gd[f].b64.n && gd[f].b64.n * 2 != gd[f].ntiles) ||
-            (gd[f].b128.n && gd[f].b128.n * 4 != gd[f].ntiles))
-            throw Error{SEEDCG_ERR_ARG, "internal: bricks do not tile the lattice"};
         gd[f].part = cv.take<double>((size_t)ns * gd[f].ntiles);
         gd[f].part2 = cv.take<double>((size_t)ns * gd[f].ntiles);
         gd[f].tile0 = tile0;
@@ -1180,15 +1031,14 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
 
     // ---- the iteration chunk (graph-captured) ----
     const int gx = rblocks;
-    const Brk b64 = gd[0].b64, b128 = gd[0].b128;
     // FP64: one kernel, its grid rows by a rule; FP32: the autotuner's choice
     int rpb = 8;
     if constexpr (sizeof(R) == 8) rpb = fix_grid_y(tiles, nsys_max);
-    else if (nrows > 0) rpb = autotune_rpb<R>(groups, tiles, b64, b128, gdev, ng, rows, C, st);
+    else if (nrows > 0) rpb = autotune_rpb<R>(groups, tiles, gdev, ng, rows, C, st);
     out.rpb = rpb;
     auto chunk = [&](cudaStream_t s) {
         for (int it = 0; it < poll; it++) {
-            launch_op<R>(eo, rpb, tiles, b64, b128, s, gdev, ng, rows, C, true);   // steps 1-3
+            launch_op<R>(eo, rpb, tiles, s, gdev, ng, rows, C, true);   // steps 1-3
             launch_pdl(C.pdl, k_mf_beta<R>, rows_cap, 256, 0, s, gdev, rows, C);
             launch_pdl(C.pdl, k_mf_xp<R>, dim3(gx, rows_cap), kRedThreads, 0, s, gdev, rows, C);
         }

@@ -23,8 +23,8 @@ struct CgResult {
     std::vector<std::vector<double>> true_resid;
     int reliable_updates = 0;
     int graph_chunks = 0;
-    int rpb = 0;          // the operator's launch shape chosen by the autotuner (warps per
-                          // 32-site tile, or TB * 1000 + groups for the brick kernel)
+    int rpb = 0;          // the operator's launch shape: warps per 32-site tile chosen by the autotuner
+                          // (FP32), grid rows of the fixed-point kernel (FP64)
 };
 
 // Run CG on every system of every group until ||b - M x|| <= tol ||b|| in FP64.

@@ -108,6 +108,30 @@ __device__ __forceinline__ void store_spinor(float2* __restrict__ p, int vol, in
         q[(size_t)c * vol] = make_float4(a.x, a.y, b.x, b.y);
     }
 }
+// The warp's index within its block, computed so that the compiler knows it is the same for all lanes: what
+// depends on it (the right-hand side, its field's plane addresses) then lives in uniform registers, and a gather is
+// one load at [uniform plane base + 32-bit lane offset] without 64-bit address arithmetic per plane.
+__device__ __forceinline__ int uniform_warp(int w) { return __shfl_sync(0xffffffffu, w, 0); }
+// neighbour of a site in each direction, as byte offsets (16 * site) of the gathers
+struct OffNbr {
+    unsigned f[4], b[4];
+};
+// spinor at byte offset `off` (16 * site) of an FP32 field whose planes are `plane` bytes apart
+__device__ __forceinline__ void load_spinor_at(const char* field, size_t plane, unsigned off, Spinor<float>& out) {
+#pragma unroll
+    for (int c = 0; c < 6; c++) {
+        const float4 z = __ldg(reinterpret_cast<const float4*>(field + c * plane + off));
+        out.c[(2 * c) / 3][(2 * c) % 3] = make_float2(z.x, z.y);
+        out.c[(2 * c + 1) / 3][(2 * c + 1) % 3] = make_float2(z.z, z.w);
+    }
+}
+__device__ __forceinline__ void store_spinor_at(char* field, size_t plane, unsigned off, const Spinor<float>& v) {
+#pragma unroll
+    for (int c = 0; c < 6; c++) {
+        const float2 a = v.c[(2 * c) / 3][(2 * c) % 3], b = v.c[(2 * c + 1) / 3][(2 * c + 1) % 3];
+        *reinterpret_cast<float4*>(field + c * plane + off) = make_float4(a.x, a.y, b.x, b.y);
+    }
+}
 // coherent loads, for a field that the same kernel writes back at the same site
 __device__ __forceinline__ void load_spinor_rw(const float2* p, int vol, int s, Spinor<float>& out) {
     const float4* q = reinterpret_cast<const float4*>(p) + s;
@@ -176,6 +200,38 @@ __device__ __forceinline__ Nbr neighbours(const Geom& g, int s) {
     return n;
 }
 
+__device__ __forceinline__ OffNbr offsets_of(const Nbr& nb, int shift) {
+    OffNbr o;
+#pragma unroll
+    for (int mu = 0; mu < 4; mu++) {
+        o.f[mu] = (unsigned)(nb.f[mu] >> shift) * 16u;
+        o.b[mu] = (unsigned)(nb.b[mu] >> shift) * 16u;
+    }
+    return o;
+}
+
+// Staging of a tile's links [fwd/bwd][mu][3a+b][NS sites] in shared memory: a warp takes whole rows (direction, mu, entry), a
+// lane a site.  src(dir, mu, j, site, scale) gives the link's site and factor, false for sites past the end.
+template <int NS, typename Src>
+__device__ __forceinline__ void stage_tile_links(float2* sl, const float2* __restrict__ u, int vol, Src src) {
+    static_assert(NS == 32, "a lane per site");
+    const int nw = blockDim.x >> 5, j = threadIdx.x & 31;
+    for (int row = uniform_warp(threadIdx.x >> 5); row < 72; row += nw) {
+        const int dir = row / 36, mu = (row / 9) % 4, c = row % 9;
+        float2 z = make_float2(0.f, 0.f);
+        unsigned site;
+        float scale;
+        if (src(dir, mu, j, site, scale)) z = cscale(__ldg(u + (size_t)(mu * 9 + c) * vol + site), scale);
+        sl[row * NS + j] = z;
+    }
+}
+
+// Blocks per SM of the tile kernels with `rpb` warps: between 24 and 32 warps at 64 to 80 registers.  D + D^dag
+// on 12 fields of 16^3 x 32 in ms: 3 warps x 9 blocks 0.260, 4 x 7 0.262 (x 6 0.278, x 8 0.264, x 9 0.369: spills), 6 x 5
+// 0.264, 8 x 4 0.273, 12 x 2 0.289; three uneven fields 0.279, 0.284, 0.269, 0.284, 0.355; five systems of 10x6x14x12
+// 0.036, 0.032, 0.025, 0.023, 0.029.  The autotuner chooses among them.
+constexpr int tile_blocks(int rpb) { return rpb <= 3 ? 9 : rpb <= 4 ? 7 : rpb <= 6 ? 5 : rpb <= 8 ? 4 : 2; }
+
 // ---------------------------------------------------------------------------
 // one hop: acc += coef * P U psi_nbr  (forward: U = U_mu(x); backward: U = U_mu(x-mu)^dag)
 // LinkAt(a, b) returns U[a][b] for the link in use.
@@ -227,23 +283,24 @@ __device__ __forceinline__ void wilson_site(const Nbr& n, int s, LoadNbr load, F
     load(n.b[3], nb); hop<3, SB, true>(out, nb, [&](int a, int b) { return bl(3, 3 * a + b); }, n.bwrap_t ? kappa : mk_);
 }
 
-// Same, with links that already carry -kappa and the boundary sign (staged
-// that way by the multi-RHS kernel): out = psi(x) + sum of hops, no scaling.
-template <int DAG, typename R, typename LoadNbr, typename Fwd, typename Bwd>
-__device__ __forceinline__ void wilson_site_prescaled(const Nbr& n, int s, LoadNbr load, Fwd fl,
-                                                      Bwd bl, Spinor<R>& out) {
+// Same, with links that already carry the coefficient and the boundary sign (staged that way by the
+// tile kernels): out += sum of hops, no scaling.  n.f / n.b are what `load` takes (sites or offsets).
+// One neighbour is always in flight while another is multiplied: the gathers' latency bounds these kernels, and
+// with the fields' plane addresses in uniform registers the second spinor still leaves 28 warps per SM.
+template <int DAG, typename R, typename N, typename LoadNbr, typename Fwd, typename Bwd>
+__device__ __forceinline__ void wilson_hops_prescaled(const N& n, LoadNbr load, Fwd fl, Bwd bl, Spinor<R>& out) {
     constexpr int SF = DAG ? 1 : -1;
     constexpr int SB = -SF;
-    load(s, out);
-    Spinor<R> nb;
+    Spinor<R> pa, pb;
+    load(n.f[0], pa);
 #define SEEDCG_HOP(MU)                                                                          \
     {                                                                                           \
         auto lf = [&](int a, int b) { return fl(MU, 3 * a + b); };                              \
         auto lb = [&](int a, int b) { return bl(MU, 3 * a + b); };                              \
-        load(n.f[MU], nb);                                                                      \
-        hop<MU, SF, false, R, decltype(lf), false>(out, nb, lf, R(1));                          \
-        load(n.b[MU], nb);                                                                      \
-        hop<MU, SB, true, R, decltype(lb), false>(out, nb, lb, R(1));                           \
+        load(n.b[MU], pb);                                                                      \
+        hop<MU, SF, false, R, decltype(lf), false>(out, pa, lf, R(1));                          \
+        if (MU < 3) load(n.f[(MU + 1) & 3], pa);                                                \
+        hop<MU, SB, true, R, decltype(lb), false>(out, pb, lb, R(1));                           \
     }
     SEEDCG_HOP(0)
     SEEDCG_HOP(1)
@@ -251,36 +308,11 @@ __device__ __forceinline__ void wilson_site_prescaled(const Nbr& n, int s, LoadN
     SEEDCG_HOP(3)
 #undef SEEDCG_HOP
 }
-
-// Same result as wilson_site_prescaled, written for a looser register budget:
-// the forward and backward neighbours of each direction are loaded together and
-// the next direction's pair is requested before the current one is consumed,
-// so two to four spinors are in flight per thread instead of one.
-template <int DAG, typename R, typename LoadNbr, typename Fwd, typename Bwd>
-__device__ __forceinline__ void wilson_site_prescaled_pipe(const Nbr& n, int s, LoadNbr load, Fwd fl,
-                                                           Bwd bl, Spinor<R>& out) {
-    constexpr int SF = DAG ? 1 : -1;
-    constexpr int SB = -SF;
-    Spinor<R> pf, pb, qf, qb;
-    load(n.f[0], pf);
-    load(n.b[0], pb);
+// out = psi(s) + sum of hops
+template <int DAG, typename R, typename N, typename S, typename LoadNbr, typename Fwd, typename Bwd>
+__device__ __forceinline__ void wilson_site_prescaled(const N& n, S s, LoadNbr load, Fwd fl, Bwd bl, Spinor<R>& out) {
     load(s, out);
-#define SEEDCG_HOP2(MU, CF, CB, NF, NB, NEXT)                                                   \
-    {                                                                                           \
-        auto lf = [&](int a, int b) { return fl(MU, 3 * a + b); };                              \
-        auto lb = [&](int a, int b) { return bl(MU, 3 * a + b); };                              \
-        if (NEXT) {                                                                             \
-            load(n.f[(MU + 1) & 3], NF);                                                        \
-            load(n.b[(MU + 1) & 3], NB);                                                        \
-        }                                                                                       \
-        hop<MU, SF, false, R, decltype(lf), false>(out, CF, lf, R(1));                          \
-        hop<MU, SB, true, R, decltype(lb), false>(out, CB, lb, R(1));                           \
-    }
-    SEEDCG_HOP2(0, pf, pb, qf, qb, true)
-    SEEDCG_HOP2(1, qf, qb, pf, pb, true)
-    SEEDCG_HOP2(2, pf, pb, qf, qb, true)
-    SEEDCG_HOP2(3, qf, qb, pf, pb, false)
-#undef SEEDCG_HOP2
+    wilson_hops_prescaled<DAG, R>(n, load, fl, bl, out);
 }
 
 }  // namespace seedcg
