@@ -106,7 +106,7 @@ k_dslash(Geom g, const float2* __restrict__ u, float kappa, const float2* __rest
     } else {
         auto fl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + s); };
         auto bl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + n.b[mu]); };
-        wilson_site<DAG, float>(n, s, load, fl, bl, kappa, res);
+        wilson_site_ahead<DAG, 2>(n, s, load, fl, bl, kappa, res);
     }
     put_site(out, blockIdx.y, vol, s, res);
 }

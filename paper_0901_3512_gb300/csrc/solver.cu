@@ -51,6 +51,16 @@ inline int site_blocks(int vol) { return (vol + kRedThreads - 1) / kRedThreads; 
 // waves (16.4 -> 14.6 us for D with the L2 warm)
 constexpr int kSiteThreads = 128;
 inline int site_blocks_lz(int vol) { return (vol + kSiteThreads - 1) / kSiteThreads; }
+// Blocks per SM of the operator kernels, by which the registers and the neighbours in flight go. A lattice that has at
+// most two or three blocks of 128 per SM is bound by the chain of a thread's eight gathers, one L2 latency after the
+// other: four in flight, at up to 255 or 168 registers, make it two long. D + D^dag + update in us, one gather at 72
+// registers -> now: 10 x 6 x 14 x 12 (79 blocks) 26.9 -> 21.5, 8^3 x 16 (64) 23.9 -> 20.7, 12^3 x 24 (324) 34.7 ->
+// 33.5. Larger ones have the warps to cover the latency and keep seven blocks, one wave of 16^3 x 32, with a second
+// gather in flight: 71.1 -> 67.4 with V in BF16, 74.4 -> 66.8 with V in FP32 (v_i is stored once there).
+inline int lz_blocks_per_sm(int sites) {
+    const int blocks = (sites + kSiteThreads - 1) / kSiteThreads;
+    return blocks <= 2 * 152 ? 2 : blocks <= 3 * 152 ? 3 : 7;
+}
 
 // blocks for a streaming pass that ends in one grid reduction: two per SM.  Every
 // block takes the reduction's atomic ticket, and thousands of tickets on one
@@ -122,20 +132,28 @@ __device__ __forceinline__ R lz_inv(const LzDev& L, int i) {
     return R(1) / (R)(i == 1 ? L.ctl->beta0 : L.beta[i - 2]);
 }
 
+// A row of V that holds v_i in the vector's own type is v_i: the vector apart from it exists only in the iterations
+// that re-orthogonalise, whose products want v_i and f side by side
+template <typename C, typename VT>
+__device__ __forceinline__ bool lz_own_v(const C* v, const VT* Vrow) {
+    if constexpr (sizeof(C) != sizeof(VT)) return true;
+    else return (const void*)v != (const void*)Vrow;
+}
+
 // v_i and its row of V at one site
 template <typename R, typename VT>
 __device__ __forceinline__ void lz_put_v(const Spinor<R>& w, R inv, cx_t<R>* v, VT* Vrow, int vol, int s) {
     Spinor<R> sc;
 #pragma unroll
     for (int k = 0; k < 12; k++) sc.c[k / 3][k % 3] = cscale(w.c[k / 3][k % 3], inv);
-    store_spinor(v, vol, s, sc);
+    if (lz_own_v(v, Vrow)) store_spinor(v, vol, s, sc);
 #pragma unroll
     for (int k = 0; k < 12; k++) st_cx(Vrow, sidx(k, s, vol), sc.c[k / 3][k % 3]);
 }
 
 // v_i = w / ||w||, t = D v_i
-template <typename R, typename VT>
-__global__ void __launch_bounds__(kSiteThreads, 7)
+template <typename R, typename VT, int BPS>
+__global__ void __launch_bounds__(kSiteThreads, BPS)
 k_lz_D(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict__ w, cx_t<R>* __restrict__ v,
        VT* __restrict__ Vrow, cx_t<R>* __restrict__ t, int i, LzDev L) {
     pdl_enter();
@@ -151,7 +169,7 @@ k_lz_D(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict
     auto load = [&](int y, Spinor<R>& p) { load_spinor(w, vol, y, p); };
     auto fl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + s); };
     auto bl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + n.b[mu]); };
-    wilson_site<0, R>(n, s, load, fl, bl, kappa, res);
+    wilson_site_ahead<0, (BPS < 4 ? 4 : 2)>(n, s, load, fl, bl, kappa, res);
 #pragma unroll
     for (int k = 0; k < 12; k++) res.c[k / 3][k % 3] = cscale(res.c[k / 3][k % 3], inv);
     store_spinor(t, vol, s, res);
@@ -159,8 +177,8 @@ k_lz_D(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict
 
 // Step 5 (and 2): f = D^dag t - beta_{i-1} v_{i-1}; alpha_i = Re v_i^dag f.
 // Step 6 scalars (and 3): gamma_{i-1}, delta_i, zeta_i.
-template <typename R>
-__global__ void __launch_bounds__(kSiteThreads, 7)
+template <typename R, int BPS>
+__global__ void __launch_bounds__(kSiteThreads, BPS)
 k_lz_Ddag(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict__ t,
           const cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ vprev,
           cx_t<R>* __restrict__ f, int i, LzDev L) {
@@ -176,7 +194,7 @@ k_lz_Ddag(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restr
         auto load = [&](int y, Spinor<R>& p) { load_spinor(t, vol, y, p); };
         auto fl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + s); };
         auto bl = [&](int mu, int e) { return __ldg(u + (size_t)(mu * 9 + e) * vol + n.b[mu]); };
-        wilson_site<1, R>(n, s, load, fl, bl, kappa, res);
+        wilson_site_ahead<1, (BPS < 4 ? 4 : 2)>(n, s, load, fl, bl, kappa, res);
         R part = 0;
 #pragma unroll
         for (int k = 0; k < 12; k++) {
@@ -283,8 +301,10 @@ struct LzFixEpi {
             if (KIND == LZ_PUT) {
                 const double2 wa = w[ix], wb = w[ix + 1];
                 const double2 sa = cscale(wa, inv), sb = cscale(wb, inv);
-                vout[ix] = sa;
-                vout[ix + 1] = sb;
+                if (lz_own_v(vout, Vrow)) {
+                    vout[ix] = sa;
+                    vout[ix + 1] = sb;
+                }
                 Vrow[ix] = sa;
                 Vrow[ix + 1] = sb;
                 a = cscale(a, inv);
@@ -1171,13 +1191,18 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> po_ev;
     int m = 0, m_conv = 0, po_count = 0, lz_status = SEEDCG_OK, breakdown = 0;
     if (beta0 > 0.0) {
-        cx_t<R>* v = vA;
-        cx_t<R>* vprev = vB;
+        cx_t<R>* vprev = nullptr;
         int i = 1;
         const int sbh = site_blocks(vol / 2);
+        const int bps = lz_blocks_per_sm(vol);
+        cx_t<R>* slot = vA;
         const R kk = (R)(h->kappa * h->kappa);
         for (; i <= m_max; i++) {
             VT* Vrow = Vb + (size_t)(i - 1) * n;
+            const bool po_now = k_po > 0 && i >= 2 && (i % k_po) == 0;
+            cx_t<R>* v = slot;
+            if (sizeof(VT) == sizeof(cx_t<R>) && !po_now) v = reinterpret_cast<cx_t<R>*>(Vrow);   // lz_own_v
+            else slot = slot == vA ? vB : vA;
             const cx_t<R>* w = i == 1 ? R0 : fv;   // v_i = w / ||w||
             if constexpr (sizeof(R) == 8) {
                 lz_apply_f64(fix_of(h), eo, w, v, vprev, Vrow, runE, tv, ev, fv, i, L, st);
@@ -1189,8 +1214,14 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                 launch_pdl(pdl, k_lz_eo<R, VT, 2>, sbh, kRedThreads, 0, st, h->g, U, kk, tv, none, ev, v, none, Vrow, i, L);
                 launch_pdl(pdl, k_lz_eo<R, VT, 3>, sbh, kRedThreads, 0, st, h->g, U, kk, ev, tv, fv, v, vprev, Vrow, i, L);
             } else {
-                launch_pdl(pdl, k_lz_D<R, VT>, site_blocks_lz(vol), kSiteThreads, 0, st, h->g, U, kap, w, v, Vrow, tv, i, L);
-                launch_pdl(pdl, k_lz_Ddag<R>, site_blocks_lz(vol), kSiteThreads, 0, st, h->g, U, kap, tv, v, vprev, fv, i, L);
+                const int sbl = site_blocks_lz(vol);
+#define SEEDCG_LZ(BPS)                                                                                                \
+    launch_pdl(pdl, k_lz_D<R, VT, BPS>, sbl, kSiteThreads, 0, st, h->g, U, kap, w, v, Vrow, tv, i, L);                \
+    launch_pdl(pdl, k_lz_Ddag<R, BPS>, sbl, kSiteThreads, 0, st, h->g, U, kap, tv, v, vprev, fv, i, L);
+                if (bps == 2) { SEEDCG_LZ(2) }
+                else if (bps == 3) { SEEDCG_LZ(3) }
+                else { SEEDCG_LZ(7) }
+#undef SEEDCG_LZ
             }
             if (literal) {
                 for (int j0 = 2; j0 <= nrhs; j0 += 8) {
@@ -1199,7 +1230,6 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                                                                  L.counters + CTR_ETA0 + j0);
                 }
             }
-            const bool po_now = k_po > 0 && i >= 2 && (i % k_po) == 0;
             if (literal)
                 launch_pdl(pdl, k_lz_update<R, true>, rb, kRedThreads, 0, st, 
                     v, fv, wv, reinterpret_cast<cx_t<R>*>(X64), nrhs, n, i, po_now ? 0 : 1, L);
@@ -1223,7 +1253,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                 cudaEventRecord(e1, st);
                 po_ev.push_back({e0, e1});
             }
-            std::swap(v, vprev);
+            vprev = v;
             if (i % poll == 0 || i == m_max) {
                 SEEDCG_CUDA_TRY(cudaMemcpyAsync(pin, L.ctl, sizeof(int) * 8, cudaMemcpyDeviceToHost, st));
                 SEEDCG_CUDA_TRY(cudaStreamSynchronize(st));

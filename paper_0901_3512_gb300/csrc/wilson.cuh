@@ -17,6 +17,8 @@
 //   mu=t: h0 = p0 + S   p2, h1 = p1 + S   p3;  full = (r0, r1,  S   r0,  S   r1)
 #pragma once
 
+#include <type_traits>
+
 #include "internal.cuh"
 
 namespace seedcg {
@@ -283,6 +285,50 @@ __device__ __forceinline__ void wilson_site(const Nbr& n, int s, LoadNbr load, F
     load(n.b[3], nb); hop<3, SB, true>(out, nb, [&](int a, int b) { return bl(3, 3 * a + b); }, n.bwrap_t ? kappa : mk_);
 }
 
+// The eight hops in their order (forward, backward of x, y, z, t) with DEPTH neighbours in flight: step(k, spinor) is
+// called for k = 0 .. 7 with the neighbour that load(index) fetched for index(k).
+template <int DEPTH, typename R, typename Index, typename LoadNbr, typename Step>
+__device__ __forceinline__ void hops_in_flight(Index index, LoadNbr load, Step step) {
+    Spinor<R> p[DEPTH];
+#pragma unroll
+    for (int k = 0; k < DEPTH; k++) load(index(k), p[k]);
+#define SEEDCG_STEP(K)                                                                          \
+    step(std::integral_constant<int, K>{}, p[K % DEPTH]);                                       \
+    if constexpr (K + DEPTH < 8) load(index(K + DEPTH), p[K % DEPTH]);
+    SEEDCG_STEP(0)
+    SEEDCG_STEP(1)
+    SEEDCG_STEP(2)
+    SEEDCG_STEP(3)
+    SEEDCG_STEP(4)
+    SEEDCG_STEP(5)
+    SEEDCG_STEP(6)
+    SEEDCG_STEP(7)
+#undef SEEDCG_STEP
+}
+template <typename N> __device__ __forceinline__ auto hop_index(const N& n, int k) {
+    return (k & 1) ? n.b[k >> 1] : n.f[k >> 1];
+}
+
+// wilson_site with DEPTH neighbours in flight, for the FP32 kernels with one thread per site: two where the lattice
+// fills the chip (the Lanczos D at 16^3 x 32: 19.3 -> 16.4 us; in FP64 the second spinor's registers cost more than
+// they give), four on small lattices, where a thread may have the registers.
+template <int DAG, int DEPTH, typename LoadNbr, typename Fwd, typename Bwd>
+__device__ __forceinline__ void wilson_site_ahead(const Nbr& n, int s, LoadNbr load, Fwd fl, Bwd bl, float kappa,
+                                                  Spinor<float>& out) {
+    constexpr int SF = DAG ? 1 : -1;
+    load(s, out);
+    hops_in_flight<DEPTH, float>(
+        [&](int k) { return hop_index(n, k); }, load, [&](auto kk, const Spinor<float>& nb) {
+            constexpr int K = decltype(kk)::value, MU = K >> 1, BACK = K & 1;
+            if constexpr (BACK)
+                hop<MU, -SF, true>(out, nb, [&](int a, int b) { return bl(MU, 3 * a + b); },
+                                   MU == 3 && n.bwrap_t ? kappa : -kappa);
+            else
+                hop<MU, SF, false>(out, nb, [&](int a, int b) { return fl(MU, 3 * a + b); },
+                                   MU == 3 && n.fwrap_t ? kappa : -kappa);
+        });
+}
+
 // Same, with links that already carry the coefficient and the boundary sign (staged that way by the
 // tile kernels): out += sum of hops, no scaling.  n.f / n.b are what `load` takes (sites or offsets).
 // One neighbour is always in flight while another is multiplied: the gathers' latency bounds these kernels, and
@@ -290,23 +336,11 @@ __device__ __forceinline__ void wilson_site(const Nbr& n, int s, LoadNbr load, F
 template <int DAG, typename R, typename N, typename LoadNbr, typename Fwd, typename Bwd>
 __device__ __forceinline__ void wilson_hops_prescaled(const N& n, LoadNbr load, Fwd fl, Bwd bl, Spinor<R>& out) {
     constexpr int SF = DAG ? 1 : -1;
-    constexpr int SB = -SF;
-    Spinor<R> pa, pb;
-    load(n.f[0], pa);
-#define SEEDCG_HOP(MU)                                                                          \
-    {                                                                                           \
-        auto lf = [&](int a, int b) { return fl(MU, 3 * a + b); };                              \
-        auto lb = [&](int a, int b) { return bl(MU, 3 * a + b); };                              \
-        load(n.b[MU], pb);                                                                      \
-        hop<MU, SF, false, R, decltype(lf), false>(out, pa, lf, R(1));                          \
-        if (MU < 3) load(n.f[(MU + 1) & 3], pa);                                                \
-        hop<MU, SB, true, R, decltype(lb), false>(out, pb, lb, R(1));                           \
-    }
-    SEEDCG_HOP(0)
-    SEEDCG_HOP(1)
-    SEEDCG_HOP(2)
-    SEEDCG_HOP(3)
-#undef SEEDCG_HOP
+    hops_in_flight<2, R>([&](int k) { return hop_index(n, k); }, load, [&](auto kk, const Spinor<R>& nb) {
+        constexpr int K = decltype(kk)::value, MU = K >> 1, BACK = K & 1;
+        auto l = [&](int a, int b) { return BACK ? bl(MU, 3 * a + b) : fl(MU, 3 * a + b); };
+        hop<MU, BACK ? -SF : SF, BACK != 0, R, decltype(l), false>(out, nb, l, R(1));
+    });
 }
 // out = psi(s) + sum of hops
 template <int DAG, typename R, typename N, typename S, typename LoadNbr, typename Fwd, typename Bwd>
