@@ -76,7 +76,7 @@ k_gemm_t(const AT* __restrict__ A, long lda, int na, const cx_t<R>* __restrict__
             v[2 * (t * NB + c)] = acc[t][c].x;
             v[2 * (t * NB + c) + 1] = acc[t][c].y;
         }
-    block_sum<2 * TA * NB>(v);
+    block_sum_all<2 * TA * NB>(v);
     // part layout [slice][a][b] with b over the full nb
     for (int k = threadIdx.x; k < TA * NB; k += blockDim.x) {
         int t = k / NB, c = k % NB;

@@ -82,6 +82,7 @@ struct CgS {
     double tol, delta2;
     int maxiter;
     int rows_cap;   // rows of every per-row array (grid of the per-row kernels)
+    int share_t;    // threads that add a row's shares (share_threads of the longest row)
     bool pdl;       // programmatic dependent launch of the iteration's kernels
 };
 
@@ -350,66 +351,81 @@ void mf_fix(int tiles, int gy, cudaStream_t s, const GroupDev<double>* gdev, int
     launch_pdl(C.pdl, k_mf_fix<EO, STAGE>, dim3(tiles, gy), kFixThreads, kFixSmem, s, gdev, ng, rows, C);
 }
 
-// a row's shares, summed in a fixed order (one block per row); four independent
-// partial sums per thread keep four loads in flight
+// A row's shares, summed in a fixed order by one block; every thread has the result. The row's one SM adds them,
+// so its FP64 pipe and the chain of loads bound it: long rows go over 1024 threads with four loads in flight
+// each, and the warps' sums are taken on the integer pipe (warp_sum).
+constexpr int kShareThreads = 256, kShareThreadsLong = 1024;
+inline int share_threads(int ntiles) { return ntiles > 4 * kShareThreads ? kShareThreadsLong : kShareThreads; }
 __device__ __forceinline__ double row_shares(const double* __restrict__ sh, int ntiles) {
+    __shared__ double s_w[kShareThreadsLong / 32];
     const int bd = blockDim.x;
-    double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0;
-    int b = threadIdx.x;
-    for (; b + 3 * bd < ntiles; b += 4 * bd) {
-        v0 += sh[b];
-        v1 += sh[b + bd];
-        v2 += sh[b + 2 * bd];
-        v3 += sh[b + 3 * bd];
+    double v = 0.0;
+    for (int b0 = 0; b0 < ntiles; b0 += 4 * bd) {
+        double p[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int b = b0 + u * bd + threadIdx.x;
+            p[u] = b < ntiles ? sh[b] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (b0 + u * bd < ntiles) v += p[u];
     }
-    for (; b < ntiles; b += bd) v0 += sh[b];
-    double v[1] = {(v0 + v1) + (v2 + v3)};
-    block_sum<1>(v);
-    return v[0];
+    const double t = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = t;
+    __syncthreads();
+    return warp_sum((int)(threadIdx.x & 31) < bd / 32 ? s_w[threadIdx.x & 31] : 0.0);
 }
 
-// 2: alpha = ||r||^2 / ||D p||^2 (one block per row)
+// 2: alpha = ||r||^2 / ||D p||^2 (one block per row). The per-row scalars are read before the sum, which waits for
+// the shares anyway.
 template <typename R>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kShareThreadsLong)
 k_mf_alpha(const GroupDev<R>* __restrict__ G, Rows rows, CgS C) {
     pdl_enter();
     const int row = blockIdx.x;
-    const int f = rows.group[row];
+    const int f = rows.group[row], local = rows.local[row], act = C.active[row];
+    const double rr = C.rr[row];
     if (f < 0) return;
-    if (!C.active[row]) {
+    if (!act) {
         // a system that stopped keeps its x and r: the updates of steps 3 and 5 add 0
         if (threadIdx.x == 0) C.alpha[row] = 0.0;
         return;
     }
     const GroupDev<R>& gd = G[f];
-    const double den = row_shares(gd.part + (size_t)rows.local[row] * gd.ntiles, gd.ntiles);
-    if (threadIdx.x == 0) C.alpha[row] = C.rr[row] / den;
+    const double den = row_shares(gd.part + (size_t)local * gd.ntiles, gd.ntiles);
+    if (threadIdx.x == 0) C.alpha[row] = rr / den;
 }
 
-// 4: beta = the new ||r||^2 over the old, and the per-row flags (one block per row)
+// 4: beta = the new ||r||^2 over the old, and the per-row flags (one block per row; the division and the root, about
+// 900 clocks each, on two warps)
 template <typename R>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kShareThreadsLong)
 k_mf_beta(const GroupDev<R>* __restrict__ G, Rows rows, CgS C) {
     pdl_enter();
     const int row = blockIdx.x;
-    const int f = rows.group[row];
-    if (f < 0 || !C.active[row]) return;
+    const int f = rows.group[row], local = rows.local[row], act = C.active[row], done = C.iters[row] + 1;
+    const double rr = C.rr[row], bn = C.bn[row], ru = C.rr_ru[row];
+    if (f < 0 || !act) return;
     const GroupDev<R>& gd = G[f];
-    const double rn = row_shares(gd.part2 + (size_t)rows.local[row] * gd.ntiles, gd.ntiles);
-    if (threadIdx.x != 0) return;
-    C.beta[row] = rn / C.rr[row];
-    C.rr[row] = rn;
-    C.iters[row] += 1;
+    const double rn = row_shares(gd.part2 + (size_t)local * gd.ntiles, gd.ntiles);
+    // every thread has read the row's scalars: row_shares has a barrier
+    if (threadIdx.x == 0) {
+        C.beta[row] = rn / rr;
+        C.rr[row] = rn;
+        C.iters[row] = done;
+    }
+    if (threadIdx.x != 32) return;
     if (!isfinite(rn)) {
         C.flag[row] = 3;
         C.active[row] = 0;
-    } else if (sqrt(rn) <= C.tol * C.bn[row]) {
+    } else if (sqrt(rn) <= C.tol * bn) {
         C.flag[row] = 2;
         C.active[row] = 0;
-    } else if (C.iters[row] >= C.maxiter) {
+    } else if (done >= C.maxiter) {
         C.flag[row] = 3;
         C.active[row] = 0;
-    } else if (C.delta2 > 0.0 && rn < C.delta2 * C.rr_ru[row]) {
+    } else if (C.delta2 > 0.0 && rn < C.delta2 * ru) {
         C.flag[row] = 1;
     }
 }
@@ -425,13 +441,12 @@ __device__ __forceinline__ void rowsum(double (&v)[NV], double* partials, unsign
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < NV; k++) part[(size_t)k * nblk + blockIdx.x] = v[k];
-        __threadfence();
-        unsigned t = atomicAdd(counters + row, 1u);
+        unsigned t;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(counters + row) : "memory");
         s_last = (t == nblk - 1);
     }
     __syncthreads();
     if (!s_last) return;
-    __threadfence();
     double tot[NV];
 #pragma unroll
     for (int k = 0; k < NV; k++) tot[k] = 0.0;
@@ -442,7 +457,6 @@ __device__ __forceinline__ void rowsum(double (&v)[NV], double* partials, unsign
     if (threadIdx.x == 0) {
         fin(tot);
         counters[row] = 0u;
-        __threadfence();
     }
 }
 
@@ -531,14 +545,15 @@ __global__ void k_mf_ru_flush(const int* __restrict__ slot, const int* __restric
          e += (long)gridDim.x * blockDim.x) {
         cx_t<R> d = xr[e];
         double2 xv = x[e];
-        xv.x += (double)d.x;
-        xv.y += (double)d.y;
+        xv.x += widen(d.x);
+        xv.y += widen(d.y);
         x[e] = xv;
         gk[e] = xv;
         xr[e] = mk<R>(0, 0);
     }
 }
 
+// (the FP64 pipe bounds it, not the 40 bytes per entry: the roundings to FP32 are done with integers)
 // r64 = b - (M x)[k]; r_R[slot] = r64; rr, rr_ru, true residual; active flag
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
@@ -556,7 +571,7 @@ k_mf_ru_resid(const int* __restrict__ row_of, const int* __restrict__ slot,
          e += (long)gridDim.x * blockDim.x) {
         double2 bv = b[e], mv = mx[e];
         double rx = bv.x - mv.x, ry = bv.y - mv.y;
-        r[e] = mk<R>((R)rx, (R)ry);
+        r[e] = mk<R>(to_real<R>(rx), to_real<R>(ry));
         part += rx * rx + ry * ry;
     }
     double red[1] = {part};
@@ -636,7 +651,7 @@ template <typename R>
 void launch_op(bool eo, int code, int tiles, cudaStream_t s, const GroupDev<R>* gdev, int ng, Rows rows, const CgS& C, bool with_alpha) {
     auto alpha = [&]() {
         if (!with_alpha) return;
-        launch_pdl(C.pdl, k_mf_alpha<R>, C.rows_cap, 256, 0, s, gdev, rows, C);
+        launch_pdl(C.pdl, k_mf_alpha<R>, C.rows_cap, C.share_t, 0, s, gdev, rows, C);
     };
     if constexpr (sizeof(R) == 8) {
         // code = the grid rows (systems side by side)
@@ -812,7 +827,7 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
     Carve2 cv{ws.as<char>()};
     std::vector<GroupDev<R>> gd(ng);
     std::vector<double2*> Gx(ng), MX(ng), T64(ng);
-    int tile0 = 0;
+    int tile0 = 0, tiles_max = 0;
     for (int f = 0; f < ng; f++) {
         seedcg_handle* h = groups[f].h;
         const long n = 12L * nsites(groups[f]);
@@ -836,6 +851,7 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
         gd[f].part2 = cv.take<double>((size_t)ns * gd[f].ntiles);
         gd[f].tile0 = tile0;
         tile0 += gd[f].ntiles;
+        tiles_max = std::max(tiles_max, gd[f].ntiles);
         SEEDCG_CUDA_TRY(cudaMemsetAsync(gd[f].xr, 0, (size_t)ns * n * cxR, st));
     }
     GroupDev<R>* gdev = cv.take<GroupDev<R>>(kMaxGroups);
@@ -863,6 +879,7 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
     C.delta2 = reliable_delta > 0.0 ? reliable_delta * reliable_delta : 0.0;
     C.maxiter = maxiter;
     C.rows_cap = rows_cap;
+    C.share_t = share_threads(tiles_max);
     C.pdl = pdl_for(entries);
     SEEDCG_CUDA_TRY(cudaMemsetAsync(C.counters, 0, sizeof(unsigned) * (rows_cap + 64), st));
     SEEDCG_CUDA_TRY(cudaMemsetAsync(C.iters, 0, sizeof(int) * rows_cap, st));
@@ -1039,7 +1056,7 @@ void batched_cg(std::vector<CgGroup>& groups, double tol, double reliable_delta,
     auto chunk = [&](cudaStream_t s) {
         for (int it = 0; it < poll; it++) {
             launch_op<R>(eo, rpb, tiles, s, gdev, ng, rows, C, true);   // steps 1-3
-            launch_pdl(C.pdl, k_mf_beta<R>, rows_cap, 256, 0, s, gdev, rows, C);
+            launch_pdl(C.pdl, k_mf_beta<R>, rows_cap, C.share_t, 0, s, gdev, rows, C);
             launch_pdl(C.pdl, k_mf_xp<R>, dim3(gx, rows_cap), kRedThreads, 0, s, gdev, rows, C);
         }
     };

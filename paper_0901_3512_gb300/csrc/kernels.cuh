@@ -24,6 +24,7 @@ struct LzCtl {
     double past_factor;
     double nv;        // scratch: norm of v_i during re-orthogonalisation
     double2 dvf;      // scratch: v_i^dag f during re-orthogonalisation
+    int i_x;          // the last iteration that added its term to half of x^1 (k_lz_update_v)
 };
 
 struct LzDev {

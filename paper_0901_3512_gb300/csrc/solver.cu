@@ -66,7 +66,9 @@ inline int lz_blocks_per_sm(int sites) {
 // block takes the reduction's atomic ticket, and thousands of tickets on one
 // counter cost more than the pass's loads (the 16^3x32 Lanczos update: 23 us at
 // 304 blocks against 35 us at 3072)
-inline int lean_blocks(long n, int w) { return std::min(vec_blocks(n, w), 2 * 152); }
+// (those blocks are of 256 threads; vectors with less than a group per thread are spread over the SMs, and
+// their FP64 pipes, in smaller ones)
+inline int lean_threads(long n, int w) { return n / w <= 304 * 64 ? 64 : n / w <= 304 * 256 ? 128 : 256; }
 
 // ===========================================================================
 // phase A kernels.  Every kernel of iteration i returns at once when i
@@ -74,51 +76,68 @@ inline int lean_blocks(long n, int w) { return std::min(vec_blocks(n, w), 2 * 15
 // may queue iterations ahead of its next poll.
 // ===========================================================================
 
-// |zeta_i / delta_i| of the residual estimate, known before beta_i
-__device__ __forceinline__ double lz_ratio(const LzDev& L, int i) { return fabs(L.zeta[i - 1] / L.delta[i - 1]); }
+// What step 9 needs besides beta_i (grid_sum's aux): |zeta_i / delta_i| of the residual estimate and the scalars read
+struct LzBetaPre {
+    enum { RATIO, ALPHA, DELTA, BOUND, SMALL, BETA };
+};
+__device__ __forceinline__ void lz_beta_pre(const LzDev& L, int i, double* pre) {
+    const LzCtl* c = L.ctl;
+    const double z = L.zeta[i - 1], d = L.delta[i - 1], a = L.alpha[i - 1];
+    pre[LzBetaPre::ALPHA] = a;
+    pre[LzBetaPre::DELTA] = d;
+    pre[LzBetaPre::BOUND] = c->m_conv == 0 ? c->tol * c->bnorm1 : -1.0;   // converged: no estimate is below
+    pre[LzBetaPre::SMALL] = 1e-14 * fabs(a);
+    pre[LzBetaPre::BETA] = L.beta[i - 1];   // before a PO step makes it final
+    pre[LzBetaPre::RATIO] = fabs(z / d);
+}
 
-// Algorithm 1 step 9 bookkeeping after beta_i is final (ratio: lz_ratio).
-__device__ void lz_after_beta(const LzDev& L, int i, double ratio) {
+// Algorithm 1 step 9 bookkeeping once beta_i = b is final
+__device__ __forceinline__ void lz_after_beta(const LzDev& L, int i, double b, const double* pre) {
     LzCtl* c = L.ctl;
-    const double b = L.beta[i - 1], a = L.alpha[i - 1];
-    const double d = L.delta[i - 1];
-    if (!isfinite(b) || !isfinite(d) || !isfinite(a)) {
+    if (!isfinite(b) || !isfinite(pre[LzBetaPre::DELTA]) || !isfinite(pre[LzBetaPre::ALPHA])) {
         c->status = SEEDCG_ERR_NAN;
         c->m = i;
         return;
     }
-    const double est = b * ratio;
-    if (c->m_conv == 0 && est <= c->tol * c->bnorm1) {
+    const double est = b * pre[LzBetaPre::RATIO];
+    if (est <= pre[LzBetaPre::BOUND]) {
         c->m_conv = i;
         int m1 = i + c->extra_iters;
         int m2 = (int)ceil(c->past_factor * (double)i);
         int m = m1 > m2 ? m1 : m2;
         c->m = m < c->m_max ? m : c->m_max;
     }
-    if (b <= 1e-14 * fabs(a)) {
+    if (b <= pre[LzBetaPre::SMALL]) {
         c->breakdown = 1;
         c->m = i;
     }
 }
 
-// gamma_{i-1} = beta_{i-1} / delta_{i-1}, known before alpha_i
-__device__ __forceinline__ double lz_gamma(const LzDev& L, int i) {
-    return i == 1 ? 0.0 : L.beta[i - 2] / L.delta[i - 2];
+// gamma_{i-1} = beta_{i-1} / delta_{i-1} and what else of step i-1 the LU recurrence takes, known before alpha_i
+struct LzAlphaPre {
+    enum { GAMMA, BETA, ZETA };
+};
+__device__ __forceinline__ void lz_alpha_pre(const LzDev& L, int i, double* pre) {
+    const double b = i == 1 ? L.ctl->beta0 : L.beta[i - 2];
+    pre[LzAlphaPre::BETA] = b;
+    pre[LzAlphaPre::ZETA] = i == 1 ? 0.0 : L.zeta[i - 2];
+    pre[LzAlphaPre::GAMMA] = i == 1 ? 0.0 : b / L.delta[i - 2];
 }
 
 // alpha_i is final: the LU recurrence of T (Algorithm 1 steps 3 and 6, Eq. 2)
-__device__ __forceinline__ void lz_alpha_fin(const LzDev& L, int i, double a, double gm) {
+__device__ __forceinline__ void lz_alpha_fin(const LzDev& L, int i, double a, const double* pre) {
     L.alpha[i - 1] = a;
+    double d = a;
     if (i == 1) {
-        L.delta[0] = a;
-        L.zeta[0] = L.ctl->beta0;
+        L.zeta[0] = pre[LzAlphaPre::BETA];   // beta_0
     } else {
-        const double bp = L.beta[i - 2];
+        const double gm = pre[LzAlphaPre::GAMMA];
+        d = a - gm * pre[LzAlphaPre::BETA];
         L.gamma[i - 2] = gm;
-        L.delta[i - 1] = a - gm * bp;
-        L.zeta[i - 1] = -gm * L.zeta[i - 2];
+        L.zeta[i - 1] = -gm * pre[LzAlphaPre::ZETA];
     }
-    if (L.delta[i - 1] == 0.0) {
+    L.delta[i - 1] = d;
+    if (d == 0.0) {
         L.ctl->status = SEEDCG_ERR_BREAKDOWN;
         L.ctl->m = i;
     }
@@ -211,8 +230,8 @@ k_lz_Ddag(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restr
         }
         red[0] = (double)part;
     }
-    grid_sum<1>(red, L.partials, L.counters + CTR_B, [&] { return lz_gamma(L, i); },
-                    [&](double* tot, double gm) { lz_alpha_fin(L, i, tot[0], gm); });
+    grid_sum<1>(red, L.partials, L.counters + CTR_B, [&](double* pre) { lz_alpha_pre(L, i, pre); },
+                    [&](double* tot, const double* pre) { lz_alpha_fin(L, i, tot[0], pre); });
 }
 
 // Even-odd system (Section 3): M = A^dag A on odd-site half vectors, A = 1 - kappa^2 H_oe H_eo,
@@ -267,8 +286,8 @@ k_lz_eo(Geom g, const cx_t<R>* __restrict__ u, R kk, const cx_t<R>* __restrict__
         }
     }
     if (STAGE == 3)
-        grid_sum<1>(red, L.partials, L.counters + CTR_B, [&] { return lz_gamma(L, i); },
-                    [&](double* tot, double gm) { lz_alpha_fin(L, i, tot[0], gm); });
+        grid_sum<1>(red, L.partials, L.counters + CTR_B, [&](double* pre) { lz_alpha_pre(L, i, pre); },
+                    [&](double* tot, const double* pre) { lz_alpha_fin(L, i, tot[0], pre); });
 }
 
 // FP64 runs apply the operator in fixed point (fixhop.cuh).  The epilogues: PUT (D, or A's second hop)
@@ -283,7 +302,7 @@ struct LzFixEpi {
     double2* vout;
     double2* Vrow;
     int* runE;              // running exponents of the stored rows
-    double inv;
+    const double* inv;      // in shared memory, there before the tile's first barrier
     const double2* v;       // LZ_LAST
     const double2* vprev;   // null: no beta_{i-1} v_{i-1}
     double bprev;
@@ -291,6 +310,7 @@ struct LzFixEpi {
     double part;
     __device__ __forceinline__ double operator()(int, int plane, int idx, int, bool live, double2 a, double2 b) {
         const size_t ix = ((size_t)plane * vo + idx) * 2;
+        const double inv = KIND == LZ_PUT ? *this->inv : 1.0;
         if (KIND == LZ_PUT) {
             // groups of 8 lanes hold a block of 16 entries and are live or not as a whole
             const double2 za = live ? cscale(w[ix], inv) : make_double2(0.0, 0.0);
@@ -336,12 +356,15 @@ k_lz_fix(FixDev F, FixOp op, const double2* __restrict__ w, double2* __restrict_
     pdl_enter();
     if (i > L.ctl->m) return;
     extern __shared__ __align__(16) unsigned char fix_smem[];
+    // one thread divides (an FP64 division by all of them would hold the pipe for 1 us per block)
+    __shared__ double s_inv;
+    if (KIND == LZ_PUT && threadIdx.x == blockDim.x - 1) s_inv = lz_inv<double>(L, i);
     LzFixEpi<KIND> epi{out,
                        w,
                        v,
                        Vrow,
                        runE,
-                       KIND == LZ_PUT ? lz_inv<double>(L, i) : 1.0,
+                       &s_inv,
                        v,
                        KIND == LZ_LAST && i > 1 ? vprev : nullptr,
                        KIND == LZ_LAST && i > 1 ? L.beta[i - 2] : 0.0,
@@ -350,8 +373,8 @@ k_lz_fix(FixDev F, FixOp op, const double2* __restrict__ w, double2* __restrict_
     fix_tile(F, op, blockIdx.x, 0, 1, 1, fix_smem, epi);
     if (KIND == LZ_LAST) {
         double red[1] = {epi.part};
-        grid_sum<1>(red, L.partials, L.counters + CTR_B, [&] { return lz_gamma(L, i); },
-                    [&](double* tot, double gm) { lz_alpha_fin(L, i, tot[0], gm); });
+        grid_sum<1>(red, L.partials, L.counters + CTR_B, [&](double* pre) { lz_alpha_pre(L, i, pre); },
+                    [&](double* tot, const double* pre) { lz_alpha_fin(L, i, tot[0], pre); });
     }
 }
 
@@ -462,47 +485,58 @@ k_lz_update(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, cx_t<R>* __r
         }
     }
     double red[1] = {(double)part};
-    grid_sum<1>(red, L.partials, L.counters + CTR_D, [&] { return lz_ratio(L, i); }, [&](double* tot, double ratio) {
-        L.beta[i - 1] = sqrt(tot[0]);
-        if (final_beta) lz_after_beta(L, i, ratio);
+    grid_sum<1>(red, L.partials, L.counters + CTR_D, [&](double* pre) { lz_beta_pre(L, i, pre); }, [&](double* tot, const double* pre) {
+        const double b = sqrt(tot[0]);
+        L.beta[i - 1] = b;
+        if (final_beta) lz_after_beta(L, i, b, pre);
     });
 }
 
-// The blocked modes' pass with 16-byte accesses: a thread owns 16 / sizeof(cx_t<R>)
+// The blocked modes' pass with 16-byte accesses: a thread owns W = 16 / sizeof(cx_t<R>)
 // consecutive complex entries (two in FP32, one in FP64; n is a multiple of 4).
-// X1: also steps 3 and 6 for RHS 1, w_i = (v_i - beta_{i-1} w_{i-1}) / delta_i in R
+// Steps 3 and 6 for RHS 1 too: w_i = (v_i - beta_{i-1} w_{i-1}) / delta_i in R
 // and x^1 += zeta_i w_i accumulated in FP64 (x1 = the FP64 solution of RHS 1; the
-// systems j >= 2 take Eq. (1) after the run).  X1 = false: f -= alpha v and beta only.
-template <typename R, bool X1>
+// systems j >= 2 take Eq. (1) after the run).
+//
+// x^1 is the widest stream, and its FP64 arithmetic is as long as the pass's traffic (68 clocks per warp and operation),
+// so each iteration takes half of the entries (blocks of 128 groups in turn) two terms further,
+// zeta_{i-1} w_{i-1} and zeta_i w_i in their order, with the w_{i-1} that it reads anyway: the same
+// sums, half of the traffic. k_lz_flush_x adds the terms that are left at the end. One
+// thread of a block divides by delta_i, beside the block's loads (all of them: 2 us of the pipe per SM).
+// An iteration of Lanczos (operator, this pass and the reductions, without re-orthogonalisation): 16^3 x 32 with V in
+// BF16 67.6 -> 64.6 us, 10 x 6 x 14 x 12 in FP32 21.4 -> 19.9, 4^3 x 4 in FP64 24.0 -> 20.6.
+__device__ __forceinline__ bool lz_x_turn(long g, int i) { return ((int)(g >> 7) & 1) == (i & 1); }
+
+template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
 k_lz_update_v(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, cx_t<R>* __restrict__ w,
               double2* __restrict__ x1, long n, int i, int final_beta, LzDev L) {
     pdl_enter();
-    if (i > L.ctl->m) return;
     constexpr int W = 16 / (int)sizeof(cx_t<R>);
-    const R a = (R)L.alpha[i - 1];
-    R bp = 0, idl = 0;
-    double zt = 0.0;
-    if (X1) {
-        bp = i > 1 ? (R)L.beta[i - 2] : R(0);
-        idl = (R)(1.0 / L.delta[i - 1]);
-        zt = L.zeta[i - 1];
-    }
+    __shared__ R s_idl;
+    // (all read before the test, which waits for its own)
+    const int m = L.ctl->m;
+    const double alpha = L.alpha[i - 1], zt = L.zeta[i - 1];
+    const double beta = i > 1 ? L.beta[i - 2] : 0.0, ztp = i > 1 ? L.zeta[i - 2] : 0.0;
+    const double delta = L.delta[i - 1];
+    if (i > m) return;
+    if (threadIdx.x == blockDim.x - 1) s_idl = (R)(1.0 / delta);
+    const R a = (R)alpha, bp = (R)beta;
     R part = 0;
     const long ng = n / W;
     const long st = (long)gridDim.x * blockDim.x;
+    const long b0 = blockIdx.x * (long)blockDim.x;
     // two 16-byte groups per thread and trip, every load of both issued before the
     // arithmetic: the grid is two blocks per SM, so each thread keeps more bytes in flight
-    for (long g0 = blockIdx.x * (long)blockDim.x + threadIdx.x; g0 < ng; g0 += 2 * st) {
-        const bool two = g0 + st < ng;
-        cx_t<R> vv[2][W], fv[2][W], ww[2][W];
+    for (long gb = b0; gb < ng; gb += 2 * st) {
+        const long g0 = gb + threadIdx.x;
+        cx_t<R> vv[2][W], fv[2][W], wo[2][W];
         double2 xv[2][W];
 #pragma unroll
         for (int h = 0; h < 2; h++) {
-            if (h == 1 && !two) break;
             const long g = g0 + h * st;
-            if (X1) {
-                // the FP64 x^1 is the widest stream of the pass
+            if (g >= ng) break;
+            if (lz_x_turn(g, i)) {
 #pragma unroll
                 for (int k = 0; k < W; k++) xv[h][k] = __ldcs(x1 + g * W + k);
             }
@@ -511,54 +545,76 @@ k_lz_update_v(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, cx_t<R>* _
                 const float4 b4 = reinterpret_cast<const float4*>(f)[g];
                 vv[h][0] = mk<R>(a4.x, a4.y); vv[h][1] = mk<R>(a4.z, a4.w);
                 fv[h][0] = mk<R>(b4.x, b4.y); fv[h][1] = mk<R>(b4.z, b4.w);
-                if (X1) {
-                    const float4 c4 = i > 1 ? __ldcs(reinterpret_cast<const float4*>(w) + g) : make_float4(0, 0, 0, 0);
-                    ww[h][0] = mk<R>(c4.x, c4.y); ww[h][1] = mk<R>(c4.z, c4.w);
-                }
+                const float4 c4 = i > 1 ? __ldcs(reinterpret_cast<const float4*>(w) + g) : make_float4(0, 0, 0, 0);
+                wo[h][0] = mk<R>(c4.x, c4.y); wo[h][1] = mk<R>(c4.z, c4.w);
             } else {
                 vv[h][0] = v[g];
                 fv[h][0] = f[g];
-                if (X1) ww[h][0] = i > 1 ? __ldcs(reinterpret_cast<const double2*>(w) + g) : mk<R>(0, 0);
+                wo[h][0] = i > 1 ? __ldcs(reinterpret_cast<const double2*>(w) + g) : mk<R>(0, 0);
             }
         }
+        if (gb == b0) __syncthreads();
+        const R idl = s_idl;
 #pragma unroll
         for (int h = 0; h < 2; h++) {
-            if (h == 1 && !two) break;
             const long g = g0 + h * st;
+            if (g >= ng) break;
+            cx_t<R> ww[W];
 #pragma unroll
             for (int k = 0; k < W; k++) {
                 fv[h][k].x -= a * vv[h][k].x;
                 fv[h][k].y -= a * vv[h][k].y;
                 part += fv[h][k].x * fv[h][k].x + fv[h][k].y * fv[h][k].y;
-                if (X1) {
-                    ww[h][k].x = (vv[h][k].x - bp * ww[h][k].x) * idl;
-                    ww[h][k].y = (vv[h][k].y - bp * ww[h][k].y) * idl;
-                }
+                ww[k].x = (vv[h][k].x - bp * wo[h][k].x) * idl;
+                ww[k].y = (vv[h][k].y - bp * wo[h][k].y) * idl;
             }
-            // w and x^1 are streamed (evict-first): each is touched once per iteration, and
-            // caching them would push the operator's links and vectors out of L2
+            // w and x^1 are streamed (evict-first): caching them would push the operator's
+            // links and vectors out of L2
             if constexpr (W == 2) {
                 reinterpret_cast<float4*>(f)[g] = make_float4(fv[h][0].x, fv[h][0].y, fv[h][1].x, fv[h][1].y);
-                if (X1) __stcs(reinterpret_cast<float4*>(w) + g, make_float4(ww[h][0].x, ww[h][0].y, ww[h][1].x, ww[h][1].y));
+                __stcs(reinterpret_cast<float4*>(w) + g, make_float4(ww[0].x, ww[0].y, ww[1].x, ww[1].y));
             } else {
                 f[g] = fv[h][0];
-                if (X1) __stcs(reinterpret_cast<double2*>(w) + g, make_double2(ww[h][0].x, ww[h][0].y));
+                __stcs(reinterpret_cast<double2*>(w) + g, make_double2(ww[0].x, ww[0].y));
             }
-            if (X1) {
+            if (lz_x_turn(g, i)) {
 #pragma unroll
                 for (int k = 0; k < W; k++) {
-                    xv[h][k].x = fma(zt, (double)ww[h][k].x, xv[h][k].x);
-                    xv[h][k].y = fma(zt, (double)ww[h][k].y, xv[h][k].y);
+                    if (i > 1) {
+                        xv[h][k].x = fma(ztp, widen(wo[h][k].x), xv[h][k].x);
+                        xv[h][k].y = fma(ztp, widen(wo[h][k].y), xv[h][k].y);
+                    }
+                    xv[h][k].x = fma(zt, widen(ww[k].x), xv[h][k].x);
+                    xv[h][k].y = fma(zt, widen(ww[k].y), xv[h][k].y);
                     __stcs(x1 + g * W + k, xv[h][k]);
                 }
             }
         }
     }
     double red[1] = {(double)part};
-    grid_sum<1>(red, L.partials, L.counters + CTR_D, [&] { return lz_ratio(L, i); }, [&](double* tot, double ratio) {
-        L.beta[i - 1] = sqrt(tot[0]);
-        if (final_beta) lz_after_beta(L, i, ratio);
+    grid_sum<1>(red, L.partials, L.counters + CTR_D, [&](double* pre) { lz_beta_pre(L, i, pre); },
+                [&](double* tot, const double* pre) {
+        const double b = sqrt(tot[0]);
+        L.beta[i - 1] = b;
+        L.ctl->i_x = i;
+        if (final_beta) lz_after_beta(L, i, b, pre);
     });
+}
+
+// x^1 += zeta w of the last iteration, where k_lz_update_v has not had its turn
+template <typename R>
+__global__ void __launch_bounds__(kRedThreads)
+k_lz_flush_x(const cx_t<R>* __restrict__ w, double2* __restrict__ x1, long n, LzDev L) {
+    constexpr int W = 16 / (int)sizeof(cx_t<R>);
+    const int i = L.ctl->i_x;
+    const double zt = L.zeta[i - 1];
+    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n; e += (long)gridDim.x * blockDim.x) {
+        if (lz_x_turn(e / W, i)) continue;
+        double2 x = x1[e];
+        x.x = fma(zt, (double)w[e].x, x.x);
+        x.y = fma(zt, (double)w[e].y, x.y);
+        x1[e] = x;
+    }
 }
 
 // ---- step 8: periodic re-orthogonalisation (classical Gram-Schmidt) ----
@@ -742,7 +798,10 @@ k_po_normalise(cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f, VT* __res
                long n, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
-    const R inv = (R)(1.0 / L.ctl->nv);
+    __shared__ R s_inv;
+    if (threadIdx.x == blockDim.x - 1) s_inv = (R)(1.0 / L.ctl->nv);   // once per block, not per thread
+    __syncthreads();
+    const R inv = s_inv;
     R pr = 0, pi = 0;
     for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n;
          e += (long)gridDim.x * blockDim.x) {
@@ -776,18 +835,18 @@ k_po_finish(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, long n, int 
         part += fv.x * fv.x + fv.y * fv.y;
     }
     double red[1] = {(double)part};
-    grid_sum<1>(red, L.partials, L.counters + CTR_PO4, [&] { return lz_ratio(L, i); }, [&](double* tot, double ratio) {
+    grid_sum<1>(red, L.partials, L.counters + CTR_PO4, [&](double* pre) { lz_beta_pre(L, i, pre); }, [&](double* tot, const double* pre) {
         const double bnew = sqrt(tot[0]);
         L.ctl->po_count += 1;
         // an orthogonal projection never lengthens f; growth means the stored
         // basis is far from orthonormal: end the run at i - 1
-        if (L.ctl->guard ? !(bnew <= 1.01 * L.beta[i - 1]) : !isfinite(bnew)) {
+        if (L.ctl->guard ? !(bnew <= 1.01 * pre[LzBetaPre::BETA]) : !isfinite(bnew)) {
             L.ctl->breakdown = 3;
             L.ctl->m = i - 1;
             return;
         }
         L.beta[i - 1] = bnew;
-        lz_after_beta(L, i, ratio);
+        lz_after_beta(L, i, bnew, pre);
     });
 }
 
@@ -1195,6 +1254,9 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
         int i = 1;
         const int sbh = site_blocks(vol / 2);
         const int bps = lz_blocks_per_sm(vol);
+        const long lean_g = n * (long)sizeof(cx_t<R>) / 16;
+        const int lean_t = lean_threads(n, 16 / (int)sizeof(cx_t<R>));
+        const int lean = (int)std::min<long>((lean_g + lean_t - 1) / lean_t, 2 * 152);
         cx_t<R>* slot = vA;
         const R kk = (R)(h->kappa * h->kappa);
         for (; i <= m_max; i++) {
@@ -1234,8 +1296,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                 launch_pdl(pdl, k_lz_update<R, true>, rb, kRedThreads, 0, st, 
                     v, fv, wv, reinterpret_cast<cx_t<R>*>(X64), nrhs, n, i, po_now ? 0 : 1, L);
             else
-                launch_pdl(pdl, k_lz_update_v<R, true>, lean_blocks(n, 16 / (int)sizeof(cx_t<R>)), kRedThreads, 0, st, 
-                    v, fv, wv, X64, n, i, po_now ? 0 : 1, L);
+                launch_pdl(pdl, k_lz_update_v<R>, lean, lean_t, 0, st, v, fv, wv, X64, n, i, po_now ? 0 : 1, L);
             if (po_now) {
                 cudaEvent_t e0, e1;
                 cudaEventCreate(&e0);
@@ -1262,6 +1323,10 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
         }
         SEEDCG_CUDA_TRY(cudaMemcpyAsync(pin, L.ctl, sizeof(int) * 8, cudaMemcpyDeviceToHost, st));
         SEEDCG_CUDA_TRY(cudaStreamSynchronize(st));
+        if (!literal) {
+            k_lz_flush_x<R><<<vec_blocks(n, 16 / (int)sizeof(cx_t<R>)), kRedThreads, 0, st>>>(wv, X64, n, L);
+            SEEDCG_CHECK_LAUNCH();
+        }
         m = std::min(pin[0], m_max);
         m_conv = pin[1];
         lz_status = pin[2];
