@@ -35,15 +35,28 @@ __global__ void k_to_internal_f64(const double2* __restrict__ in, double2* __res
     for (int k = 0; k < 12; k++) dst[sidx(k, s, vol)] = src[k];
 }
 
+// (with 16-byte stores every 32-byte sector is written twice: 12 fields of 16^3 x 32, 196 us against 88 in whole sectors; `wide`: out
+// is 32-byte aligned, as a spinor is a multiple of it)
 __global__ void k_from_internal_f64(const double2* __restrict__ in, double2* __restrict__ out,
-                                    int vol, int n) {
+                                    int vol, int n, int wide) {
     long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (t >= (long)vol * n) return;
     int r = (int)(t / vol), s = (int)(t % vol);
     const double2* src = in + (size_t)r * 12 * vol;
     double2* dst = out + ((size_t)r * vol + s) * 12;
+    double2 z[12];
 #pragma unroll
-    for (int k = 0; k < 12; k++) dst[k] = src[sidx(k, s, vol)];
+    for (int k = 0; k < 12; k++) z[k] = src[sidx(k, s, vol)];
+#pragma unroll
+    for (int k = 0; k < 12; k += 2) {
+        if (wide) {
+            asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(dst + k), "d"(z[k].x), "d"(z[k].y),
+                         "d"(z[k + 1].x), "d"(z[k + 1].y) : "memory");
+        } else {
+            dst[k] = z[k];
+            dst[k + 1] = z[k + 1];
+        }
+    }
 }
 
 __global__ void k_to_internal_f32(const double2* __restrict__ in, float2* __restrict__ out,
@@ -283,7 +296,7 @@ void to_internal_f64(const double* in, double2* out, int vol, int n, cudaStream_
 void from_internal_f64(const double2* in, double* out, int vol, int n, cudaStream_t s) {
     if ((long)vol * n == 0) return;
     k_from_internal_f64<<<blocks_for((long)vol * n, 256), 256, 0, s>>>(
-        in, reinterpret_cast<double2*>(out), vol, n);
+        in, reinterpret_cast<double2*>(out), vol, n, (reinterpret_cast<uintptr_t>(out) & 31) == 0);
     SEEDCG_CHECK_LAUNCH();
 }
 void to_internal_f32(const double* in, float2* out, int vol, int n, cudaStream_t s) {

@@ -279,10 +279,12 @@ k_g_first(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, cons
     st_site(site_ptr(h, warp, vol, x), r);
 }
 
-// layer 3 (8 -> 1): eight warps transport one input channel each for direction d + 1 while six warps add
-// direction d, a (colour, spin pair) each, over the eight channels; the buffer of a direction is reused two later.
-// 16^3 x 32: 346 us with one thread per site, 214 us here (issue 62 % busy, shared memory 74 %).
-__global__ void __launch_bounds__(448)
+// layer 3 (8 -> 1): eight warps transport one input channel each for direction d + 1 while three warps add
+// direction d, a colour's four spins each, over the eight channels; the buffer of a direction is reused two later.
+// Shared memory bounds it (two wavefronts per value read): with four spins per value instead of two 16^3 x 32 takes
+// 195 us instead of 214 (346 with one thread per site).
+constexpr int kLastThreads = 352;
+__global__ void __launch_bounds__(kLastThreads, 2)
 k_g_last(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const bf2* __restrict__ in,
          bf2* __restrict__ z) {
     extern __shared__ __align__(16) unsigned char last_smem[];
@@ -295,14 +297,16 @@ k_g_last(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, x = x0 + lane;
     const bool live = x < vol;
     stage_links<false>(gm, u, x0, sl, snb);
-    // weights [d][ci][input spin][output spin]: one 16-byte load gives the two output spins of a warp
+    // weights [d][ci][input spin][output spin]: two 16-byte loads give the four output spins
     for (int t = threadIdx.x; t < 72 * 16; t += blockDim.x)
         sw[t / 16][(t % 4) * 4 + (t / 4) % 4] = __bfloat1622float2(W[t]);
     __syncthreads();
     const bool producer = warp < 8;
     if (producer && live) stage_gather(in + (size_t)warp * vol * 12, x, 0, sl, snb, lane, sg + 12 * warp);
-    const int cw = warp - 8, c = cw % 3, s0 = cw < 3 ? 0 : 2;   // consumer: spins s0, s0 + 1 of colour c
-    float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+    const int c = warp - 8;   // consumer: colour c
+    float2 acc[4];
+#pragma unroll
+    for (int s = 0; s < 4; s++) acc[s] = make_float2(0.f, 0.f);
 #pragma unroll 1
     for (int d = 0; d < 9; d++) {
         __syncthreads();
@@ -317,16 +321,19 @@ k_g_last(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const
 #pragma unroll
                 for (int sp = 0; sp < 4; sp++) {
                     const float2 gv = g[12 * ci + 3 * sp + c][lane];
-                    const float4 ww = *reinterpret_cast<const float4*>(w + 4 * sp + s0);
-                    a0 = cfma(make_float2(ww.x, ww.y), gv, a0);
-                    a1 = cfma(make_float2(ww.z, ww.w), gv, a1);
+                    const float4 w0 = *reinterpret_cast<const float4*>(w + 4 * sp);
+                    const float4 w1 = *reinterpret_cast<const float4*>(w + 4 * sp + 2);
+                    acc[0] = cfma(make_float2(w0.x, w0.y), gv, acc[0]);
+                    acc[1] = cfma(make_float2(w0.z, w0.w), gv, acc[1]);
+                    acc[2] = cfma(make_float2(w1.x, w1.y), gv, acc[2]);
+                    acc[3] = cfma(make_float2(w1.z, w1.w), gv, acc[3]);
                 }
             }
         }
     }
     if (!producer) {
-        so[lane][3 * s0 + c] = __float22bfloat162_rn(a0);
-        so[lane][3 * s0 + 3 + c] = __float22bfloat162_rn(a1);
+#pragma unroll
+        for (int s = 0; s < 4; s++) so[lane][3 * s + c] = __float22bfloat162_rn(acc[s]);
     }
     __syncthreads();
     // the block's results are contiguous in z: [site][12]
@@ -872,13 +879,20 @@ __device__ __forceinline__ size_t pidx(int s, int k, int vol) {
 }
 
 // a0 = b / ||b|| in bf16 [V][12]
+// One thread of a block divides (an FP64 operation takes the pipe 68 clocks per warp, a division a dozen of
+// them), and roundings to and from FP32 move bits, with four entries in flight. 16^3 x 32: k_g_scale_in 22.8 -> 16.4 us,
+// k_g_loss 47 -> 41 us.
 __global__ void k_g_scale_in(const double2* __restrict__ b, const double* __restrict__ nb, bf2* __restrict__ a0,
                              int vol) {
-    const double inv = 1.0 / *nb;
+    __shared__ double s_inv;
+    if (threadIdx.x == 0) s_inv = 1.0 / *nb;
+    __syncthreads();
+    const double inv = s_inv;
+#pragma unroll 4
     for (long o = blockIdx.x * (long)blockDim.x + threadIdx.x; o < 12L * vol; o += (long)gridDim.x * blockDim.x) {
         const int s = (int)(o / 12), k = (int)(o % 12);
         const double2 z = b[pidx(s, k, vol)];
-        a0[o] = __float22bfloat162_rn(make_float2((float)(z.x * inv), (float)(z.y * inv)));
+        a0[o] = __float22bfloat162_rn(make_float2(narrow(z.x * inv), narrow(z.y * inv)));
     }
 }
 
@@ -886,10 +900,11 @@ __global__ void k_g_scale_in(const double2* __restrict__ b, const double* __rest
 __global__ void k_g_scale_out(const bf2* __restrict__ z3, const double* __restrict__ nb, double2* __restrict__ x0,
                               int vol) {
     const double s = *nb;
+#pragma unroll 4
     for (long o = blockIdx.x * (long)blockDim.x + threadIdx.x; o < 12L * vol; o += (long)gridDim.x * blockDim.x) {
         const int st = (int)(o / 12), k = (int)(o % 12);
         const float2 z = __bfloat1622float2(z3[o]);
-        x0[pidx(st, k, vol)] = make_double2(s * z.x, s * z.y);
+        x0[pidx(st, k, vol)] = make_double2(s * widen(z.x), s * widen(z.y));
     }
 }
 
@@ -899,15 +914,19 @@ k_g_loss(const bf2* __restrict__ z3, const double2* __restrict__ x, const double
          const double* __restrict__ nx, double inv_batch, bf2* __restrict__ dz3, int vol,
          double* partials, unsigned* ctr, double* loss_acc) {
     const double s = *nb, xn2 = (*nx) * (*nx);
+    __shared__ double s_f;
+    if (threadIdx.x == 0) s_f = s * 2.0 * inv_batch / xn2;
+    __syncthreads();
+    const double f = s_f;
     double part = 0.0;
+#pragma unroll 4
     for (long o = blockIdx.x * (long)blockDim.x + threadIdx.x; o < 12L * vol; o += (long)gridDim.x * blockDim.x) {
         const int st = (int)(o / 12), k = (int)(o % 12);
         const float2 z = __bfloat1622float2(z3[o]);
         const double2 xv = x[pidx(st, k, vol)];
-        const double rx = s * z.x - xv.x, ry = s * z.y - xv.y;
+        const double rx = s * widen(z.x) - xv.x, ry = s * widen(z.y) - xv.y;
         part += rx * rx + ry * ry;
-        const double f = s * 2.0 * inv_batch / xn2;
-        dz3[o] = __float22bfloat162_rn(make_float2((float)(f * rx), (float)(f * ry)));
+        dz3[o] = __float22bfloat162_rn(make_float2(narrow(f * rx), narrow(f * ry)));
     }
     double red[1] = {part};
     grid_sum<1>(red, partials, ctr, [&](double* tot) { *loss_acc += tot[0] / xn2 * inv_batch; });
@@ -1053,7 +1072,7 @@ void forward(seedcg_handle* h, GuessState* G, const Acts& A, const double2* b64,
     double* partials = A.nb + 64;
     unsigned* ctr = reinterpret_cast<unsigned*>(partials + 8192);
     k_norm2_public(b64, n, partials, ctr, A.nb, st);
-    k_g_scale_in<<<std::min<long>((n + 255) / 256, 4096), 256, 0, st>>>(b64, A.nb, A.a0, gm.vol);
+    k_g_scale_in<<<std::min<long>((n + 255) / 256, 8 * 152), 256, 0, st>>>(b64, A.nb, A.a0, gm.vol);
     SEEDCG_CHECK_LAUNCH();
     const int tiles = (gm.vol + SL - 1) / SL;
     k_g_first<<<tiles, 288, 0, st>>>(gm, u, W, A.a0, keep_z ? A.z1 : nullptr, A.h1);
@@ -1062,7 +1081,7 @@ void forward(seedcg_handle* h, GuessState* G, const Acts& A, const double2* b64,
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_g_last, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLastSmem);
     SEEDCG_CUDA_TRY(attr);
-    k_g_last<<<tiles, 448, kLastSmem, st>>>(gm, u, W + GuessState::NW1 + GuessState::NW2, A.h2, A.z3);
+    k_g_last<<<tiles, kLastThreads, kLastSmem, st>>>(gm, u, W + GuessState::NW1 + GuessState::NW2, A.h2, A.z3);
     SEEDCG_CHECK_LAUNCH();
 }
 
@@ -1097,7 +1116,7 @@ void backward_pair(seedcg_handle* h, GuessState* G, const Acts& A, const double2
     double* partials = A.nb + 64;
     unsigned* ctr = reinterpret_cast<unsigned*>(partials + 8192);
     k_norm2_public(x64, n, partials, ctr, A.nx, st);
-    k_g_loss<<<std::min<long>((n + 1023) / 1024, 1216), kRedThreads, 0, st>>>(A.z3, x64, A.nb, A.nx, inv_batch,
+    k_g_loss<<<std::min<long>((n + 1023) / 1024, 4 * 152), kRedThreads, 0, st>>>(A.z3, x64, A.nb, A.nx, inv_batch,
                                                                              A.d3, gm.vol, partials, ctr + 1, A.loss);
     SEEDCG_CHECK_LAUNCH();
     // layer 3 (8 -> 1)
@@ -1204,7 +1223,7 @@ void guess_predict(seedcg_handle* h, int n_fields, const double2* B, double2* X0
     SEEDCG_CUDA_TRY(cudaMemsetAsync(A.nb, 0, G->scal.bytes, st));
     for (int k = 0; k < n_fields; k++) {
         forward(h, G, A, B + (size_t)k * n, false, st);
-        k_g_scale_out<<<std::min<long>((n + 255) / 256, 4096), 256, 0, st>>>(A.z3, A.nb, X0 + (size_t)k * n,
+        k_g_scale_out<<<std::min<long>((n + 255) / 256, 8 * 152), 256, 0, st>>>(A.z3, A.nb, X0 + (size_t)k * n,
                                                                             h->g.vol);
         SEEDCG_CHECK_LAUNCH();
     }
