@@ -35,8 +35,8 @@ __global__ void k_to_internal_f64(const double2* __restrict__ in, double2* __res
     for (int k = 0; k < 12; k++) dst[sidx(k, s, vol)] = src[k];
 }
 
-// (with 16-byte stores every 32-byte sector is written twice: 12 fields of 16^3 x 32, 196 us against 88 in whole sectors; `wide`: out
-// is 32-byte aligned, as a spinor is a multiple of it)
+// (with 16-byte stores every 32-byte sector is written twice: 12 fields of 16^3 x 32 take 196 us, in whole
+// sectors 88; `wide`: out is 32-byte aligned, and so is every spinor)
 __global__ void k_from_internal_f64(const double2* __restrict__ in, double2* __restrict__ out,
                                     int vol, int n, int wide) {
     long t = blockIdx.x * (long)blockDim.x + threadIdx.x;

@@ -206,11 +206,23 @@ __device__ __forceinline__ void staged_link(const float2 (*sl)[SL], int lane, bo
         }
 }
 
-// g_d(x) of one channel into sg[12][lane]
-__device__ __forceinline__ void stage_gather(const bf2* __restrict__ in_ch, int x, int d, const float2 (*sl)[SL],
-                                             const int (*snb)[SL], int lane, float2 (*sg)[SL]) {
+// g_d(x) of one channel into sg[12][lane], in two parts: the source site's values on their way, and the rest
+__device__ __forceinline__ void gather_load(const bf2* __restrict__ in_ch, int x, int d, const int (*snb)[SL], int lane,
+                                            uint4 (&q)[3]) {
+    const uint4* p = reinterpret_cast<const uint4*>(in_ch + (size_t)(d == 0 ? x : snb[d - 1][lane]) * 12);
+#pragma unroll
+    for (int j = 0; j < 3; j++) q[j] = __ldg(p + j);
+}
+__device__ __forceinline__ void gather_put(const uint4 (&q)[3], int d, const float2 (*sl)[SL], int lane,
+                                           float2 (*sg)[SL]) {
     float2 v[12];
-    ld_site(in_ch + (size_t)(d == 0 ? x : snb[d - 1][lane]) * 12, v);
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        v[4 * j + 0] = unpack_bf2(q[j].x);
+        v[4 * j + 1] = unpack_bf2(q[j].y);
+        v[4 * j + 2] = unpack_bf2(q[j].z);
+        v[4 * j + 3] = unpack_bf2(q[j].w);
+    }
     if (d == 0) {
 #pragma unroll
         for (int k = 0; k < 12; k++) sg[k][lane] = v[k];
@@ -250,7 +262,11 @@ k_g_first(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, cons
     const bool live = x < vol;
     stage_links<false>(gm, u, x0, sl, snb);
     __syncthreads();
-    if (live) stage_gather(in, x, warp, sl, snb, lane, sg + 12 * warp);
+    if (live) {
+        uint4 q[3];
+        gather_load(in, x, warp, snb, lane, q);
+        gather_put(q, warp, sl, lane, sg + 12 * warp);
+    }
     __syncthreads();
     if (warp >= 8 || !live) return;
     float2 acc[4][3];
@@ -282,7 +298,7 @@ k_g_first(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, cons
 // layer 3 (8 -> 1): eight warps transport one input channel each for direction d + 1 while three warps add
 // direction d, a colour's four spins each, over the eight channels; the buffer of a direction is reused two later.
 // Shared memory bounds it (two wavefronts per value read): with four spins per value instead of two 16^3 x 32 takes
-// 195 us instead of 214 (346 with one thread per site).
+// 190 us instead of 214 (346 with one thread per site); a producer loads a direction ahead.
 constexpr int kLastThreads = 352;
 __global__ void __launch_bounds__(kLastThreads, 2)
 k_g_last(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const bf2* __restrict__ in,
@@ -302,7 +318,13 @@ k_g_last(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const
         sw[t / 16][(t % 4) * 4 + (t / 4) % 4] = __bfloat1622float2(W[t]);
     __syncthreads();
     const bool producer = warp < 8;
-    if (producer && live) stage_gather(in + (size_t)warp * vol * 12, x, 0, sl, snb, lane, sg + 12 * warp);
+    const bf2* in_ch = in + (size_t)warp * vol * 12;   // (producers)
+    uint4 raw[3];
+    if (producer && live) {
+        gather_load(in_ch, x, 0, snb, lane, raw);
+        gather_put(raw, 0, sl, lane, sg + 12 * warp);
+        gather_load(in_ch, x, 1, snb, lane, raw);
+    }
     const int c = warp - 8;   // consumer: colour c
     float2 acc[4];
 #pragma unroll
@@ -311,8 +333,10 @@ k_g_last(Geom gm, const float2* __restrict__ u, const bf2* __restrict__ W, const
     for (int d = 0; d < 9; d++) {
         __syncthreads();
         if (producer) {
-            if (d < 8 && live)
-                stage_gather(in + (size_t)warp * vol * 12, x, d + 1, sl, snb, lane, sg + ((d + 1) & 1) * 96 + 12 * warp);
+            if (d < 8 && live) {
+                gather_put(raw, d + 1, sl, lane, sg + ((d + 1) & 1) * 96 + 12 * warp);
+                if (d < 7) gather_load(in_ch, x, d + 2, snb, lane, raw);
+            }
         } else {
             const float2 (*g)[SL] = sg + (d & 1) * 96;
 #pragma unroll
