@@ -182,7 +182,7 @@ seedcg_status seedcg_batch_solve(seedcg_handle** hs, int nfields, const int* nrh
  * arithmetic, 1 = FP32 arithmetic (inputs rounded to FP32, result widened).
  * in/out: device pointers, complex128 [n][V][4][3]; they may not overlap.
  * multi = 1 uses the multi-RHS kernel (links staged once per site tile for
- * all n fields), 0 the single-RHS kernel n times.
+ * all n fields), 0 the single-RHS kernel n times; FP64 has one kernel for both.
  */
 seedcg_status seedcg_apply(seedcg_handle* h, int op, int prec, int multi, int n,
                            const double* in, double* out, void* stream);

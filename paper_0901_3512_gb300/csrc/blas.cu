@@ -20,20 +20,6 @@ inline int nblocks(long n, int per_block, int cap) {
     return (int)(b < cap ? b : cap);
 }
 
-template <typename R>
-__global__ void __launch_bounds__(kRedThreads)
-k_dot(const cx_t<R>* __restrict__ a, const cx_t<R>* __restrict__ b, long n, double* partials,
-      unsigned* ctr, double2* res) {
-    double v[2] = {0.0, 0.0};
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n;
-         e += (long)gridDim.x * blockDim.x) {
-        cx_t<R> x = a[e], y = b[e];
-        v[0] += (double)x.x * y.x + (double)x.y * y.y;
-        v[1] += (double)x.x * y.y - (double)x.y * y.x;
-    }
-    grid_sum<2>(v, partials, ctr, [&](double* t) { *res = make_double2(t[0], t[1]); });
-}
-
 // ---------------------------------------------------------------------------
 // gemm_t: block (tile of TA rows of A) x (slice of the entries); every thread
 // keeps TA x NB complex accumulators in R, the block reduces them in FP64 and
@@ -382,14 +368,6 @@ void k_norm2_public(const double2* x, long n, double* partials, unsigned* ctr, d
     SEEDCG_CHECK_LAUNCH();
 }
 
-template <typename R>
-void dot(const cx_t<R>* a, const cx_t<R>* b, long n, double* partials, unsigned* ctr,
-         double2* res, cudaStream_t s) {
-    int nb = nblocks(n, kRedThreads * 8, kMaxRedBlocks);
-    k_dot<R><<<nb, kRedThreads, 0, s>>>(a, b, n, partials, ctr, res);
-    SEEDCG_CHECK_LAUNCH();
-}
-
 template <typename R, typename AT>
 void gemm_t(const AT* A, long lda, int na, const cx_t<R>* B, long ldb, int nb, long n,
             double2* C, int ldc, double2* scratch, size_t scratch_elems, cudaStream_t s) {
@@ -502,31 +480,22 @@ void convert(const ST* src, DT* dst, long n, cudaStream_t s) {
 }
 
 // explicit instantiations
-template void dot<double>(const double2*, const double2*, long, double*, unsigned*, double2*, cudaStream_t);
-template void dot<float>(const float2*, const float2*, long, double*, unsigned*, double2*, cudaStream_t);
 
 template void gemm_t<double, double2>(const double2*, long, int, const double2*, long, int, long, double2*, int, double2*, size_t, cudaStream_t);
 template void gemm_t<float, float2>(const float2*, long, int, const float2*, long, int, long, double2*, int, double2*, size_t, cudaStream_t);
 template void gemm_t<float, __nv_bfloat162>(const __nv_bfloat162*, long, int, const float2*, long, int, long, double2*, int, double2*, size_t, cudaStream_t);
 
-template void proj<double, double2>(const double2*, long, int, const double2*, long, int, long, double2*, int, double2*, size_t, cudaStream_t);
 template void proj<float, float2>(const float2*, long, int, const float2*, long, int, long, double2*, int, double2*, size_t, cudaStream_t);
 template void proj<float, __nv_bfloat162>(const __nv_bfloat162*, long, int, const float2*, long, int, long, double2*, int, double2*, size_t, cudaStream_t);
-template size_t proj_scratch_elems<double, double2>(long, int);
 template size_t proj_scratch_elems<float, float2>(long, int);
 template size_t proj_scratch_elems<float, __nv_bfloat162>(long, int);
 
 template void gemm_n<double, double2, double2>(const double2*, long, int, const double2*, int, int, double2*, long, long, double, cudaStream_t);
-template void gemm_n<float, float2, float2>(const float2*, long, int, const double2*, int, int, float2*, long, long, double, cudaStream_t);
 template void gemm_n<float, float2, double2>(const float2*, long, int, const double2*, int, int, double2*, long, long, double, cudaStream_t);
-template void gemm_n<float, __nv_bfloat162, float2>(const __nv_bfloat162*, long, int, const double2*, int, int, float2*, long, long, double, cudaStream_t);
 template void gemm_n<float, __nv_bfloat162, double2>(const __nv_bfloat162*, long, int, const double2*, int, int, double2*, long, long, double, cudaStream_t);
 
 template void convert<double2, double2>(const double2*, double2*, long, cudaStream_t);
 template void convert<float2, double2>(const float2*, double2*, long, cudaStream_t);
-template void convert<double2, float2>(const double2*, float2*, long, cudaStream_t);
 template void convert<__nv_bfloat162, double2>(const __nv_bfloat162*, double2*, long, cudaStream_t);
-template void convert<float2, float2>(const float2*, float2*, long, cudaStream_t);
-template void convert<float2, __nv_bfloat162>(const float2*, __nv_bfloat162*, long, cudaStream_t);
 
 }  // namespace seedcg

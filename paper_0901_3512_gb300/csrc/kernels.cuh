@@ -43,11 +43,6 @@ struct LzDev {
 enum { CTR_B = 0, CTR_D, CTR_PO1, CTR_PO2, CTR_PO3, CTR_PO4, CTR_NORM, CTR_ETA0, CTR_COUNT = 64 };
 
 // ----- generic reductions (blas.cu) -----
-// res[0] = sum conj(a) b over n complex entries (a, b flat internal vectors)
-template <typename R>
-void dot(const cx_t<R>* a, const cx_t<R>* b, long n, double* partials, unsigned* ctr,
-         double2* res, cudaStream_t s);
-
 // C[a][b] = sum_e conj(A[a][e]) B[b][e] for a < na, b < nb (A rows of type AT,
 // B rows of cx_t<R>); C is double2 [na][ldc].  scratch holds the split partials.
 template <typename R, typename AT>

@@ -1109,10 +1109,11 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     const bool seeds_streamed = !fp64 && !(std::is_same<VT, __nv_bfloat162>::value && o.use_tensor_cores);
     // also room for three row segments of the PO subtraction (k_po_sub_seg partials)
     const size_t seg3 = 3 * 2 * (size_t)n * sizeof(cx_t<R>) / sizeof(double2);
-    const size_t split_elems = std::max<size_t>(
-        std::max<size_t>(std::max<size_t>(coef_elems * 48, (size_t)1 << 20), seg3),
-        fp64 ? proj_fix_scratch(n, m_max)
-             : seeds_streamed ? proj_scratch_elems<R, VT>(n, m_max) : proj_scratch_elems<R, VT>(n, m_max) / 2);
+    size_t proj_elems;
+    if constexpr (sizeof(R) == 8) proj_elems = proj_fix_scratch(n, m_max);
+    else proj_elems = proj_scratch_elems<R, VT>(n, m_max) / (seeds_streamed ? 1 : 2);
+    const size_t split_elems =
+        std::max<size_t>({coef_elems * 48, (size_t)1 << 20, seg3, proj_elems});
     h->coef.ensure((coef_elems + split_elems) * sizeof(double2));
     double2* Cc = h->coef.as<double2>();
     double2* split = Cc + coef_elems;
