@@ -61,6 +61,7 @@ __global__ void k_from_internal_f64(const double2* __restrict__ in, double2* __r
 
 __global__ void k_to_internal_f32(const double2* __restrict__ in, float2* __restrict__ out,
                                   int vol, int n) {
+    pdl_enter();
     long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (t >= (long)vol * n) return;
     int r = (int)(t / vol), s = (int)(t % vol);
@@ -100,6 +101,7 @@ __device__ __forceinline__ void put_site(const OutF64& o, int r, int vol, int s,
 template <int DAG, bool PRE, typename Out>
 __global__ void __launch_bounds__(kThreads)
 k_dslash(Geom g, const float2* __restrict__ u, float kappa, const float2* __restrict__ in, Out out) {
+    pdl_enter();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.vol) return;
     const int vol = g.vol;
@@ -136,6 +138,7 @@ constexpr int TS = 32;
 template <int DAG, int RPB, typename Out>
 __global__ void __launch_bounds__(TS * RPB, tile_blocks(RPB))
 k_dslash_mrhs(Geom g, const float2* __restrict__ u, float kappa, int n, const float2* __restrict__ in, Out out) {
+    pdl_enter();
     __shared__ float2 sl[72 * TS];
     __shared__ OffNbr snb[TS];
     __shared__ int sb[4][TS];
@@ -177,9 +180,8 @@ k_dslash_mrhs(Geom g, const float2* __restrict__ u, float kappa, int n, const fl
 template <int RPB, typename Out>
 void mrhs_go(const Geom& g, const float2* u, float kappa, int dag, int n, const float2* in, Out out, cudaStream_t st) {
     const int nb = blocks_for(g.vol, TS);
-    if (dag) k_dslash_mrhs<1, RPB, Out><<<nb, TS * RPB, 0, st>>>(g, u, kappa, n, in, out);
-    else k_dslash_mrhs<0, RPB, Out><<<nb, TS * RPB, 0, st>>>(g, u, kappa, n, in, out);
-    SEEDCG_CHECK_LAUNCH();
+    launch_pdl(pdl_for_apply(12L * g.vol * n), dag ? k_dslash_mrhs<1, RPB, Out> : k_dslash_mrhs<0, RPB, Out>, nb, TS * RPB,
+               0, st, g, u, kappa, n, in, out);
 }
 
 template <bool PRE, typename Out>
@@ -192,9 +194,8 @@ void launch_dslash(const Geom& g, const float2* u, float kappa, int dag, int n, 
         Out o = out;
         if constexpr (std::is_same<Out, OutF64>::value) o.p += 2 * off;
         else o.p += off;
-        if (dag) k_dslash<1, PRE, Out><<<grid, kThreads, 0, s>>>(g, u, kappa, in + off, o);
-        else k_dslash<0, PRE, Out><<<grid, kThreads, 0, s>>>(g, u, kappa, in + off, o);
-        SEEDCG_CHECK_LAUNCH();
+        launch_pdl(pdl_for(12L * g.vol), dag ? k_dslash<1, PRE, Out> : k_dslash<0, PRE, Out>, grid, kThreads, 0, s,
+                   g, u, kappa, in + off, o);
     }
 }
 

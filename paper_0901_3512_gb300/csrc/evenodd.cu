@@ -33,6 +33,7 @@ template <int DAG, typename Out>
 __global__ void __launch_bounds__(EOT * 12, 2)
 k_eo_hop(Geom g, const float2* __restrict__ u, int p_out, int n, const float2* __restrict__ other,
          const float2* __restrict__ same, float c_diag, float c_hop, Out out) {
+    pdl_enter();
     __shared__ float2 sl[2][4][9][EOT];
     __shared__ Nbr snb[EOT];
     __shared__ int ssite[EOT];
@@ -80,9 +81,8 @@ void eo_hop(const Geom& g, const float2* u, int dag, int p_out, int n, const flo
     // tiles alone do not fill two blocks per SM
     const int gy = std::min(n, std::max((n + 11) / 12, (304 + tiles - 1) / tiles));
     const int per = std::min(12, (n + gy - 1) / gy);
-    if (dag) k_eo_hop<1, Out><<<dim3(tiles, gy), EOT * per, 0, st>>>(g, u, p_out, n, other, same, c_diag, c_hop, out);
-    else k_eo_hop<0, Out><<<dim3(tiles, gy), EOT * per, 0, st>>>(g, u, p_out, n, other, same, c_diag, c_hop, out);
-    SEEDCG_CHECK_LAUNCH();
+    launch_pdl(pdl_for_apply(6L * g.vol * n), dag ? k_eo_hop<1, Out> : k_eo_hop<0, Out>, dim3(tiles, gy), EOT * per, 0,
+               st, g, u, p_out, n, other, same, c_diag, c_hop, out);
 }
 
 // y_o = A x_o (dag = 0) or A^dag x_o (dag = 1), n half vectors; t: even-site scratch

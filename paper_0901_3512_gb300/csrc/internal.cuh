@@ -64,6 +64,11 @@ __device__ __forceinline__ void pdl_enter() {
 // takes 37.0 ms without it and 33.4 ms with it, but at 16^3 x 32 the early blocks take slots that the running
 // kernel's own blocks would have used (250.6 against 254.1 ms; even-odd 113.1 against 115.5 ms).
 inline bool pdl_for(long entries) { return entries <= 12L * 49152; }
+// The launches of one FP32 application, `entries` over all of its fields: kernels of 10 to 20 us, of which the launch
+// is still a part: M of twelve fields of 8^3 x 16 (1.2 M entries) 48.2 -> 45.0 us, A^dag A of six half vectors of
+// 12^3 x 24 (1.5 M) 115.5 -> 107.1 us. The line lies next above the sizes measured, far below the 19 M of
+// twelve fields of 16^3 x 32, where a launch is 3 % of a kernel and early blocks cost more.
+inline bool pdl_for_apply(long entries) { return entries <= 12L * 196608; }
 template <typename... P, typename... A>
 void launch_pdl(bool early, void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchAttribute at[1];
