@@ -6,12 +6,10 @@
 // depend on block scheduling, so repeated runs are bitwise identical.
 #pragma once
 
+#include "grids.h"
 #include "internal.cuh"
 
 namespace seedcg {
-
-constexpr int kRedThreads = 256;  // every reducing kernel uses this block size
-constexpr int kMaxRedBlocks = 4096;
 
 // warp sum in the value's own precision (FP32 sums stay off the scarce FP64 pipe)
 template <typename T> __device__ __forceinline__ T warp_sum_t(T v) {

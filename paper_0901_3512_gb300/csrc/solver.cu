@@ -28,29 +28,6 @@ namespace seedcg {
 
 namespace {
 
-inline int red_blocks(long n) {
-    long b = (n + kRedThreads * 4 - 1) / (kRedThreads * 4);
-    if (b < 1) b = 1;
-    return (int)std::min<long>(b, 152 * 8);
-}
-
-// blocks for a kernel whose thread handles one 16-byte group of entries (n / w
-// groups), in equal rounds of at most kMaxRedBlocks blocks
-inline int vec_blocks(long n, int w) {
-    long b = (n / w + kRedThreads - 1) / kRedThreads;
-    if (b < 1) b = 1;
-    const long rounds = (b + kMaxRedBlocks - 1) / kMaxRedBlocks;
-    return (int)((b + rounds - 1) / rounds);
-}
-
-inline int site_blocks(int vol) { return (vol + kRedThreads - 1) / kRedThreads; }
-
-// The single-RHS operator kernels of the Lanczos loop (one thread per site) run in
-// blocks of 128 with at most 72 registers in FP32: 7 blocks per SM then hold a
-// 16^3x32 lattice in one wave, where 256-thread blocks at 77 registers need 1.12
-// waves (16.4 -> 14.6 us for D with the L2 warm)
-constexpr int kSiteThreads = 128;
-inline int site_blocks_lz(int vol) { return (vol + kSiteThreads - 1) / kSiteThreads; }
 // Blocks per SM of the operator kernels, by which the registers and the neighbours in flight go. A lattice that has at
 // most two or three blocks of 128 per SM is bound by the chain of a thread's eight gathers, one L2 latency after the
 // other: four in flight, at up to 255 or 168 registers, make it two long. D + D^dag + update in us, one gather at 72
@@ -385,7 +362,7 @@ void lz_fix(const FixDev& F, const FixOp& op, const double2* w, double2* v, cons
         cudaFuncSetAttribute(k_lz_fix<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
     SEEDCG_CUDA_TRY(attr);
     const int sites = op.parity < 0 ? F.g.vol : F.g.vol / 2;
-    launch_pdl(pdl_for(12L * sites), k_lz_fix<KIND>, (sites + 31) / 32, kFixThreads, kFixSmem, st, F, op, w, v, vprev,
+    launch_pdl(pdl_for(12L * sites), k_lz_fix<KIND>, fix_tiles(sites), kFixThreads, kFixSmem, st, F, op, w, v, vprev,
                Vrow, runE, out, i, L);
 }
 
@@ -1072,11 +1049,16 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     double* bnorm = cs.take<double>(nrhs + 2);
     double* tr_dev = cs.take<double>(nrhs + 2);
     const int rb = red_blocks(n);
-    const size_t part_doubles = (size_t)std::max(kMaxRedBlocks, rb * (nrhs + 2)) * 64;
+    const size_t part_doubles = lz_partial_doubles(n, nrhs, fp64);
     h->red.ensure(part_doubles * sizeof(double) + 8192 * sizeof(unsigned));
     L.partials = h->red.as<double>();
     L.counters = reinterpret_cast<unsigned*>(h->red.as<double>() + part_doubles);
     SEEDCG_CUDA_TRY(cudaMemsetAsync(L.counters, 0, 8192 * sizeof(unsigned), st));
+    // a grid that ends in a reduction writes its partials there and has its counters right behind them
+    auto reducing = [&](long blocks) {
+        if (blocks < 1 || (size_t)blocks > part_doubles) throw Error{SEEDCG_ERR_ARG, "internal: reduction workspace"};
+        return (unsigned)blocks;
+    };
     // V basis and coefficient scratch
     const size_t vrow = (size_t)n * sizeof(VT);
     if (h->vbasis.bytes < vrow * (size_t)m_max) {
@@ -1163,7 +1145,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                                                                           kRedThreads, 0));
     constexpr int kW = 16 / (int)sizeof(VT);
     if (n % 4 != 0) throw Error{SEEDCG_ERR_ARG, "spinor length not a multiple of 4"};
-    const long po_gb = (n / kW + kRedThreads - 1) / kRedThreads;
+    const long po_gb = entry_blocks(n, kW);
     const long seg_cap = (long)(split_elems * sizeof(double2) / (2 * (size_t)n * sizeof(cx_t<R>)));
     auto po_subtract = [&](int na, int cvcol, cx_t<R>* vv, cx_t<R>* ff, int i) {
         long nseg = 1;
@@ -1177,7 +1159,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                            Cc, cvcol, vv, ff, n, sp, i, L);
                 launch_pdl(pdl, k_po_sub_fin<R>, rb, kRedThreads, 0, st, sp, ns, vv, ff, n, i, L);
             } else {
-                launch_pdl(pdl, k_po_sub_fix<false>, dim3((unsigned)po_gb), kRedThreads, 0, st, Vb, n, na, na, runE, Cc,
+                launch_pdl(pdl, k_po_sub_fix<false>, reducing(po_gb), kRedThreads, 0, st, Vb, n, na, na, runE, Cc,
                            cvcol, vv, ff, n, sp, i, L);
             }
             return;
@@ -1253,7 +1235,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     if (beta0 > 0.0) {
         cx_t<R>* vprev = nullptr;
         int i = 1;
-        const int sbh = site_blocks(vol / 2);
+        const int sbh = reducing(site_blocks(vol / 2));
         const int bps = lz_blocks_per_sm(vol);
         const long lean_g = n * (long)sizeof(cx_t<R>) / 16;
         const int lean_t = lean_threads(n, 16 / (int)sizeof(cx_t<R>));
@@ -1268,6 +1250,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
             else slot = slot == vA ? vB : vA;
             const cx_t<R>* w = i == 1 ? R0 : fv;   // v_i = w / ||w||
             if constexpr (sizeof(R) == 8) {
+                reducing(fix_tiles((int)(n / 12)));
                 lz_apply_f64(fix_of(h), eo, w, v, vprev, Vrow, runE, tv, ev, fv, i, L, st);
             } else if (eo) {
                 // f = A^dag A v - beta v_prev, alpha: four half-lattice hops
@@ -1277,7 +1260,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                 launch_pdl(pdl, k_lz_eo<R, VT, 2>, sbh, kRedThreads, 0, st, h->g, U, kk, tv, none, ev, v, none, Vrow, i, L);
                 launch_pdl(pdl, k_lz_eo<R, VT, 3>, sbh, kRedThreads, 0, st, h->g, U, kk, ev, tv, fv, v, vprev, Vrow, i, L);
             } else {
-                const int sbl = site_blocks_lz(vol);
+                const int sbl = reducing(site_blocks_lz(vol));
 #define SEEDCG_LZ(BPS)                                                                                                \
     launch_pdl(pdl, k_lz_D<R, VT, BPS>, sbl, kSiteThreads, 0, st, h->g, U, kap, w, v, Vrow, tv, i, L);                \
     launch_pdl(pdl, k_lz_Ddag<R, BPS>, sbl, kSiteThreads, 0, st, h->g, U, kap, tv, v, vprev, fv, i, L);
