@@ -235,7 +235,7 @@ k_gemm_n_wide(const AT* __restrict__ A, long lda, int na, const double2* __restr
 // ---------------------------------------------------------------------------
 template <typename R, typename VT, int NV, int RPW, int CHUNK>
 __global__ void __launch_bounds__(256, (sizeof(R) == 4 && NV == 2) ? 4 : 1)
-k_proj_partial(const VT* __restrict__ V, long ldv, int na, const cx_t<R>* __restrict__ X,
+k_proj_partial(const VT* V, long ldv, int na, const cx_t<R>* X,
                long ldx, int nv, long n, int chunk, int rg, double2* __restrict__ part) {
     pdl_enter();
     // block (x, y): one chunk of entries (X chunk staged in shared memory)
@@ -302,7 +302,7 @@ k_proj_partial(const VT* __restrict__ V, long ldv, int na, const cx_t<R>* __rest
 // C[a][j] = sum over blocks of part[b][a][j]: one warp per output, lanes stride
 // over the blocks, then a fixed shuffle tree (deterministic)
 template <int NV>
-__global__ void k_proj_reduce(const double2* __restrict__ part, int nblk, int na, int nv,
+__global__ void k_proj_reduce(const double2* part, int nblk, int na, int nv,
                               double2* __restrict__ C, int ldc, int c0) {
     pdl_enter();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;

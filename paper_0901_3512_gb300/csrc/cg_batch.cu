@@ -356,7 +356,7 @@ void mf_fix(int tiles, int gy, cudaStream_t s, const GroupDev<double>* gdev, int
 // each, and the warps' sums are taken on the integer pipe (warp_sum).
 constexpr int kShareThreads = 256, kShareThreadsLong = 1024;
 inline int share_threads(int ntiles) { return ntiles > 4 * kShareThreads ? kShareThreadsLong : kShareThreads; }
-__device__ __forceinline__ double row_shares(const double* __restrict__ sh, int ntiles) {
+__device__ __forceinline__ double row_shares(const double* sh, int ntiles) {
     __shared__ double s_w[kShareThreadsLong / 32];
     const int bd = blockDim.x;
     double v = 0.0;
@@ -497,9 +497,9 @@ k_mf_xp(const GroupDev<R>* __restrict__ G, Rows rows, CgS C) {
     if (f < 0) return;
     const GroupDev<R>& gd = G[f];
     const size_t off = (size_t)rows.local[row] * gd.n;
-    T* __restrict__ x = reinterpret_cast<T*>(gd.xr + off);
-    const T* __restrict__ r = reinterpret_cast<const T*>(gd.r + off);
-    T* __restrict__ p = reinterpret_cast<T*>(gd.p + off);
+    T* x = reinterpret_cast<T*>(gd.xr + off);
+    const T* r = reinterpret_cast<const T*>(gd.r + off);
+    T* p = reinterpret_cast<T*>(gd.p + off);
     const R a = (R)C.alpha[row], b = (R)C.beta[row];
     const long ng = gd.n / W;
     const long st = (long)gridDim.x * blockDim.x;

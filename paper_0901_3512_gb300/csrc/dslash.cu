@@ -59,7 +59,7 @@ __global__ void k_from_internal_f64(const double2* __restrict__ in, double2* __r
     }
 }
 
-__global__ void k_to_internal_f32(const double2* __restrict__ in, float2* __restrict__ out,
+__global__ void k_to_internal_f32(const double2* in, float2* __restrict__ out,
                                   int vol, int n) {
     pdl_enter();
     long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
@@ -100,7 +100,7 @@ __device__ __forceinline__ void put_site(const OutF64& o, int r, int vol, int s,
 // ---------------------------------------------------------------------------
 template <int DAG, bool PRE, typename Out>
 __global__ void __launch_bounds__(kThreads)
-k_dslash(Geom g, const float2* __restrict__ u, float kappa, const float2* __restrict__ in, Out out) {
+k_dslash(Geom g, const float2* __restrict__ u, float kappa, const float2* in, Out out) {
     pdl_enter();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.vol) return;
@@ -137,7 +137,7 @@ constexpr int TS = 32;
 
 template <int DAG, int RPB, typename Out>
 __global__ void __launch_bounds__(TS * RPB, tile_blocks(RPB))
-k_dslash_mrhs(Geom g, const float2* __restrict__ u, float kappa, int n, const float2* __restrict__ in, Out out) {
+k_dslash_mrhs(Geom g, const float2* __restrict__ u, float kappa, int n, const float2* in, Out out) {
     pdl_enter();
     __shared__ float2 sl[72 * TS];
     __shared__ OffNbr snb[TS];
@@ -169,6 +169,7 @@ k_dslash_mrhs(Geom g, const float2* __restrict__ u, float kappa, int n, const fl
     auto bl = [&](int mu, int e) { return sl[(36 + mu * 9 + e) * TS + j]; };
     const size_t plane = (size_t)vol * 16;
     for (int r = q; r < n; r += RPB) {
+        links_stay_shared();
         const char* inr = reinterpret_cast<const char*>(in) + r * (6 * plane);
         Spinor<float> res;
         auto load = [&](unsigned o, Spinor<float>& p) { load_spinor_at(inr, plane, o, p); };

@@ -27,7 +27,7 @@ __device__ __forceinline__ int eo_site(const Geom& g, int h, int p) {
 // the half vector `other` at index >> 1; the antiperiodic sign on hops that wrap t.
 // Fwd(mu, e) / Bwd(mu, e) give element e = 3a+b of U_mu(s) / U_mu(s - mu).
 template <typename R, int DAG, typename Fwd, typename Bwd>
-__device__ __forceinline__ void eo_hops(const Nbr& nb, Fwd fl, Bwd bl, const cx_t<R>* __restrict__ other, int vh,
+__device__ __forceinline__ void eo_hops(const Nbr& nb, Fwd fl, Bwd bl, const cx_t<R>* other, int vh,
                                         R c_hop, Spinor<R>& acc) {
     constexpr int SF = DAG ? 1 : -1;
     constexpr int SB = -SF;
@@ -52,8 +52,8 @@ __device__ __forceinline__ void eo_hops(const Nbr& nb, Fwd fl, Bwd bl, const cx_
 // (same may be null: no diagonal term)
 template <typename R, int DAG>
 __device__ __forceinline__ void eo_site_apply(const Geom& g, const cx_t<R>* __restrict__ u, int p_out, int h,
-                                              const cx_t<R>* __restrict__ other,
-                                              const cx_t<R>* __restrict__ same, R c_diag, R c_hop,
+                                              const cx_t<R>* other,
+                                              const cx_t<R>* same, R c_diag, R c_hop,
                                               Spinor<R>& acc) {
     const int vh = g.vol / 2;
     const int s = eo_site(g, h, p_out);

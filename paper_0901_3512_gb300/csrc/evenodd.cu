@@ -31,8 +31,8 @@ constexpr int EOT = 32;   // half sites per block (a lane each); a warp per fiel
 // field and hop on 12^3 x 24, 41 us for six; here 21 us).
 template <int DAG, typename Out>
 __global__ void __launch_bounds__(EOT * 12, 2)
-k_eo_hop(Geom g, const float2* __restrict__ u, int p_out, int n, const float2* __restrict__ other,
-         const float2* __restrict__ same, float c_diag, float c_hop, Out out) {
+k_eo_hop(Geom g, const float2* __restrict__ u, int p_out, int n, const float2* other,
+         const float2* same, float c_diag, float c_hop, Out out) {
     pdl_enter();
     __shared__ float2 sl[2][4][9][EOT];
     __shared__ Nbr snb[EOT];
@@ -58,6 +58,7 @@ k_eo_hop(Geom g, const float2* __restrict__ u, int p_out, int n, const float2* _
     auto bl = [&](int mu, int e) { return sl[1][mu][e][j]; };
     const size_t hf = (size_t)vh * 12;
     for (int r = blockIdx.y * (blockDim.x / EOT) + threadIdx.x / EOT; r < n; r += gridDim.y * (blockDim.x / EOT)) {
+        links_stay_shared();
         Spinor<float> acc;
         if (same) {
             load_spinor(same + r * hf, vh, h, acc);

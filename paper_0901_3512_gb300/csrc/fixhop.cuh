@@ -135,7 +135,7 @@ static __device__ __noinline__ void fix_slow(const FixDev& F, int dag, int s, co
         } else {
             const double2* q = in.p + (size_t)r * in.field + (size_t)y * in.site;
 #pragma unroll
-            for (int k = 0; k < 12; k++) p.c[k / 3][k % 3] = __ldg(q + (size_t)(k >> 1) * in.pair + (k & 1));
+            for (int k = 0; k < 12; k++) p.c[k / 3][k % 3] = q[(size_t)(k >> 1) * in.pair + (k & 1)];
         }
     };
     if (dag) wilson_site<1, double>(idx, -1, load, fl, bl, F.kappa, acc);
@@ -252,7 +252,7 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
         {
             double2 p[12];   // 0-5: spins 0 and 1; 6-8: spin q0; 9-11: spin q1
             const double2* q = pin + (size_t)r * op.in.field;
-            auto at = [&](int k) { return __ldg(q + (size_t)(k >> 1) * op.in.pair + (k & 1)); };
+            auto at = [&](int k) { return q[(size_t)(k >> 1) * op.in.pair + (k & 1)]; };
 #pragma unroll
             for (int c = 0; c < 6; c++) p[c] = at(c);
 #pragma unroll

@@ -14,8 +14,8 @@ namespace {
 // seed vectors against 634 rows: 5.1 -> 1.6 ms, and their X += V Y 5.7 -> 1.9 ms.
 template <int NV, int RPW, int CHUNK>
 __global__ void __launch_bounds__(256, 2)
-k_proj_fix(const double2* __restrict__ V, long ldv, int na, const int* __restrict__ runE,
-           const double2* __restrict__ X, long ldx, int nv, long n, int chunk, int rg, double2* __restrict__ part) {
+k_proj_fix(const double2* V, long ldv, int na, const int* runE,
+           const double2* X, long ldx, int nv, long n, int chunk, int rg, double2* __restrict__ part) {
     static_assert(RPW * NV * 2 <= 32, "one lane per value");
     pdl_enter();
     __shared__ int4 sx[NV][CHUNK];
@@ -126,7 +126,7 @@ k_proj_fix(const double2* __restrict__ V, long ldv, int na, const int* __restric
 
 // C[a][j] = sum over blocks of part[b][a][j]: one warp per output, fixed order
 template <int NV>
-__global__ void k_proj_fix_reduce(const double2* __restrict__ part, int nblk, int na, int nv, double2* __restrict__ C,
+__global__ void k_proj_fix_reduce(const double2* part, int nblk, int na, int nv, double2* __restrict__ C,
                                   int ldc, int c0) {
     pdl_enter();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;

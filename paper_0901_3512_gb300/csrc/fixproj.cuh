@@ -49,8 +49,8 @@ struct FixColumns {
 
 // av[j] = sum over rows [r0, r1) of V[a][e] coef[a * ldc + col[j]]; every thread of the block (256) calls it
 template <int NB>
-__device__ __forceinline__ void fix_accumulate(const double2* __restrict__ V, long ldv, int r0, int r1,
-                                               const int* __restrict__ runE, const double2* __restrict__ coef, int ldc,
+__device__ __forceinline__ void fix_accumulate(const double2* V, long ldv, int r0, int r1,
+                                               const int* runE, const double2* coef, int ldc,
                                                const int (&col)[NB], long e, bool live, double2 (&av)[NB],
                                                FixColumns<NB>& S) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -55,6 +55,10 @@ extern std::atomic<unsigned long long> g_kernel_launches;
 // one still runs, and pdl_enter, the first statement of every such kernel, waits until that one is complete
 // and visible, then lets the kernel after it come up.  Every kernel launched this way has to call it on every
 // path: one that returned without waiting would let its successor overtake its predecessor.
+// Such a kernel is resident while its predecessor writes, so what it reads is not constant during its life: only links
+// and tables written long before come through __ldg or a __restrict__ pointer (which let the compiler take the
+// read-only path, or move a load above the wait); fields, partials and coefficients are loaded plainly, and
+// __restrict__ stays on outputs that the kernel never reads.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -189,10 +189,10 @@ __device__ __forceinline__ void grid_sum(double (&v)[NV], double* partials, unsi
 // loads of one complex entry from the three storage types, widened to R
 // ---------------------------------------------------------------------------
 template <typename R> __device__ __forceinline__ cx_t<R> ld_cx(const double2* p, size_t i) {
-    double2 z = __ldg(p + i); return mk<R>((R)z.x, (R)z.y);
+    double2 z = p[i]; return mk<R>((R)z.x, (R)z.y);
 }
 template <typename R> __device__ __forceinline__ cx_t<R> ld_cx(const float2* p, size_t i) {
-    float2 z = __ldg(p + i); return mk<R>((R)z.x, (R)z.y);
+    float2 z = p[i]; return mk<R>((R)z.x, (R)z.y);
 }
 template <typename R> __device__ __forceinline__ cx_t<R> ld_cx(const __nv_bfloat162* p, size_t i) {
     float2 z = __bfloat1622float2(p[i]); return mk<R>((R)z.x, (R)z.y);

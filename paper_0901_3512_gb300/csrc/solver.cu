@@ -150,7 +150,7 @@ __device__ __forceinline__ void lz_put_v(const Spinor<R>& w, R inv, cx_t<R>* v, 
 // v_i = w / ||w||, t = D v_i
 template <typename R, typename VT, int BPS>
 __global__ void __launch_bounds__(kSiteThreads, BPS)
-k_lz_D(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict__ w, cx_t<R>* __restrict__ v,
+k_lz_D(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* w, cx_t<R>* __restrict__ v,
        VT* __restrict__ Vrow, cx_t<R>* __restrict__ t, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
@@ -175,8 +175,8 @@ k_lz_D(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict
 // Step 6 scalars (and 3): gamma_{i-1}, delta_i, zeta_i.
 template <typename R, int BPS>
 __global__ void __launch_bounds__(kSiteThreads, BPS)
-k_lz_Ddag(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restrict__ t,
-          const cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ vprev,
+k_lz_Ddag(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* t,
+          const cx_t<R>* v, const cx_t<R>* vprev,
           cx_t<R>* __restrict__ f, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
@@ -220,9 +220,9 @@ k_lz_Ddag(Geom g, const cx_t<R>* __restrict__ u, R kappa, const cx_t<R>* __restr
 //            (the hops of D^dag give A^dag = g5 A g5), with the LU finaliser of k_lz_Ddag.
 template <typename R, typename VT, int STAGE>
 __global__ void __launch_bounds__(kRedThreads)
-k_lz_eo(Geom g, const cx_t<R>* __restrict__ u, R kk, const cx_t<R>* __restrict__ other,
-        const cx_t<R>* __restrict__ same, cx_t<R>* __restrict__ out, cx_t<R>* __restrict__ v,
-        const cx_t<R>* __restrict__ vprev, VT* __restrict__ Vrow, int i, LzDev L) {
+k_lz_eo(Geom g, const cx_t<R>* __restrict__ u, R kk, const cx_t<R>* other,
+        const cx_t<R>* same, cx_t<R>* __restrict__ out, cx_t<R>* v,
+        const cx_t<R>* vprev, VT* __restrict__ Vrow, int i, LzDev L) {
     pdl_enter();
     constexpr int DAG = STAGE >= 2 ? 1 : 0;
     constexpr int POUT = (STAGE & 1) ? 1 : 0;
@@ -327,8 +327,8 @@ struct LzFixEpi {
 
 template <int KIND>
 __global__ void __launch_bounds__(kFixThreads, 2)
-k_lz_fix(FixDev F, FixOp op, const double2* __restrict__ w, double2* __restrict__ v,
-         const double2* __restrict__ vprev, double2* __restrict__ Vrow, int* __restrict__ runE,
+k_lz_fix(FixDev F, FixOp op, const double2* w, double2* v,
+         const double2* vprev, double2* __restrict__ Vrow, int* runE,
          double2* __restrict__ out, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
@@ -386,7 +386,7 @@ void lz_apply_f64(const FixDev& F, bool eo, const double2* w, double2* v, const 
 // j = j0 .. j0+NE-1 (r_0^j at r0 + (j-1) * n).
 template <typename R, int NE>
 __global__ void __launch_bounds__(kRedThreads)
-k_lz_eta(const cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ r0, long n, int j0, int ne,
+k_lz_eta(const cx_t<R>* v, const cx_t<R>* r0, long n, int j0, int ne,
          int i, LzDev L, unsigned* ctr) {
     pdl_enter();
     if (i > L.ctl->m) return;
@@ -425,8 +425,8 @@ k_lz_eta(const cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ r0, long n, 
 // 6-7: w_i = (v_i - beta_{i-1} w_{i-1}) / delta_i, x^1 += zeta_i w_i, x^j += eta^j w_i.
 template <typename R, bool LIT>
 __global__ void __launch_bounds__(kRedThreads)
-k_lz_update(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, cx_t<R>* __restrict__ w,
-            cx_t<R>* __restrict__ X, int nrhs, long n, int i, int final_beta, LzDev L) {
+k_lz_update(const cx_t<R>* v, cx_t<R>* f, cx_t<R>* w,
+            cx_t<R>* X, int nrhs, long n, int i, int final_beta, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
     const R a = (R)L.alpha[i - 1];
@@ -486,8 +486,8 @@ __device__ __forceinline__ bool lz_x_turn(long g, int i) { return ((int)(g >> 7)
 
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
-k_lz_update_v(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, cx_t<R>* __restrict__ w,
-              double2* __restrict__ x1, long n, int i, int final_beta, LzDev L) {
+k_lz_update_v(const cx_t<R>* v, cx_t<R>* f, cx_t<R>* w,
+              double2* x1, long n, int i, int final_beta, LzDev L) {
     pdl_enter();
     constexpr int W = 16 / (int)sizeof(cx_t<R>);
     __shared__ R s_idl;
@@ -603,8 +603,8 @@ k_lz_flush_x(const cx_t<R>* __restrict__ w, double2* __restrict__ x1, long n, Lz
 // shared memory.  Every thread of the block calls it (it synchronises);
 // `live` marks threads that own entries.
 template <typename R, typename VT>
-__device__ __forceinline__ void po_accumulate(const VT* __restrict__ V, long ldv, int r0, int r1,
-                                              const double2* __restrict__ coef, int cv, long e,
+__device__ __forceinline__ void po_accumulate(const VT* V, long ldv, int r0, int r1,
+                                              const double2* coef, int cv, long e,
                                               bool live, cx_t<R> (&av)[VLoad<R, VT>::N],
                                               cx_t<R> (&af)[VLoad<R, VT>::N],
                                               cx_t<R> (*sc)[2]) {
@@ -657,8 +657,8 @@ __device__ __forceinline__ void po_check_nv(const LzDev& L, int i, double nv2) {
 // (n is a multiple of W, host-checked)
 template <typename R, typename VT>
 __global__ void __launch_bounds__(kRedThreads)
-k_po_sub(const VT* __restrict__ V, long ldv, int na, const double2* __restrict__ coef, int cv,
-         cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, long n, int i, LzDev L) {
+k_po_sub(const VT* V, long ldv, int na, const double2* coef, int cv,
+         cx_t<R>* v, cx_t<R>* f, long n, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
     constexpr int W = VLoad<R, VT>::N;
@@ -689,7 +689,7 @@ k_po_sub(const VT* __restrict__ V, long ldv, int na, const double2* __restrict__
 // to part[s][0 / 1][n]; k_po_sub_fin adds the segments in a fixed order.
 template <typename R, typename VT>
 __global__ void __launch_bounds__(kRedThreads)
-k_po_sub_seg(const VT* __restrict__ V, long ldv, int na, int seg, const double2* __restrict__ coef,
+k_po_sub_seg(const VT* V, long ldv, int na, int seg, const double2* coef,
              int cv, long n, cx_t<R>* __restrict__ part, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
@@ -715,8 +715,8 @@ k_po_sub_seg(const VT* __restrict__ V, long ldv, int na, int seg, const double2*
 // part, as k_po_sub_seg.  8^3 x 16, 320 rows on average: 460 us on the FP64 pipe, 190 us here.
 template <bool SEG>
 __global__ void __launch_bounds__(kRedThreads, 2)
-k_po_sub_fix(const double2* __restrict__ V, long ldv, int na, int seg, const int* __restrict__ runE,
-             const double2* __restrict__ coef, int cv, double2* __restrict__ v, double2* __restrict__ f, long n,
+k_po_sub_fix(const double2* V, long ldv, int na, int seg, const int* runE,
+             const double2* coef, int cv, double2* v, double2* f, long n,
              double2* __restrict__ part, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
@@ -747,8 +747,8 @@ k_po_sub_fix(const double2* __restrict__ V, long ldv, int na, int seg, const int
 
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
-k_po_sub_fin(const cx_t<R>* __restrict__ part, int nseg, cx_t<R>* __restrict__ v,
-             cx_t<R>* __restrict__ f, long n, int i, LzDev L) {
+k_po_sub_fin(const cx_t<R>* part, int nseg, cx_t<R>* v,
+             cx_t<R>* f, long n, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
     R acc = 0;
@@ -771,7 +771,7 @@ k_po_sub_fin(const cx_t<R>* __restrict__ part, int nseg, cx_t<R>* __restrict__ v
 // v_i /= ||v_i|| (and its row of V); dvf = v_i^dag f
 template <typename R, typename VT>
 __global__ void __launch_bounds__(kRedThreads)
-k_po_normalise(cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f, VT* __restrict__ Vrow, int* __restrict__ runE,
+k_po_normalise(cx_t<R>* v, const cx_t<R>* f, VT* __restrict__ Vrow, int* runE,
                long n, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
@@ -799,7 +799,7 @@ k_po_normalise(cx_t<R>* __restrict__ v, const cx_t<R>* __restrict__ f, VT* __res
 // f -= (v_i^dag f) v_i; beta_i = ||f||; step 9 bookkeeping
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
-k_po_finish(const cx_t<R>* __restrict__ v, cx_t<R>* __restrict__ f, long n, int i, LzDev L) {
+k_po_finish(const cx_t<R>* v, cx_t<R>* f, long n, int i, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
     const double2 d = L.ctl->dvf;

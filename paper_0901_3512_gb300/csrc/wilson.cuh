@@ -91,12 +91,12 @@ __host__ __device__ __forceinline__ size_t sidx(int k, int s, int vol) {
     return ((size_t)(k >> 1) * (size_t)vol + (size_t)s) * 2 + (size_t)(k & 1);
 }
 
-__device__ __forceinline__ void load_spinor(const float2* __restrict__ p, int vol, int s,
+__device__ __forceinline__ void load_spinor(const float2* p, int vol, int s,
                                             Spinor<float>& out) {
     const float4* q = reinterpret_cast<const float4*>(p) + s;
 #pragma unroll
     for (int c = 0; c < 6; c++) {
-        const float4 z = __ldg(q + (size_t)c * vol);
+        const float4 z = q[(size_t)c * vol];
         out.c[(2 * c) / 3][(2 * c) % 3] = make_float2(z.x, z.y);
         out.c[(2 * c + 1) / 3][(2 * c + 1) % 3] = make_float2(z.z, z.w);
     }
@@ -122,7 +122,7 @@ struct OffNbr {
 __device__ __forceinline__ void load_spinor_at(const char* field, size_t plane, unsigned off, Spinor<float>& out) {
 #pragma unroll
     for (int c = 0; c < 6; c++) {
-        const float4 z = __ldg(reinterpret_cast<const float4*>(field + c * plane + off));
+        const float4 z = *reinterpret_cast<const float4*>(field + c * plane + off);
         out.c[(2 * c) / 3][(2 * c) % 3] = make_float2(z.x, z.y);
         out.c[(2 * c + 1) / 3][(2 * c + 1) % 3] = make_float2(z.z, z.w);
     }
@@ -148,10 +148,10 @@ __device__ __forceinline__ void load_spinor_rw(const double2* p, int vol, int s,
 #pragma unroll
     for (int k = 0; k < 12; k++) out.c[k / 3][k % 3] = p[sidx(k, s, vol)];
 }
-__device__ __forceinline__ void load_spinor(const double2* __restrict__ p, int vol, int s,
+__device__ __forceinline__ void load_spinor(const double2* p, int vol, int s,
                                             Spinor<double>& out) {
 #pragma unroll
-    for (int k = 0; k < 12; k++) out.c[k / 3][k % 3] = __ldg(p + sidx(k, s, vol));
+    for (int k = 0; k < 12; k++) out.c[k / 3][k % 3] = p[sidx(k, s, vol)];
 }
 __device__ __forceinline__ void store_spinor(double2* __restrict__ p, int vol, int s,
                                              const Spinor<double>& v) {
@@ -227,6 +227,10 @@ __device__ __forceinline__ void stage_tile_links(float2* sl, const float2* __res
         sl[row * NS + j] = z;
     }
 }
+
+// First in each round of a tile kernel's loop over fields: the compiler would otherwise read all 72 links before the
+// loop and spill them (632 bytes per thread at 80 registers).
+__device__ __forceinline__ void links_stay_shared() { asm volatile("" ::: "memory"); }
 
 // Blocks per SM of the tile kernels with `rpb` warps: between 24 and 32 warps at 64 to 80 registers.  D + D^dag
 // on 12 fields of 16^3 x 32 in ms: 3 warps x 9 blocks 0.260, 4 x 7 0.262 (x 6 0.278, x 8 0.264, x 9 0.369: spills), 6 x 5
