@@ -345,9 +345,7 @@ k_mf_fix(const GroupDev<double>* __restrict__ G, int ng, Rows rows, CgS C) {
 
 template <int EO, int STAGE>
 void mf_fix(int tiles, int gy, cudaStream_t s, const GroupDev<double>* gdev, int ng, Rows rows, const CgS& C) {
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_mf_fix<EO, STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
-    SEEDCG_CUDA_TRY(attr);
+    allow_smem<k_mf_fix<EO, STAGE>>(kFixSmem);
     launch_pdl(C.pdl, k_mf_fix<EO, STAGE>, dim3(tiles, gy), kFixThreads, kFixSmem, s, gdev, ng, rows, C);
 }
 

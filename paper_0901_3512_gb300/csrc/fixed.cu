@@ -75,9 +75,7 @@ __global__ void __launch_bounds__(kFixThreads, 2) k_fix_apply(FixDev F, FixOp op
 void fix_go(const FixDev& F, const FixOp& op, double2* out, const FixView& layout, int n, cudaStream_t s) {
     if (n <= 0) return;
     const FixStore st{out, layout, (reinterpret_cast<uintptr_t>(out) & 31) == 0};
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_fix_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
-    SEEDCG_CUDA_TRY(attr);
+    allow_smem<k_fix_apply>(kFixSmem);
     const int sites = op.parity < 0 ? F.g.vol : F.g.vol / 2, tiles = (sites + 31) / 32;
     k_fix_apply<<<dim3(tiles, fix_grid_y(tiles, n)), kFixThreads, kFixSmem, s>>>(F, op, st, n);
     SEEDCG_CHECK_LAUNCH();

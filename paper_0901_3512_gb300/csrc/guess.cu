@@ -1058,14 +1058,8 @@ void layer2_tc(seedcg_handle* h, GuessState* G, int mode, const bf2* in, const b
     const Geom& gm = h->g;
     const int blocks = (gm.vol + TC_SITES - 1) / TC_SITES;
     const uint4* img = reinterpret_cast<const uint4*>(G->wimg.as<uint8_t>() + (mode ? 9 * TC_B_BYTES : 0));
-    static bool attr[2] = {false, false};
-    if (!attr[mode]) {
-        if (mode == 0)
-            SEEDCG_CUDA_TRY(cudaFuncSetAttribute(k_g_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
-        else
-            SEEDCG_CUDA_TRY(cudaFuncSetAttribute(k_g_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
-        attr[mode] = true;
-    }
+    if (mode == 0) allow_smem<k_g_tc<0>>(TC_SMEM);
+    else allow_smem<k_g_tc<1>>(TC_SMEM);
     if (mode == 0)
         k_g_tc<0><<<blocks, 256, TC_SMEM, st>>>(gm, h->u32.as<float2>(), in, img, zprev, out0, out1, err);
     else
@@ -1102,9 +1096,7 @@ void forward(seedcg_handle* h, GuessState* G, const Acts& A, const double2* b64,
     k_g_first<<<tiles, 288, 0, st>>>(gm, u, W, A.a0, keep_z ? A.z1 : nullptr, A.h1);
     SEEDCG_CHECK_LAUNCH();
     layer2_tc(h, G, 0, A.h1, nullptr, keep_z ? A.z2 : nullptr, A.h2, A.tc_err, st);
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_g_last, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLastSmem);
-    SEEDCG_CUDA_TRY(attr);
+    allow_smem<k_g_last>(kLastSmem);
     k_g_last<<<tiles, kLastThreads, kLastSmem, st>>>(gm, u, W + GuessState::NW1 + GuessState::NW2, A.h2, A.z3);
     SEEDCG_CHECK_LAUNCH();
 }
@@ -1120,9 +1112,7 @@ void weight_grad(seedcg_handle* h, GuessState* G, const bf2* a, const bf2* dout,
     constexpr int NO = CO * CI * 16;
     const size_t ne = (size_t)9 * NO;
     G->part.ensure((size_t)nslice * 2 * ne * sizeof(float2));
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_g_tw<CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TW_SMEM);
-    SEEDCG_CUDA_TRY(attr);
+    allow_smem<k_g_tw<CI, CO>>(TW_SMEM);
     k_g_tw<CI, CO><<<dim3(nslice, groups), TW_THREADS, TW_SMEM, st>>>(gm, h->u32.as<float2>(), a, dout, G->part.as<float>(), err);
     SEEDCG_CHECK_LAUNCH();
     k_g_reduce_w<<<(int)((ne + 31) / 32), 256, 0, st>>>(G->part.as<float2>(), 2 * nslice, (int)ne, grad);

@@ -21,6 +21,7 @@
 #include <string>
 
 #include "../../include/seedcg.h"
+#include "device_once.h"
 
 namespace seedcg {
 
@@ -49,6 +50,17 @@ extern std::atomic<unsigned long long> g_kernel_launches;
         ::seedcg::g_kernel_launches.fetch_add(1, std::memory_order_relaxed);               \
         SEEDCG_CUDA_TRY(cudaGetLastError());                                               \
     } while (0)
+
+// Dynamic shared memory above 48 KB for a kernel, on the device that is current (the attribute belongs to a device)
+template <auto Kernel>
+inline void allow_smem(size_t bytes) {
+    static DeviceOnce once;
+    int dev = 0;
+    SEEDCG_CUDA_TRY(cudaGetDevice(&dev));
+    once.run(dev, [&]() {
+        SEEDCG_CUDA_TRY(cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    });
+}
 
 // Programmatic dependent launch for the kernels of the iteration loops, which are a few
 // microseconds each: launch_pdl lets the next kernel of the stream be placed on the SMs while the previous

@@ -358,9 +358,7 @@ k_lz_fix(FixDev F, FixOp op, const double2* w, double2* v,
 template <int KIND>
 void lz_fix(const FixDev& F, const FixOp& op, const double2* w, double2* v, const double2* vprev, double2* Vrow,
             int* runE, double2* out, int i, const LzDev& L, cudaStream_t st) {
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_lz_fix<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
-    SEEDCG_CUDA_TRY(attr);
+    allow_smem<k_lz_fix<KIND>>(kFixSmem);
     const int sites = op.parity < 0 ? F.g.vol : F.g.vol / 2;
     launch_pdl(pdl_for(12L * sites), k_lz_fix<KIND>, fix_tiles(sites), kFixThreads, kFixSmem, st, F, op, w, v, vprev,
                Vrow, runE, out, i, L);

@@ -282,10 +282,9 @@ void launch_tc_shape(const CUtensorMap& ma, const CUtensorMap& mb, int rows, lon
     const int nkb = (int)((kelems + BK - 1) / BK);
     const int tiles = (rows + BM - 1) / BM;
     const int groups = (tiles + R - 1) / R;
-    static int occ = 0, nsm = 0;
+    allow_smem<k_tc_proj<NB, R, KC>>(SM::BYTES);
+    static int occ = 0, nsm = 0;   // the same on every GPU that this library's code runs on
     if (!occ) {
-        SEEDCG_CUDA_TRY(cudaFuncSetAttribute(k_tc_proj<NB, R, KC>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::BYTES));
         int dev = 0;
         SEEDCG_CUDA_TRY(cudaGetDevice(&dev));
         SEEDCG_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
