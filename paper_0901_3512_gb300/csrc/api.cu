@@ -2,7 +2,9 @@
 // the dispatch to the solver and the dslash kernels.  No exception crosses
 // the ABI: every entry point converts failures into a seedcg_status and a
 // message kept in the handle.
+#include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -13,7 +15,59 @@ using seedcg::Error;
 
 namespace seedcg {
 std::atomic<unsigned long long> g_kernel_launches{0};
+
+namespace {
+struct Kept {
+    std::mutex mu;
+    std::vector<KeptScratch*> all;
+};
+Kept& kept() {
+    static Kept* k = new Kept;   // outlives every handle
+    return *k;
 }
+}  // namespace
+
+KeptScratch::KeptScratch() {
+    std::lock_guard<std::mutex> lk(kept().mu);
+    kept().all.push_back(this);
+}
+KeptScratch::~KeptScratch() {
+    std::lock_guard<std::mutex> lk(kept().mu);
+    auto& a = kept().all;
+    a.erase(std::find(a.begin(), a.end(), this));
+    buf_.release();
+}
+KeptScratch::Use::Use(KeptScratch& s, size_t bytes) : s_(s) {
+    {
+        std::lock_guard<std::mutex> lk(kept().mu);
+        s_.busy_ = true;
+    }
+    try {
+        s_.buf_.ensure(bytes);
+    } catch (...) {
+        std::lock_guard<std::mutex> lk(kept().mu);
+        s_.busy_ = false;
+        throw;
+    }
+}
+KeptScratch::Use::~Use() {
+    std::lock_guard<std::mutex> lk(kept().mu);
+    s_.busy_ = false;
+    size_t total = 0;
+    for (const KeptScratch* k : kept().all) total += k->buf_.bytes;
+    if (total > kKeptBytes) s_.buf_.release();
+}
+bool give_back_scratch() {
+    std::lock_guard<std::mutex> lk(kept().mu);
+    bool any = false;
+    for (KeptScratch* k : kept().all)
+        if (!k->busy_ && k->buf_.p) {
+            k->buf_.release();
+            any = true;
+        }
+    return any;
+}
+}  // namespace seedcg
 
 namespace {
 
@@ -257,16 +311,15 @@ seedcg_status seedcg_apply(seedcg_handle* h, int op, int prec, int multi, int n,
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     try {
         SEEDCG_CUDA_TRY(cudaSetDevice(h->device));
-        // the operator reads and writes the caller's fields; what lies between is kept in the handle
+        // the operator reads and writes the caller's fields; what lies between is in scratch
         const size_t nf = (size_t)n * h->g.vol * 12;
-        if (prec == 0) {
-            if (op == 2) h->apply.ensure(nf * sizeof(double2));
-            seedcg::apply_spinors_f64(seedcg::fix_of(h), op, n, in, out, h->apply.as<double2>(), st);
-        } else {
-            h->apply.ensure((op == 2 ? 2 : 1) * nf * sizeof(float2));
+        seedcg::KeptScratch::Use work(h->apply, prec == 0 ? (op == 2 ? nf * sizeof(double2) : 0)
+                                                          : (op == 2 ? 2 : 1) * nf * sizeof(float2));
+        if (prec == 0)
+            seedcg::apply_spinors_f64(seedcg::fix_of(h), op, n, in, out, work.as<double2>(), st);
+        else
             seedcg::apply_spinors_f32(h->g, h->u32.as<float2>(), (float)h->kappa, op, multi, false, n, in, out,
-                                      h->apply.as<float2>(), st);
-        }
+                                      work.as<float2>(), st);
         SEEDCG_CUDA_TRY(cudaStreamSynchronize(st));
         return SEEDCG_OK;
     } catch (const Error& e) {
@@ -544,7 +597,6 @@ void seedcg_destroy(seedcg_handle* h) {
     h->tcbuf.release();
     h->cgbuf.release();
     h->hostio.release();
-    h->apply.release();
     seedcg::guess_free(h);
     h->staging.release();
     if (h->pinned) cudaFreeHost(h->pinned);

@@ -106,17 +106,17 @@ bool eo_dims_ok(const Geom& g) {
 
 void apply_eo_f64(seedcg_handle* h, int op, int n, const double* in, double* out, cudaStream_t st) {
     const size_t hf = (size_t)h->g.vol / 2 * 12 * n;
-    h->apply.ensure((op == 2 ? 2 : 1) * hf * sizeof(double2));
-    double2* te = h->apply.as<double2>();
+    KeptScratch::Use work(h->apply, (op == 2 ? 2 : 1) * hf * sizeof(double2));
+    double2* te = work.as<double2>();
     apply_eo_spinors_f64(fix_of(h), op, n, in, out, te, te + hf, st);
     SEEDCG_CUDA_TRY(cudaStreamSynchronize(st));
 }
 
 void apply_eo_f32(seedcg_handle* h, int op, int n, const double* in, double* out, cudaStream_t st) {
     const size_t hf = (size_t)h->g.vol / 2 * 12 * n;
-    h->apply.ensure((op == 2 ? 3 : 2) * hf * sizeof(float2));
+    KeptScratch::Use work(h->apply, (op == 2 ? 3 : 2) * hf * sizeof(float2));
     const float2* u = h->u32.as<float2>();
-    float2* X = h->apply.as<float2>();
+    float2* X = work.as<float2>();
     float2* T = X + hf;
     float2* Y = T + hf;   // op 2 only
     to_internal_f32(in, X, h->g.vol / 2, n, st);

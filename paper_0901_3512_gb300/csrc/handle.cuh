@@ -29,8 +29,7 @@ struct seedcg_handle {
     seedcg::DevBuf tcbuf;         // tensor-core projection: bf16 B operand + FP32 partials
     seedcg::DevBuf cgbuf;         // batched CG engine workspace
     seedcg::DevBuf hostio;        // device copies of host B / X passed to seedcg_solve
-    seedcg::DevBuf apply;         // scratch of the operator applications, kept between calls (each call
-                                  // returns after its work); given up when a solve's basis has to grow
+    seedcg::KeptScratch apply;    // of the operator applications
     std::vector<double> alpha, beta, delta;  // Lanczos scalars of the last solve
     int last_m = 0;
     int last_m_conv = 0, last_po_count = 0, last_lz_status = 0;

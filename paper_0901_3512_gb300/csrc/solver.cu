@@ -1060,7 +1060,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     // V basis and coefficient scratch
     const size_t vrow = (size_t)n * sizeof(VT);
     if (h->vbasis.bytes < vrow * (size_t)m_max) {
-        h->apply.release();   // scratch of earlier operator applications must not stand in a basis's way
+        give_back_scratch();   // scratch that operator applications keep must not stand in a basis's way
         // refuse a basis that cannot fit before allocating it (m_max rows of one vector each)
         size_t free_b = 0, total_b = 0;
         SEEDCG_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));

@@ -1,0 +1,55 @@
+"""Device memory at its limits: what operator applications keep between calls is bounded and is given up when another
+call needs it."""
+import pytest
+
+from paper_0901_3512_gb300 import seedcg, workloads as W
+from tests.gpu_helpers import need_gpu
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+DIMS = (8, 8, 8, 8)
+FIELD = 8 ** 4 * 12 * 16   # bytes of one FP64 field
+
+
+def _solver():
+    return seedcg.Solver(DIMS, W.gauge_field(DIMS, 0.5, 11), 0.2)
+
+
+def _apply_m(s, n):
+    x = torch.ones(n, 8 ** 4, 4, 3, dtype=torch.complex128, device="cuda")
+    y = torch.empty_like(x)
+    s.apply(seedcg.OP_M, x, y, prec=0, multi=1)
+    return x, y
+
+
+def test_large_scratch_is_given_back_when_the_call_returns():
+    need_gpu()
+    s = _solver()
+    _apply_m(s, 1)
+    n = (640 << 20) // FIELD
+    x = torch.ones(n, 8 ** 4, 4, 3, dtype=torch.complex128, device="cuda")
+    y = torch.empty_like(x)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    s.apply(seedcg.OP_M, x, y, prec=0, multi=1)   # an intermediate of 640 MB
+    assert torch.cuda.mem_get_info()[0] >= before - (64 << 20)
+    s.close()
+
+
+def test_kept_scratch_makes_room_for_another_handle():
+    need_gpu()
+    a, b = _solver(), _solver()
+    n = (300 << 20) // FIELD
+    x, y = _apply_m(a, n)                         # a keeps 300 MB
+    _apply_m(b, 1)
+    torch.cuda.empty_cache()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - (150 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        y.zero_()
+        b.apply(seedcg.OP_M, x, y, prec=0, multi=1)   # needs 300 MB of which 150 are free
+        assert y[0].abs().max().item() > 0 and torch.equal(y[0], y[-1])
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+        a.close()
+        b.close()
