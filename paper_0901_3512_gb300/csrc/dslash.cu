@@ -188,9 +188,9 @@ void mrhs_go(const Geom& g, const float2* u, float kappa, int dag, int n, const 
 template <bool PRE, typename Out>
 void launch_dslash(const Geom& g, const float2* u, float kappa, int dag, int n, const float2* in, Out out,
                    cudaStream_t s) {
-    // fields side by side in the grid (at most 65535 per launch)
-    for (int r0 = 0; r0 < n; r0 += 65535) {
-        const dim3 grid(blocks_for(g.vol, kThreads), std::min(n - r0, 65535));
+    // fields side by side in the grid
+    for (int r0 = 0; r0 < n; r0 += kMaxGridY) {
+        const dim3 grid(blocks_for(g.vol, kThreads), std::min(n - r0, kMaxGridY));
         const size_t off = (size_t)r0 * 12 * g.vol;
         Out o = out;
         if constexpr (std::is_same<Out, OutF64>::value) o.p += 2 * off;

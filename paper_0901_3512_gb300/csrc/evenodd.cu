@@ -80,7 +80,7 @@ void eo_hop(const Geom& g, const float2* u, int dag, int p_out, int n, const flo
     const int tiles = (g.vol / 2 + EOT - 1) / EOT;
     // fields side by side: all of them in balanced passes of at most 12 warps, split over the grid while the
     // tiles alone do not fill two blocks per SM
-    const int gy = std::min(n, std::max((n + 11) / 12, (304 + tiles - 1) / tiles));
+    const int gy = std::min({n, kMaxGridY, std::max((n + 11) / 12, (304 + tiles - 1) / tiles)});
     const int per = std::min(12, (n + gy - 1) / gy);
     launch_pdl(pdl_for_apply(6L * g.vol * n), dag ? k_eo_hop<1, Out> : k_eo_hop<0, Out>, dim3(tiles, gy), EOT * per, 0,
                st, g, u, p_out, n, other, same, c_diag, c_hop, out);

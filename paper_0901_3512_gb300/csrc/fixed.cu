@@ -99,8 +99,11 @@ __global__ void k_eo_move(Geom g, int p, int scatter, double2* __restrict__ full
 }
 
 void eo_move(const Geom& g, int p, int scatter, int n, double2* full, double2* half, cudaStream_t st) {
-    k_eo_move<<<dim3((g.vol / 2 + 127) / 128, n), 128, 0, st>>>(g, p, scatter, full, half);
-    SEEDCG_CHECK_LAUNCH();
+    for (int r0 = 0; r0 < n; r0 += kMaxGridY) {
+        const dim3 grid((g.vol / 2 + 127) / 128, std::min(n - r0, kMaxGridY));
+        k_eo_move<<<grid, 128, 0, st>>>(g, p, scatter, full + (size_t)r0 * 12 * g.vol, half + (size_t)r0 * 6 * g.vol);
+        SEEDCG_CHECK_LAUNCH();
+    }
 }
 
 }  // namespace

@@ -43,6 +43,8 @@ struct Error {
         }                                                                                  \
     } while (0)
 
+constexpr int kMaxGridY = 65535;   // the most blocks of a grid in y: fields side by side beyond it take another launch
+
 // every kernel launch site ends with this: it checks the launch and counts it
 extern std::atomic<unsigned long long> g_kernel_launches;
 #define SEEDCG_CHECK_LAUNCH()                                                              \
