@@ -117,20 +117,27 @@ void fix_links(const Geom& g, const double2* u, double kappa, int4* L, int* k, i
     SEEDCG_CHECK_LAUNCH();
     SEEDCG_CUDA_TRY(cudaMemcpyAsync(range, rb.p, sizeof(range), cudaMemcpyDeviceToHost, s));
     SEEDCG_CUDA_TRY(cudaStreamSynchronize(s));
-    // |kappa U| < 2^ex for every component; L = kappa U 2^k stays within 2^55, and the diagonal term's
-    // significand within 2^58 (k <= 57).  Links of very different size would lose relative
-    // accuracy (more than 2^8 apart), as would a scale far from the diagonal's: plain FP64 then.
-    int ex = 0;
-    const bool finite = range[0] < 0x7ff00000u - 1u && std::isfinite(kappa);
-    double mx = 0.0;
-    if (finite) {
-        const unsigned long long bits = (unsigned long long)(range[0] + 1u) << 32;
-        std::memcpy(&mx, &bits, sizeof(mx));
-        if (range[0] == 0) mx = 0.0;
-        frexp(mx * std::fabs(kappa), &ex);
+    // |kappa U| < 2^ex for every component, and L = kappa U 2^k stays within 2^55: the exponents are added, as the
+    // product need not be a normal number.  Plain FP64 takes links of very different size (more than 2^8 apart: the
+    // weak ones would lose relative accuracy), and scales so far from the diagonal term's that one of the two, or the
+    // factor kappa 2^k, could leave the range.
+    *ok = 0;
+    *k = 55;
+    if (range[0] < 0x7ff00000u - 1u && std::isfinite(kappa)) {
+        if (range[0] == 0 || kappa == 0.0) {
+            *ok = 1;
+        } else {
+            const unsigned long long bits = (unsigned long long)(range[0] + 1u) << 32;
+            double mx = 0.0;
+            std::memcpy(&mx, &bits, sizeof(mx));
+            int em = 0, ek = 0, e = 0;
+            const double fm = frexp(mx, &em), fk = frexp(std::fabs(kappa), &ek);
+            frexp(fm * fk, &e);
+            const int ex = em + ek + e;
+            *k = 55 - ex;
+            *ok = ex >= -100 && ex < 16 && std::abs(ek) <= 500 && std::abs(em) <= 500 && range[1] + (8u << 20) >= range[0];
+        }
     }
-    *k = std::min(57, 55 - ex);
-    *ok = finite && ex < 16 && (range[0] == 0 || range[1] + (8u << 20) >= range[0]) ? 1 : 0;
     if (!*ok) *k = 0;
     k_fix_links<<<(int)((36L * g.vol + 255) / 256), 256, 0, s>>>(g, u, *ok ? kappa : 0.0, *k, L);
     SEEDCG_CHECK_LAUNCH();

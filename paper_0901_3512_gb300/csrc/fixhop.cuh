@@ -65,34 +65,39 @@ __device__ __forceinline__ long long fix_sra(long long v, int n) {
     return r;
 }
 
-// S 2^(-1 - k) 2^(E - 1022) rounded to FP64 (S != 0, exponents within range)
-__device__ __forceinline__ double fix_to_double(long long S, int E, int k) {
+// Sums are integers in units of 2^(-1 - kFixUnit) 2^(E - 1022): E is the neighbours' exponent, moved by the links' scale
+// (L = -kappa U 2^k: E + kFixUnit - k), so the unit follows the hop's size whatever kappa is, and every exponent
+// below stays a normal one for k in (39, 155].
+constexpr int kFixUnit = 57;
+
+// S in that unit, rounded to FP64 (S != 0)
+__device__ __forceinline__ double fix_to_double(long long S, int E) {
     const unsigned long long a = S < 0 ? (unsigned long long)(-S) : (unsigned long long)S;
     const int n = __clzll((long long)a);
     const unsigned long long t = a << n;
     const unsigned long long q = (t >> 11) + ((t >> 10) & 1ull);   // 53 bits, rounded half up
-    const long long eb = (long long)(E + 63 - n - k);
+    const long long eb = (long long)(E + 63 - n - kFixUnit);
     const unsigned long long bits = ((unsigned long long)(eb - 1) << 52) + q;
     return __longlong_as_double((long long)(bits | (S < 0 ? 0x8000000000000000ull : 0ull)));
 }
 
 // diag * p + sgn * S, the diagonal term p in FP64 (diag 0 or 1)
-__device__ __forceinline__ double fix_combine(long long S, int E, int k, int diag, double p) {
+__device__ __forceinline__ double fix_combine(long long S, int E, int diag, double p) {
     if (S == 0) return diag ? p : 0.0;
-    if (!diag) return fix_to_double(S, E, k);
+    if (!diag) return fix_to_double(S, E);
     const unsigned h = (unsigned)__double2hiint(p), l = (unsigned)__double2loint(p);
     const int e = (int)((h >> 20) & 0x7ffu);
-    if (e == 0) return fix_to_double(S, E, k);   // zero, or below every step of S
+    if (e == 0) return fix_to_double(S, E);   // zero, or below every step of S
     const int Ec = e > E ? e : E;
     const unsigned long long m = ((unsigned long long)((h & 0x000fffffu) | 0x00100000u) << 32) | l;
-    // p's significand in S's unit: m 2^(2 - (Ec - e)) 2^(k + 1 - 55)
-    const int sh = k - 52 - (Ec - e);
+    // p's significand (below 2^53) in the unit of Ec
+    const int sh = kFixUnit - 52 - (Ec - e);
     unsigned long long P;
     if (sh >= 0) P = m << sh;
     else asm("shr.u64 %0, %1, %2;" : "=l"(P) : "l"(m), "r"(-sh));
     const long long sp = (int)h < 0 ? -(long long)P : (long long)P;
     const long long T = fix_sra(S, Ec - E) + sp;
-    return T == 0 ? 0.0 : fix_to_double(T, Ec, k);
+    return T == 0 ? 0.0 : fix_to_double(T, Ec);
 }
 
 // FP64 fields as the tiles read them: entry k of site y of field r at p[r * field + y * site + (k / 2) * pair + k % 2].
@@ -371,10 +376,11 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
                     x1 = -x1;
                     y1 = -y1;
                 }
-                va.x = fix_combine(x0, Em, F.k, op.diag, pa.x);
-                va.y = fix_combine(y0, Em, F.k, op.diag, pa.y);
-                vb.x = fix_combine(x1, Em, F.k, op.diag, pb.x);
-                vb.y = fix_combine(y1, Em, F.k, op.diag, pb.y);
+                const int Eh = Em + kFixUnit - F.k;
+                va.x = fix_combine(x0, Eh, op.diag, pa.x);
+                va.y = fix_combine(y0, Eh, op.diag, pa.y);
+                vb.x = fix_combine(x1, Eh, op.diag, pb.x);
+                vb.y = fix_combine(y1, Eh, op.diag, pb.y);
             }
             const double part = epi(r, warp, idx, s, live, va, vb);
             if (Epi::kShare) {
