@@ -290,7 +290,7 @@ struct MfFixEpi {
     const double* alpha;  // of this group's slot 0
     double* shares;       // null: none
     long stride;
-    int ntiles, tile, vo;
+    int ntiles, vo;
     __device__ __forceinline__ double operator()(int q, int plane, int idx, int, bool live, double2 a, double2 b) {
         if (!live) return 0.0;
         const size_t ix = (size_t)q * stride + ((size_t)plane * vo + idx) * 2;
@@ -307,7 +307,7 @@ struct MfFixEpi {
         }
         return shares ? a.x * a.x + a.y * a.y + (b.x * b.x + b.y * b.y) : 0.0;
     }
-    __device__ __forceinline__ void put(int q, double v) {
+    __device__ __forceinline__ void put(int q, int tile, double v) {
         if (shares) shares[(size_t)q * ntiles + tile] = v;
     }
 };
@@ -338,8 +338,12 @@ k_mf_fix(const GroupDev<double>* __restrict__ G, int ng, Rows rows, CgS C) {
                  STAGE == 3 ? gd.part2 : (STAGE == 1 || !EO) ? gd.part : nullptr,
                  gd.n,
                  gd.ntiles,
-                 tile,
                  EO ? gd.g.vol / 2 : gd.g.vol};
+    if (!gd.fix.ok) {
+        const int rows_here = min((int)gridDim.y, nsys);
+        fix_plain(gd.fix, op, blockIdx.y * gd.ntiles + tile, rows_here * gd.ntiles, gd.ntiles, nsys, epi);
+        return;
+    }
     fix_tile(gd.fix, op, tile, blockIdx.y, nsys, gridDim.y, fix_smem, epi);
 }
 

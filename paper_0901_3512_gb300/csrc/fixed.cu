@@ -60,7 +60,7 @@ struct FixStore {
         }
         return 0.0;
     }
-    __device__ __forceinline__ void put(int, double) {}
+    __device__ __forceinline__ void put(int, int, double) {}
 };
 
 // At most 128 registers: two blocks per SM.  Instruction issue bounds it: 1270 warp instructions per
@@ -69,6 +69,10 @@ struct FixStore {
 // 12 %; 1037 us from and to the boundary's spinors, where two layout passes took another 303 us.
 __global__ void __launch_bounds__(kFixThreads, 2) k_fix_apply(FixDev F, FixOp op, FixStore st, int n) {
     extern __shared__ __align__(16) unsigned char fix_smem[];
+    if (!F.ok) {
+        fix_plain(F, op, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y, gridDim.x, n, st);
+        return;
+    }
     fix_tile(F, op, blockIdx.x, blockIdx.y, n, gridDim.y, fix_smem, st);
 }
 

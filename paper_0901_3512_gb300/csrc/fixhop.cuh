@@ -22,8 +22,8 @@
 // field at 8^3 x 16 in the Lanczos loop 31 -> 8.2 us, at 4^4 31 -> 5.5 us.
 //
 // Sites whose neighbourhood holds values that the fixed point cannot take (infinities, NaN,
-// magnitudes beyond 2^+-800) and handles whose links differ in size by more than 2^8
-// (ok = 0; never SU(3) links) are computed by fix_slow: the plain FP64 chain.
+// magnitudes beyond 2^+-800) are computed by the plain FP64 chain (fix_chain), and so is every site of a handle whose
+// links differ in size by more than 2^8 (ok = 0; never SU(3) links): there a warp takes 32 sites of one field (fix_plain).
 #pragma once
 
 #include "eo.cuh"
@@ -115,10 +115,8 @@ inline FixView fix_spinors(const double2* p, const Geom& g, int half) {
     return FixView{p, 12L * (g.vol >> half), 12, 2, half};
 }
 
-// The two complex entries of pair-plane `plane` of -kappa H psi (dag: of D^dag's hopping term) at full
-// site s, by the plain FP64 chain; psi: field r of `in`.
-static __device__ __noinline__ void fix_slow(const FixDev& F, int dag, int s, const FixView& in, int r, int plane,
-                                             double2* a, double2* b) {
+// -kappa H psi (dag: of D^dag's hopping term) at full site s, by the plain FP64 chain; psi: field r of `in`
+static __device__ __noinline__ void fix_chain(const FixDev& F, int dag, int s, const FixView& in, int r, double2* out) {
     const Geom& g = F.g;
     const Nbr nb = neighbours(g, s);
     const int vol = g.vol, sh = in.half;
@@ -146,11 +144,7 @@ static __device__ __noinline__ void fix_slow(const FixDev& F, int dag, int s, co
     if (dag) wilson_site<1, double>(idx, -1, load, fl, bl, F.kappa, acc);
     else wilson_site<0, double>(idx, -1, load, fl, bl, F.kappa, acc);
 #pragma unroll
-    for (int k = 0; k < 6; k++)
-        if (k == plane) {
-            *a = acc.c[(2 * k) / 3][(2 * k) % 3];
-            *b = acc.c[(2 * k + 1) / 3][(2 * k + 1) % 3];
-        }
+    for (int k = 0; k < 12; k++) out[k] = acc.c[k / 3][k % 3];
 }
 
 // What one call computes at every site of a tile: val = diag * same(site) + hsgn * (-kappa H in)(site).
@@ -203,7 +197,7 @@ __device__ __forceinline__ void fix_gather(const long long* R, const int (&D)[8]
 
 // One tile of 32 sites, right-hand sides r0, r0 + rstep, ... < nr.  Every thread of the block (256) calls
 // it.  epi(r, plane, idx, live, a, b) receives the two finished entries of pair-plane `plane` at tile
-// index idx and returns this thread's share of a sum; with Epi::kShare, epi.put(r, total) follows (one thread).
+// index idx and returns this thread's share of a sum; with Epi::kShare, epi.put(r, tile, total) follows (one thread).
 template <class Epi>
 __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int tile, int r0, int nr, int rstep,
                                          unsigned char* smem, Epi& epi) {
@@ -270,7 +264,7 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
             for (int c = 0; c < 12; c++)
                 mx = max(mx, max(__double2hiint(p[c].x) & 0x7fffffff, __double2hiint(p[c].y) & 0x7fffffff));
             int E = mx >> 20;
-            if ((mx != 0 && (E < kFixEMin || E > kFixEMax)) || !F.ok) E = kFixBad;
+            if (mx != 0 && (E < kFixEMin || E > kFixEMax)) E = kFixBad;
             sE[warp * 32 + lane] = E;
             // an all-zero spinor (E = 0) still needs an exponent that shifts its components out
             const int eb = (E == kFixBad || E == 0 ? kFixEMax : E) << 20;
@@ -321,7 +315,7 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
         __syncthreads();
         if (Epi::kShare && rprev >= 0 && threadIdx.x == 6 * 32) {
             const double* sh = s_share + (buf ^ 1) * 8;
-            epi.put(rprev, ((sh[0] + sh[1]) + (sh[2] + sh[3])) + (sh[4] + sh[5]));
+            epi.put(rprev, tile, ((sh[0] + sh[1]) + (sh[2] + sh[3])) + (sh[4] + sh[5]));
         }
         rprev = r;
         if (warp < 6) {
@@ -348,7 +342,10 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
                 return h != 0 && ((h >> 20) < kFixEMin || (h >> 20) > kFixEMax);
             };
             if (bad || (op.diag && (far(pa.x) || far(pa.y) || far(pb.x) || far(pb.y)))) {
-                fix_slow(F, op.dag, s, op.in, r, warp, &va, &vb);
+                double2 c[12];
+                fix_chain(F, op.dag, s, op.in, r, c);
+                va = c[2 * warp];
+                vb = c[2 * warp + 1];
                 const double hs = (double)op.hsgn;
                 va = make_double2(pa.x + hs * va.x, pa.y + hs * va.y);
                 vb = make_double2(pb.x + hs * vb.x, pb.y + hs * vb.y);
@@ -393,7 +390,47 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
         __syncthreads();
         if (threadIdx.x == 6 * 32) {
             const double* sh = s_share + (buf ^ 1) * 8;
-            epi.put(rprev, ((sh[0] + sh[1]) + (sh[2] + sh[3])) + (sh[4] + sh[5]));
+            epi.put(rprev, tile, ((sh[0] + sh[1]) + (sh[2] + sh[3])) + (sh[4] + sh[5]));
+        }
+    }
+}
+
+// The same for links out of the fixed point's range: block `block` of the `nblocks` that share ntiles tiles and nr fields.
+// A warp takes a tile of one field at a time and no barrier, so the chain is formed once per site and bounded by the
+// FP64 pipe; with few fields the first blocks do all of it, eight warps each.  Every thread of the block calls it.
+// D on 12 fields of 16^3 x 32: 14.6 ms when the gathering warps each formed the chain, 2.5 ms here.
+template <class Epi>
+__device__ __forceinline__ void fix_plain(const FixDev& F, const FixOp& op, int block, int nblocks, int ntiles, int nr,
+                                          Epi& epi) {
+    const Geom& g = F.g;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nsite = op.parity < 0 ? g.vol : g.vol / 2;
+    __syncthreads();   // what the block has put into shared memory for the epilogue
+    for (long p = block * 8L + warp; p < (long)ntiles * nr; p += nblocks * 8L) {
+        const int tile = (int)(p % ntiles), r = (int)(p / ntiles);
+        int idx = tile * 32 + lane;
+        const bool live = idx < nsite;
+        if (!live) idx = nsite - 1;
+        const int s = op.parity < 0 ? idx : eo_site(g, idx, op.parity);
+        double2 c[12];
+        fix_chain(F, op.dag, s, op.in, r, c);
+        const double hs = (double)op.hsgn;
+        const double2* q = op.same.p + (size_t)r * op.same.field + (size_t)(op.same.half ? idx : s) * op.same.site;
+        double part = 0.0;
+#pragma unroll 1
+        for (int plane = 0; plane < 6; plane++) {
+            double2 v[2];
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                const double2 z = c[2 * plane + k];
+                const double2 d = op.diag ? q[(size_t)plane * op.same.pair + k] : make_double2(0.0, 0.0);
+                v[k] = make_double2(d.x + hs * z.x, d.y + hs * z.y);
+            }
+            part += epi(r, plane, idx, s, live, v[0], v[1]);
+        }
+        if (Epi::kShare) {
+            const double t = warp_sum(part);
+            if (lane == 0) epi.put(r, tile, t);
         }
     }
 }

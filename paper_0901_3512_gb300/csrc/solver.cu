@@ -322,7 +322,7 @@ struct LzFixEpi {
         }
         return 0.0;
     }
-    __device__ __forceinline__ void put(int, double) {}
+    __device__ __forceinline__ void put(int, int, double) {}
 };
 
 template <int KIND>
@@ -347,7 +347,8 @@ k_lz_fix(FixDev F, FixOp op, const double2* w, double2* v,
                        KIND == LZ_LAST && i > 1 ? L.beta[i - 2] : 0.0,
                        op.parity < 0 ? F.g.vol : F.g.vol / 2,
                        0.0};
-    fix_tile(F, op, blockIdx.x, 0, 1, 1, fix_smem, epi);
+    if (F.ok) fix_tile(F, op, blockIdx.x, 0, 1, 1, fix_smem, epi);
+    else fix_plain(F, op, blockIdx.x, gridDim.x, gridDim.x, 1, epi);
     if (KIND == LZ_LAST) {
         double red[1] = {epi.part};
         grid_sum<1>(red, L.partials, L.counters + CTR_B, [&](double* pre) { lz_alpha_pre(L, i, pre); },
