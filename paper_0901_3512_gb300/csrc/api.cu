@@ -167,10 +167,23 @@ seedcg_status seedcg_create(seedcg_handle** out, const int dims[4], const double
             src = tmp.as<double>();
         }
         seedcg::gauge_to_internal(src, h->u64.as<double2>(), h->u32.as<float2>(), (int)vol, 0);
-        h->fix.ensure(nl * sizeof(int4));
-        seedcg::fix_links(h->g, h->u64.as<double2>(), kappa, h->fix.as<int4>(), &h->fix_k, &h->fix_ok, 0);
+        seedcg::fix_scale(h->g, h->u64.as<double2>(), kappa, &h->fix_k, &h->fix_ok, 0);
         SEEDCG_CUDA_TRY(cudaDeviceSynchronize());
         tmp.release();
+        if (h->fix_ok) {
+            // 576 bytes a site beside the 864 of the other links: a lattice that leaves no room for them
+            // keeps the plain FP64 operator
+            try {
+                h->fix.ensure(nl * sizeof(int4));
+            } catch (const Error& e) {
+                if (e.code != SEEDCG_ERR_OOM) throw;
+                h->fix_ok = 0;
+            }
+        }
+        if (h->fix_ok) {
+            seedcg::fix_links(h->g, h->u64.as<double2>(), kappa, h->fix_k, h->fix.as<int4>(), 0);
+            SEEDCG_CUDA_TRY(cudaDeviceSynchronize());
+        }
     } catch (const Error& e) {
         g_create_error = e.msg;
         seedcg_destroy(h);

@@ -112,7 +112,7 @@ void eo_move(const Geom& g, int p, int scatter, int n, double2* full, double2* h
 
 }  // namespace
 
-void fix_links(const Geom& g, const double2* u, double kappa, int4* L, int* k, int* ok, cudaStream_t s) {
+void fix_scale(const Geom& g, const double2* u, double kappa, int* k, int* ok, cudaStream_t s) {
     DevBuf rb;
     rb.ensure(2 * sizeof(unsigned));
     unsigned range[2] = {0u, 0x7fffffffu};
@@ -142,8 +142,10 @@ void fix_links(const Geom& g, const double2* u, double kappa, int4* L, int* k, i
             *ok = ex >= -100 && ex < 16 && std::abs(ek) <= 500 && std::abs(em) <= 500 && range[1] + (8u << 20) >= range[0];
         }
     }
-    if (!*ok) *k = 0;
-    k_fix_links<<<(int)((36L * g.vol + 255) / 256), 256, 0, s>>>(g, u, *ok ? kappa : 0.0, *k, L);
+}
+
+void fix_links(const Geom& g, const double2* u, double kappa, int k, int4* L, cudaStream_t s) {
+    k_fix_links<<<(int)((36L * g.vol + 255) / 256), 256, 0, s>>>(g, u, kappa, k, L);
     SEEDCG_CHECK_LAUNCH();
 }
 

@@ -15,7 +15,7 @@ struct seedcg_handle {
     int device = 0;
     seedcg::DevBuf u64, u32;      // links [4][9][V] double2 / float2
     seedcg::DevBuf fix;           // links in fixed point [4][9][V] int4 (the FP64 operator)
-    int fix_k = 0, fix_ok = 0;    // their scale, and whether every link fits it
+    int fix_k = 0, fix_ok = 0;    // their scale, and whether they are there: every link fits it, and memory had room
     // workspaces
     seedcg::DevBuf vbasis;        // stored Krylov basis V, m_cap rows
     int vbasis_prec = -1;         // precision mode V was written in

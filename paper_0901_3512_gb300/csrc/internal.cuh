@@ -159,7 +159,7 @@ inline Geom make_geom(const int dims[4]) {
 
 // One gauge field for the FP64 operator (fixhop.cuh): the links in fixed point,
 // L = -kappa U 2^k with the antiperiodic sign, [4][9][V] (re hi, re lo, im hi, im lo),
-// and the FP64 links for what the fixed point cannot take (ok = 0: for every site).
+// and the FP64 links for what the fixed point cannot take (ok = 0: for every site; there is no L then).
 struct FixDev {
     Geom g;
     const int4* L;
@@ -281,8 +281,9 @@ void apply_spinors_f64(const FixDev& F, int op, int n, const double* in, double*
 // A, A^dag or A^dag A on complex128 half fields (te: n half vectors of scratch; tmp: n more, op 2 only)
 void apply_eo_spinors_f64(const FixDev& F, int op, int n, const double* in, double* out, double2* te, double2* tmp,
                           cudaStream_t s);
-// the links of a handle in fixed point: L from u, and the scale k and range flag ok (synchronises)
-void fix_links(const Geom& g, const double2* u, double kappa, int4* L, int* k, int* ok, cudaStream_t s);
+// the scale k of a handle's links in fixed point, and whether they fit it (synchronises); the links themselves
+void fix_scale(const Geom& g, const double2* u, double kappa, int* k, int* ok, cudaStream_t s);
+void fix_links(const Geom& g, const double2* u, double kappa, int k, int4* L, cudaStream_t s);
 
 // even-odd preconditioned system (fixed.cu), FP64 half vectors in the internal layout:
 // out_r = A x_r (dag = 0) or A^dag x_r, A = 1 - kappa^2 H_oe H_eo, n fields (te: n even half

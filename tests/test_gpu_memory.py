@@ -53,3 +53,28 @@ def test_kept_scratch_makes_room_for_another_handle():
         torch.cuda.empty_cache()
         a.close()
         b.close()
+
+
+def test_create_without_room_for_the_fixed_point_links():
+    """Room for the FP64 and FP32 links (864 bytes a site) but not for the 576 of the fixed point: the handle works, in
+    plain FP64.  Bar: a site's sum has 73 terms, each rounded a few times at 2^-53 of the largest."""
+    need_gpu()
+    dims, vol = (16, 16, 16, 32), 16 ** 3 * 32
+    u = torch.from_numpy(W.gauge_field(dims, 0.5, 12)).cuda()
+    x = torch.view_as_complex(torch.randn(1, vol, 4, 3, 2, dtype=torch.float64, device="cuda"))
+    y, z = torch.empty_like(x), torch.empty_like(x)
+    roomy = seedcg.Solver(dims, u, 0.2)
+    roomy.apply(seedcg.OP_D, x, y, prec=0, multi=1)
+    roomy.close()
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - 864 * vol - (30 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        tight = seedcg.Solver(dims, u, 0.2)
+        tight.apply(seedcg.OP_D, x, z, prec=0, multi=1)
+        assert float((y - z).abs().max()) <= 64 * 2.0 ** -52 * (1 + 8 * 0.2) * float(x.abs().max())
+        assert not torch.equal(y, z)     # another path
+        tight.close()
+    finally:
+        del hog
+        torch.cuda.empty_cache()
