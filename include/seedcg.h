@@ -134,8 +134,9 @@ void seedcg_default_options(seedcg_options* opt);
  * gauge: host or device, complex128 [V][4][3][3]; copied, the caller keeps
  * ownership.  kappa: hopping parameter.  opt may be NULL (defaults).
  * The handle holds the links three times, in FP64, FP32 and (for the FP64 operator) fixed
- * point: 1440 bytes per site.  Where device memory has no room for the last 576, or the links
- * differ in size by more than 2^8, the FP64 operator runs in plain FP64, 2.4 times as long.
+ * point: 1440 bytes per site.  Where device memory has no room for the last 576, or the
+ * links' largest components differ by more than a factor 2.5 (those of SU(3) links never
+ * do), the FP64 operator runs in plain FP64 and takes 2.4 times as long.
  * Returns SEEDCG_ERR_ARG for bad dims/pointers, SEEDCG_ERR_OOM/CUDA on
  * device failures; *h is NULL on failure.
  */

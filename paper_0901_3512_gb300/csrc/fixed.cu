@@ -122,24 +122,27 @@ void fix_scale(const Geom& g, const double2* u, double kappa, int* k, int* ok, c
     SEEDCG_CUDA_TRY(cudaMemcpyAsync(range, rb.p, sizeof(range), cudaMemcpyDeviceToHost, s));
     SEEDCG_CUDA_TRY(cudaStreamSynchronize(s));
     // |kappa U| < 2^ex for every component, and L = kappa U 2^k stays within 2^55: the exponents are added, as the
-    // product need not be a normal number.  Plain FP64 takes links of very different size (more than 2^8 apart: the
-    // weak ones would lose relative accuracy), and scales so far from the diagonal term's that one of the two, or the
-    // factor kappa 2^k, could leave the range.
+    // product need not be a normal number.  Plain FP64 takes links whose largest components are more than 2.5 apart
+    // (those of SU(3) links lie between 0.408 = 1 / sqrt(6) and 1): a link is held to 2^-56 of the largest, and next to
+    // a point source a hop over links of 1, 1/2, 1/4 of it has an error of 0.88, 1.33, 2.40 times 2^-53 against the
+    // chain's 1.06.  It also takes scales so far from the diagonal term's that one of the two, or the factor
+    // kappa 2^k, could leave the range.
     *ok = 0;
     *k = 55;
     if (range[0] < 0x7ff00000u - 1u && std::isfinite(kappa)) {
         if (range[0] == 0 || kappa == 0.0) {
             *ok = 1;
         } else {
-            const unsigned long long bits = (unsigned long long)(range[0] + 1u) << 32;
-            double mx = 0.0;
-            std::memcpy(&mx, &bits, sizeof(mx));
+            const unsigned long long bits[2] = {(unsigned long long)(range[0] + 1u) << 32, (unsigned long long)range[1] << 32};
+            double mx = 0.0, mn = 0.0;
+            std::memcpy(&mx, &bits[0], sizeof(mx));
+            std::memcpy(&mn, &bits[1], sizeof(mn));
             int em = 0, ek = 0, e = 0;
             const double fm = frexp(mx, &em), fk = frexp(std::fabs(kappa), &ek);
             frexp(fm * fk, &e);
             const int ex = em + ek + e;
             *k = 55 - ex;
-            *ok = ex >= -100 && ex < 16 && std::abs(ek) <= 500 && std::abs(em) <= 500 && range[1] + (8u << 20) >= range[0];
+            *ok = ex >= -100 && ex < 16 && std::abs(ek) <= 500 && std::abs(em) <= 500 && mx <= 2.5 * mn;
         }
     }
 }

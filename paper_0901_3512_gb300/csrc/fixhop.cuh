@@ -23,7 +23,7 @@
 //
 // Sites whose neighbourhood holds values that the fixed point cannot take (infinities, NaN,
 // magnitudes beyond 2^+-800) are computed by the plain FP64 chain (fix_chain), and so is every site of a handle whose
-// links differ in size by more than 2^8 (ok = 0; never SU(3) links): there a warp takes 32 sites of one field (fix_plain).
+// links differ in size by more than 2.5 (ok = 0; never SU(3) links): there a warp takes 32 sites of one field (fix_plain).
 #pragma once
 
 #include "eo.cuh"
