@@ -623,7 +623,6 @@ void launch_mf(int rpb, int dag, int tiles, cudaStream_t s, const GroupDev<float
     else if (rpb == 12) { SEEDCG_MF(12) }
     else { SEEDCG_MF(8) }
 #undef SEEDCG_MF
-    SEEDCG_CHECK_LAUNCH();
 }
 
 void launch_mf_eo(int rpb, int stage, int tiles, cudaStream_t s, const GroupDev<float>* gdev, int ng, Rows rows,
@@ -641,7 +640,6 @@ void launch_mf_eo(int rpb, int stage, int tiles, cudaStream_t s, const GroupDev<
     else if (rpb == 12) { SEEDCG_MFE(12) }
     else { SEEDCG_MFE(8) }
 #undef SEEDCG_MFE
-    SEEDCG_CHECK_LAUNCH();
 }
 
 // Launch shape of the operator, chosen by the autotuner: warps per tile of TS sites (FP32), or the grid rows of
