@@ -36,6 +36,21 @@ __device__ __forceinline__ float narrow(double x) {
     const unsigned r = (unsigned)((v + 0x0fffffffull + ((v >> 29) & 1u)) >> 29);
     return __uint_as_float((u == 0 ? 0u : r) | ((unsigned)((unsigned long long)b >> 32) & 0x80000000u));
 }
+// 1 / x rounded once: FP32 in two floats (x = h + l), as an FP64 division by every thread holds its pipe for 1 us per
+// block.  Far from 1 the scaling of l would leave FP32's range: the FP64 division.
+template <typename R> __device__ __forceinline__ R inverse(double x) {
+    if constexpr (sizeof(R) == 8) {
+        return 1.0 / x;
+    } else {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+        const unsigned e = (unsigned)(b >> 52);
+        if (e - 960u >= 128u) return (float)(1.0 / x);   // also negative, infinite or NaN
+        const float h = __uint_as_float((unsigned)((b - (896ull << 52)) >> 29));
+        const float l = (float)(unsigned)(b & 0x1fffffffu) * __uint_as_float((e - 948u) << 23);
+        const float r = 1.f / h;
+        return fmaf(r, fmaf(-l, r, fmaf(-h, r, 1.f)), r);
+    }
+}
 template <typename R> __device__ __forceinline__ R to_real(double x) {
     if constexpr (sizeof(R) == 4) return narrow(x);
     else return x;

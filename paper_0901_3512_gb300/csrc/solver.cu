@@ -120,12 +120,22 @@ __device__ __forceinline__ void lz_alpha_fin(const LzDev& L, int i, double a, co
     }
 }
 
-// Steps 2 and 9, folded into the operator's first kernel: v_i = w / ||w|| with w = f of the last iteration
-// (||w|| = beta_{i-1}) or r_0^1 (beta_0).  The kernel applies D to w and scales the result, and every thread
-// forms its own entries of v_i and stores them as vector and as row of V (a PO step rewrites both).
+// v_1 = r_0^1 / beta_0 (step 2); beta_0 already in ctl
+template <typename R>
+__global__ void k_lz_start(const cx_t<R>* __restrict__ r0, cx_t<R>* __restrict__ w, long n, LzDev L) {
+    const double inv = 1.0 / L.ctl->beta0;
+    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n; e += (long)gridDim.x * blockDim.x) {
+        const cx_t<R> z = r0[e];
+        w[e] = mk<R>((R)(z.x * inv), (R)(z.y * inv));
+    }
+}
+
+// Step 9, folded into the operator's first kernel: v_i = w / ||w|| with w = f of the last iteration
+// (||w|| = beta_{i-1}); in the first iteration w is v_1.  The kernel applies D to w and scales the result, and every
+// thread forms its own entries of v_i and stores them as vector and as row of V (a PO step rewrites both).
 template <typename R>
 __device__ __forceinline__ R lz_inv(const LzDev& L, int i) {
-    return R(1) / (R)(i == 1 ? L.ctl->beta0 : L.beta[i - 2]);
+    return i == 1 ? R(1) : inverse<R>(L.beta[i - 2]);
 }
 
 // A row of V that holds v_i in the vector's own type is v_i: the vector apart from it exists only in the iterations
@@ -1232,6 +1242,8 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> po_ev;
     int m = 0, m_conv = 0, po_count = 0, lz_status = SEEDCG_OK, breakdown = 0;
     if (beta0 > 0.0) {
+        k_lz_start<R><<<rb, kRedThreads, 0, st>>>(R0, fv, n, L);
+        SEEDCG_CHECK_LAUNCH();
         cx_t<R>* vprev = nullptr;
         int i = 1;
         const int sbh = reducing(site_blocks(vol / 2));
@@ -1247,7 +1259,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
             cx_t<R>* v = slot;
             if (sizeof(VT) == sizeof(cx_t<R>) && !po_now) v = reinterpret_cast<cx_t<R>*>(Vrow);   // lz_own_v
             else slot = slot == vA ? vB : vA;
-            const cx_t<R>* w = i == 1 ? R0 : fv;   // v_i = w / ||w||
+            const cx_t<R>* w = fv;   // v_i = w / ||w||
             if constexpr (sizeof(R) == 8) {
                 reducing(fix_tiles((int)(n / 12)));
                 lz_apply_f64(fix_of(h), eo, w, v, vprev, Vrow, runE, tv, ev, fv, i, L, st);
