@@ -146,13 +146,15 @@ __device__ __forceinline__ void fix_accumulate(const double2* V, long ldv, int r
 #pragma unroll
         for (int q = 0; q < 2; q++) {
             const int k = 2 * j + q;
-            // 96 bits: the upper word is the sign unless thousands of rows add up
+            // 96 bits: the upper word is the sign until products of one sign near the largest fill 64 bits (about 128 rows
+            // of them); then as many bits are dropped as the upper word takes, which leaves at least 62
             const bool fits = hi[k] == (int)(lo[k] >> 63);
-            const long long t = fits ? lo[k] : (long long)(((unsigned long long)(unsigned)hi[k] << 32) | ((unsigned long long)lo[k] >> 32));
+            const int drop = fits ? 0 : 33 - __clz(hi[k] ^ (hi[k] >> 31));
+            const long long t = fits ? lo[k] : (long long)(((unsigned long long)(long long)hi[k] << (64 - drop)) | ((unsigned long long)lo[k] >> drop));
             const int ec = S.ebits[j] >> 20;
             // unit of hi x hi: 2^(54 - 2 * 1077 + Ev + Ec)
             v[q] = bad || ec > kFixEMax ? __longlong_as_double(0x7ff8000000000000ll)
-                                        : ldexp((double)t, Ev + ec - 2100 + (fits ? 0 : 32));
+                                        : ldexp((double)t, Ev + ec - 2100 + drop);
         }
         av[j] = make_double2(v[0], v[1]);
     }
