@@ -195,7 +195,7 @@ void launch_dslash(const Geom& g, const float2* u, float kappa, int dag, int n, 
         Out o = out;
         if constexpr (std::is_same<Out, OutF64>::value) o.p += 2 * off;
         else o.p += off;
-        launch_pdl(pdl_for(12L * g.vol), dag ? k_dslash<1, PRE, Out> : k_dslash<0, PRE, Out>, grid, kThreads, 0, s,
+        launch_pdl(pdl_for_apply(12L * g.vol * (int)grid.y), dag ? k_dslash<1, PRE, Out> : k_dslash<0, PRE, Out>, grid, kThreads, 0, s,
                    g, u, kappa, in + off, o);
     }
 }

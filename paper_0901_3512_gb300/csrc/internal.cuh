@@ -82,11 +82,13 @@ __device__ __forceinline__ void pdl_enter() {
 // takes 37.0 ms without it and 33.4 ms with it, but at 16^3 x 32 the early blocks take slots that the running
 // kernel's own blocks would have used (250.6 against 254.1 ms; even-odd 113.1 against 115.5 ms).
 inline bool pdl_for(long entries) { return entries <= 12L * 49152; }
-// The launches of one FP32 application, `entries` over all of its fields: kernels of 10 to 20 us, of which the launch
-// is still a part: M of twelve fields of 8^3 x 16 (1.2 M entries) 48.2 -> 45.0 us, A^dag A of six half vectors of
-// 12^3 x 24 (1.5 M) 115.5 -> 107.1 us. The line lies next above the sizes measured, far below the 19 M of
-// twelve fields of 16^3 x 32, where a launch is 3 % of a kernel and early blocks cost more.
-inline bool pdl_for_apply(long entries) { return entries <= 12L * 196608; }
+// The launches of one FP32 application, `entries` over all of the fields of a launch: two to four kernels in a row, where
+// the early launch hides the next one's start. us without -> with it, M / M by single-field kernels / A^dag A:
+//   8^3 x 16:  12 fields 48.4 -> 43.8 / 45.1 -> 42.6 / 69.4 -> 70.3; 48 fields 120.3 -> 115.2 / 113.2 -> 106.8 / 116.6 -> 107.3
+//   12^3 x 24:  6 fields 96.9 -> 94.1 / 89.3 -> 83.8 / 112.2 -> 105.1; 18 fields 210.2 -> 206.6 / 193.4 -> 187.3 / 247.2 -> 238.4
+//   16^3 x 32:  2 fields 93.5 -> 89.0 / 92.7 -> 88.2 / 172.5 -> 167.1; 12 fields 392.6 -> 390.2 / 377.3 -> 367.7 / 395.1 -> 385.2
+// The gain ends at the last (19 M entries): the line.
+inline bool pdl_for_apply(long entries) { return entries <= 12L * 1572864; }
 template <typename... P, typename... A>
 void launch_pdl(bool early, void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchAttribute at[1];

@@ -11,8 +11,8 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dims,n,multi", [((8, 8, 8, 16), 24, 1), ((8, 8, 8, 16), 25, 1), ((16, 16, 16, 12), 2, 0),
-                                          ((16, 16, 16, 14), 2, 0), ((16, 16, 16, 12), 5, 1), ((2, 2, 2, 2), 3, 1)])
+@pytest.mark.parametrize("dims,n,multi", [((8, 8, 8, 16), 192, 1), ((8, 8, 8, 16), 193, 1), ((16, 16, 16, 32), 12, 0),
+                                          ((16, 16, 16, 32), 13, 0), ((16, 16, 16, 12), 5, 1), ((2, 2, 2, 2), 3, 1)])
 def test_single_precision_applications(dims, n, multi):
     need_gpu()
     u = W.gauge_field(dims, 0.5, 81)
