@@ -3,17 +3,17 @@
 // GB300 executes FP64 at 1.6 lanes per clock and SM (a DFMA or DADD occupies an SM
 // partition for 68 clocks, measured), against 54 for a 32 x 32 + 64 bit integer
 // multiply-add.  A hop's 3 x 3 complex products are therefore formed exactly in
-// integers: a spinor becomes 24 fixed-point numbers relative to its largest
-// component's exponent E (55 fraction bits: one step is 2^-55 of a power of two at
+// integers: each half spinor of the projection becomes 12 fixed-point numbers relative to the exponent E of the
+// largest component that goes into it (55 fraction bits: one step is 2^-55 of a power of two at
 // most twice that component), a link is L = -kappa U 2^k with |L| <= 2^55 (prepared
 // once per handle, the antiperiodic sign included), both split into a 27-bit low and
 // a 29-bit high limb.  A product needs three 32 x 32 multiply-adds (high x high and the two
 // cross terms; low x low is below 2^-57 of the result), sums are exact, and the sums
-// of the eight hops are aligned to the largest E among the neighbours and added to the
-// diagonal term before the one rounding to FP64.  The error per site is at most a few
-// 2^-55 of the largest neighbour component: below that of the FP64 chain it replaces,
-// which rounds about 20 times per component (4^4 and 16^3 x 32, random spinors, against another
-// program's FP64: 1.4e-16 of the norm, most of it the reference's; the FP64 chain 1.9e-16).
+// of the eight hops are aligned to the largest E among them and added to the
+// diagonal term before the one rounding to FP64.  The error is at most a few 2^-55 of the largest
+// component among the spins that an output spin takes from the neighbours: below that of the FP64 chain it replaces,
+// which rounds about 20 times per component, on dense fields and for each spin.  A single colour far below its
+// spin's others counts against those.
 //
 // One block owns 32 sites and one warp one of the eight directions, so a link stays in
 // registers for all right-hand sides of the block; the eight warps meet in shared memory,
@@ -36,9 +36,9 @@ namespace seedcg {
 constexpr int kFixThreads = 256;
 constexpr int kFixEMin = 200, kFixEMax = 1900;   // biased exponents the fixed point accepts
 constexpr int kFixBad = 0x7fffffff;
-// two buffers of [8 directions][12 components][32 sites] 64-bit sums and [8][32] exponents, the
+// two buffers of [8 directions][12 components][32 sites] 64-bit sums and [2 spins][8][32] exponents, the
 // six planes' shares per buffer
-constexpr size_t kFixBufBytes = 8 * 12 * 32 * sizeof(long long) + 8 * 32 * sizeof(int);
+constexpr size_t kFixBufBytes = 8 * 12 * 32 * sizeof(long long) + 2 * 8 * 32 * sizeof(int);
 constexpr size_t kFixSmem = 2 * kFixBufBytes + 2 * 8 * sizeof(double);
 
 // x (a double with sign flipped where flip has bit 31) as two limbs x = (hi 2^27 + lo) 2^(E - 1022 - 55);
@@ -259,20 +259,27 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
                 p[6 + c] = at(3 * q0 + c);
                 p[9 + c] = at(3 * q1 + c);
             }
-            int mx = 0;
+            int ebits[2];   // each half spinor's own exponent: a spin far below the others keeps its digits
 #pragma unroll
-            for (int c = 0; c < 12; c++)
-                mx = max(mx, max(__double2hiint(p[c].x) & 0x7fffffff, __double2hiint(p[c].y) & 0x7fffffff));
-            int E = mx >> 20;
-            if (mx != 0 && (E < kFixEMin || E > kFixEMax)) E = kFixBad;
-            sE[warp * 32 + lane] = E;
-            // an all-zero spinor (E = 0) still needs an exponent that shifts its components out
-            const int eb = (E == kFixBad || E == 0 ? kFixEMax : E) << 20;
+            for (int v = 0; v < 2; v++) {
+                int mx = 0;
+#pragma unroll
+                for (int c = 3 * v; c < 3 * v + 3; c++) {
+                    mx = max(mx, max(__double2hiint(p[c].x) & 0x7fffffff, __double2hiint(p[c].y) & 0x7fffffff));
+                    mx = max(mx, max(__double2hiint(p[6 + c].x) & 0x7fffffff, __double2hiint(p[6 + c].y) & 0x7fffffff));
+                }
+                int E = mx >> 20;
+                if (mx != 0 && (E < kFixEMin || E > kFixEMax)) E = kFixBad;
+                sE[(v * 8 + warp) * 32 + lane] = E;
+                // all zero (E = 0) still needs an exponent that shifts the components out
+                ebits[v] = (E == kFixBad || E == 0 ? kFixEMax : E) << 20;
+            }
             int hh[6][2], hl[6][2], nh[6], nl[6];   // limbs of h (re, im) and of -im
 #pragma unroll
             for (int c = 0; c < 6; c++) {
                 const double2 w = p[6 + c];
                 const double wr = swap ? w.y : w.x, wi = swap ? w.x : w.y;
+                const int eb = ebits[c / 3];
                 int a, b, x, y;
                 fix_limbs(p[c].x, eb, 0u, a, b);
                 fix_limbs(wr, eb, c < 3 ? fr0 : fr1, x, y);
@@ -319,15 +326,26 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
         }
         rprev = r;
         if (warp < 6) {
-            int D[8], Em = 0;
+            // exponents of the half spinors that an output spin takes from the x, y and the z, t directions, the largest of
+            // them, and the others' distance from it
+            auto shifts = [&](int spin, int (&D)[8]) {
+                const int* xy = sE + (spin == 1 || spin == 2 ? 8 * 32 : 0) + lane;
+                const int* zt = sE + (spin & 1 ? 8 * 32 : 0) + lane;
+                int Em = 0;
 #pragma unroll
-            for (int d = 0; d < 8; d++) {
-                D[d] = sE[d * 32 + lane];
-                Em = max(Em, D[d]);
-            }
-            const bool bad = Em == kFixBad;
+                for (int d = 0; d < 8; d++) {
+                    D[d] = (d < 4 ? xy : zt)[d * 32];
+                    Em = max(Em, D[d]);
+                }
 #pragma unroll
-            for (int d = 0; d < 8; d++) D[d] = Em - D[d];
+                for (int d = 0; d < 8; d++) D[d] = Em - D[d];
+                return Em;
+            };
+            // the plane's two entries are of one spin, or (warps 1 and 4) of two
+            const int spin0 = 2 * warp / 3, spin1 = (2 * warp + 1) / 3;
+            int D[8];
+            const int E0 = shifts(spin0, D);
+            int E1 = E0;
             double2 pa = make_double2(0.0, 0.0), pb = pa;
             if (op.diag) {
                 const int si = op.same.half ? idx : s;
@@ -341,7 +359,21 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
                 const int h = __double2hiint(x) & 0x7fffffff;
                 return h != 0 && ((h >> 20) < kFixEMin || (h >> 20) > kFixEMax);
             };
-            if (bad || (op.diag && (far(pa.x) || far(pa.y) || far(pb.x) || far(pb.y)))) {
+            bool slow = E0 == kFixBad || (op.diag && (far(pa.x) || far(pa.y) || far(pb.x) || far(pb.y)));
+            long long x0 = 0, y0 = 0, x1 = 0, y1 = 0;
+            if (!slow) {
+                if (warp < 3) fix_gather<0>(R, D, 2 * warp, lane, x0, y0);
+                else if (warp == 3) fix_gather<2>(R, D, 0, lane, x0, y0);
+                else if (warp == 4) fix_gather<2>(R, D, 2, lane, x0, y0);
+                else fix_gather<3>(R, D, 1, lane, x0, y0);
+                if (spin1 != spin0) E1 = shifts(spin1, D);
+                if (warp < 3) fix_gather<0>(R, D, 2 * warp + 1, lane, x1, y1);
+                else if (warp == 3) fix_gather<2>(R, D, 1, lane, x1, y1);
+                else if (warp == 4) fix_gather<3>(R, D, 0, lane, x1, y1);
+                else fix_gather<3>(R, D, 2, lane, x1, y1);
+                slow = E1 == kFixBad;
+            }
+            if (slow) {
                 double2 c[12];
                 fix_chain(F, op.dag, s, op.in, r, c);
                 va = c[2 * warp];
@@ -350,22 +382,6 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
                 va = make_double2(pa.x + hs * va.x, pa.y + hs * va.y);
                 vb = make_double2(pb.x + hs * vb.x, pb.y + hs * vb.y);
             } else {
-                long long x0, y0, x1, y1;
-                if (warp < 3) {
-                    fix_gather<0>(R, D, 2 * warp, lane, x0, y0);
-                    fix_gather<0>(R, D, 2 * warp + 1, lane, x1, y1);
-                } else {
-                    if (warp == 3) {
-                        fix_gather<2>(R, D, 0, lane, x0, y0);
-                        fix_gather<2>(R, D, 1, lane, x1, y1);
-                    } else if (warp == 4) {
-                        fix_gather<2>(R, D, 2, lane, x0, y0);
-                        fix_gather<3>(R, D, 0, lane, x1, y1);
-                    } else {
-                        fix_gather<3>(R, D, 1, lane, x0, y0);
-                        fix_gather<3>(R, D, 2, lane, x1, y1);
-                    }
-                }
                 const bool neg = (op.hsgn < 0) != (op.dag && warp >= 3);
                 if (neg) {
                     x0 = -x0;
@@ -373,11 +389,11 @@ __device__ __forceinline__ void fix_tile(const FixDev& F, const FixOp& op, int t
                     x1 = -x1;
                     y1 = -y1;
                 }
-                const int Eh = Em + kFixUnit - F.k;
-                va.x = fix_combine(x0, Eh, op.diag, pa.x);
-                va.y = fix_combine(y0, Eh, op.diag, pa.y);
-                vb.x = fix_combine(x1, Eh, op.diag, pb.x);
-                vb.y = fix_combine(y1, Eh, op.diag, pb.y);
+                const int H0 = E0 + kFixUnit - F.k, H1 = E1 + kFixUnit - F.k;
+                va.x = fix_combine(x0, H0, op.diag, pa.x);
+                va.y = fix_combine(y0, H0, op.diag, pa.y);
+                vb.x = fix_combine(x1, H1, op.diag, pb.x);
+                vb.y = fix_combine(y1, H1, op.diag, pb.y);
             }
             const double part = epi(r, warp, idx, s, live, va, vb);
             if (Epi::kShare) {
