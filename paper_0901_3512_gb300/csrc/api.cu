@@ -54,7 +54,8 @@ KeptScratch::Use::~Use() {
     std::lock_guard<std::mutex> lk(kept().mu);
     s_.busy_ = false;
     size_t total = 0;
-    for (const KeptScratch* k : kept().all) total += k->buf_.bytes;
+    for (const KeptScratch* k : kept().all)
+        if (!k->busy_) total += k->buf_.bytes;   // one in use may be growing in its own thread, and counts when that ends
     if (total > kKeptBytes) s_.buf_.release();
 }
 bool give_back_scratch() {

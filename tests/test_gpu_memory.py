@@ -78,3 +78,40 @@ def test_create_without_room_for_the_fixed_point_links():
     finally:
         del hog
         torch.cuda.empty_cache()
+
+
+def test_threads_with_their_own_handles_keep_within_the_bound():
+    """Scratch that grows in one thread while another thread's call ends and counts what is kept."""
+    need_gpu()
+    import threading
+    handles = [_solver() for _ in range(3)]
+    x = torch.view_as_complex(torch.randn((288 << 20) // FIELD, 8 ** 4, 4, 3, 2, dtype=torch.float64, device="cuda"))
+    want = torch.empty_like(x)
+    handles[0].apply(seedcg.OP_M, x, want, prec=0, multi=1)
+    outs = [torch.empty_like(x) for _ in handles]
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    wrong = []
+
+    def work(s, y):
+        try:
+            for n in (1, 7, len(x), 3, len(x)):
+                y.zero_()
+                torch.cuda.synchronize()
+                s.apply(seedcg.OP_M, x[:n], y[:n], prec=0, multi=1)
+                if not torch.equal(y[:n], want[:n]):
+                    wrong.append(n)
+        except Exception as e:   # reported by the assertion below, in the test's own thread
+            wrong.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=a) for a in zip(handles, outs)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
+    torch.cuda.synchronize()
+    # 288 MB were kept before; 512 MB at most are now, and torch's own allocations for the comparisons
+    assert torch.cuda.mem_get_info()[0] >= free - (512 << 20)
+    for s in handles:
+        s.close()
