@@ -137,6 +137,9 @@ void seedcg_default_options(seedcg_options* opt);
  * point: 1440 bytes per site.  Where device memory has no room for the last 576, or the
  * links' largest components differ by more than a factor 2.5 (those of SU(3) links never
  * do), the FP64 operator runs in plain FP64 and takes 2.4 times as long.
+ * In fixed point its error is at most a few 2^-55 of the largest component among the spins of a
+ * site's neighbours that enter a spin of the result: in norm below that of plain FP64; a
+ * colour far below the others of its spin may keep fewer digits than there.
  * Returns SEEDCG_ERR_ARG for bad dims/pointers, SEEDCG_ERR_OOM/CUDA on
  * device failures; *h is NULL on failure.
  */
@@ -236,11 +239,12 @@ seedcg_status seedcg_eo_reconstruct(seedcg_handle* h, int n, const double* x_odd
  * counterpart: this is a property of the library, not of the method.)
  * Same arguments, layouts and results as seedcg_apply; in and out are the
  * caller's device buffers on the handle's GPU (host, pinned or unregistered
- * memory is refused with SEEDCG_ERR_ARG before any kernel runs).  The scratch (internal copies of in, the
- * intermediate and the output) is one fixed 16 MiB device array that every
+ * memory is refused with SEEDCG_ERR_ARG before any kernel runs).  The scratch (the field between the two
+ * operators of M, and for prec 1 the rounded input) is one fixed 16 MiB device array that every
  * GPU loading this library holds until the process exits; the call returns
  * SEEDCG_ERR_ARG, with a message, when 3 * n * V * 12 * (16 B for prec 0,
- * 8 B for prec 1) exceeds 16 MiB.  No device memory is allocated or freed.
+ * 8 B for prec 1) exceeds 16 MiB (more than the fields there take; the limit is part of
+ * the interface).  No device memory is allocated or freed.
  * The first call on a device looks up the array's device address
  * (cudaGetSymbolAddress, with that device current); make that first call
  * before any stream capture.  All calls share the one array and every call

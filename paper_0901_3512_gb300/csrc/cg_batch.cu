@@ -677,8 +677,8 @@ void launch_op(bool eo, int code, int tiles, cudaStream_t s, const GroupDev<R>* 
     }
 }
 
-std::string tune_key(const std::vector<CgGroup>& groups, bool fp64) {
-    std::string k = fp64 ? "mf_dslash f64" : "mf_dslash f32";
+std::string tune_key(const std::vector<CgGroup>& groups) {
+    std::string k = "mf_dslash f32";   // FP64 has nothing to tune
     if (!groups.empty() && groups[0].h->eo_active) k += " eo";
     k += " t32";   // the launch shapes: entries of caches written for other shapes are not read
     for (auto& g : groups) {
@@ -725,7 +725,7 @@ std::vector<std::pair<std::string, int>>& tune_table() {
 
 template <typename R>
 int autotune_rpb(const std::vector<CgGroup>& groups, int tiles, const GroupDev<R>* gdev, int ng, Rows rows, const CgS& C, cudaStream_t st) {
-    const std::string key = tune_key(groups, sizeof(R) == 8);
+    const std::string key = tune_key(groups);
     {
         std::lock_guard<std::mutex> lk(tune_mutex());
         for (auto& e : tune_table())

@@ -7,7 +7,7 @@ namespace seedcg {
 namespace {
 
 // Block (x, y): a chunk of entries against the rows of group y, like k_proj_partial: the chunk of X in shared memory
-// as limbs, a warp takes RPW rows at a time, a lane every 32nd entry.  A lane adds at most 32 entries (64
+// as limbs, a warp takes RPW rows at a time, a lane every 32nd entry.  A lane adds at most 16 entries (32
 // products of at most 2^56), so 64 bits hold its sums; the warp's sum is formed exactly from three 22-bit
 // parts.  RPW * NV * 2 values per warp are converted to FP64 side by side.  8^3 x 16, 320 rows on average, two
 // vectors: 570 us on the FP64 pipe, 160 us here (issue-bound; the rows take 75 us at the measured HBM rate); eleven

@@ -17,8 +17,8 @@
 //   B = the layer's weights in real form (64 x 64 bf16 per direction),
 //   D = 128 x 64 FP32 accumulators in TMEM, one per colour.
 // The backward pass through the data of layer 2 is the same GEMM with the
-// adjoint transport and the adjoint weights.  Layers 1 and 3 (one channel on one
-// side) and the weight gradients run on SIMT.
+// adjoint transport and the adjoint weights, and the weight gradients of all layers run on
+// tcgen05 too (k_g_tw).  Layers 1 and 3 (one channel on one side) run on SIMT.
 //
 // Activations are bf16x2 [C][V][12] (entry k = 3 spin + colour of site x at
 // (c V + x) 12 + k); weights of a layer are [9][CO][CI][4][4] complex, directions

@@ -1,6 +1,6 @@
 // seedcg_apply_noalloc: the operator application of seedcg_apply for callers
-// that cannot allocate device memory.  Its scratch (the internal-layout copies
-// of the input and of the intermediate / output fields) lives in one fixed
+// that cannot allocate device memory.  Its scratch (the field between the two
+// operators of M, and in FP32 the rounded input) lives in one fixed
 // file-scope device array instead of per-call cudaMalloc buffers.
 #include <cstring>
 #include <mutex>

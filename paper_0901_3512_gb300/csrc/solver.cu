@@ -39,12 +39,10 @@ inline int lz_blocks_per_sm(int sites) {
     return blocks <= 2 * 152 ? 2 : blocks <= 3 * 152 ? 3 : 7;
 }
 
-// blocks for a streaming pass that ends in one grid reduction: two per SM.  Every
-// block takes the reduction's atomic ticket, and thousands of tickets on one
-// counter cost more than the pass's loads (the 16^3x32 Lanczos update: 23 us at
-// 304 blocks against 35 us at 3072)
-// (those blocks are of 256 threads; vectors with less than a group per thread are spread over the SMs, and
-// their FP64 pipes, in smaller ones)
+// Threads per block of a streaming pass that ends in one grid reduction, whose grid is at most two blocks per SM: every
+// block takes the reduction's atomic ticket, and thousands of tickets on one counter cost more than the pass's
+// loads (the 16^3x32 Lanczos update: 23 us at 304 blocks of 256 threads against 35 us at 3072).  Vectors with less than a
+// 16-byte group per thread are spread over the SMs, and their FP64 pipes, in smaller blocks.
 inline int lean_threads(long n, int w) { return n / w <= 304 * 64 ? 64 : n / w <= 304 * 256 ? 128 : 256; }
 
 // ===========================================================================
@@ -429,22 +427,16 @@ k_lz_eta(const cx_t<R>* v, const cx_t<R>* r0, long n, int j0, int ne,
     });
 }
 
-// Steps 5-7 vector part: f -= alpha_i v_i; beta_i = ||f|| (final unless PO
-// follows).  LIT (the literal seeding of FP64 runs) also does, in R, steps 3 and
-// 6-7: w_i = (v_i - beta_{i-1} w_{i-1}) / delta_i, x^1 += zeta_i w_i, x^j += eta^j w_i.
-template <typename R, bool LIT>
+// Steps 5-7 vector part of the literal seeding (FP64 runs): f -= alpha_i v_i; beta_i = ||f|| (final unless PO
+// follows), and, in R, steps 3 and 6-7: w_i = (v_i - beta_{i-1} w_{i-1}) / delta_i, x^1 += zeta_i w_i, x^j += eta^j w_i.
+template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
 k_lz_update(const cx_t<R>* v, cx_t<R>* f, cx_t<R>* w,
             cx_t<R>* X, int nrhs, long n, int i, int final_beta, LzDev L) {
     pdl_enter();
     if (i > L.ctl->m) return;
     const R a = (R)L.alpha[i - 1];
-    R dl = 0, bp = 0, zt = 0;
-    if (LIT) {
-        dl = (R)L.delta[i - 1];
-        bp = i > 1 ? (R)L.beta[i - 2] : R(0);
-        zt = (R)L.zeta[i - 1];
-    }
+    const R dl = (R)L.delta[i - 1], bp = i > 1 ? (R)L.beta[i - 2] : R(0), zt = (R)L.zeta[i - 1];
     R part = 0;
     for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n;
          e += (long)gridDim.x * blockDim.x) {
@@ -453,21 +445,19 @@ k_lz_update(const cx_t<R>* v, cx_t<R>* f, cx_t<R>* w,
         fv.y -= a * vv.y;
         f[e] = fv;
         part += fv.x * fv.x + fv.y * fv.y;
-        if (LIT) {
-            cx_t<R> ww = i > 1 ? w[e] : mk<R>(0, 0);
-            ww.x = (vv.x - bp * ww.x) / dl;
-            ww.y = (vv.y - bp * ww.y) / dl;
-            w[e] = ww;
-            cx_t<R> x1 = X[e];
-            x1.x += zt * ww.x;
-            x1.y += zt * ww.y;
-            X[e] = x1;
-            for (int j = 1; j < nrhs; j++) {
-                double2 et = L.eta[j - 1];
-                cx_t<R> xj = X[(size_t)j * n + e];
-                xj = cfma(mk<R>((R)et.x, (R)et.y), ww, xj);
-                X[(size_t)j * n + e] = xj;
-            }
+        cx_t<R> ww = i > 1 ? w[e] : mk<R>(0, 0);
+        ww.x = (vv.x - bp * ww.x) / dl;
+        ww.y = (vv.y - bp * ww.y) / dl;
+        w[e] = ww;
+        cx_t<R> x1 = X[e];
+        x1.x += zt * ww.x;
+        x1.y += zt * ww.y;
+        X[e] = x1;
+        for (int j = 1; j < nrhs; j++) {
+            double2 et = L.eta[j - 1];
+            cx_t<R> xj = X[(size_t)j * n + e];
+            xj = cfma(mk<R>((R)et.x, (R)et.y), ww, xj);
+            X[(size_t)j * n + e] = xj;
         }
     }
     double red[1] = {(double)part};
@@ -1288,7 +1278,7 @@ seedcg_status run_solve(seedcg_handle* h, int nrhs, const double2* B64, double2*
                 }
             }
             if (literal)
-                launch_pdl(pdl, k_lz_update<R, true>, rb, kRedThreads, 0, st, 
+                launch_pdl(pdl, k_lz_update<R>, rb, kRedThreads, 0, st, 
                     v, fv, wv, reinterpret_cast<cx_t<R>*>(X64), nrhs, n, i, po_now ? 0 : 1, L);
             else
                 launch_pdl(pdl, k_lz_update_v<R>, lean, lean_t, 0, st, v, fv, wv, X64, n, i, po_now ? 0 : 1, L);
