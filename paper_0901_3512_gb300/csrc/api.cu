@@ -4,6 +4,7 @@
 // message kept in the handle.
 #include <algorithm>
 #include <cstring>
+#include <exception>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -37,7 +38,7 @@ KeptScratch::~KeptScratch() {
     a.erase(std::find(a.begin(), a.end(), this));
     buf_.release();
 }
-KeptScratch::Use::Use(KeptScratch& s, size_t bytes) : s_(s) {
+KeptScratch::Use::Use(KeptScratch& s, size_t bytes) : s_(s), exceptions_(std::uncaught_exceptions()) {
     {
         std::lock_guard<std::mutex> lk(kept().mu);
         s_.busy_ = true;
@@ -56,7 +57,8 @@ KeptScratch::Use::~Use() {
     size_t total = 0;
     for (const KeptScratch* k : kept().all)
         if (!k->busy_) total += k->buf_.bytes;   // one in use may be growing in its own thread, and counts when that ends
-    if (total > kKeptBytes) s_.buf_.release();
+    // a call that failed may have left work running on its stream: cudaFree waits for it
+    if (total > kKeptBytes || std::uncaught_exceptions() > exceptions_) s_.buf_.release();
 }
 bool give_back_scratch() {
     std::lock_guard<std::mutex> lk(kept().mu);

@@ -241,6 +241,7 @@ public:
     KeptScratch& operator=(const KeptScratch&) = delete;
     class Use {   // the scratch for one call, which ends with its device work
         KeptScratch& s_;
+        int exceptions_;   // in flight when the call began
 
     public:
         Use(KeptScratch& s, size_t bytes);
