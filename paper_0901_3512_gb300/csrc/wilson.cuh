@@ -302,11 +302,11 @@ template <typename N> __device__ __forceinline__ auto hop_index(const N& n, int 
 // wilson_site with DEPTH neighbours in flight, for the FP32 kernels with one thread per site: two where the lattice
 // fills the chip (the Lanczos D at 16^3 x 32: 19.3 -> 16.4 us; in FP64 the second spinor's registers cost more than
 // they give), four on small lattices, where a thread may have the registers.
+// wilson_hops_ahead adds the hops to what `out` holds.
 template <int DAG, int DEPTH, typename LoadNbr, typename Fwd, typename Bwd>
-__device__ __forceinline__ void wilson_site_ahead(const Nbr& n, int s, LoadNbr load, Fwd fl, Bwd bl, float kappa,
+__device__ __forceinline__ void wilson_hops_ahead(const Nbr& n, LoadNbr load, Fwd fl, Bwd bl, float kappa,
                                                   Spinor<float>& out) {
     constexpr int SF = DAG ? 1 : -1;
-    load(s, out);
     hops_in_flight<DEPTH, float>(
         [&](int k) { return hop_index(n, k); }, load, [&](auto kk, const Spinor<float>& nb) {
             constexpr int K = decltype(kk)::value, MU = K >> 1, BACK = K & 1;
@@ -317,6 +317,13 @@ __device__ __forceinline__ void wilson_site_ahead(const Nbr& n, int s, LoadNbr l
                 hop<MU, SF, false>(out, nb, [&](int a, int b) { return fl(MU, 3 * a + b); },
                                    MU == 3 && n.fwrap_t ? kappa : -kappa);
         });
+}
+
+template <int DAG, int DEPTH, typename LoadNbr, typename Fwd, typename Bwd>
+__device__ __forceinline__ void wilson_site_ahead(const Nbr& n, int s, LoadNbr load, Fwd fl, Bwd bl, float kappa,
+                                                  Spinor<float>& out) {
+    load(s, out);
+    wilson_hops_ahead<DAG, DEPTH>(n, load, fl, bl, kappa, out);
 }
 
 // Same, with links that already carry the coefficient and the boundary sign (staged that way by the
