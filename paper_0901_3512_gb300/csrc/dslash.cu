@@ -67,8 +67,11 @@ __global__ void k_to_internal_f32(const double2* in, float2* __restrict__ out,
     int r = (int)(t / vol), s = (int)(t % vol);
     const double2* src = in + ((size_t)r * vol + s) * 12;
     float2* dst = out + (size_t)r * 12 * vol;
+    double2 z[12];
 #pragma unroll
-    for (int k = 0; k < 12; k++) dst[sidx(k, s, vol)] = make_float2((float)src[k].x, (float)src[k].y);
+    for (int k = 0; k < 12; k++) z[k] = src[k];
+#pragma unroll
+    for (int k = 0; k < 12; k++) dst[sidx(k, s, vol)] = make_float2((float)z[k].x, (float)z[k].y);
 }
 
 __global__ void k_gauge_to_internal(const double2* __restrict__ in, double2* __restrict__ u64,

@@ -65,8 +65,8 @@ struct FixStore {
 
 // At most 128 registers: two blocks per SM.  Instruction issue bounds it: 1270 warp instructions per
 // 32 sites, direction and field, 216 of them multiply-adds of 32 x 32 + 64 bits and 380 the conversion of the
-// neighbour.  16^3 x 32, 12 fields: 900 us between internal fields, issue 44 % busy at 16 warps per SM, DRAM
-// 12 %; 1037 us from and to the boundary's spinors, where two layout passes took another 303 us.
+// neighbour.  16^3 x 32, 12 fields: 898 us between internal fields; 996 us from and to the boundary's spinors, issue 40 %
+// busy at 16 warps per SM, DRAM 12 %, where two layout passes took another 303 us.
 __global__ void __launch_bounds__(kFixThreads, 2) k_fix_apply(FixDev F, FixOp op, FixStore st, int n) {
     extern __shared__ __align__(16) unsigned char fix_smem[];
     if (!F.ok) {
